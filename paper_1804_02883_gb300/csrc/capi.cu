@@ -17,7 +17,6 @@
 
 namespace epdlb {
 
-cudaError_t configure_prop_kernels();
 cudaError_t configure_epd_kernels();
 
 cudaError_t configure_kernels()
@@ -25,8 +24,7 @@ cudaError_t configure_kernels()
     // once per process (a function-local static is initialised exactly once,
     // also when handles are created on several threads)
     static const cudaError_t status = [] {
-        cudaError_t e = configure_prop_kernels();
-        if (e == cudaSuccess) e = configure_epd_kernels();
+        cudaError_t e = configure_epd_kernels();
         if (e == cudaSuccess) e = configure_step3d_kernels();
         return e;
     }();
@@ -187,6 +185,67 @@ static int radix_plan(int n, int *f)
     return k;
 }
 
+// Radices of the in-place transforms (fftg.cuh) of an even length 2^a 3^b 5^c:
+// the first from {2, 4, 6, 8, 10, 12, 16}, the last from {1, 2, 3, 4, 5, 8, 9,
+// 10, 15, 16}, {3, 4, 5, 8, 9} between (every such length to 2048 has a plan
+// of at most four).  Cost per plan: instructions per point of each radix, the
+// twiddles and shared-memory trip of each pass, a shorter contiguous run of
+// the first pass's legs (0.5 r_0), and w times the largest radix, the serial
+// instructions of one thread.  Large radices save passes where every SM has
+// warps to spare; on small grids (few points per SM) and in FP64 (few warps
+// hide each other's latency at 2 FP64 lanes per SM) the thread's own chain is
+// the time, so w grows there.  Measured: FP64 64 x 64 (N_s = 32), 10 steps:
+// 4.4.4 8.7 ms, 8.8 12.4, 4.16 16.3; FP64 4 x 256 x 512: 256 as 4.8.8 15.6 ms,
+// as 16.16 16.1 (one batch alone 17.9 and 22.2); FP64 64 x 128 x 128 box: 128
+// as 8.16 16.1 ms, as 4.4.8 16.7; FP32 128 x 128: 4.4.8 0.76 ms, 8.16 0.84;
+// FP32 48 x 90 x 96 box: 96 as 6.16 0.80 ms, as 12.8 1.04; FP32 64 x 150 x
+// 150: 10.15 14.3 ms, 6.5.5 18.5.  The choice depends on one run's grid only, so a run's
+// results do not depend on the batch it is in.
+LinePlan line_plan(int n, long long sites, bool fp64)
+{
+    static const int first[] = {2, 4, 6, 8, 10, 12, 16}, inner[] = {3, 4, 5, 8, 9}, last[] = {1, 2, 3, 4, 5, 8, 9, 10, 15, 16};
+    const double w = fp64 ? (sites <= (1 << 15) ? 2.0 : (sites < (1 << 20) ? 1.0 : 0.3)) : (sites <= (1 << 14) ? 1.0 : 0.3);
+    auto cost = [](int r) {
+        static const double c[17] = {0, 0, 2, 4, 4, 7.2, 6, 0, 6.5, 9.8, 9.2, 0, 8, 0, 0, 11.2, 10};
+        return c[r] + 8.0;
+    };
+    LinePlan best = {0, 0};
+    double least = 1e30;
+    int r[4];
+    auto close = [&](int rest, int nf, double c) {  // rest as the last radix
+        for (int v : last)
+            if (v == rest) {
+                int mx = v;
+                for (int i = 0; i < nf; ++i) mx = std::max(mx, r[i]);
+                c += cost(v) + w * mx + 0.5 * r[0];
+                if (c >= least) return;
+                least = c;
+                best.w = 0;
+                r[nf] = v;
+                best.nf = nf + 1;
+                for (int i = 0; i <= nf; ++i) best.w |= (unsigned long long)r[i] << (8 * i);
+            }
+    };
+    for (int r0 : first) {
+        if (n % r0 || (r0 == 2 && n % 4 == 0)) continue;
+        r[0] = r0;
+        const int n1 = n / r0;
+        close(n1, 1, cost(r0));
+        for (int a : inner) {
+            if (n1 % a) continue;
+            r[1] = a;
+            const int n2 = n1 / a;
+            close(n2, 2, cost(r0) + cost(a));
+            for (int b : inner) {
+                if (n2 % b) continue;
+                r[2] = b;
+                close(n2 / b, 3, cost(r0) + cost(a) + cost(b));
+            }
+        }
+    }
+    return best;
+}
+
 // Largest divisor of n not above cap (at least 1).
 static int divisor_at_most(int n, int cap)
 {
@@ -213,6 +272,9 @@ static void fill_geom(Group &G)
     g.logy = g.pow2 ? ilog2(p.ny) : 0;
     g.nfx = radix_plan(p.nx, g.fx);
     g.nfy = radix_plan(p.ny, g.fy);
+    const bool fp64 = p.precision == EPD_LB_PLAIN_FP64;
+    g.px = line_plan(p.nx, (long long)p.nx * p.ny, fp64);
+    g.py = line_plan(p.ny, (long long)p.nx * p.ny, fp64);
     g.ns = p.ns;
     g.na = (int)std::lround(p.f_a * (double)p.ns);
     g.jr = p.junction_rule;
@@ -244,14 +306,9 @@ static void fill_geom(Group &G)
 static void default_shapes(Group &G)
 {
     const int nx = G.g.nx, ny = G.g.ny;
-    const bool f32 = G.prec == EPD_LB_MIXED_FP32;
-    G.sh.rows_prop = std::max(1, std::min(ny, 2048 / nx));
-    G.sh.cols_prop = std::min(nx, std::max(f32 ? 4 : 2, 2048 / ny));
     G.sh.rows_epd = std::max(1, std::min(ny, 2048 / nx));
     G.sh.cols_epd = std::min(nx, std::max(2, 2048 / ny));
     if (!G.g.pow2) {  // tiles must divide the axes
-        G.sh.rows_prop = divisor_at_most(ny, G.sh.rows_prop);
-        G.sh.cols_prop = divisor_at_most(nx, G.sh.cols_prop);
         G.sh.rows_epd = divisor_at_most(ny, G.sh.rows_epd);
         G.sh.cols_epd = divisor_at_most(nx, G.sh.cols_epd);
     }
@@ -1334,13 +1391,14 @@ static size_t solve3_layout(const epd_lb_params *p, int nz, Solve3 &S, char *bas
     S.vz.pow2 = pow2(nxy) && pow2(nz);
     S.vz.logx = S.vz.pow2 ? ilog2(nxy) : 0;
     S.vz.logy = S.vz.pow2 ? ilog2(nz) : 0;
-    S.vz.nfy = radix_plan(nz, S.vz.fy);
-    S.rows_x = divisor_at_most(nyz, std::max(1, 2048 / nx));
-    S.cols_y = divisor_at_most(nx, std::max(2, 2048 / ny));
-    S.cols_z = divisor_at_most(nxy, std::max(2, 2048 / nz));
-    if (nyz / S.rows_x > kMaxPart / 2) return 0;  // Q partials of the row pass
+    const bool fp64 = p->precision == EPD_LB_PLAIN_FP64;
+    S.vx.px = line_plan(nx, n3, fp64);
+    S.vy.py = line_plan(ny, n3, fp64);
+    S.vz.py = line_plan(nz, n3, fp64);
+    // the boxes this entry point takes: at most kMaxPart / 2 tiles of whole
+    // rows of at most 2048 sites (Q partials)
+    if (nyz / divisor_at_most(nyz, std::max(1, 2048 / nx)) > kMaxPart / 2) return 0;
     S.prec = p->precision;
-    if (solve3d_smem_max(S) > 200 * 1024) return 0;
     const size_t tb = p->precision == EPD_LB_MIXED_FP32 ? sizeof(float) : sizeof(double);
     size_t off = 0;
     auto take = [&](size_t bytes) -> void * {

@@ -16,8 +16,18 @@ namespace epdlb {
 // Parameters every kernel of a group needs, by value.
 constexpr int kMaxFactors = 16;  // radices of one axis (mixed-radix transforms)
 
+// Radices of one axis for the in-place transforms of fftg.cuh: nf of them,
+// radix i in byte i.
+struct LinePlan {
+    unsigned long long w;
+    int nf;
+    __host__ __device__ int r(int i) const { return (int)((w >> (8 * i)) & 255u); }
+};
+LinePlan line_plan(int n, long long sites, bool fp64);  // of a length on a grid of `sites` sites (capi.cu)
+
 struct GroupGeom {
     int nx, ny, logx, logy;  // logx, logy: 0 unless both axes are powers of two
+    LinePlan px, py;         // radices of each axis' in-place transforms
     int pow2;                // both axes powers of two; else the mixed-radix radix-2-family passes
     int nfx, nfy;            // radix plans (4, 2, 3, 5) of each axis for the mixed-radix transforms
     int fx[kMaxFactors], fy[kMaxFactors];
@@ -52,8 +62,7 @@ __host__ __device__ inline int half_step_block(int jr, int chain, int m, int ns,
 
 // Launch shapes of the transform passes (chosen at init, see tune_shapes).
 struct Shapes {
-    int rows_prop, cols_prop;  // rows per CTA of the propagator row pass, columns per CTA of its column pass
-    int rows_epd, cols_epd;    // the same for the FP64 EPD/force passes
+    int rows_epd, cols_epd;  // rows per CTA of the EPD/force row passes, columns per CTA of the column passes
 };
 
 // One batch of runs with identical grid, contour and model parameters.
@@ -224,7 +233,6 @@ cudaError_t launch_selftest_wait(int *err, long long limit_cycles, cudaStream_t 
 // rows) carrying the node factors, history and contour sums.
 struct Solve3 {
     GroupGeom vx, vy, vz;        // the three views (vx holds the chain geometry)
-    int rows_x, cols_y, cols_z;  // tiles of the x-row, y-column and z-column passes
     void *chain, *hist, *efac;   // bulk precision: [n3] complex, [half_lo + 1][n3] complex, [n3] complex
     double *ia, *ib, *part;
     void *twx, *twy, *twz, *kx, *ky, *kz;  // bulk precision tables (full twiddle tables)
@@ -232,7 +240,6 @@ struct Solve3 {
     int prec;
 };
 cudaError_t launch_solve3d(const Solve3 &S, const double *omega, double *phi, double *q, cudaStream_t s);
-size_t solve3d_smem_max(const Solve3 &S);  // largest dynamic shared memory of the three passes
 // One axis of the FP64 3D transforms of the coupled 3D step.
 struct Axis3 {
     int n, pow2, logn, nf;

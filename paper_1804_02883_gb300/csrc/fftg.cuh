@@ -1,0 +1,445 @@
+// fftg.cuh -- in-place transforms of any length 2^a 3^b 5^c in shared memory
+// (FP32 and FP64), for the passes that run on every grid.
+//
+// A sequence of N points is transformed with decimation in frequency over the
+// radices r_0, r_1, .., r_last of its plan: the butterfly of pass i reads and
+// writes the same R points, M_i = N / (r_0 .. r_i) apart, so a pass needs one
+// buffer and one barrier, and the spectrum ends in digit-reversed order.  A
+// spectral operator acts on it there, by the natural bin of each position
+// (line_bin), and the inverse runs the passes backwards (decimation in time),
+// so the order never has to be restored.  The last forward pass, the operator
+// and the first inverse pass are one: a length up to 256 is two radices, three
+// trips through shared memory for a whole transform pair.
+//
+// Radices up to 16: a pass costs the tile one trip through shared memory and
+// one twiddle per point whatever its radix, so few large ones win (150 = 10 x
+// 15).  Butterflies of coprime factors (6, 10, 12, 15) are prime-factor
+// transforms (Good 1958, Thomas 1963) without inner twiddles.
+//
+// The first forward pass takes its points from global memory and the last
+// inverse pass hands its points to the caller's epilogue, both templated on
+// the plan's first radix; the passes between are called by radix.
+#pragma once
+
+#include "common.cuh"
+#include "engine.h"
+
+namespace epdlb {
+
+// (x, y) -> i (x, y) times the direction's sign: forward -i, inverse +i
+template <bool INV, typename V> __device__ __forceinline__ V mul_i(V a)
+{
+    V r;
+    r.x = INV ? -a.y : a.y;
+    r.y = INV ? a.x : -a.x;
+    return r;
+}
+
+// a conj(b)
+template <typename V> __device__ __forceinline__ V cmul_conj(V a, V b)
+{
+    V r;
+    r.x = a.x * b.x + a.y * b.y;
+    r.y = a.y * b.x - a.x * b.y;
+    return r;
+}
+
+// DFT of R points in registers, natural order in and out.
+template <typename T, int R, bool INV> struct DftN;
+
+template <typename T, bool INV> struct DftN<T, 1, INV> {
+    static __device__ __forceinline__ void run(V2<T> *) {}
+};
+template <typename T, bool INV> struct DftN<T, 2, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        const V2<T> a = x[0], b = x[1];
+        x[0] = cadd(a, b);
+        x[1] = csub(a, b);
+    }
+};
+template <typename T, bool INV> struct DftN<T, 3, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        const T h = (T)0.86602540378443864676;  // sin(2 pi / 3)
+        const V2<T> s = cadd(x[1], x[2]), d = mul_i<INV>(csub(x[1], x[2]));
+        const V2<T> m = mk<T>(x[0].x - (T)0.5 * s.x, x[0].y - (T)0.5 * s.y);
+        x[0] = cadd(x[0], s);
+        x[1] = mk<T>(m.x + h * d.x, m.y + h * d.y);
+        x[2] = mk<T>(m.x - h * d.x, m.y - h * d.y);
+    }
+};
+template <typename T, bool INV> struct DftN<T, 4, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        const V2<T> s02 = cadd(x[0], x[2]), d02 = csub(x[0], x[2]);
+        const V2<T> s13 = cadd(x[1], x[3]), d13 = mul_i<INV>(csub(x[1], x[3]));
+        x[0] = cadd(s02, s13);
+        x[2] = csub(s02, s13);
+        x[1] = cadd(d02, d13);
+        x[3] = csub(d02, d13);
+    }
+};
+template <typename T, bool INV> struct DftN<T, 5, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        const T c1 = (T)0.30901699437494742410, c2 = (T)-0.80901699437494742410;  // cos(2 pi / 5), cos(4 pi / 5)
+        const T s1 = (T)0.95105651629515357212, s2 = (T)0.58778525229247312917;   // sin(2 pi / 5), sin(4 pi / 5)
+        const V2<T> a1 = cadd(x[1], x[4]), a2 = cadd(x[2], x[3]);
+        const V2<T> b1 = mul_i<INV>(csub(x[1], x[4])), b2 = mul_i<INV>(csub(x[2], x[3]));
+        const V2<T> m1 = mk<T>(x[0].x + c1 * a1.x + c2 * a2.x, x[0].y + c1 * a1.y + c2 * a2.y);
+        const V2<T> m2 = mk<T>(x[0].x + c2 * a1.x + c1 * a2.x, x[0].y + c2 * a1.y + c1 * a2.y);
+        const V2<T> n1 = mk<T>(s1 * b1.x + s2 * b2.x, s1 * b1.y + s2 * b2.y);
+        const V2<T> n2 = mk<T>(s2 * b1.x - s1 * b2.x, s2 * b1.y - s1 * b2.y);
+        x[0] = cadd(x[0], cadd(a1, a2));
+        x[1] = cadd(m1, n1);
+        x[4] = csub(m1, n1);
+        x[2] = cadd(m2, n2);
+        x[3] = csub(m2, n2);
+    }
+};
+template <typename T, bool INV> struct DftN<T, 8, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        V2<T> e[4] = {x[0], x[2], x[4], x[6]}, o[4] = {x[1], x[3], x[5], x[7]};
+        DftN<T, 4, INV>::run(e);
+        DftN<T, 4, INV>::run(o);
+        const T h = (T)0.70710678118654752440;
+        // W8 o_1 = h (o_1 + (-+i) o_1), W8^3 o_3 = h ((-+i) o_3 - o_3): the
+        // factor h goes into the sums
+        const V2<T> o1 = cadd(o[1], mul_i<INV>(o[1])), o2 = mul_i<INV>(o[2]), o3 = csub(mul_i<INV>(o[3]), o[3]);
+        x[0] = cadd(e[0], o[0]);
+        x[4] = csub(e[0], o[0]);
+        x[1] = mk<T>(e[1].x + h * o1.x, e[1].y + h * o1.y);
+        x[5] = mk<T>(e[1].x - h * o1.x, e[1].y - h * o1.y);
+        x[2] = cadd(e[2], o2);
+        x[6] = csub(e[2], o2);
+        x[3] = mk<T>(e[3].x + h * o3.x, e[3].y + h * o3.y);
+        x[7] = mk<T>(e[3].x - h * o3.x, e[3].y - h * o3.y);
+    }
+};
+// x times exp(-+2 pi i / n) given its cosine and sine
+template <typename T, bool INV> __device__ __forceinline__ V2<T> rot(V2<T> v, T c, T s)
+{
+    if (!INV) s = -s;
+    return mk<T>(v.x * c - v.y * s, v.x * s + v.y * c);
+}
+// 9 = 3 x 3 and 16 = 4 x 4: X[k1 + P k2] = DFT over n2 of W^(n2 k1) DFT over n1 of x[P n1 + n2]
+template <typename T, bool INV> struct DftN<T, 9, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        const T c1 = (T)0.76604444311897803520, s1 = (T)0.64278760968653932632;   // 2 pi / 9
+        const T c2 = (T)0.17364817766693034885, s2 = (T)0.98480775301220805937;   // 4 pi / 9
+        const T c4 = (T)-0.93969262078590838405, s4 = (T)0.34202014332566873304;  // 8 pi / 9
+        V2<T> y[3][3];
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) {
+            y[n2][0] = x[n2];
+            y[n2][1] = x[3 + n2];
+            y[n2][2] = x[6 + n2];
+            DftN<T, 3, INV>::run(y[n2]);
+        }
+        y[1][1] = rot<T, INV>(y[1][1], c1, s1);
+        y[1][2] = rot<T, INV>(y[1][2], c2, s2);
+        y[2][1] = rot<T, INV>(y[2][1], c2, s2);
+        y[2][2] = rot<T, INV>(y[2][2], c4, s4);
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) {
+            V2<T> v[3] = {y[0][k1], y[1][k1], y[2][k1]};
+            DftN<T, 3, INV>::run(v);
+#pragma unroll
+            for (int k2 = 0; k2 < 3; ++k2) x[k1 + 3 * k2] = v[k2];
+        }
+    }
+};
+template <typename T, bool INV> struct DftN<T, 16, INV> {
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        const T c = (T)0.92387953251128675613, s = (T)0.38268343236508977173, h = (T)0.70710678118654752440;
+        V2<T> y[4][4];
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+            y[n2][0] = x[n2];
+            y[n2][1] = x[4 + n2];
+            y[n2][2] = x[8 + n2];
+            y[n2][3] = x[12 + n2];
+            DftN<T, 4, INV>::run(y[n2]);
+        }
+        auto w2 = [&](V2<T> v) { return cscale(cadd(v, mul_i<INV>(v)), h); };   // exp(-+2 pi i 2 / 16)
+        auto w6 = [&](V2<T> v) { return cscale(csub(mul_i<INV>(v), v), h); };   // exp(-+2 pi i 6 / 16)
+        y[1][1] = rot<T, INV>(y[1][1], c, s);
+        y[1][2] = w2(y[1][2]);
+        y[1][3] = rot<T, INV>(y[1][3], s, c);
+        y[2][1] = w2(y[2][1]);
+        y[2][2] = mul_i<INV>(y[2][2]);
+        y[2][3] = w6(y[2][3]);
+        y[3][1] = rot<T, INV>(y[3][1], s, c);
+        y[3][2] = w6(y[3][2]);
+        y[3][3] = rot<T, INV>(y[3][3], -c, -s);
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            V2<T> v[4] = {y[0][k1], y[1][k1], y[2][k1], y[3][k1]};
+            DftN<T, 4, INV>::run(v);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) x[k1 + 4 * k2] = v[k2];
+        }
+    }
+};
+// Prime-factor transform of A B points, gcd(A, B) = 1: input n = B n1 + A n2
+// (mod AB), output the k with k = k1 (mod A), k = k2 (mod B).
+template <typename T, int A, int B, bool INV> struct DftPf {
+    static constexpr int out(int k1, int k2)
+    {
+        for (int k = 0; k < A * B; ++k)
+            if (k % A == k1 && k % B == k2) return k;
+        return 0;
+    }
+    static __device__ __forceinline__ void run(V2<T> *x)
+    {
+        V2<T> y[B][A];
+#pragma unroll
+        for (int n2 = 0; n2 < B; ++n2) {
+#pragma unroll
+            for (int n1 = 0; n1 < A; ++n1) y[n2][n1] = x[(B * n1 + A * n2) % (A * B)];
+            DftN<T, A, INV>::run(y[n2]);
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            V2<T> v[B];
+#pragma unroll
+            for (int n2 = 0; n2 < B; ++n2) v[n2] = y[n2][k1];
+            DftN<T, B, INV>::run(v);
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) x[out(k1, k2)] = v[k2];
+        }
+    }
+};
+template <typename T, bool INV> struct DftN<T, 6, INV> : DftPf<T, 2, 3, INV> {};
+template <typename T, bool INV> struct DftN<T, 10, INV> : DftPf<T, 2, 5, INV> {};
+template <typename T, bool INV> struct DftN<T, 12, INV> : DftPf<T, 3, 4, INV> {};
+template <typename T, bool INV> struct DftN<T, 15, INV> : DftPf<T, 3, 5, INV> {};
+
+// Tile of B = 2^logb sequences of n points: point p of sequence b at
+// (p + pad (p / rl)) bp + b, rl the plan's last radix, pad = 1 where it is
+// even.  Every pass but the middle one has legs a multiple of rl apart, so
+// the pad only changes their constant distance, and the middle one's blocks
+// start an odd number of points apart.  Columns: bp = B, consecutive threads
+// on consecutive sequences; rows: bp odd, and consecutive threads on
+// consecutive points (the global order) where the legs are far enough apart.
+// No access then meets the same bank more than twice.
+struct LineTile {
+    int n, logb, bp, rl, pad;
+    bool row;
+    __host__ __device__ LineTile(bool row_, int n_, int logb_, LinePlan pl)
+        : n(n_), logb(logb_), bp(row_ ? (1 << logb_) | 1 : 1 << logb_), rl(pl.r(pl.nf - 1)), pad(rl % 2 ? 0 : 1), row(row_)
+    {
+    }
+    __host__ __device__ size_t points() const { return (size_t)(n + pad * (n / rl)) * bp; }
+    // distance of points M apart (M a multiple of rl)
+    __device__ int leg(int M) const { return (M + pad * (M / rl)) * bp; }
+};
+// sequence b and butterfly t of butterfly number bf (dq.d per sequence)
+__device__ __forceinline__ void line_split(const LineTile &tl, bool bfast, const FastDiv &dq, int bf, int &b, int &t)
+{
+    if (bfast) {
+        b = bf & ((1 << tl.logb) - 1);
+        t = bf >> tl.logb;
+    } else {
+        b = dq.div(bf);
+        t = bf - b * dq.d;
+    }
+}
+
+// Natural bin of position p of a spectrum in the plan's digit-reversed order.
+__device__ __forceinline__ int line_bin(LinePlan pl, int n, int p)
+{
+    int m = n, s = 1, k = 0;
+    for (int i = 0; i < pl.nf; ++i) {
+        m /= pl.r(i);
+        const int v = p / m;
+        p -= v * m;
+        k += s * v;
+        s *= pl.r(i);
+    }
+    return k;
+}
+
+// Twiddles of a butterfly, w[u] = tw[u j] (tw[i] = exp(-2 pi i i / n)), read
+// before its points: with few warps per SM the reads' latency is exposed, and
+// taken one by one next to their uses it cost the FP64 passes 40%.
+template <int R, typename V> __device__ __forceinline__ void line_twiddles(V (&w)[R], const V *__restrict__ tw, int j)
+{
+#pragma unroll
+    for (int u = 1; u < R; ++u) w[u] = __ldg(&tw[u * j]);
+}
+
+// One pass: radix R, M = points between the legs of a butterfly, S = product
+// of the radices before it; tw[i] = exp(-2 pi i i / n).
+template <typename T, int R, bool INV>
+__device__ __forceinline__ void line_pass(V2<T> *buf, LineTile tl, int M, int S, const V2<T> *__restrict__ tw)
+{
+    const int q = tl.n / R, total = q << tl.logb, leg = tl.leg(M);
+    const FastDiv dq(q), dm(M), dl(tl.rl);
+    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+        int b, t;
+        line_split(tl, !tl.row || M < 8, dq, bf, b, t);
+        const int blk = dm.div(t), j = t - blk * M;
+        V2<T> *p = buf + (j + (tl.pad ? dl.div(j) : 0)) * tl.bp + blk * R * leg + b;
+        V2<T> x[R], w[R];
+        line_twiddles(w, tw, j * S);
+#pragma unroll
+        for (int u = 0; u < R; ++u) x[u] = p[u * leg];
+        if (INV) {
+#pragma unroll
+            for (int u = 1; u < R; ++u) x[u] = cmul_conj(x[u], w[u]);
+            DftN<T, R, true>::run(x);
+        } else {
+            DftN<T, R, false>::run(x);
+#pragma unroll
+            for (int u = 1; u < R; ++u) x[u] = cmul(x[u], w[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u) p[u * leg] = x[u];
+    }
+    __syncthreads();
+}
+
+// Last forward pass, operator, first inverse pass (adjacent points).
+// op(op.pre(b, bin), v): the operator applied to natural bin `bin` of
+// sequence b (pre: what it reads from memory, ahead of the points).
+// FWD, BWD: which halves run.
+template <typename T, int R, bool FWD, bool BWD, class Op>
+__device__ __forceinline__ void line_middle(V2<T> *buf, LineTile tl, LinePlan pl, const Op &op)
+{
+    const int q = tl.n / R, total = q << tl.logb;
+    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+        const int b = bf & ((1 << tl.logb) - 1), t = bf >> tl.logb;
+        int bin = t;  // digits of the block, reversed (one radix before the last: the digit itself)
+        if (pl.nf > 2) {
+            int m = q, p = t, s = 1;
+            bin = 0;
+            for (int i = 0; i + 1 < pl.nf; ++i) {
+                m /= pl.r(i);
+                const int v = p / m;
+                p -= v * m;
+                bin += s * v;
+                s *= pl.r(i);
+            }
+        }
+        V2<T> *p = buf + t * (R + tl.pad) * tl.bp + b;
+        V2<T> x[R];
+        typename Op::Pre f[R];
+#pragma unroll
+        for (int u = 0; u < R; ++u) f[u] = op.pre(b, bin + u * q);
+#pragma unroll
+        for (int u = 0; u < R; ++u) x[u] = p[u * tl.bp];
+        if (FWD) DftN<T, R, false>::run(x);
+#pragma unroll
+        for (int u = 0; u < R; ++u) x[u] = op(f[u], x[u]);
+        if (BWD) DftN<T, R, true>::run(x);
+#pragma unroll
+        for (int u = 0; u < R; ++u) p[u * tl.bp] = x[u];
+    }
+    __syncthreads();
+}
+
+template <typename T, bool INV>
+__device__ __forceinline__ void line_pass_any(int R, V2<T> *buf, LineTile tl, int M, int S, const V2<T> *tw)
+{
+    switch (R) {
+    case 3: line_pass<T, 3, INV>(buf, tl, M, S, tw); break;
+    case 4: line_pass<T, 4, INV>(buf, tl, M, S, tw); break;
+    case 5: line_pass<T, 5, INV>(buf, tl, M, S, tw); break;
+    case 8: line_pass<T, 8, INV>(buf, tl, M, S, tw); break;
+    default: line_pass<T, 9, INV>(buf, tl, M, S, tw); break;
+    }
+}
+template <typename T, bool FWD, bool BWD, class Op>
+__device__ __forceinline__ void line_middle_any(V2<T> *buf, LineTile tl, LinePlan pl, const Op &op)
+{
+    switch (pl.r(pl.nf - 1)) {
+    case 1: line_middle<T, 1, FWD, BWD>(buf, tl, pl, op); break;
+    case 2: line_middle<T, 2, FWD, BWD>(buf, tl, pl, op); break;
+    case 3: line_middle<T, 3, FWD, BWD>(buf, tl, pl, op); break;
+    case 4: line_middle<T, 4, FWD, BWD>(buf, tl, pl, op); break;
+    case 5: line_middle<T, 5, FWD, BWD>(buf, tl, pl, op); break;
+    case 8: line_middle<T, 8, FWD, BWD>(buf, tl, pl, op); break;
+    case 9: line_middle<T, 9, FWD, BWD>(buf, tl, pl, op); break;
+    case 10: line_middle<T, 10, FWD, BWD>(buf, tl, pl, op); break;
+    case 15: line_middle<T, 15, FWD, BWD>(buf, tl, pl, op); break;
+    default: line_middle<T, 16, FWD, BWD>(buf, tl, pl, op); break;
+    }
+}
+// The passes between the first and the middle one, forward or back.
+template <typename T, bool INV>
+__device__ __forceinline__ void line_inner(V2<T> *buf, LineTile tl, LinePlan pl, const V2<T> *tw)
+{
+    if (!INV) {
+        int S = pl.r(0);
+        for (int i = 1; i + 1 < pl.nf; ++i) {
+            const int r = pl.r(i);
+            line_pass_any<T, false>(r, buf, tl, tl.n / (S * r), S, tw);
+            S *= r;
+        }
+    } else {
+        int S = tl.n / pl.r(pl.nf - 1);
+        for (int i = pl.nf - 2; i >= 1; --i) {
+            const int r = pl.r(i);
+            S /= r;
+            line_pass_any<T, true>(r, buf, tl, tl.n / (S * r), S, tw);
+        }
+    }
+}
+// First pass of a forward transform (R0 = the plan's first radix):
+// src(b, t, q, x) gives the points t + u q, u < R0, of sequence b.
+template <typename T, int R0, class Src>
+__device__ __forceinline__ void line_open(V2<T> *buf, LineTile tl, const V2<T> *__restrict__ tw, const Src &src)
+{
+    const int q = tl.n / R0, total = q << tl.logb, leg = tl.leg(q);
+    const FastDiv dq(q), dl(tl.rl);
+    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+        int b, t;
+        line_split(tl, !tl.row, dq, bf, b, t);
+        V2<T> x[R0], w[R0];
+        src(b, t, q, x);
+        line_twiddles(w, tw, t);
+        DftN<T, R0, false>::run(x);
+        V2<T> *p = buf + (t + (tl.pad ? dl.div(t) : 0)) * tl.bp + b;
+        p[0] = x[0];
+#pragma unroll
+        for (int u = 1; u < R0; ++u) p[u * leg] = cmul(x[u], w[u]);
+    }
+    __syncthreads();
+}
+// Last pass of an inverse transform: sink(b, t, q, x) takes the points t + u q.
+template <typename T, int R0, class Sink>
+__device__ __forceinline__ void line_close(const V2<T> *buf, LineTile tl, const V2<T> *__restrict__ tw, const Sink &sink)
+{
+    const int q = tl.n / R0, total = q << tl.logb, leg = tl.leg(q);
+    const FastDiv dq(q), dl(tl.rl);
+    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+        int b, t;
+        line_split(tl, !tl.row, dq, bf, b, t);
+        const V2<T> *p = buf + (t + (tl.pad ? dl.div(t) : 0)) * tl.bp + b;
+        V2<T> x[R0], w[R0];
+        line_twiddles(w, tw, t);
+        x[0] = p[0];
+#pragma unroll
+        for (int u = 1; u < R0; ++u) x[u] = cmul_conj(p[u * leg], w[u]);
+        DftN<T, R0, true>::run(x);
+        sink(b, t, q, x);
+    }
+}
+// Forward transform, operator, inverse transform of the tile's sequences.
+template <typename T, int R0, class Src, class Op, class Sink>
+__device__ __forceinline__ void line_pair(V2<T> *buf, LineTile tl, LinePlan pl, const V2<T> *tw, const Src &src, const Op &op,
+                                          const Sink &sink)
+{
+    line_open<T, R0>(buf, tl, tw, src);
+    line_inner<T, false>(buf, tl, pl, tw);
+    line_middle_any<T, true, true>(buf, tl, pl, op);
+    line_inner<T, true>(buf, tl, pl, tw);
+    line_close<T, R0>(buf, tl, tw, sink);
+}
+
+} // namespace epdlb

@@ -28,46 +28,9 @@
 #include "common.cuh"
 #include "engine.h"
 #include "fft8.cuh"
+#include "prop_line.cuh"
 
 namespace epdlb {
-
-template <typename T> struct PropK {
-    GroupGeom g;
-    V2<T> *chain;
-    V2<T> *hist;          // [run][hnodes][n]: nodes 0..half_lo, or all N_s + 1 (reference of a differential solve)
-    V2<T> *hd;            // differential solve: (dg, dg') at every node, [run][N_s + 1][n]
-    const float2 *rho;    // differential solve: (rho_A, rho_B), [run][n]
-    int hnodes;
-    const V2<T> *efac;
-    double *ia, *ib, *part;
-    const V2<T> *twx, *twy;
-    const T *kx, *ky;
-    int rows, logc, cols;  // tile rows (row pass), columns and their log2 (column pass; logc when pow2)
-};
-
-// Trapezoid weights on [0, s_{N_A}] (block A) and [s_{N_A}, 1] (block B).
-__device__ __forceinline__ double weight_a(int j, int na, double ds)
-{
-    if (na == 0 || j > na) return 0.0;
-    return (j == 0 || j == na) ? 0.5 * ds : ds;
-}
-__device__ __forceinline__ double weight_b(int j, int na, int ns, double ds)
-{
-    if (na == ns || j < na) return 0.0;
-    return (j == na || j == ns) ? 0.5 * ds : ds;
-}
-
-// Node j of g carries w_A iff j < N_A; node j of g' carries the field of node ns - j.
-// Boltzmann factor (E_A, E_B) of the half-step at node j of chain g (fac_g)
-// or g' (fac_gp), arriving or departing (half_step_block)
-template <typename T> __device__ __forceinline__ T fac_g(V2<T> e, const GroupGeom &g, int j, bool arriving)
-{
-    return half_step_block(g.jr, 0, j, g.ns, g.na, arriving) ? e.y : e.x;
-}
-template <typename T> __device__ __forceinline__ T fac_gp(V2<T> e, const GroupGeom &g, int j, bool arriving)
-{
-    return half_step_block(g.jr, 1, j, g.ns, g.na, arriving) ? e.y : e.x;
-}
 
 template <typename T> __device__ __forceinline__ T exp_t(T v);
 template <> __device__ __forceinline__ float exp_t<float>(float v) { return expf(v); }
@@ -120,189 +83,31 @@ __global__ void __launch_bounds__(kThreads) prop_start(PropK<T> k)
     }
 }
 
-// Column pass: Ty = IFFT_y Ky FFT_y on a tile of C adjacent columns (radix-2
-// transforms on power-of-two grids, mixed-radix ones otherwise).
-template <typename T>
-__global__ void __launch_bounds__(kThreads) prop_col(PropK<T> k)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const bool p2 = k.g.pow2;
-    const int ny = k.g.ny, nx = k.g.nx, logy = k.g.logy, logc = k.logc, C = k.cols;
-    const int tile = ny * C, ntw = p2 ? ny / 2 : ny;
-    V2<T> *a = reinterpret_cast<V2<T> *>(smem_raw);
-    V2<T> *b = a + tile;
-    V2<T> *tw = b + tile;
-    T *ky = reinterpret_cast<T *>(tw + ntw);
-    const int run = blockIdx.y, x0 = blockIdx.x * C;
-    V2<T> *data = k.chain + (size_t)run * k.g.n;
-    auto at = [&](int i) { return p2 ? (size_t)(i >> logc) * nx + x0 + (i & (C - 1)) : (size_t)(i / C) * nx + x0 + i % C; };
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) a[i] = data[at(i)];
-    for (int i = threadIdx.x; i < ntw; i += blockDim.x) tw[i] = k.twy[i];
-    for (int i = threadIdx.x; i < ny; i += blockDim.x) ky[i] = k.ky[i];
-    __syncthreads();
-    V2<T> *r = p2 ? fft_smem<T, false, true>(a, b, logy, logc, 1, C, tw)
-                  : fft_smem_mr<T, false, true>(a, b, ny, k.g.nfy, k.g.fy, C, 1, C, tw);
-    V2<T> *o = (r == a) ? b : a;
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) r[i] = cscale(r[i], ky[p2 ? i >> logc : i / C]);
-    __syncthreads();
-    r = p2 ? fft_smem<T, true, true>(r, o, logy, logc, 1, C, tw) : fft_smem_mr<T, true, true>(r, o, ny, k.g.nfy, k.g.fy, C, 1, C, tw);
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) data[at(i)] = r[i];
-}
-
-// Row pass producing contour node m (1 <= m <= ns): Tx, node factors, history
-// store / contour accumulation, Q_P partial sums at m = ns, next half step.
-// Differential solve (DIFF): the chain carries the change d a of the state
-// E_d g; with U = T(d a_{m-1}) and the reference node g~_m from the history,
-//   dg_m = E'_a U + rho_a g~_m,   d a_m = E'_d dg_m + E_d rho_d g~_m
-// (E' = E (1 + rho)), the exact differences of g_m = E'_a T(a_{m-1}) and
-// a_m = E'_d g_m from the reference solve's g~_m = E_a T(a~_{m-1}) and
-// a~_m = E_d g~_m; dg_m is stored at every node, dQ_P partials at m = ns.
-constexpr int RB = 4;  // points per thread whose loads the row pass's epilogue issues together
-template <typename T, bool DIFF>
-__global__ void __launch_bounds__(kThreads) prop_row(PropK<T> k, int m)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[32];
-    const bool p2 = k.g.pow2;
-    const int nx = k.g.nx, logx = k.g.logx, rows = k.rows;
-    const int tile = rows * nx, ntw = p2 ? nx / 2 : nx;
-    V2<T> *a = reinterpret_cast<V2<T> *>(smem_raw);
-    V2<T> *b = a + tile;
-    V2<T> *tw = b + tile;
-    T *kx = reinterpret_cast<T *>(tw + ntw);
-    const int run = blockIdx.y;
-    const long long n = k.g.n;
-    const long long base = (long long)blockIdx.x * tile;
-    V2<T> *data = k.chain + (size_t)run * n + base;
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) a[i] = data[i];
-    for (int i = threadIdx.x; i < ntw; i += blockDim.x) tw[i] = k.twx[i];
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) kx[i] = k.kx[i];
-    __syncthreads();
-    const int logb = p2 ? ilog2(rows) : 0;
-    V2<T> *r = p2 ? fft_smem<T, false, false>(a, b, logx, logb, nx, 1, tw)
-                  : fft_smem_mr<T, false, false>(a, b, nx, k.g.nfx, k.g.fx, rows, nx, 1, tw);
-    V2<T> *o = (r == a) ? b : a;
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) r[i] = cscale(r[i], kx[p2 ? i & (nx - 1) : i % nx]);
-    __syncthreads();
-    r = p2 ? fft_smem<T, true, false>(r, o, logx, logb, nx, 1, tw) : fft_smem_mr<T, true, false>(r, o, nx, k.g.nfx, k.g.fx, rows, nx, 1, tw);
-
-    const int ns = k.g.ns, na = k.g.na, hlo = k.g.half_lo, hhi = k.g.half_hi;
-    const double ds = k.g.ds;
-    const V2<T> *efac = k.efac + (size_t)run * n + base;
-    V2<T> *hist = k.hist + (size_t)run * k.hnodes * n + base;
-    double qsum = 0.0;
-    if constexpr (DIFF) {
-        const float2 *rho = k.rho + (size_t)run * n + base;
-        V2<T> *hd = k.hd + ((size_t)run * (ns + 1) + m) * n + base;
-        const V2<T> *gref = hist + (size_t)m * n;
-        const int bag = half_step_block(k.g.jr, 0, m, ns, na, true), bap = half_step_block(k.g.jr, 1, m, ns, na, true);
-        const int bdg = half_step_block(k.g.jr, 0, m, ns, na, false), bdp = half_step_block(k.g.jr, 1, m, ns, na, false);
-        // batches of RB points per thread: the loads first, then the stores
-        for (int i0 = threadIdx.x; i0 < tile; i0 += RB * blockDim.x) {
-            V2<T> eb[RB], grb[RB];
-            float2 qb[RB];
-#pragma unroll
-            for (int b = 0; b < RB; ++b) {
-                const int i = i0 + b * blockDim.x;
-                if (i < tile) {
-                    eb[b] = efac[i];
-                    grb[b] = gref[i];
-                    qb[b] = rho[i];
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < RB; ++b) {
-                const int i = i0 + b * blockDim.x;
-                if (i >= tile) break;
-                const V2<T> e = eb[b], gr = grb[b], u = r[i];
-                const float2 q = qb[b];
-                const T ea = bag ? e.y : e.x, eap = bap ? e.y : e.x, qa = bag ? q.y : q.x, qap = bap ? q.y : q.x;
-                const V2<T> dg = mk<T>(ea * ((T)1 + qa) * u.x + qa * gr.x, eap * ((T)1 + qap) * u.y + qap * gr.y);
-                hd[i] = dg;
-                if (m == ns) {
-                    qsum += (double)dg.x;
-                } else {
-                    const T ed = bdg ? e.y : e.x, edp = bdp ? e.y : e.x, qd = bdg ? q.y : q.x, qdp = bdp ? q.y : q.x;
-                    data[i] = mk<T>(ed * ((T)1 + qd) * dg.x + ed * qd * gr.x, edp * ((T)1 + qdp) * dg.y + edp * qdp * gr.y);
-                }
-            }
-        }
-        if (m == ns) {
-            const double s = block_sum(qsum, red);
-            if (threadIdx.x == 0) k.part[(size_t)run * kMaxPart + blockIdx.x] = s;
-        }
-        return;
-    }
-    const bool store_all = k.hnodes == ns + 1;
-    double *ia = k.ia + (size_t)run * n + base, *ib = k.ib + (size_t)run * n + base;
-    const int s2 = ns - m;
-    // batches of RB points per thread: the loads first, then the stores
-    for (int i0 = threadIdx.x; i0 < tile; i0 += RB * blockDim.x) {
-        V2<T> eb[RB], hvb[RB];
-        double iab[RB], ibb[RB];
-#pragma unroll
-        for (int b = 0; b < RB; ++b) {
-            const int i = i0 + b * blockDim.x;
-            if (i < tile) {
-                eb[b] = efac[i];
-                if (m >= hhi && s2 != m) hvb[b] = hist[(size_t)s2 * n + i];
-                if (m > hhi) {
-                    iab[b] = ia[i];
-                    ibb[b] = ib[i];
-                }
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < RB; ++b) {
-            const int i = i0 + b * blockDim.x;
-            if (i >= tile) break;
-            const V2<T> e = eb[b];
-            // z = (g_m, g'_m): the arriving half-step's factor; the chain goes on
-            // with the departing one
-            const T eg = fac_g<T>(e, k.g, m, true), egp = fac_gp<T>(e, k.g, m, true);
-            const V2<T> h = r[i];
-            const V2<T> z = mk<T>(eg * h.x, egp * h.y);
-            if (m <= hlo || store_all) hist[(size_t)m * n + i] = z;
-            if (m >= hhi) {
-                const V2<T> hv = (s2 == m) ? z : hvb[b];
-                const double t1 = (double)z.x * (double)hv.y;  // g(s_m) g'(1 - s_m)
-                double va = weight_a(m, na, ds) * t1, vb = weight_b(m, na, ns, ds) * t1;
-                if (s2 != m) {
-                    const double t2 = (double)hv.x * (double)z.y;  // g(s_{ns-m}) g'(s_m)
-                    va += weight_a(s2, na, ds) * t2;
-                    vb += weight_b(s2, na, ns, ds) * t2;
-                }
-                if (m == hhi) { ia[i] = va; ib[i] = vb; }
-                else { ia[i] = iab[b] + va; ib[i] = ibb[b] + vb; }
-            }
-            if (m == ns) qsum += (double)z.x;
-            else data[i] = mk<T>(fac_g<T>(e, k.g, m, false) * z.x, fac_gp<T>(e, k.g, m, false) * z.y);
-        }
-    }
-    if (m == ns) {
-        const double s = block_sum(qsum, red);
-        if (threadIdx.x == 0) k.part[(size_t)run * kMaxPart + blockIdx.x] = s;
-    }
-}
-
 // Normalisation, Eqs. (9)-(11) with Q as spatial means.
 // ia2/ib2 (may be null): sums of the second chain's terms (cluster solve).
 __global__ void __launch_bounds__(kThreads) prop_finalize(GroupGeom g, int nrow_blocks, int nprep_blocks, const double *ia,
                                                       const double *ib, const double *ia2, const double *ib2,
                                                       const double *part, double *phi, double *q, int *err)
 {
-    __shared__ double bc;
+    __shared__ double bc, fac[2];
     const int run = blockIdx.y;
     const long long n = g.n;
     const double *pr = part + (size_t)run * kMaxPart;
-    const double qp = sum_partials(pr, nrow_blocks, 1, &bc) / (double)n;
-    const double qs = sum_partials(pr + kMaxPart / 2, nprep_blocks, 1, &bc) / (double)n;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        q[2 * run] = qp;
-        q[2 * run + 1] = qs;
-        if (!(qp > 0.0) || !(qs > 0.0) || !isfinite(qp) || !isfinite(qs)) atomicOr(err, 1);
+    const double sp = sum_partials(pr, nrow_blocks, 1, &bc), ss = sum_partials(pr + kMaxPart / 2, nprep_blocks, 1, &bc);
+    // the FP64 divisions once per block: a division is tens of FP64
+    // instructions, at 2 lanes per SM and cycle
+    if (threadIdx.x == 0) {
+        const double qp = sp / (double)n, qs = ss / (double)n;
+        fac[0] = g.phi_p / qp;
+        fac[1] = (1.0 - g.phi_p) / qs;
+        if (blockIdx.x == 0) {
+            q[2 * run] = qp;
+            q[2 * run + 1] = qs;
+            if (!(qp > 0.0) || !(qs > 0.0) || !isfinite(qp) || !isfinite(qs)) atomicOr(err, 1);
+        }
     }
-    const double cp = g.phi_p / qp, cs = (1.0 - g.phi_p) / qs;
+    __syncthreads();
+    const double cp = fac[0], cs = fac[1];
     double *pa = phi + (size_t)run * 3 * n, *pb = pa + n, *ps = pb + n;
     const double *ja = ia + (size_t)run * n, *jb = ib + (size_t)run * n;
     const double *ja2 = ia2 ? ia2 + (size_t)run * n : nullptr, *jb2 = ib2 ? ib2 + (size_t)run * n : nullptr;
@@ -530,7 +335,7 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
                                                                 double *phi, double *q, const double *phi_ref,
                                                                 const double *q_ref, int *err)
 {
-    __shared__ double bc;
+    __shared__ double bc, fac[4];
     const int run = blockIdx.y, ns = g.ns, na = g.na;
     const long long n = g.n;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -553,6 +358,21 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
         if (wa != 0.f) kadd(sa, ca, wa * t);
         if (wb != 0.f) kadd(sb, cb, wb * t);
     };
+    // plain solve: the product's rounding error (exact, by FMA) joins the
+    // carried one, so the sums are those of the exact products to ~2^-46
+    auto add_exact = [&](int j, float x, float y) {
+        const float wa = (na == 0 || j > na) ? 0.f : ((j == 0 || j == na) ? 0.5f : 1.f);
+        const float wb = (na == ns || j < na) ? 0.f : ((j == na || j == ns) ? 0.5f : 1.f);
+        const float t = x * y, e = fmaf(x, y, -t);
+        if (wa != 0.f) {
+            kadd(sa, ca, wa * t);
+            ca -= wa * e;
+        }
+        if (wb != 0.f) {
+            kadd(sb, cb, wb * t);
+            cb -= wb * e;
+        }
+    };
     const int half = ns / 2;
     constexpr int U = DIFF ? 4 : 8;
     for (int m0 = 0; m0 <= (valid ? half : -1); m0 += U) {
@@ -574,8 +394,8 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
             const int m = m0 + u;
             if (m > half) break;
             if (!DIFF) {
-                add(m, zl[u].x * zr[u].y);
-                if (ns - m != m) add(ns - m, zr[u].x * zl[u].y);
+                add_exact(m, zl[u].x, zr[u].y);
+                if (ns - m != m) add_exact(ns - m, zr[u].x, zl[u].y);
             } else {
                 // node m: g_m g'_{ns-m}; node ns - m: g_{ns-m} g'_m
                 add(m, zl[u].x * dr[u].y + dl[u].x * zr[u].y + dl[u].x * dr[u].y);
@@ -584,30 +404,38 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
         }
     }
     // Q from the partials (after the streaming loop, so that its latency
-    // overlaps other blocks' loads; every thread of the block takes part)
+    // overlaps other blocks' loads; every thread of the block takes part).
+    // The FP64 divisions once per block, by one thread.
     const double *pr = part + (size_t)run * kMaxPart;
-    const double sq = sum_partials(pr, nrow_blocks, 1, &bc) / (double)n;
-    const double ss = sum_partials(pr + kMaxPart / 2, nprep_blocks, 1, &bc) / (double)n;
-    const double qp = DIFF ? q_ref[2 * run] + sq : sq, qs = DIFF ? q_ref[2 * run + 1] + ss : ss;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        q[2 * run] = qp;
-        q[2 * run + 1] = qs;
-        if (!(qp > 0.0) || !(qs > 0.0) || !isfinite(qp) || !isfinite(qs)) atomicOr(err, 1);
+    const double tp = sum_partials(pr, nrow_blocks, 1, &bc), ts = sum_partials(pr + kMaxPart / 2, nprep_blocks, 1, &bc);
+    if (threadIdx.x == 0) {
+        const double sq = tp / (double)n, ss = ts / (double)n;
+        const double qp = DIFF ? q_ref[2 * run] + sq : sq, qs = DIFF ? q_ref[2 * run + 1] + ss : ss;
+        fac[0] = g.phi_p * g.ds / qp;
+        fac[1] = (1.0 - g.phi_p) / qs;
+        fac[2] = sq / qp;
+        fac[3] = ss / qs;
+        if (blockIdx.x == 0) {
+            q[2 * run] = qp;
+            q[2 * run + 1] = qs;
+            if (!(qp > 0.0) || !(qs > 0.0) || !isfinite(qp) || !isfinite(qs)) atomicOr(err, 1);
+        }
     }
+    __syncthreads();
     if (!valid) return;
     const double ia = (double)sa - (double)ca, ib = (double)sb - (double)cb;
+    const double cp = fac[0], cs = fac[1];
     double *ph = phi + (size_t)run * 3 * n;
     if (!DIFF) {
-        const double c = g.phi_p * g.ds / qp;
-        ph[i] = c * ia;
-        ph[n + i] = c * ib;
-        ph[2 * n + i] *= (1.0 - g.phi_p) / qs;
+        ph[i] = cp * ia;
+        ph[n + i] = cp * ib;
+        ph[2 * n + i] *= cs;
     } else {
         const double *pt = phi_ref + (size_t)run * 3 * n;
-        const double rq = 1.0 / qp, c = g.phi_p * g.ds;
-        ph[i] = pt[i] + (c * ia - pt[i] * sq) * rq;
-        ph[n + i] = pt[n + i] + (c * ib - pt[n + i] * sq) * rq;
-        ph[2 * n + i] = pt[2 * n + i] + ((1.0 - g.phi_p) * ph[2 * n + i] - pt[2 * n + i] * ss) / qs;
+        const double rp = fac[2], rs = fac[3], pa = pt[i], pb = pt[n + i], ps = pt[2 * n + i];
+        ph[i] = pa + (cp * ia - pa * rp);
+        ph[n + i] = pb + (cp * ib - pb * rp);
+        ph[2 * n + i] = ps + (cs * ph[2 * n + i] - ps * rs);
     }
 }
 
@@ -776,19 +604,6 @@ static int grid_for(long long n)
 }
 
 template <typename T>
-static size_t col_smem(const Group &G)
-{
-    return (size_t)2 * (G.g.ny * G.sh.cols_prop) * sizeof(V2<T>) + (G.g.pow2 ? G.g.ny / 2 : G.g.ny) * sizeof(V2<T>) +
-           G.g.ny * sizeof(T);
-}
-template <typename T>
-static size_t row_smem(const Group &G)
-{
-    return (size_t)2 * (G.sh.rows_prop * G.g.nx) * sizeof(V2<T>) + (G.g.pow2 ? G.g.nx / 2 : G.g.nx) * sizeof(V2<T>) +
-           G.g.nx * sizeof(T);
-}
-
-template <typename T>
 static PropK<T> prop_args(const Group &G)
 {
     PropK<T> k;
@@ -806,9 +621,6 @@ static PropK<T> prop_args(const Group &G)
     k.twy = reinterpret_cast<const V2<T> *>(G.twy);
     k.kx = reinterpret_cast<const T *>(G.kx);
     k.ky = reinterpret_cast<const T *>(G.ky);
-    k.rows = G.sh.rows_prop;
-    k.logc = G.g.pow2 ? ilog2(G.sh.cols_prop) : 0;
-    k.cols = G.sh.cols_prop;
     return k;
 }
 
@@ -816,24 +628,22 @@ static PropK<T> prop_args(const Group &G)
 static int stream8_row_blocks(const GroupGeom &g) { return (int)(g.n / (g.nx >= 2048 ? g.nx : 2048)); }
 
 // The contour loop of the generic streaming solve (column pass, row pass per
-// node); returns the row pass grid (its x extent = the Q partial blocks).
-template <typename T, bool DIFF>
-static dim3 generic_loop(const Group &G, PropK<T> &k, cudaStream_t s, const SolveProbe *probe)
+// node); blocks: the Q partials of the last row pass per run.
+template <typename T>
+static cudaError_t generic_loop(const PropK<T> &k, bool diff, int *blocks, cudaStream_t s, const SolveProbe *probe)
 {
-    const GroupGeom &g = G.g;
-    const dim3 gc(g.nx / G.sh.cols_prop, g.nruns), gr(g.ny / G.sh.rows_prop, g.nruns);
-    const size_t sc = col_smem<T>(G), sr = row_smem<T>(G);
-    for (int m = 1; m <= g.ns; ++m) {
+    cudaError_t e = cudaSuccess;
+    for (int m = 1; m <= k.g.ns && !e; ++m) {
         const bool pa = probe && m == probe->m_acc, ps = probe && m == probe->m_store;
         if (pa) cudaEventRecordWithFlags(probe->ev[2], s, cudaEventRecordExternal);
-        prop_col<T><<<gc, kThreads, sc, s>>>(k);
+        e = line_col(k, s);
         if (pa) cudaEventRecordWithFlags(probe->ev[3], s, cudaEventRecordExternal);
         if (ps) cudaEventRecordWithFlags(probe->ev[0], s, cudaEventRecordExternal);
-        prop_row<T, DIFF><<<gr, kThreads, sr, s>>>(k, m);
+        if (!e) e = line_row(k, m, diff, blocks, s);
         if (ps) cudaEventRecordWithFlags(probe->ev[1], s, cudaEventRecordExternal);
         if (pa) cudaEventRecordWithFlags(probe->ev[4], s, cudaEventRecordExternal);
     }
-    return gr;
+    return e;
 }
 
 template <typename T>
@@ -858,8 +668,13 @@ static cudaError_t solve_t(Group &G, const double *omega, double *phi, double *q
         return cudaGetLastError();
     }
     prop_start<T, false><<<dim3(pg, g.nruns), kThreads, 0, s>>>(k);
-    const dim3 gr = generic_loop<T, false>(G, k, s, probe);
-    prop_finalize<<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, gr.x, pg, G.ia, G.ib, nullptr, nullptr, G.part, phi, q, G.err);
+    int blocks = 0;
+    if (cudaError_t e = generic_loop<T>(k, false, &blocks, s, probe)) return e;
+    if (sizeof(T) == sizeof(float) && k.hnodes == g.ns + 1)  // full history: the sums are one pass over it
+        prop_contour_stream<false><<<dim3((unsigned)((g.n + kThreads - 1) / kThreads), g.nruns), kThreads, 0, s>>>(
+            g, reinterpret_cast<const float2 *>(G.hist), nullptr, blocks, pg, G.part, phi, q, nullptr, nullptr, G.err);
+    else
+        prop_finalize<<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, blocks, pg, G.ia, G.ib, nullptr, nullptr, G.part, phi, q, G.err);
     return cudaGetLastError();
 }
 
@@ -881,9 +696,10 @@ static cudaError_t stream_delta(Group &G, int pg, double *phi, double *q, const 
     }
     PropK<float> k = prop_args<float>(G);
     prop_start<float, true><<<dim3(pg, g.nruns), kThreads, 0, s>>>(k);
-    const dim3 gr = generic_loop<float, true>(G, k, s, probe);
+    int blocks = 0;
+    if (cudaError_t e = generic_loop<float>(k, true, &blocks, s, probe)) return e;
     prop_contour_stream<true><<<gcon, kThreads, 0, s>>>(g, reinterpret_cast<const float2 *>(G.hist),
-                                                       reinterpret_cast<const float2 *>(G.hd), (int)gr.x, pg, G.part, phi,
+                                                       reinterpret_cast<const float2 *>(G.hd), blocks, pg, G.part, phi,
                                                        q, phi_ref, q_ref, G.err);
     return cudaGetLastError();
 }
@@ -916,26 +732,9 @@ cudaError_t launch_solve_delta(Group &G, cudaStream_t s, const SolveProbe *probe
 // three axes' factors, each applied inside its own axis transform), the row
 // pass carrying the node factors, history and contour sums as in 2D.
 template <typename T>
-static size_t smem3(const GroupGeom &g, int rows, int cols, bool row)
-{
-    if (row) return (size_t)2 * rows * g.nx * sizeof(V2<T>) + (g.pow2 ? g.nx / 2 : g.nx) * sizeof(V2<T>) + g.nx * sizeof(T);
-    return (size_t)2 * g.ny * cols * sizeof(V2<T>) + (g.pow2 ? g.ny / 2 : g.ny) * sizeof(V2<T>) + g.ny * sizeof(T);
-}
-
-size_t solve3d_smem_max(const Solve3 &S)
-{
-    auto mx = [&](auto t) {
-        using T = decltype(t);
-        return std::max(smem3<T>(S.vx, S.rows_x, 0, true), std::max(smem3<T>(S.vy, 0, S.cols_y, false), smem3<T>(S.vz, 0, S.cols_z, false)));
-    };
-    return S.prec == EPD_LB_MIXED_FP32 ? mx(0.f) : mx(0.0);
-}
-
-template <typename T>
 static cudaError_t solve3d_t(const Solve3 &S, const double *omega, double *phi, double *q, cudaStream_t s)
 {
-    auto view = [&](const GroupGeom &g, const void *tw_row, const void *tw_col, const void *k_row, const void *k_col,
-                    int rows, int cols) {
+    auto view = [&](const GroupGeom &g, const void *tw_row, const void *tw_col, const void *k_row, const void *k_col) {
         PropK<T> k;
         k.g = g;
         k.chain = reinterpret_cast<V2<T> *>(S.chain);
@@ -951,48 +750,30 @@ static cudaError_t solve3d_t(const Solve3 &S, const double *omega, double *phi, 
         k.twy = reinterpret_cast<const V2<T> *>(tw_col);
         k.kx = reinterpret_cast<const T *>(k_row);
         k.ky = reinterpret_cast<const T *>(k_col);
-        k.rows = rows;
-        k.cols = cols;
-        k.logc = g.pow2 ? ilog2(cols) : 0;
         return k;
     };
-    const PropK<T> kx = view(S.vx, S.twx, S.twy, S.kx, S.ky, S.rows_x, 1);
-    const PropK<T> ky = view(S.vy, S.twx, S.twy, S.kx, S.ky, 1, S.cols_y);
-    const PropK<T> kz = view(S.vz, S.twx, S.twz, S.kx, S.kz, 1, S.cols_z);
+    const PropK<T> kx = view(S.vx, S.twx, S.twy, S.kx, S.ky);
+    const PropK<T> ky = view(S.vy, S.twx, S.twy, S.kx, S.ky);
+    const PropK<T> kz = view(S.vz, S.twx, S.twz, S.kx, S.kz);
     const GroupGeom &g = S.vx;
     const int pg = grid_for(g.n);
     prop_prep<T><<<dim3(pg, 1), kThreads, 0, s>>>(g, omega, reinterpret_cast<V2<T> *>(S.efac), phi, S.part);
     prop_start<T, false><<<dim3(pg, 1), kThreads, 0, s>>>(kx);
-    const dim3 gz(S.vz.nx / S.cols_z, 1), gy(S.vy.nx / S.cols_y, S.vy.nruns), gr(S.vx.ny / S.rows_x, 1);
-    const size_t sz = smem3<T>(S.vz, 0, S.cols_z, false), sy = smem3<T>(S.vy, 0, S.cols_y, false),
-                 sr = smem3<T>(S.vx, S.rows_x, 0, true);
-    for (int m = 1; m <= g.ns; ++m) {
-        prop_col<T><<<gz, kThreads, sz, s>>>(kz);
-        prop_col<T><<<gy, kThreads, sy, s>>>(ky);
-        prop_row<T, false><<<gr, kThreads, sr, s>>>(kx, m);
+    int blocks = 0;
+    cudaError_t e = cudaSuccess;
+    for (int m = 1; m <= g.ns && !e; ++m) {
+        e = line_col(kz, s);
+        if (!e) e = line_col(ky, s);
+        if (!e) e = line_row(kx, m, false, &blocks, s);
     }
-    prop_finalize<<<dim3(pg, 1), kThreads, 0, s>>>(g, gr.x, pg, S.ia, S.ib, nullptr, nullptr, S.part, phi, q, S.err);
+    if (e) return e;
+    prop_finalize<<<dim3(pg, 1), kThreads, 0, s>>>(g, blocks, pg, S.ia, S.ib, nullptr, nullptr, S.part, phi, q, S.err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_solve3d(const Solve3 &S, const double *omega, double *phi, double *q, cudaStream_t s)
 {
     return S.prec == EPD_LB_MIXED_FP32 ? solve3d_t<float>(S, omega, phi, q, s) : solve3d_t<double>(S, omega, phi, q, s);
-}
-
-cudaError_t configure_prop_kernels()
-{
-    cudaError_t e = cudaSuccess;
-    const int lim = 200 * 1024;
-    e = cudaFuncSetAttribute(prop_col<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e) return e;
-    e = cudaFuncSetAttribute(prop_row<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e) return e;
-    e = cudaFuncSetAttribute(prop_row<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e) return e;
-    e = cudaFuncSetAttribute(prop_col<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if (e) return e;
-    return cudaFuncSetAttribute(prop_row<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
 } // namespace epdlb

@@ -1,0 +1,306 @@
+// prop_line.cuh -- the streaming propagator passes that run on every grid
+// (Sec. 2, Eqs. (6)-(10) of arXiv:1804.02883): one contour step is a column
+// pass and a row pass over the packed chain z = g + i g', each a forward
+// transform, the axis' Fourier factor and an inverse transform of every line
+// (fftg.cuh).  Included by one translation unit per precision.
+//
+// What bounds them.  FP32: L2 traffic and, on small grids, the latency of a
+// pass; FP64: the FP64 unit (2 lanes per SM and cycle), so what counts there
+// is FP64 instructions per point and an even load of the SMs.  A CTA holds few
+// lines (line_logb) so that every grid gives each SM several tiles.
+#pragma once
+
+#include "common.cuh"
+#include "engine.h"
+#include "fftg.cuh"
+
+namespace epdlb {
+
+template <typename T> struct PropK {
+    GroupGeom g;
+    V2<T> *chain;
+    V2<T> *hist;          // [run][hnodes][n]: nodes 0..half_lo, or all N_s + 1 (reference of a differential solve)
+    V2<T> *hd;            // differential solve: (dg, dg') at every node, [run][N_s + 1][n]
+    const float2 *rho;    // differential solve: (rho_A, rho_B), [run][n]
+    int hnodes;
+    const V2<T> *efac;
+    double *ia, *ib, *part;
+    const V2<T> *twx, *twy;
+    const T *kx, *ky;
+};
+
+// Boltzmann factor (E_A, E_B) of the half-step at node j of chain g (fac_g)
+// or g' (fac_gp), arriving or departing (half_step_block)
+template <typename T> __device__ __forceinline__ T fac_g(V2<T> e, const GroupGeom &g, int j, bool arriving)
+{
+    return half_step_block(g.jr, 0, j, g.ns, g.na, arriving) ? e.y : e.x;
+}
+template <typename T> __device__ __forceinline__ T fac_gp(V2<T> e, const GroupGeom &g, int j, bool arriving)
+{
+    return half_step_block(g.jr, 1, j, g.ns, g.na, arriving) ? e.y : e.x;
+}
+
+// Trapezoid weights on [0, s_{N_A}] (block A) and [s_{N_A}, 1] (block B).
+__host__ __device__ inline double weight_a(int j, int na, double ds)
+{
+    if (na == 0 || j > na) return 0.0;
+    return (j == 0 || j == na) ? 0.5 * ds : ds;
+}
+__host__ __device__ inline double weight_b(int j, int na, int ns, double ds)
+{
+    if (na == ns || j < na) return 0.0;
+    return (j == na || j == ns) ? 0.5 * ds : ds;
+}
+
+// log2 of the lines per CTA: at most 2^maxlog, halved down to 2^minlog while
+// the launch has fewer than four CTAs per SM (152 SMs) or a tile more than
+// 40 KB; then doubled while the launch has more than maxblocks CTAs per run
+// (the partials a row pass writes).
+inline int line_logb(bool row, int n, LinePlan pl, long long nseq, int nruns, size_t elem, int maxlog, int minlog, long long maxblocks)
+{
+    auto tiles = [&](int l) { return (nseq + (1 << l) - 1) >> l; };
+    int l = maxlog;
+    while (l > 0 && LineTile(row, n, l, pl).points() * elem > 40 * 1024) --l;
+    while (l > minlog && tiles(l) * nruns < 4 * 152) --l;
+    while (tiles(l) > maxblocks) ++l;
+    return l;
+}
+// threads of a tile: one butterfly of the first pass each, in whole warps
+inline int line_threads(int n, int r0, int logb)
+{
+    const int t = (((n / r0) << logb) + 31) / 32 * 32;
+    return t > 256 ? 256 : t;
+}
+
+// Launches of one contour step are dependents of the one before
+// (griddepcontrol): the next one's CTAs are placed while its last CTAs finish.
+__device__ __forceinline__ void line_dependents()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename T> struct LineScale {  // the Fourier factor of Eq. (8)
+    const T *__restrict__ kf;
+    using Pre = T;
+    __device__ __forceinline__ T pre(int, int bin) const { return __ldg(&kf[bin]); }
+    __device__ __forceinline__ V2<T> operator()(T f, V2<T> v) const { return cscale(v, f); }
+};
+
+// Column pass: Ty = IFFT_y Ky FFT_y on 2^logb adjacent columns.
+template <typename T, int R0>
+__global__ void __launch_bounds__(256) prop_col(PropK<T> k, int logb)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V2<T> *buf = reinterpret_cast<V2<T> *>(smem_raw);
+    const int ny = k.g.ny, nx = k.g.nx, x0 = blockIdx.x << logb;
+    V2<T> *data = k.chain + (size_t)blockIdx.y * k.g.n + x0;
+    line_dependents();
+    line_pair<T, R0>(
+        buf, LineTile(false, ny, logb, k.g.py), k.g.py, k.twy,
+        [&](int b, int t, int q, V2<T>(&x)[R0]) {
+            const bool in = x0 + b < nx;
+            const int i0 = t * nx + b, di = q * nx;
+#pragma unroll
+            for (int u = 0; u < R0; ++u) x[u] = in ? data[i0 + u * di] : mk<T>((T)0, (T)0);
+        },
+        LineScale<T>{k.ky},
+        [&](int b, int t, int q, V2<T>(&x)[R0]) {
+            if (x0 + b >= nx) return;
+            const int i0 = t * nx + b, di = q * nx;
+#pragma unroll
+            for (int u = 0; u < R0; ++u) data[i0 + u * di] = x[u];
+        });
+}
+
+// What a row pass adds to the contour sums: the trapezoid weights of node m
+// (block A, B) and of its mirror N_s - m.
+struct RowWeights {
+    double a1, b1, a2, b2;
+};
+
+// Row pass producing contour node m (1 <= m <= ns): Tx, node factors, history
+// store / contour accumulation, Q_P partial sums at m = ns, next half step.
+// Differential solve (DIFF): the chain carries the change d a of the state
+// E_d g; with U = T(d a_{m-1}) and the reference node g~_m from the history,
+//   dg_m = E'_a U + rho_a g~_m,   d a_m = E'_d dg_m + E_d rho_d g~_m
+// (E' = E (1 + rho)), the exact differences of g_m = E'_a T(a_{m-1}) and
+// a_m = E'_d g_m from the reference solve's g~_m = E_a T(a~_{m-1}) and
+// a~_m = E_d g~_m; dg_m is stored at every node, dQ_P partials at m = ns.
+// With the full history (hnodes = N_s + 1) the contour sums are a pass of
+// their own (prop_contour_stream); otherwise node m >= N_s / 2 meets its
+// mirror from the half history here.
+template <typename T, int R0, bool DIFF>
+__global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, RowWeights w)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[32];
+    V2<T> *buf = reinterpret_cast<V2<T> *>(smem_raw);
+    const int nx = k.g.nx, ny = k.g.ny, run = blockIdx.y, y0 = blockIdx.x << logb;
+    const int ns = k.g.ns, na = k.g.na, jr = k.g.jr, hlo = k.g.half_lo, hhi = k.g.half_hi, s2 = ns - m;
+    const long long n = k.g.n, base = (long long)y0 * nx;
+    V2<T> *data = k.chain + (size_t)run * n + base;
+    const V2<T> *efac = k.efac + (size_t)run * n + base;
+    V2<T> *hist = k.hist + (size_t)run * k.hnodes * n + base;
+    // blocks of the arriving and departing half-steps of both chains
+    const bool bag = half_step_block(jr, 0, m, ns, na, true), bap = half_step_block(jr, 1, m, ns, na, true);
+    const bool bdg = half_step_block(jr, 0, m, ns, na, false), bdp = half_step_block(jr, 1, m, ns, na, false);
+    double qsum = 0.0;
+    // points whose loads are issued together, ahead of the stores
+    constexpr int CH = R0 % 4 == 0 ? 4 : (R0 % 5 == 0 ? 5 : (R0 % 3 == 0 ? 3 : 2));
+    line_dependents();
+    line_pair<T, R0>(
+        buf, LineTile(true, nx, logb, k.g.px), k.g.px, k.twx,
+        [&](int b, int t, int q, V2<T>(&x)[R0]) {
+            const bool in = y0 + b < ny;
+            const int i0 = b * nx + t;
+#pragma unroll
+            for (int u = 0; u < R0; ++u) x[u] = in ? data[i0 + u * q] : mk<T>((T)0, (T)0);
+        },
+        LineScale<T>{k.kx},
+        [&](int b, int t, int q, V2<T>(&x)[R0]) {
+            if (y0 + b >= ny) return;
+            const int i0 = b * nx + t;
+            if constexpr (DIFF) {
+                const float2 *rho = k.rho + (size_t)run * n + base;
+                V2<T> *hd = k.hd + ((size_t)run * (ns + 1) + m) * n + base;
+                const V2<T> *gref = hist + (size_t)m * n;
+#pragma unroll
+                for (int u0 = 0; u0 < R0; u0 += CH) {
+                    V2<T> eb[CH], grb[CH];
+                    float2 qb[CH];
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        const int i = i0 + (u0 + c) * q;
+                        eb[c] = efac[i];
+                        grb[c] = gref[i];
+                        qb[c] = rho[i];
+                    }
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        const int i = i0 + (u0 + c) * q;
+                        const V2<T> e = eb[c], gr = grb[c], h = x[u0 + c];
+                        const float2 r = qb[c];
+                        const T ea = bag ? e.y : e.x, eap = bap ? e.y : e.x, qa = bag ? r.y : r.x, qap = bap ? r.y : r.x;
+                        const V2<T> dg = mk<T>(ea * ((T)1 + qa) * h.x + qa * gr.x, eap * ((T)1 + qap) * h.y + qap * gr.y);
+                        hd[i] = dg;
+                        if (m == ns) {
+                            qsum += (double)dg.x;
+                        } else {
+                            const T ed = bdg ? e.y : e.x, edp = bdp ? e.y : e.x, qd = bdg ? r.y : r.x, qdp = bdp ? r.y : r.x;
+                            data[i] = mk<T>(ed * ((T)1 + qd) * dg.x + ed * qd * gr.x,
+                                            edp * ((T)1 + qdp) * dg.y + edp * qdp * gr.y);
+                        }
+                    }
+                }
+            } else {
+                const bool store_all = k.hnodes == ns + 1, acc = !store_all && m >= hhi;
+                // only the block(s) with a weight at this node or its mirror
+                const bool use_a = acc && (m == hhi || w.a1 != 0.0 || w.a2 != 0.0);
+                const bool use_b = acc && (m == hhi || w.b1 != 0.0 || w.b2 != 0.0);
+                double *ia = k.ia + (size_t)run * n + base, *ib = k.ib + (size_t)run * n + base;
+#pragma unroll
+                for (int u0 = 0; u0 < R0; u0 += CH) {
+                    V2<T> eb[CH], hvb[CH];
+                    double iab[CH], ibb[CH];
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        const int i = i0 + (u0 + c) * q;
+                        eb[c] = efac[i];
+                        iab[c] = ibb[c] = 0.0;
+                        if (acc && s2 != m) hvb[c] = hist[(size_t)s2 * n + i];
+                        if (use_a && m > hhi) iab[c] = ia[i];
+                        if (use_b && m > hhi) ibb[c] = ib[i];
+                    }
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        const int i = i0 + (u0 + c) * q;
+                        const V2<T> e = eb[c], h = x[u0 + c];
+                        // z = (g_m, g'_m): the arriving half-step's factor; the
+                        // chain goes on with the departing one
+                        const V2<T> z = mk<T>((bag ? e.y : e.x) * h.x, (bap ? e.y : e.x) * h.y);
+                        if (m <= hlo || store_all) hist[(size_t)m * n + i] = z;
+                        if (acc) {
+                            const V2<T> hv = (s2 == m) ? z : hvb[c];
+                            const double t1 = (double)z.x * (double)hv.y;                  // g(s_m) g'(1 - s_m)
+                            const double t2 = s2 == m ? 0.0 : (double)hv.x * (double)z.y;  // g(s_{ns-m}) g'(s_m)
+                            if (use_a) ia[i] = iab[c] + (w.a1 * t1 + w.a2 * t2);
+                            if (use_b) ib[i] = ibb[c] + (w.b1 * t1 + w.b2 * t2);
+                        }
+                        if (m == ns) qsum += (double)z.x;
+                        else data[i] = mk<T>((bdg ? e.y : e.x) * z.x, (bdp ? e.y : e.x) * z.y);
+                    }
+                }
+            }
+        });
+    if (m == ns) {
+        const double s = block_sum(qsum, red);
+        if (threadIdx.x == 0) k.part[(size_t)run * kMaxPart + blockIdx.x] = s;
+    }
+}
+
+template <typename K, typename... A>
+cudaError_t launch_line(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename T> cudaError_t line_col_t(const PropK<T> &k, cudaStream_t s)
+{
+    const int n = k.g.ny, nx = k.g.nx, r0 = k.g.py.r(0);
+    const int maxlog = sizeof(T) == 4 ? 3 : 2;  // 64-byte row segments
+    const int l = line_logb(false, n, k.g.py, nx, k.g.nruns, sizeof(V2<T>), maxlog, sizeof(T) == 4 ? 1 : 0, 1LL << 30);
+    const dim3 grid((nx + (1 << l) - 1) >> l, k.g.nruns);
+    const size_t sm = LineTile(false, n, l, k.g.py).points() * sizeof(V2<T>);
+    const int th = line_threads(n, r0, l);
+    switch (r0) {
+    case 2: return launch_line(prop_col<T, 2>, grid, th, sm, s, k, l);
+    case 4: return launch_line(prop_col<T, 4>, grid, th, sm, s, k, l);
+    case 6: return launch_line(prop_col<T, 6>, grid, th, sm, s, k, l);
+    case 8: return launch_line(prop_col<T, 8>, grid, th, sm, s, k, l);
+    case 10: return launch_line(prop_col<T, 10>, grid, th, sm, s, k, l);
+    case 12: return launch_line(prop_col<T, 12>, grid, th, sm, s, k, l);
+    default: return launch_line(prop_col<T, 16>, grid, th, sm, s, k, l);
+    }
+}
+
+template <typename T, bool DIFF> cudaError_t line_row_t(const PropK<T> &k, int m, int *blocks, cudaStream_t s)
+{
+    const int n = k.g.nx, ny = k.g.ny, r0 = k.g.px.r(0), ns = k.g.ns, na = k.g.na;
+    const int l = line_logb(true, n, k.g.px, ny, k.g.nruns, sizeof(V2<T>), 3, 0, kMaxPart / 2);
+    const dim3 grid((ny + (1 << l) - 1) >> l, k.g.nruns);
+    *blocks = (int)grid.x;
+    const size_t sm = LineTile(true, n, l, k.g.px).points() * sizeof(V2<T>);
+    const int th = line_threads(n, r0, l), s2 = ns - m;
+    const double ds = k.g.ds;
+    const RowWeights w = {weight_a(m, na, ds), weight_b(m, na, ns, ds), s2 == m ? 0.0 : weight_a(s2, na, ds),
+                          s2 == m ? 0.0 : weight_b(s2, na, ns, ds)};
+    switch (r0) {
+    case 2: return launch_line(prop_row<T, 2, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 4: return launch_line(prop_row<T, 4, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 6: return launch_line(prop_row<T, 6, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 8: return launch_line(prop_row<T, 8, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 10: return launch_line(prop_row<T, 10, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 12: return launch_line(prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
+    default: return launch_line(prop_row<T, 16, DIFF>, grid, th, sm, s, k, m, l, w);
+    }
+}
+
+// One column pass; one row pass producing node m (blocks: its Q partials per
+// run); instantiated in prop_line_f32.cu and prop_line_f64.cu.
+cudaError_t line_col(const PropK<float> &k, cudaStream_t s);
+cudaError_t line_col(const PropK<double> &k, cudaStream_t s);
+cudaError_t line_row(const PropK<float> &k, int m, bool diff, int *blocks, cudaStream_t s);
+cudaError_t line_row(const PropK<double> &k, int m, bool diff, int *blocks, cudaStream_t s);
+
+} // namespace epdlb
