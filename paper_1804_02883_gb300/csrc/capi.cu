@@ -17,19 +17,6 @@
 
 namespace epdlb {
 
-cudaError_t configure_epd_kernels();
-
-cudaError_t configure_kernels()
-{
-    // once per process (a function-local static is initialised exactly once,
-    // also when handles are created on several threads)
-    static const cudaError_t status = [] {
-        cudaError_t e = configure_epd_kernels();
-        if (e == cudaSuccess) e = configure_step3d_kernels();
-        return e;
-    }();
-    return status;
-}
 
 static size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -173,18 +160,6 @@ static Group run_view(const Group &G, int r)
 
 static bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
-// Radix plan of an axis: radix 4 while it divides, then 2, 3, 5.
-static int radix_plan(int n, int *f)
-{
-    int k = 0;
-    for (int p : {4, 2, 3, 5})
-        while (n % p == 0 && k < kMaxFactors) {
-            f[k++] = p;
-            n /= p;
-        }
-    return k;
-}
-
 // Radices of the in-place transforms (fftg.cuh) of an even length 2^a 3^b 5^c:
 // the first from {2, 4, 6, 8, 10, 12, 16}, the last from {1, 2, 3, 4, 5, 8, 9,
 // 10, 15, 16}, {3, 4, 5, 8, 9} between (every such length to 2048 has a plan
@@ -270,8 +245,6 @@ static void fill_geom(Group &G)
     g.pow2 = pow2(p.nx) && pow2(p.ny);
     g.logx = g.pow2 ? ilog2(p.nx) : 0;
     g.logy = g.pow2 ? ilog2(p.ny) : 0;
-    g.nfx = radix_plan(p.nx, g.fx);
-    g.nfy = radix_plan(p.ny, g.fy);
     const bool fp64 = p.precision == EPD_LB_PLAIN_FP64;
     g.px = line_plan(p.nx, (long long)p.nx * p.ny, fp64);
     g.py = line_plan(p.ny, (long long)p.nx * p.ny, fp64);
@@ -302,20 +275,7 @@ static void fill_geom(Group &G)
     g.vscale = p.dx / p.dt;
 }
 
-// Launch shapes: about 2048 points per CTA, column tiles at least 32 bytes wide.
-static void default_shapes(Group &G)
-{
-    const int nx = G.g.nx, ny = G.g.ny;
-    G.sh.rows_epd = std::max(1, std::min(ny, 2048 / nx));
-    G.sh.cols_epd = std::min(nx, std::max(2, 2048 / ny));
-    if (!G.g.pow2) {  // tiles must divide the axes
-        G.sh.rows_epd = divisor_at_most(ny, G.sh.rows_epd);
-        G.sh.cols_epd = divisor_at_most(nx, G.sh.cols_epd);
-    }
-}
-
-// Twiddles exp(-2 pi i t / n), t < n (the radix-2 passes read t < n/2), and
-// Fourier factors exp(-R_G^2 k^2 ds) / n of the propagator (Eq. (8)), on the
+// Twiddles exp(-2 pi i t / n), t < n, and Fourier factors exp(-R_G^2 k^2 ds) / n of the propagator (Eq. (8)), on the
 // host in FP64.
 template <typename T>
 static void host_tables(const Group &G, std::vector<T> &twx, std::vector<T> &twy, std::vector<T> &kx, std::vector<T> &ky,
@@ -483,7 +443,6 @@ static void form_groups(const epd_lb_params *p, int nruns, std::vector<Group> &g
     }
     for (auto &G : groups) {
         fill_geom(G);
-        default_shapes(G);
     }
 }
 
@@ -709,10 +668,6 @@ extern "C" int epd_lb_init(const epd_lb_params *p, int32_t nruns, void *workspac
         epd_lb_destroy(h);
         return code;
     };
-    if (cudaError_t e = configure_kernels()) {
-        (void)e;
-        return bail(EPD_LB_ECUDA);
-    }
     if (workspace) {
         if (workspace_bytes < need || ((uintptr_t)workspace & 255)) return bail(EPD_LB_ENOMEM);
         h->ws = workspace;
@@ -1461,7 +1416,6 @@ extern "C" int epd_prop_solve3d(const epd_lb_params *p, int32_t nz, const double
     const size_t need = solve3_layout(p, nz, S, nullptr);
     if (!need) return EPD_LB_EINVAL;
     if (workspace_bytes < need || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
-    if (configure_kernels() != cudaSuccess) return EPD_LB_ECUDA;
     solve3_layout(p, nz, S, (char *)workspace_dev);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const double ds = 1.0 / (double)p->ns;
@@ -1490,30 +1444,15 @@ extern "C" int epd_lb3d_step(const epd_lb_params *p, int32_t nz, const double *p
 
 // The coupled 3D step: the 3D solve's layout plus the step's fields and the
 // FP64 transform buffers and tables.
-static Axis3 axis3(int n)
-{
-    Axis3 a = Axis3();
-    a.n = n;
-    a.pow2 = pow2(n);
-    a.logn = a.pow2 ? ilog2(n) : 0;
-    a.nf = radix_plan(n, a.f);
-    return a;
-}
-
 static size_t step3_layout(const epd_lb_params *p, int nz, Step3 &T, char *base)
 {
     const size_t sb = solve3_layout(p, nz, T.S, base);
     if (!sb) return 0;
     const int nx = p->nx, ny = p->ny;
     const long long n = (long long)nx * ny * nz;
-    Fft3 &F = T.F;
-    F.ax = axis3(nx);
-    F.ay = axis3(ny);
-    F.az = axis3(nz);
-    F.rows_x = divisor_at_most(ny * nz, std::max(1, 2048 / nx));
-    F.cols_y = divisor_at_most(nx, std::max(1, 2048 / ny));
-    F.cols_z = divisor_at_most(nx * ny, std::max(1, 2048 / nz));
-    if (fft3_smem(F) > 200 * 1024) return 0;
+    T.nx = nx;
+    T.ny = ny;
+    T.nz = nz;
     size_t off = sb;
     auto take = [&](size_t bytes) -> void * {
         off = align_up(off);
@@ -1529,9 +1468,9 @@ static size_t step3_layout(const epd_lb_params *p, int nz, Step3 &T, char *base)
     T.pop2 = (double *)take(19 * n * sizeof(double));
     T.b0 = (double2 *)take(n * sizeof(double2));
     T.b1 = (double2 *)take(n * sizeof(double2));
-    F.twx = (const double2 *)take(nx * sizeof(double2));
-    F.twy = (const double2 *)take(ny * sizeof(double2));
-    F.twz = (const double2 *)take(nz * sizeof(double2));
+    T.twx = (const double2 *)take(nx * sizeof(double2));
+    T.twy = (const double2 *)take(ny * sizeof(double2));
+    T.twz = (const double2 *)take(nz * sizeof(double2));
     T.f0_lat = p->f0 * fstar_lattice(*p);
     return align_up(off);
 }
@@ -1555,7 +1494,6 @@ extern "C" int epd_step3d(const epd_lb_params *p, int32_t nz, double *omega_dev,
     const size_t need = step3_layout(p, nz, T, nullptr);
     if (!need) return EPD_LB_EINVAL;
     if (workspace_bytes < need || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
-    if (configure_kernels() != cudaSuccess) return EPD_LB_ECUDA;
     step3_layout(p, nz, T, (char *)workspace_dev);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const double ds = 1.0 / (double)p->ns;
@@ -1568,9 +1506,9 @@ extern "C" int epd_step3d(const epd_lb_params *p, int32_t nz, double *omega_dev,
     if (!e) e = up(p->ny, T.S.twy, T.S.ky);
     if (!e) e = up(nz, T.S.twz, T.S.kz);
     // FP64 twiddles of the EPD transforms
-    if (!e) e = upload_axis<double>(p->nx, p->dx, p->rg, ds, (void *)T.F.twx, nullptr, s);
-    if (!e) e = upload_axis<double>(p->ny, p->dx, p->rg, ds, (void *)T.F.twy, nullptr, s);
-    if (!e) e = upload_axis<double>(nz, p->dx, p->rg, ds, (void *)T.F.twz, nullptr, s);
+    if (!e) e = upload_axis<double>(p->nx, p->dx, p->rg, ds, (void *)T.twx, nullptr, s);
+    if (!e) e = upload_axis<double>(p->ny, p->dx, p->rg, ds, (void *)T.twy, nullptr, s);
+    if (!e) e = upload_axis<double>(nz, p->dx, p->rg, ds, (void *)T.twz, nullptr, s);
     if (!e) e = launch_step3d(T, omega_dev, pop_dev, vel_dev, phi_dev, q_dev, force_dev, s);
     return e ? EPD_LB_ECUDA : EPD_LB_OK;
 }
@@ -1617,7 +1555,6 @@ extern "C" int epd_prop_solve(const epd_lb_params *p, const double *omega_dev, d
     Group G;
     if (!solve_group(p, G) || !omega_dev || !phi_dev || !q_dev || !workspace_dev) return EPD_LB_EINVAL;
     if (workspace_bytes < carve_solve(G, nullptr) || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
-    if (configure_kernels() != cudaSuccess) return EPD_LB_ECUDA;
     carve_solve(G, (char *)workspace_dev);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (cudaMemsetAsync(G.err, 0, sizeof(int), s) != cudaSuccess) return EPD_LB_ECUDA;
@@ -1685,7 +1622,6 @@ extern "C" int epd_prop_solve_noalloc(const epd_lb_params *p, const double *omeg
     G.prec = p->precision;
     fill_geom(G);
     G.g.nruns = 1;
-    default_shapes(G);
     if (carve_solve(G, nullptr) > kNoallocBytes) return EPD_LB_ETOOLARGE;
 
     int dev = 0;
@@ -1695,7 +1631,6 @@ extern "C" int epd_prop_solve_noalloc(const epd_lb_params *p, const double *omeg
         if (cudaGetSymbolAddress(&base, g_noalloc_scratch) != cudaSuccess || !base) return EPD_LB_ECUDA;
         g_noalloc_addr[dev].store(base);
     }
-    if (configure_kernels() != cudaSuccess) return EPD_LB_ECUDA;
     carve_solve(G, (char *)base);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // the error word must start at zero; every other scratch buffer is written

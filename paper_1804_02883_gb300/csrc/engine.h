@@ -14,7 +14,6 @@
 namespace epdlb {
 
 // Parameters every kernel of a group needs, by value.
-constexpr int kMaxFactors = 16;  // radices of one axis (mixed-radix transforms)
 
 // Radices of one axis for the in-place transforms of fftg.cuh: nf of them,
 // radix i in byte i.
@@ -28,9 +27,7 @@ LinePlan line_plan(int n, long long sites, bool fp64);  // of a length on a grid
 struct GroupGeom {
     int nx, ny, logx, logy;  // logx, logy: 0 unless both axes are powers of two
     LinePlan px, py;         // radices of each axis' in-place transforms
-    int pow2;                // both axes powers of two; else the mixed-radix radix-2-family passes
-    int nfx, nfy;            // radix plans (4, 2, 3, 5) of each axis for the mixed-radix transforms
-    int fx[kMaxFactors], fy[kMaxFactors];
+    int pow2;                // both axes powers of two
     int ns, na;          // contour steps, A-block intervals round(f_a ns)
     int jr;              // junction rule: 0 literal, 1 segment-symmetric
     int half_lo, half_hi;  // nodes 0..half_lo are stored; nodes >= half_hi accumulate
@@ -60,16 +57,10 @@ __host__ __device__ inline int half_step_block(int jr, int chain, int m, int ns,
     return (chain == 0 ? j : ns - 1 - j) >= na;
 }
 
-// Launch shapes of the transform passes (chosen at init, see tune_shapes).
-struct Shapes {
-    int rows_epd, cols_epd;  // rows per CTA of the EPD/force row passes, columns per CTA of the column passes
-};
-
 // One batch of runs with identical grid, contour and model parameters.
 struct Group {
     epd_lb_params p;   // parameters of the first run (f0 and seed may differ per run)
     GroupGeom g;
-    Shapes sh;
     int prec;          // EPD_LB_PLAIN_FP64 or EPD_LB_MIXED_FP32
     std::vector<int> run_ids;  // handle-level run index of each member
     std::vector<epd_lb_params> run_params;
@@ -240,36 +231,22 @@ struct Solve3 {
     int prec;
 };
 cudaError_t launch_solve3d(const Solve3 &S, const double *omega, double *phi, double *q, cudaStream_t s);
-// One axis of the FP64 3D transforms of the coupled 3D step.
-struct Axis3 {
-    int n, pow2, logn, nf;
-    int f[kMaxFactors];
-};
-struct Fft3 {
-    Axis3 ax, ay, az;
-    int rows_x, cols_y, cols_z;    // tiles of the x-row, y-column and z-column transforms
-    const double2 *twx, *twy, *twz;  // FP64 twiddles exp(-2 pi i t / n), t < n
-};
-size_t fft3_smem(const Fft3 &F);
 // The coupled step on a 3D box (step3d.cu): state omega (3n), pop (19n,
 // pre-collision), vel (3n); outputs phi (3n), q (2), force (3n).
 struct Step3 {
     Solve3 S;
-    Fft3 F;
+    int nx, ny, nz;
+    const double2 *twx, *twy, *twz;           // FP64 twiddles exp(-2 pi i t / n), t < n
     double *wt, *pt, *mu, *qt, *ftot, *pop2;  // omega~, Phi~, mu / dPhi, Q~, total force, populations out
     double2 *b0, *b1;                         // complex FP64 transform buffers [n]
     double f0_lat;                            // body-force amplitude, lattice units
 };
 cudaError_t launch_step3d(const Step3 &T, double *omega, double *pop, double *vel, double *phi, double *q, double *force,
                           cudaStream_t s);
-cudaError_t configure_step3d_kernels();
 
 // D3Q19 collide-stream on an nz x ny x nx box, FP64 ([19][z][y][x] in, out).
 cudaError_t launch_lb3d_step(int nx, int ny, int nz, double gs, double gb, double gg, const double *in,
                              const double *force, double *out, double *vel, cudaStream_t s);
-
-// Kernel attributes (dynamic shared memory limits), once per process.
-cudaError_t configure_kernels();
 
 // Smallest/largest supported sizes.
 constexpr int kMinN = 8, kMaxN = 2048;

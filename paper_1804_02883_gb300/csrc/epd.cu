@@ -22,271 +22,15 @@
 
 #include "common.cuh"
 #include "engine.h"
+#include "epd.cuh"
 #include "fft8.cuh"
 
 namespace epdlb {
 
-enum RowMode { ROW_GRAD = 0, ROW_LAP = 1, ROW_FWD_S = 2, ROW_INV_FORCE = 3, ROW_DIVX = 4 };
-enum ColMode { COL_CONVECT = 0, COL_DIFFUSE = 1, COL_FORCE = 2, COL_DIVY = 3 };
-
-struct EpdK {
-    GroupGeom g;
-    const double *omega, *omega_t, *phi, *phi_t;
-    double *omega_dst;
-    double *phi_dst;  // convected densities (ROW_DIVX / COL_DIVY)
-    void *cz;  // [run][4][n] complex of the transform type
-    const void *vel;
-    void *force;
-    int bulk_double;
-    const void *twx, *twy;  // twiddles of the transform type
-    const float2 *tab8x, *tab8y;  // pass tables of each axis' best radix plan (FP32 radix-8/16 kernels)
-    const float2 *tab16y, *tab8y_r8;  // column tables of the radix-16 and radix-8 plans (tile-dependent)
-    int rows, logc, cols;  // tile rows (row passes), columns and their log2 (column passes; logc when pow2)
-    double kunit_x, kunit_y;  // 2 pi / (n dx) per axis
-    double mu_ref[3];         // mu_I at the homogeneous composition, omega = 0
-    double phibar[3];         // the homogeneous composition
-};
-
-// signed wavenumber of bin m; odd operators drop the Nyquist bin
-template <typename TT> __device__ __forceinline__ TT kvec(int m, int n, TT unit) { return unit * (TT)signed_bin(m, n); }
-template <typename TT> __device__ __forceinline__ TT kvec_odd(int m, int n, TT unit) { return (2 * m == n) ? (TT)0 : kvec<TT>(m, n, unit); }
-
-// Chemical potential of Eq. (1), mu_I = sum_{J != I} chi_IJ Phi_J + kappa_H (sum Phi - 1) - omega_I,
-// minus its homogeneous value (computed in FP64).
-__device__ __forceinline__ double2 mu_pair(const EpdK &k, const double *phi, const double *om, long long n, long long i, int pair)
-{
-    const GroupGeom &g = k.g;
-    const double pa = phi[i], pb = phi[n + i], ps = phi[2 * n + i];
-    const double inc = g.kappa_h * (pa + pb + ps - 1.0);
-    if (pair == 0)
-        return make_double2(g.chi_ab * pb + g.chi_as * ps + inc - om[i] - k.mu_ref[0],
-                            g.chi_ab * pa + g.chi_bs * ps + inc - om[n + i] - k.mu_ref[1]);
-    return make_double2(g.chi_as * pa + g.chi_bs * pb + inc - om[2 * n + i] - k.mu_ref[2], 0.0);
-}
-
-// The same in FP32 from the FP64 deviations dPhi_J = Phi_J - Phi-bar_J:
-// mu_I - mu_I(Phi-bar, 0) = sum_{J != I} chi_IJ dPhi_J + kappa_H sum_J dPhi_J - omega_I
-// (linear in Phi), so FP32 rounding scales with the fluctuations.
-__device__ __forceinline__ float2 mu_pair_f(const EpdK &k, const double *phi, const double *om, long long n, long long i, int pair)
-{
-    const GroupGeom &g = k.g;
-    const float da = (float)(phi[i] - k.phibar[0]), db = (float)(phi[n + i] - k.phibar[1]),
-                dsv = (float)(phi[2 * n + i] - k.phibar[2]);
-    const float inc = (float)g.kappa_h * (da + db + dsv);
-    if (pair == 0)
-        return make_float2((float)g.chi_ab * db + (float)g.chi_as * dsv + inc - (float)om[i],
-                           (float)g.chi_ab * da + (float)g.chi_bs * dsv + inc - (float)om[n + i]);
-    return make_float2((float)g.chi_as * da + (float)g.chi_bs * db + inc - (float)om[2 * n + i], 0.f);
-}
-
-__device__ __forceinline__ double2 vel_at(const EpdK &k, size_t idx)
-{
-    if (k.bulk_double) return reinterpret_cast<const double2 *>(k.vel)[idx];
-    const float2 v = reinterpret_cast<const float2 *>(k.vel)[idx];
-    return make_double2((double)v.x, (double)v.y);
-}
-
-template <typename TT> __device__ __forceinline__ V2<TT> to_tt(double2 v) { return mk<TT>((TT)v.x, (TT)v.y); }
-template <typename TT> __device__ __forceinline__ double2 to_d(V2<TT> v) { return make_double2((double)v.x, (double)v.y); }
-
-template <typename TT, int MODE>
-__global__ void __launch_bounds__(kThreads) epd_row(EpdK k)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const GroupGeom &g = k.g;
-    const bool p2 = g.pow2;
-    const int nx = g.nx, logx = g.logx, rows = k.rows, tile = rows * nx, ntw = p2 ? nx / 2 : nx;
-    V2<TT> *a = reinterpret_cast<V2<TT> *>(smem_raw);
-    V2<TT> *b = a + tile;
-    V2<TT> *tw = b + tile;
-    const int run = blockIdx.y, pair = blockIdx.z;
-    const long long n = g.n;
-    const long long base = (long long)blockIdx.x * tile;
-    V2<TT> *cz = reinterpret_cast<V2<TT> *>(k.cz);
-    const V2<TT> *twg = reinterpret_cast<const V2<TT> *>(k.twx);
-    for (int i = threadIdx.x; i < ntw; i += blockDim.x) tw[i] = twg[i];
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) {
-        const long long s = base + i;
-        V2<TT> v;
-        if (MODE == ROW_GRAD) {
-            const double *om = k.omega + (size_t)run * 3 * n;
-            v = pair == 0 ? mk<TT>((TT)om[s], (TT)om[n + s]) : mk<TT>((TT)om[2 * n + s], (TT)0);
-        } else if (MODE == ROW_LAP) {
-            v = to_tt<TT>(mu_pair(k, k.phi_t + (size_t)run * 3 * n, k.omega_t + (size_t)run * 3 * n, n, s, pair));
-        } else if (MODE == ROW_FWD_S) {
-            // S = sum_I dPhi_I^D / D_I, dPhi^D = Phi(t+dt) - Phi~ (Eq. (19))
-            const double *p1 = k.phi + (size_t)run * 3 * n, *p0 = k.phi_t + (size_t)run * 3 * n;
-            const double sa = (p1[s] - p0[s]) + (p1[n + s] - p0[n + s]);
-            v = mk<TT>((TT)(sa / g.d_p + (p1[2 * n + s] - p0[2 * n + s]) / g.d_s), (TT)0);
-        } else if (MODE == ROW_DIVX) {
-            // x flux v_x Phi_I, v = u_lat dx/dt
-            const double *ph = k.phi + (size_t)run * 3 * n;
-            const double vx = vel_at(k, (size_t)run * n + s).x * g.vscale;
-            v = pair == 0 ? mk<TT>((TT)(vx * ph[s]), (TT)(vx * ph[n + s])) : mk<TT>((TT)(vx * ph[2 * n + s]), (TT)0);
-        } else {
-            v = cz[((size_t)run * 4 + 2) * n + s];
-        }
-        a[i] = v;
-    }
-    __syncthreads();
-    const int logb = p2 ? ilog2(rows) : 0;
-    V2<TT> *r = a, *o = b;
-    if (MODE != ROW_INV_FORCE) {
-        r = p2 ? fft_smem<TT, false, false>(a, b, logx, logb, nx, 1, tw)
-               : fft_smem_mr<TT, false, false>(a, b, nx, g.nfx, g.fx, rows, nx, 1, tw);
-        o = (r == a) ? b : a;
-        if (MODE != ROW_FWD_S) {
-            const TT unit = (TT)k.kunit_x, inv_n = (TT)(1.0 / (double)nx);
-            for (int i = threadIdx.x; i < tile; i += blockDim.x) {
-                const int m = p2 ? i & (nx - 1) : i % nx;
-                V2<TT> v = r[i];
-                if (MODE == ROW_GRAD || MODE == ROW_DIVX) {  // i kx / nx
-                    const TT kk = kvec_odd<TT>(m, nx, unit) * inv_n;
-                    v = mk<TT>(-kk * v.y, kk * v.x);
-                } else {                 // -kx^2 / nx
-                    const TT kk = kvec<TT>(m, nx, unit);
-                    v = cscale(v, -kk * kk * inv_n);
-                }
-                r[i] = v;
-            }
-            __syncthreads();
-        }
-    }
-    if (MODE != ROW_FWD_S)
-        r = p2 ? fft_smem<TT, true, false>(r, o, logx, logb, nx, 1, tw)
-               : fft_smem_mr<TT, true, false>(r, o, nx, g.nfx, g.fx, rows, nx, 1, tw);
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) {
-        const long long s = base + i;
-        if (MODE == ROW_INV_FORCE) {
-            const V2<TT> f = cscale(r[i], (TT)(1.0 / (double)nx));
-            if (k.bulk_double) reinterpret_cast<double2 *>(k.force)[(size_t)run * n + s] = make_double2((double)f.x, (double)f.y);
-            else reinterpret_cast<float2 *>(k.force)[(size_t)run * n + s] = make_float2((float)f.x, (float)f.y);
-        } else {
-            const int plane = (MODE == ROW_FWD_S) ? 2 : pair;
-            cz[((size_t)run * 4 + plane) * n + s] = r[i];
-        }
-    }
-}
-
-template <typename TT, int MODE>
-__global__ void __launch_bounds__(kThreads) epd_col(EpdK k)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const GroupGeom &g = k.g;
-    const bool p2 = g.pow2;
-    const int ny = g.ny, nx = g.nx, logy = g.logy, logc = k.logc, C = k.cols, tile = ny * C, ntw = p2 ? ny / 2 : ny;
-    V2<TT> *a = reinterpret_cast<V2<TT> *>(smem_raw);
-    V2<TT> *b = a + tile;
-    V2<TT> *tw = b + tile;
-    const int run = blockIdx.y, pair = blockIdx.z, x0 = blockIdx.x * C;
-    // row and column of tile element i
-    auto row_of = [&](int i) { return p2 ? i >> logc : i / C; };
-    auto col_of = [&](int i) { return p2 ? i & (C - 1) : i % C; };
-    const long long n = g.n;
-    V2<TT> *cz = reinterpret_cast<V2<TT> *>(k.cz);
-    const V2<TT> *twg = reinterpret_cast<const V2<TT> *>(k.twy);
-    for (int i = threadIdx.x; i < ntw; i += blockDim.x) tw[i] = twg[i];
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) {
-        const long long s = (long long)row_of(i) * nx + x0 + col_of(i);
-        V2<TT> v;
-        if (MODE == COL_CONVECT) {
-            const double *om = k.omega + (size_t)run * 3 * n;
-            v = pair == 0 ? mk<TT>((TT)om[s], (TT)om[n + s]) : mk<TT>((TT)om[2 * n + s], (TT)0);
-        } else if (MODE == COL_DIFFUSE) {
-            v = to_tt<TT>(mu_pair(k, k.phi_t + (size_t)run * 3 * n, k.omega_t + (size_t)run * 3 * n, n, s, pair));
-        } else if (MODE == COL_DIVY) {
-            // y flux v_y Phi_I
-            const double *ph = k.phi + (size_t)run * 3 * n;
-            const double vy = vel_at(k, (size_t)run * n + s).y * g.vscale;
-            v = pair == 0 ? mk<TT>((TT)(vy * ph[s]), (TT)(vy * ph[n + s])) : mk<TT>((TT)(vy * ph[2 * n + s]), (TT)0);
-        } else {
-            v = cz[((size_t)run * 4 + 2) * n + s];
-        }
-        a[i] = v;
-    }
-    __syncthreads();
-    V2<TT> *r = p2 ? fft_smem<TT, false, true>(a, b, logy, logc, 1, C, tw)
-                   : fft_smem_mr<TT, false, true>(a, b, ny, g.nfy, g.fy, C, 1, C, tw);
-    V2<TT> *o = (r == a) ? b : a;
-    const TT uy = (TT)k.kunit_y, ux = (TT)k.kunit_x, inv_n = (TT)(1.0 / (double)ny);
-    const TT cforce = (TT)(g.inv_beta_v * g.fstar / (g.dt * (double)ny));
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) {
-        const int my = row_of(i);
-        V2<TT> v = r[i];
-        if (MODE == COL_CONVECT || MODE == COL_DIVY) {  // i ky / ny
-            const TT kk = kvec_odd<TT>(my, ny, uy) * inv_n;
-            v = mk<TT>(-kk * v.y, kk * v.x);
-        } else if (MODE == COL_DIFFUSE) { // -ky^2 / ny
-            const TT kk = kvec<TT>(my, ny, uy);
-            v = cscale(v, -kk * kk * inv_n);
-        } else {
-            // f(k) = (1/(beta v)) S(k) / dt * i k / |k|^2, Eq. (20), in lattice units;
-            // f_x + i f_y is real + i real, so one transform carries both:
-            // multiply by c (i kx - ky) / |k|^2 and invert.
-            const int mx = x0 + col_of(i);
-            const TT kx = kvec<TT>(mx, nx, ux), ky = kvec<TT>(my, ny, uy);
-            const TT k2 = kx * kx + ky * ky;
-            if (k2 == (TT)0) {
-                v = mk<TT>((TT)0, (TT)0);
-            } else {
-                const TT c = cforce / k2;
-                v = cmul(v, mk<TT>(-c * kvec_odd<TT>(my, ny, uy), c * kvec_odd<TT>(mx, nx, ux)));
-            }
-        }
-        r[i] = v;
-    }
-    __syncthreads();
-    r = p2 ? fft_smem<TT, true, true>(r, o, logy, logc, 1, C, tw) : fft_smem_mr<TT, true, true>(r, o, ny, g.nfy, g.fy, C, 1, C, tw);
-    for (int i = threadIdx.x; i < tile; i += blockDim.x) {
-        const long long s = (long long)row_of(i) * nx + x0 + col_of(i);
-        if (MODE == COL_FORCE) {
-            cz[((size_t)run * 4 + 2) * n + s] = r[i];
-        } else if (MODE == COL_DIVY) {
-            // Phi~ = Phi - dt (d/dx (v_x Phi) + d/dy (v_y Phi))
-            const double2 dy = to_d<TT>(r[i]);
-            const double2 dx = to_d<TT>(cz[((size_t)run * 4 + pair) * n + s]);
-            const double *ph = k.phi + (size_t)run * 3 * n;
-            double *pd = k.phi_dst + (size_t)run * 3 * n;
-            if (pair == 0) {
-                pd[s] = ph[s] - g.dt * (dx.x + dy.x);
-                pd[n + s] = ph[n + s] - g.dt * (dx.y + dy.y);
-            } else {
-                pd[2 * n + s] = ph[2 * n + s] - g.dt * (dx.x + dy.x);
-            }
-        } else if (MODE == COL_CONVECT) {
-            // omega~ = omega - dt v . grad omega, v = u_lat dx/dt
-            const double2 dy = to_d<TT>(r[i]);
-            const double2 dx = to_d<TT>(cz[((size_t)run * 4 + pair) * n + s]);
-            const double2 u = vel_at(k, (size_t)run * n + s);
-            const double vx = u.x * g.vscale, vy = u.y * g.vscale;
-            const double *om = k.omega + (size_t)run * 3 * n;
-            double *ot = k.omega_dst + (size_t)run * 3 * n;
-            if (pair == 0) {
-                ot[s] = om[s] - g.dt * (vx * dx.x + vy * dy.x);
-                ot[n + s] = om[n + s] - g.dt * (vx * dx.y + vy * dy.y);
-            } else {
-                ot[2 * n + s] = om[2 * n + s] - g.dt * (vx * dx.x + vy * dy.x);
-            }
-        } else {
-            // omega(t+dt) = omega~ - dt D_I Lap mu_I
-            const double2 dy = to_d<TT>(r[i]);
-            const double2 lx = to_d<TT>(cz[((size_t)run * 4 + pair) * n + s]);
-            const double *ot = k.omega_t + (size_t)run * 3 * n;
-            double *om = k.omega_dst + (size_t)run * 3 * n;
-            if (pair == 0) {
-                om[s] = ot[s] - g.dt * g.d_p * (lx.x + dy.x);
-                om[n + s] = ot[n + s] - g.dt * g.d_p * (lx.y + dy.y);
-            } else {
-                om[2 * n + s] = ot[2 * n + s] - g.dt * g.d_s * (lx.x + dy.x);
-            }
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
-// FP32 radix-8 versions of the row and column passes (MIXED_FP32, grids with
-// 64..2048 points per axis): the same operators and data flow as epd_row /
-// epd_col above, transforms and tiles (RowTile, ColTile) from fft8.cuh.
+// FP32 radix-8 row and column passes (MIXED_FP32, grids with 64..2048 points
+// per axis): the operators and data flow of epd_line.cu, transforms and tiles
+// (RowTile, ColTile) from fft8.cuh.
 // ---------------------------------------------------------------------------
 
 // i k / n (first derivative, Nyquist bin dropped) and -k^2 / n along one axis
@@ -600,9 +344,6 @@ static EpdK make_k(Group &G)
     k.tab8y = best_mr(G.g.logy) == 4 ? G.tab16y : G.tab8y;
     k.tab16y = G.tab16y;
     k.tab8y_r8 = G.tab8y;
-    k.rows = G.sh.rows_epd;
-    k.logc = G.g.pow2 ? ilog2(G.sh.cols_epd) : 0;
-    k.cols = G.sh.cols_epd;
     const double pi = 3.14159265358979323846;
     k.kunit_x = 2.0 * pi / ((double)G.g.nx * G.g.dx);
     k.kunit_y = 2.0 * pi / ((double)G.g.ny * G.g.dx);
@@ -610,25 +351,22 @@ static EpdK make_k(Group &G)
     const double fa = (double)G.g.na / (double)G.g.ns;
     const double pa = G.g.phi_p * fa, pb = G.g.phi_p * (1.0 - fa), ps = 1.0 - G.g.phi_p;
     const double inc = G.g.kappa_h * (pa + pb + ps - 1.0);
-    k.mu_ref[0] = G.g.chi_ab * pb + G.g.chi_as * ps + inc;
-    k.mu_ref[1] = G.g.chi_ab * pa + G.g.chi_bs * ps + inc;
-    k.mu_ref[2] = G.g.chi_as * pa + G.g.chi_bs * pb + inc;
+    const double mu_ref[3] = {G.g.chi_ab * pb + G.g.chi_as * ps + inc, G.g.chi_ab * pa + G.g.chi_bs * ps + inc,
+                              G.g.chi_as * pa + G.g.chi_bs * pb + inc};
+    const double chi[3][3] = {{0.0, G.g.chi_ab, G.g.chi_as}, {G.g.chi_ab, 0.0, G.g.chi_bs}, {G.g.chi_as, G.g.chi_bs, 0.0}};
+    for (int i = 0; i < 3; ++i) {
+        for (int j = 0; j < 3; ++j) k.mu_c[i][j] = chi[i][j] + G.g.kappa_h;
+        k.mu_0[i] = G.g.kappa_h + mu_ref[i];
+    }
+    k.inv_dp = 1.0 / G.g.d_p;
+    k.inv_ds = 1.0 / G.g.d_s;
     k.phibar[0] = pa;
     k.phibar[1] = pb;
     k.phibar[2] = ps;
     return k;
 }
 
-template <typename TT> static size_t row_smem(const Group &G)
-{
-    return (size_t)2 * G.sh.rows_epd * G.g.nx * sizeof(V2<TT>) + (G.g.pow2 ? G.g.nx / 2 : G.g.nx) * sizeof(V2<TT>);
-}
-template <typename TT> static size_t col_smem(const Group &G)
-{
-    return (size_t)2 * G.sh.cols_epd * G.g.ny * sizeof(V2<TT>) + (G.g.pow2 ? G.g.ny / 2 : G.g.ny) * sizeof(V2<TT>);
-}
-
-template <typename TT> static cudaError_t aux_t(Group &G, cudaStream_t s)
+static cudaError_t aux(Group &G, cudaStream_t s)
 {
     EpdK k = make_k(G);
     k.omega_dst = G.omega_t;
@@ -637,12 +375,12 @@ template <typename TT> static cudaError_t aux_t(Group &G, cudaStream_t s)
         if (row8_at<ROW_GRAD, 6>(G.g.logx, k, gz, s) && col8_at<COL_CONVECT, 6>(G.g.logy, k, gz, s, G.colw)) return cudaGetLastError();
         return cudaErrorInvalidConfiguration;
     }
-    epd_row<TT, ROW_GRAD><<<dim3(G.g.ny / G.sh.rows_epd, G.g.nruns, 2), kThreads, row_smem<TT>(G), s>>>(k);
-    epd_col<TT, COL_CONVECT><<<dim3(G.g.nx / G.sh.cols_epd, G.g.nruns, 2), kThreads, col_smem<TT>(G), s>>>(k);
-    return cudaGetLastError();
+    const bool d = G.prec == EPD_LB_PLAIN_FP64;
+    const cudaError_t e = epd_line_row(k, ROW_GRAD, d, s);
+    return e ? e : epd_line_col(k, COL_CONVECT, d, s);
 }
 
-template <typename TT> static cudaError_t diffusion_t(Group &G, cudaStream_t s)
+static cudaError_t diffusion(Group &G, cudaStream_t s)
 {
     EpdK k = make_k(G);
     k.omega_dst = G.omega;
@@ -651,12 +389,12 @@ template <typename TT> static cudaError_t diffusion_t(Group &G, cudaStream_t s)
         if (row8_at<ROW_LAP, 6>(G.g.logx, k, gz, s) && col8_at<COL_DIFFUSE, 6>(G.g.logy, k, gz, s, G.colw)) return cudaGetLastError();
         return cudaErrorInvalidConfiguration;
     }
-    epd_row<TT, ROW_LAP><<<dim3(G.g.ny / G.sh.rows_epd, G.g.nruns, 2), kThreads, row_smem<TT>(G), s>>>(k);
-    epd_col<TT, COL_DIFFUSE><<<dim3(G.g.nx / G.sh.cols_epd, G.g.nruns, 2), kThreads, col_smem<TT>(G), s>>>(k);
-    return cudaGetLastError();
+    const bool d = G.prec == EPD_LB_PLAIN_FP64;
+    const cudaError_t e = epd_line_row(k, ROW_LAP, d, s);
+    return e ? e : epd_line_col(k, COL_DIFFUSE, d, s);
 }
 
-template <typename TT> static cudaError_t force_t(Group &G, cudaStream_t s)
+static cudaError_t force(Group &G, cudaStream_t s)
 {
     EpdK k = make_k(G);
     if (use_r8(G)) {
@@ -666,10 +404,10 @@ template <typename TT> static cudaError_t force_t(Group &G, cudaStream_t s)
             return cudaGetLastError();
         return cudaErrorInvalidConfiguration;
     }
-    epd_row<TT, ROW_FWD_S><<<dim3(G.g.ny / G.sh.rows_epd, G.g.nruns, 1), kThreads, row_smem<TT>(G), s>>>(k);
-    epd_col<TT, COL_FORCE><<<dim3(G.g.nx / G.sh.cols_epd, G.g.nruns, 1), kThreads, col_smem<TT>(G), s>>>(k);
-    epd_row<TT, ROW_INV_FORCE><<<dim3(G.g.ny / G.sh.rows_epd, G.g.nruns, 1), kThreads, row_smem<TT>(G), s>>>(k);
-    return cudaGetLastError();
+    const bool d = G.prec == EPD_LB_PLAIN_FP64;
+    cudaError_t e = epd_line_row(k, ROW_FWD_S, d, s);
+    if (!e) e = epd_line_col(k, COL_FORCE, d, s);
+    return e ? e : epd_line_row(k, ROW_INV_FORCE, d, s);
 }
 
 // Column tile autotuner (radix-8 EPD column passes and streaming propagator
@@ -734,46 +472,23 @@ cudaError_t launch_convect_phi(Group &G, const double *phi, double *phi_dst, cud
     k.phi_dst = phi_dst;
     k.twx = G.twx_d;
     k.twy = G.twy_d;
-    epd_row<double, ROW_DIVX><<<dim3(G.g.ny / G.sh.rows_epd, G.g.nruns, 2), kThreads, row_smem<double>(G), s>>>(k);
-    epd_col<double, COL_DIVY><<<dim3(G.g.nx / G.sh.cols_epd, G.g.nruns, 2), kThreads, col_smem<double>(G), s>>>(k);
-    return cudaGetLastError();
+    const cudaError_t e = epd_line_row(k, ROW_DIVX, true, s);
+    return e ? e : epd_line_col(k, COL_DIVY, true, s);
 }
 
 cudaError_t launch_aux_convection(Group &G, cudaStream_t s)
 {
-    return G.prec == EPD_LB_MIXED_FP32 ? aux_t<float>(G, s) : aux_t<double>(G, s);
+    return aux(G, s);
 }
 
 cudaError_t launch_diffusion(Group &G, cudaStream_t s)
 {
-    return G.prec == EPD_LB_MIXED_FP32 ? diffusion_t<float>(G, s) : diffusion_t<double>(G, s);
+    return diffusion(G, s);
 }
 
 cudaError_t launch_force(Group &G, cudaStream_t s)
 {
-    return G.prec == EPD_LB_MIXED_FP32 ? force_t<float>(G, s) : force_t<double>(G, s);
-}
-
-template <typename TT> static cudaError_t configure_t()
-{
-    const int lim = 200 * 1024;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(epd_row<TT, ROW_GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    if ((e = cudaFuncSetAttribute(epd_row<TT, ROW_LAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    if ((e = cudaFuncSetAttribute(epd_row<TT, ROW_FWD_S>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    if ((e = cudaFuncSetAttribute(epd_row<TT, ROW_INV_FORCE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    if ((e = cudaFuncSetAttribute(epd_col<TT, COL_CONVECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    if ((e = cudaFuncSetAttribute(epd_col<TT, COL_DIFFUSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim))) return e;
-    return cudaFuncSetAttribute(epd_col<TT, COL_FORCE>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-}
-
-cudaError_t configure_epd_kernels()
-{
-    cudaError_t e = configure_t<float>();
-    if (!e) e = configure_t<double>();
-    if (!e) e = cudaFuncSetAttribute(epd_row<double, ROW_DIVX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (!e) e = cudaFuncSetAttribute(epd_col<double, COL_DIVY>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    return e;
+    return force(G, s);
 }
 
 } // namespace epdlb

@@ -442,4 +442,149 @@ __device__ __forceinline__ void line_pair(V2<T> *buf, LineTile tl, LinePlan pl, 
     line_close<T, R0>(buf, tl, tw, sink);
 }
 
+// ---------------------------------------------------------------------------
+// The same transforms on a tile filled and emptied by the caller, every pass
+// called by its radix: less code per kernel, for the operators that run once
+// per time step.
+// ---------------------------------------------------------------------------
+
+template <typename T, int R, bool INV>
+__device__ __noinline__ void line_pass_call(V2<T> *buf, LineTile tl, int M, int S, const V2<T> *tw)
+{
+    line_pass<T, R, INV>(buf, tl, M, S, tw);
+}
+template <typename T, int R, bool FWD, bool BWD, class Op>
+__device__ __noinline__ void line_middle_call(V2<T> *buf, LineTile tl, LinePlan pl, Op op)
+{
+    line_middle<T, R, FWD, BWD>(buf, tl, pl, op);
+}
+template <typename T, bool INV> __device__ __forceinline__ void line_pass_by(int R, V2<T> *buf, LineTile tl, int M, int S, const V2<T> *tw)
+{
+    switch (R) {
+    case 2: line_pass_call<T, 2, INV>(buf, tl, M, S, tw); break;
+    case 3: line_pass_call<T, 3, INV>(buf, tl, M, S, tw); break;
+    case 4: line_pass_call<T, 4, INV>(buf, tl, M, S, tw); break;
+    case 5: line_pass_call<T, 5, INV>(buf, tl, M, S, tw); break;
+    case 6: line_pass_call<T, 6, INV>(buf, tl, M, S, tw); break;
+    case 8: line_pass_call<T, 8, INV>(buf, tl, M, S, tw); break;
+    case 9: line_pass_call<T, 9, INV>(buf, tl, M, S, tw); break;
+    case 10: line_pass_call<T, 10, INV>(buf, tl, M, S, tw); break;
+    case 12: line_pass_call<T, 12, INV>(buf, tl, M, S, tw); break;
+    default: line_pass_call<T, 16, INV>(buf, tl, M, S, tw); break;
+    }
+}
+// FWD: forward transform; then op in digit-reversed order; BWD: inverse.
+template <typename T, bool FWD, bool BWD, class Op>
+__device__ __forceinline__ void line_operator(V2<T> *buf, LineTile tl, LinePlan pl, const V2<T> *tw, Op op)
+{
+    if (FWD) {
+        int S = 1;
+        for (int i = 0; i + 1 < pl.nf; ++i) {
+            const int r = pl.r(i);
+            line_pass_by<T, false>(r, buf, tl, tl.n / (S * r), S, tw);
+            S *= r;
+        }
+    }
+    switch (pl.r(pl.nf - 1)) {
+    case 1: line_middle_call<T, 1, FWD, BWD>(buf, tl, pl, op); break;
+    case 2: line_middle_call<T, 2, FWD, BWD>(buf, tl, pl, op); break;
+    case 3: line_middle_call<T, 3, FWD, BWD>(buf, tl, pl, op); break;
+    case 4: line_middle_call<T, 4, FWD, BWD>(buf, tl, pl, op); break;
+    case 5: line_middle_call<T, 5, FWD, BWD>(buf, tl, pl, op); break;
+    case 8: line_middle_call<T, 8, FWD, BWD>(buf, tl, pl, op); break;
+    case 9: line_middle_call<T, 9, FWD, BWD>(buf, tl, pl, op); break;
+    case 10: line_middle_call<T, 10, FWD, BWD>(buf, tl, pl, op); break;
+    case 15: line_middle_call<T, 15, FWD, BWD>(buf, tl, pl, op); break;
+    default: line_middle_call<T, 16, FWD, BWD>(buf, tl, pl, op); break;
+    }
+    if (BWD) {
+        int S = tl.n / pl.r(pl.nf - 1);
+        for (int i = pl.nf - 2; i >= 0; --i) {
+            const int r = pl.r(i);
+            S /= r;
+            line_pass_by<T, true>(r, buf, tl, tl.n / (S * r), S, tw);
+        }
+    }
+}
+
+// The tile elements of one thread in the global order: columns with
+// consecutive threads on consecutive sequences, rows on consecutive points.
+// (b, p) is the current element, at() its place in the tile; next() moves on.
+struct LineIter {
+    LineTile tl;
+    FastDiv dl;
+    int b, p, db, dp;
+    __device__ __forceinline__ explicit LineIter(const LineTile &t) : tl(t), dl(t.rl)
+    {
+        const int tid = threadIdx.x, nt = blockDim.x;
+        if (tl.row) {
+            b = tid / tl.n;
+            p = tid - b * tl.n;
+            db = nt / tl.n;
+            dp = nt - db * tl.n;
+        } else {
+            b = tid & ((1 << tl.logb) - 1);
+            p = tid >> tl.logb;
+            db = 0;
+            dp = nt >> tl.logb;  // at least 1: a block has 32 threads or more, a tile at most 16 columns
+        }
+    }
+    __device__ __forceinline__ void next()
+    {
+        b += db;
+        p += dp;
+        if (tl.row && p >= tl.n) {
+            p -= tl.n;
+            ++b;
+        }
+    }
+    __device__ __forceinline__ bool in() const { return tl.row ? b < (1 << tl.logb) : p < tl.n; }
+    __device__ __forceinline__ int at() const { return (p + (tl.pad ? dl.div(p) : 0)) * tl.bp + b; }
+};
+
+// f(b, p, at) for every tile element of the thread in batches of U: load
+// reads into v, use consumes (loads of a batch before its stores).
+template <int U, typename V, class Load, class Use> __device__ __forceinline__ void line_batches(const LineTile &tl, Load load, Use use)
+{
+    LineIter it(tl);
+    while (it.in()) {
+        V v[U];
+        int b[U], p[U], at[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            b[u] = -1;
+            if (it.in()) {
+                b[u] = it.b;
+                p[u] = it.p;
+                at[u] = it.at();
+                load(it.b, it.p, v[u]);
+            }
+            it.next();
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (b[u] >= 0) use(b[u], p[u], at[u], v[u]);
+    }
+}
+
+// Host: log2 of the lines per CTA: at most 2^maxlog, halved down to 2^minlog
+// while the launch has fewer than four CTAs per SM (152 SMs) or a tile more
+// than 40 KB; then doubled while the launch has more than maxblocks CTAs per
+// run.  batch: launches of nseq lines side by side (runs, fields).
+inline int line_logb(bool row, int n, LinePlan pl, long long nseq, int batch, size_t elem, int maxlog, int minlog, long long maxblocks)
+{
+    auto tiles = [&](int l) { return (nseq + (1 << l) - 1) >> l; };
+    int l = maxlog;
+    while (l > 0 && LineTile(row, n, l, pl).points() * elem > 40 * 1024) --l;
+    while (l > minlog && tiles(l) * batch < 4 * 152) --l;
+    while (tiles(l) > maxblocks) ++l;
+    return l;
+}
+// Host: threads of a tile, one butterfly of the first pass each, in whole warps
+inline int line_threads(int n, int r0, int logb)
+{
+    const int t = (((n / r0) << logb) + 31) / 32 * 32;
+    return t > 256 ? 256 : t;
+}
+
 } // namespace epdlb

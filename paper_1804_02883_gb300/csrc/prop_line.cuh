@@ -52,26 +52,6 @@ __host__ __device__ inline double weight_b(int j, int na, int ns, double ds)
     return (j == na || j == ns) ? 0.5 * ds : ds;
 }
 
-// log2 of the lines per CTA: at most 2^maxlog, halved down to 2^minlog while
-// the launch has fewer than four CTAs per SM (152 SMs) or a tile more than
-// 40 KB; then doubled while the launch has more than maxblocks CTAs per run
-// (the partials a row pass writes).
-inline int line_logb(bool row, int n, LinePlan pl, long long nseq, int nruns, size_t elem, int maxlog, int minlog, long long maxblocks)
-{
-    auto tiles = [&](int l) { return (nseq + (1 << l) - 1) >> l; };
-    int l = maxlog;
-    while (l > 0 && LineTile(row, n, l, pl).points() * elem > 40 * 1024) --l;
-    while (l > minlog && tiles(l) * nruns < 4 * 152) --l;
-    while (tiles(l) > maxblocks) ++l;
-    return l;
-}
-// threads of a tile: one butterfly of the first pass each, in whole warps
-inline int line_threads(int n, int r0, int logb)
-{
-    const int t = (((n / r0) << logb) + 31) / 32 * 32;
-    return t > 256 ? 256 : t;
-}
-
 // Launches of one contour step are dependents of the one before
 // (griddepcontrol): the next one's CTAs are placed while its last CTAs finish.
 __device__ __forceinline__ void line_dependents()
