@@ -1285,6 +1285,7 @@ static size_t carve_solve(Group &G, char *base)
 {
     const size_t n = (size_t)G.g.n;
     const size_t tb = G.prec == EPD_LB_MIXED_FP32 ? sizeof(float) : sizeof(double);
+    G.stateless = true;
     size_t off = 0;
     auto take = [&](size_t bytes) -> void * {
         off = align_up(off);

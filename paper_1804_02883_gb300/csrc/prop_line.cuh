@@ -27,6 +27,7 @@ template <typename T> struct PropK {
     double *ia, *ib, *part;
     const V2<T> *twx, *twy;
     const T *kx, *ky;
+    bool dependent;  // launches as programmatic dependents (see line_dependents)
 };
 
 // Boltzmann factor (E_A, E_B) of the half-step at node j of chain g (fac_g)
@@ -52,8 +53,14 @@ __host__ __device__ inline double weight_b(int j, int na, int ns, double ds)
     return (j == na || j == ns) ? 0.5 * ds : ds;
 }
 
-// Launches of one contour step are dependents of the one before
-// (griddepcontrol): the next one's CTAs are placed while its last CTAs finish.
+// The launches of a stateless solve are programmatic dependents of the one
+// before: the next one's CTAs are placed while its last CTAs finish (128 x 128,
+// N_s = 64: 1.03 -> 0.75 ms; 48 x 90 x 96 box 0.95 -> 0.80 ms).  Inside a
+// handle's captured step they are not: there the graph already launches
+// back to back (alone 14.4 against 14.1 ms on 64 x 150 x 150, 17.0 against 17.7
+// in FP64 on 4 x 256 x 512), and with several handles on one GPU the waiting
+// CTAs hold the other graphs' launches up (three 64 x 64 FP64 handles: 5.2 ms
+// a pass without, 8.4 with).
 __device__ __forceinline__ void line_dependents()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -220,7 +227,7 @@ __global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, Row
 }
 
 template <typename K, typename... A>
-cudaError_t launch_line(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
+cudaError_t launch_line(bool dependent, K kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -231,7 +238,7 @@ cudaError_t launch_line(K kernel, dim3 grid, int threads, size_t smem, cudaStrea
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -244,13 +251,13 @@ template <typename T> cudaError_t line_col_t(const PropK<T> &k, cudaStream_t s)
     const size_t sm = LineTile(false, n, l, k.g.py).points() * sizeof(V2<T>);
     const int th = line_threads(n, r0, l);
     switch (r0) {
-    case 2: return launch_line(prop_col<T, 2>, grid, th, sm, s, k, l);
-    case 4: return launch_line(prop_col<T, 4>, grid, th, sm, s, k, l);
-    case 6: return launch_line(prop_col<T, 6>, grid, th, sm, s, k, l);
-    case 8: return launch_line(prop_col<T, 8>, grid, th, sm, s, k, l);
-    case 10: return launch_line(prop_col<T, 10>, grid, th, sm, s, k, l);
-    case 12: return launch_line(prop_col<T, 12>, grid, th, sm, s, k, l);
-    default: return launch_line(prop_col<T, 16>, grid, th, sm, s, k, l);
+    case 2: return launch_line(k.dependent, prop_col<T, 2>, grid, th, sm, s, k, l);
+    case 4: return launch_line(k.dependent, prop_col<T, 4>, grid, th, sm, s, k, l);
+    case 6: return launch_line(k.dependent, prop_col<T, 6>, grid, th, sm, s, k, l);
+    case 8: return launch_line(k.dependent, prop_col<T, 8>, grid, th, sm, s, k, l);
+    case 10: return launch_line(k.dependent, prop_col<T, 10>, grid, th, sm, s, k, l);
+    case 12: return launch_line(k.dependent, prop_col<T, 12>, grid, th, sm, s, k, l);
+    default: return launch_line(k.dependent, prop_col<T, 16>, grid, th, sm, s, k, l);
     }
 }
 
@@ -266,13 +273,13 @@ template <typename T, bool DIFF> cudaError_t line_row_t(const PropK<T> &k, int m
     const RowWeights w = {weight_a(m, na, ds), weight_b(m, na, ns, ds), s2 == m ? 0.0 : weight_a(s2, na, ds),
                           s2 == m ? 0.0 : weight_b(s2, na, ns, ds)};
     switch (r0) {
-    case 2: return launch_line(prop_row<T, 2, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 4: return launch_line(prop_row<T, 4, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 6: return launch_line(prop_row<T, 6, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 8: return launch_line(prop_row<T, 8, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 10: return launch_line(prop_row<T, 10, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 12: return launch_line(prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
-    default: return launch_line(prop_row<T, 16, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 2: return launch_line(k.dependent, prop_row<T, 2, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 4: return launch_line(k.dependent, prop_row<T, 4, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 6: return launch_line(k.dependent, prop_row<T, 6, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 8: return launch_line(k.dependent, prop_row<T, 8, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 10: return launch_line(k.dependent, prop_row<T, 10, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 12: return launch_line(k.dependent, prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
+    default: return launch_line(k.dependent, prop_row<T, 16, DIFF>, grid, th, sm, s, k, m, l, w);
     }
 }
 
