@@ -80,13 +80,15 @@ size_t carve_group(Group &G, char *base, size_t off)
     // cluster solve (MIXED_FP32): stored states of both chains, and the
     // differential second solve's buffers; streaming MIXED solves: the
     // changes at every node and the factor changes
-    G.hc = G.hd = G.rho = G.cdiff = nullptr;
+    G.hc = G.hd = G.rho = G.cdiff = G.facp = G.facd = nullptr;
     if (cluster) {
         const size_t hs = R * cluster_state_floats2(G.g.nx, G.g.ny, G.g.ns) * sizeof(float2);
         G.hc = take(hs);
         G.hd = take(hs);
         G.rho = take(R * n * sizeof(float2));
         G.cdiff = take(R * 3 * n * sizeof(float));
+        G.facp = take(R * 3 * n * sizeof(float));
+        G.facd = take(R * 3 * n * sizeof(float));
     } else if (stream_diff) {
         G.hd = take(R * (size_t)(G.g.ns + 1) * n * sizeof(float2));
         G.rho = take(R * n * sizeof(float2));
@@ -141,6 +143,8 @@ static Group run_view(const Group &G, int r)
         V.hd = (char *)V.hd + (size_t)r * hs;
         V.rho = (char *)V.rho + (size_t)r * n * sizeof(float2);
         V.cdiff = (char *)V.cdiff + (size_t)r * 3 * n * sizeof(float);
+        V.facp = (char *)V.facp + (size_t)r * 3 * n * sizeof(float);
+        V.facd = (char *)V.facd + (size_t)r * 3 * n * sizeof(float);
     } else if (G.hd) {
         V.hd = (char *)V.hd + (size_t)r * (G.g.ns + 1) * n * sizeof(float2);
         V.rho = (char *)V.rho + (size_t)r * n * sizeof(float2);

@@ -228,6 +228,7 @@ template <typename T, bool INV> struct DftN<T, 15, INV> : DftPf<T, 3, 5, INV> {}
 // consecutive points (the global order) where the legs are far enough apart.
 // No access then meets the same bank more than twice.
 struct LineTile {
+    static constexpr bool fixed = false;
     int n, logb, bp, rl, pad;
     bool row;
     __host__ __device__ LineTile(bool row_, int n_, int logb_, LinePlan pl)
@@ -238,15 +239,65 @@ struct LineTile {
     // distance of points M apart (M a multiple of rl)
     __device__ int leg(int M) const { return (M + pad * (M / rl)) * bp; }
 };
+// The same with everything known at compile time, for the power-of-two axes
+// of the streaming solves: offsets become immediates, indices shifts, loops
+// straight code (a third fewer instructions per point than above).
+// NT: threads of the block.
+constexpr int ct_radix(int logn, int i)
+{
+    // 64 = 8.8, 128 = 16.8, 256 = 16.16, 512 = 8.8.8, 1024 = 16.8.8, 2048 = 16.8.16
+    constexpr int plan[6][4] = {{2, 8, 8, 0}, {2, 16, 8, 0}, {2, 16, 16, 0}, {3, 8, 8, 8}, {3, 16, 8, 8}, {3, 16, 8, 16}};
+    return plan[logn - 6][i + 1];
+}
+template <int LOGN> struct LinePlanCT {
+    static constexpr int nf = ct_radix(LOGN, -1);
+    static __host__ __device__ constexpr int r(int i) { return ct_radix(LOGN, i); }
+};
+template <int LOGN, int LOGB, bool ROW, int NT> struct LineTileCT {
+    static constexpr bool fixed = true;
+    static constexpr int n = 1 << LOGN, logb = LOGB, bp = ROW ? (1 << LOGB) | 1 : 1 << LOGB;
+    static constexpr int rl = LinePlanCT<LOGN>::r(LinePlanCT<LOGN>::nf - 1), pad = 1, nt = NT;
+    static constexpr bool row = ROW;
+    static constexpr int POINTS = (n + n / rl) * bp;
+    static __device__ constexpr int leg(int M) { return (M + M / rl) * bp; }
+};
+// a / d of a tile: shifts where d is known, FastDiv otherwise
+template <class Tile> struct TileDiv {
+    FastDiv f;
+    __device__ __forceinline__ explicit TileDiv(int d) : f(d) {}
+    __device__ __forceinline__ int div(int a) const { return f.div(a); }
+    __device__ __forceinline__ int d() const { return f.d; }
+};
+template <int LOGN, int LOGB, bool ROW, int NT> struct TileDiv<LineTileCT<LOGN, LOGB, ROW, NT>> {
+    int v;
+    __device__ __forceinline__ explicit TileDiv(int d) : v(d) {}
+    __device__ __forceinline__ int div(int a) const { return (int)((unsigned)a / (unsigned)v); }  // a shift once inlined
+    __device__ __forceinline__ int d() const { return v; }
+};
+// f(bf) for the thread's butterflies bf < total
+template <class Tile, class F> __device__ __forceinline__ void line_for(const Tile &, int total, F f)
+{
+    if constexpr (Tile::fixed) {
+        if (total % Tile::nt == 0) {
+#pragma unroll
+            for (int i = 0; i < total / Tile::nt; ++i) f((int)threadIdx.x + i * Tile::nt);
+        } else if ((int)threadIdx.x < total) {  // fewer butterflies than threads
+            f((int)threadIdx.x);
+        }
+    } else {
+        for (int bf = threadIdx.x; bf < total; bf += blockDim.x) f(bf);
+    }
+}
 // sequence b and butterfly t of butterfly number bf (dq.d per sequence)
-__device__ __forceinline__ void line_split(const LineTile &tl, bool bfast, const FastDiv &dq, int bf, int &b, int &t)
+template <class Tile>
+__device__ __forceinline__ void line_split(const Tile &tl, bool bfast, const TileDiv<Tile> &dq, int bf, int &b, int &t)
 {
     if (bfast) {
         b = bf & ((1 << tl.logb) - 1);
         t = bf >> tl.logb;
     } else {
         b = dq.div(bf);
-        t = bf - b * dq.d;
+        t = bf - b * dq.d();
     }
 }
 
@@ -264,43 +315,70 @@ __device__ __forceinline__ int line_bin(LinePlan pl, int n, int p)
     return k;
 }
 
-// Twiddles of a butterfly, w[u] = tw[u j] (tw[i] = exp(-2 pi i i / n)), read
-// before its points: with few warps per SM the reads' latency is exposed, and
-// taken one by one next to their uses it cost the FP64 passes 40%.
-template <int R, typename V> __device__ __forceinline__ void line_twiddles(V (&w)[R], const V *__restrict__ tw, int j)
-{
+// Twiddles of a butterfly, tw[u j] (tw[i] = exp(-2 pi i i / n)), read before
+// its points: with few warps per SM the reads' latency is exposed, and taken
+// one by one next to their uses it cost the FP64 passes 40%.  PROD: the powers
+// of two are read, the others are products, w_u = w_(u mod 8) w_(u - u mod 8)
+// (power-of-two axes in FP32: a gather at stride u j touches a line per lane,
+// and fewer factors stay in registers).
+template <int R, bool PROD, typename V> struct LineTw {
+    V w[R];
+    __device__ __forceinline__ LineTw(const V *__restrict__ tw, int j)
+    {
 #pragma unroll
-    for (int u = 1; u < R; ++u) w[u] = __ldg(&tw[u * j]);
-}
+        for (int u = 1; u < R; ++u) w[u] = __ldg(&tw[u * j]);
+    }
+    __device__ __forceinline__ V get(int u) const { return w[u]; }
+};
+template <int R, typename V> struct LineTw<R, true, V> {
+    static constexpr int NA = R < 8 ? R : 8, NB = (R + 7) / 8;
+    V a[NA], b[NB];
+    __device__ __forceinline__ LineTw(const V *__restrict__ tw, int j)
+    {
+        a[1] = __ldg(&tw[j]);
+        if constexpr (R > 2) a[2] = __ldg(&tw[2 * j]);
+        if constexpr (R > 4) a[4] = __ldg(&tw[4 * j]);
+        if constexpr (R > 8) b[1] = __ldg(&tw[8 * j]);
+        if constexpr (R > 3) a[3] = cmul(a[1], a[2]);
+        if constexpr (R > 5) a[5] = cmul(a[1], a[4]);
+        if constexpr (R > 6) a[6] = cmul(a[2], a[4]);
+        if constexpr (R > 7) a[7] = cmul(a[3], a[4]);
+    }
+    __device__ __forceinline__ V get(int u) const
+    {
+        if (u < 8) return a[u];
+        return u % 8 ? cmul(b[u / 8], a[u % 8]) : b[u / 8];
+    }
+};
 
 // One pass: radix R, M = points between the legs of a butterfly, S = product
 // of the radices before it; tw[i] = exp(-2 pi i i / n).
-template <typename T, int R, bool INV>
-__device__ __forceinline__ void line_pass(V2<T> *buf, LineTile tl, int M, int S, const V2<T> *__restrict__ tw)
+template <typename T, int R, bool INV, class Tile>
+__device__ __forceinline__ void line_pass(V2<T> *buf, Tile tl, int M, int S, const V2<T> *__restrict__ tw)
 {
     const int q = tl.n / R, total = q << tl.logb, leg = tl.leg(M);
-    const FastDiv dq(q), dm(M), dl(tl.rl);
-    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+    const TileDiv<Tile> dq(q), dm(M), dl(tl.rl);
+    line_for(tl, total, [&](int bf) {
         int b, t;
         line_split(tl, !tl.row || M < 8, dq, bf, b, t);
         const int blk = dm.div(t), j = t - blk * M;
         V2<T> *p = buf + (j + (tl.pad ? dl.div(j) : 0)) * tl.bp + blk * R * leg + b;
-        V2<T> x[R], w[R];
-        line_twiddles(w, tw, j * S);
+        V2<T> x[R];
+        const LineTw<R, Tile::fixed && sizeof(T) == 4, V2<T>> w(tw, j * S);
 #pragma unroll
         for (int u = 0; u < R; ++u) x[u] = p[u * leg];
         if (INV) {
 #pragma unroll
-            for (int u = 1; u < R; ++u) x[u] = cmul_conj(x[u], w[u]);
+            for (int u = 1; u < R; ++u) x[u] = cmul_conj(x[u], w.get(u));
             DftN<T, R, true>::run(x);
         } else {
             DftN<T, R, false>::run(x);
 #pragma unroll
-            for (int u = 1; u < R; ++u) x[u] = cmul(x[u], w[u]);
+            for (int u = 1; u < R; ++u) x[u] = cmul(x[u], w.get(u));
         }
 #pragma unroll
         for (int u = 0; u < R; ++u) p[u * leg] = x[u];
-    }
+    });
     __syncthreads();
 }
 
@@ -308,17 +386,19 @@ __device__ __forceinline__ void line_pass(V2<T> *buf, LineTile tl, int M, int S,
 // op(op.pre(b, bin), v): the operator applied to natural bin `bin` of
 // sequence b (pre: what it reads from memory, ahead of the points).
 // FWD, BWD: which halves run.
-template <typename T, int R, bool FWD, bool BWD, class Op>
-__device__ __forceinline__ void line_middle(V2<T> *buf, LineTile tl, LinePlan pl, const Op &op)
+template <typename T, int R, bool FWD, bool BWD, class Op, class Tile, class Plan>
+__device__ __forceinline__ void line_middle(V2<T> *buf, Tile tl, Plan pl, const Op &op)
 {
     const int q = tl.n / R, total = q << tl.logb;
-    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+    line_for(tl, total, [&](int bf) {
         const int b = bf & ((1 << tl.logb) - 1), t = bf >> tl.logb;
         int bin = t;  // digits of the block, reversed (one radix before the last: the digit itself)
         if (pl.nf > 2) {
             int m = q, p = t, s = 1;
             bin = 0;
-            for (int i = 0; i + 1 < pl.nf; ++i) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                if (i + 1 >= pl.nf) break;
                 m /= pl.r(i);
                 const int v = p / m;
                 p -= v * m;
@@ -339,12 +419,12 @@ __device__ __forceinline__ void line_middle(V2<T> *buf, LineTile tl, LinePlan pl
         if (BWD) DftN<T, R, true>::run(x);
 #pragma unroll
         for (int u = 0; u < R; ++u) p[u * tl.bp] = x[u];
-    }
+    });
     __syncthreads();
 }
 
-template <typename T, bool INV>
-__device__ __forceinline__ void line_pass_any(int R, V2<T> *buf, LineTile tl, int M, int S, const V2<T> *tw)
+template <typename T, bool INV, class Tile>
+__device__ __forceinline__ void line_pass_any(int R, V2<T> *buf, Tile tl, int M, int S, const V2<T> *tw)
 {
     switch (R) {
     case 3: line_pass<T, 3, INV>(buf, tl, M, S, tw); break;
@@ -354,9 +434,13 @@ __device__ __forceinline__ void line_pass_any(int R, V2<T> *buf, LineTile tl, in
     default: line_pass<T, 9, INV>(buf, tl, M, S, tw); break;
     }
 }
-template <typename T, bool FWD, bool BWD, class Op>
-__device__ __forceinline__ void line_middle_any(V2<T> *buf, LineTile tl, LinePlan pl, const Op &op)
+template <typename T, bool FWD, bool BWD, class Op, class Tile, class Plan>
+__device__ __forceinline__ void line_middle_any(V2<T> *buf, Tile tl, Plan pl, const Op &op)
 {
+    if constexpr (Tile::fixed) {
+        line_middle<T, Plan::r(Plan::nf - 1), FWD, BWD>(buf, tl, pl, op);
+        return;
+    }
     switch (pl.r(pl.nf - 1)) {
     case 1: line_middle<T, 1, FWD, BWD>(buf, tl, pl, op); break;
     case 2: line_middle<T, 2, FWD, BWD>(buf, tl, pl, op); break;
@@ -371,9 +455,14 @@ __device__ __forceinline__ void line_middle_any(V2<T> *buf, LineTile tl, LinePla
     }
 }
 // The passes between the first and the middle one, forward or back.
-template <typename T, bool INV>
-__device__ __forceinline__ void line_inner(V2<T> *buf, LineTile tl, LinePlan pl, const V2<T> *tw)
+template <typename T, bool INV, class Tile, class Plan>
+__device__ __forceinline__ void line_inner(V2<T> *buf, Tile tl, Plan pl, const V2<T> *tw)
 {
+    if constexpr (Tile::fixed) {
+        static_assert(Plan::nf <= 3, "at most one pass between");
+        if constexpr (Plan::nf == 3) line_pass<T, Plan::r(1), INV>(buf, tl, Plan::r(2), Plan::r(0), tw);
+        return;
+    }
     if (!INV) {
         int S = pl.r(0);
         for (int i = 1; i + 1 < pl.nf; ++i) {
@@ -392,47 +481,47 @@ __device__ __forceinline__ void line_inner(V2<T> *buf, LineTile tl, LinePlan pl,
 }
 // First pass of a forward transform (R0 = the plan's first radix):
 // src(b, t, q, x) gives the points t + u q, u < R0, of sequence b.
-template <typename T, int R0, class Src>
-__device__ __forceinline__ void line_open(V2<T> *buf, LineTile tl, const V2<T> *__restrict__ tw, const Src &src)
+template <typename T, int R0, class Src, class Tile>
+__device__ __forceinline__ void line_open(V2<T> *buf, Tile tl, const V2<T> *__restrict__ tw, const Src &src)
 {
     const int q = tl.n / R0, total = q << tl.logb, leg = tl.leg(q);
-    const FastDiv dq(q), dl(tl.rl);
-    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+    const TileDiv<Tile> dq(q), dl(tl.rl);
+    line_for(tl, total, [&](int bf) {
         int b, t;
         line_split(tl, !tl.row, dq, bf, b, t);
-        V2<T> x[R0], w[R0];
+        V2<T> x[R0];
         src(b, t, q, x);
-        line_twiddles(w, tw, t);
+        const LineTw<R0, Tile::fixed && sizeof(T) == 4, V2<T>> w(tw, t);
         DftN<T, R0, false>::run(x);
         V2<T> *p = buf + (t + (tl.pad ? dl.div(t) : 0)) * tl.bp + b;
         p[0] = x[0];
 #pragma unroll
-        for (int u = 1; u < R0; ++u) p[u * leg] = cmul(x[u], w[u]);
-    }
+        for (int u = 1; u < R0; ++u) p[u * leg] = cmul(x[u], w.get(u));
+    });
     __syncthreads();
 }
 // Last pass of an inverse transform: sink(b, t, q, x) takes the points t + u q.
-template <typename T, int R0, class Sink>
-__device__ __forceinline__ void line_close(const V2<T> *buf, LineTile tl, const V2<T> *__restrict__ tw, const Sink &sink)
+template <typename T, int R0, class Sink, class Tile>
+__device__ __forceinline__ void line_close(const V2<T> *buf, Tile tl, const V2<T> *__restrict__ tw, const Sink &sink)
 {
     const int q = tl.n / R0, total = q << tl.logb, leg = tl.leg(q);
-    const FastDiv dq(q), dl(tl.rl);
-    for (int bf = threadIdx.x; bf < total; bf += blockDim.x) {
+    const TileDiv<Tile> dq(q), dl(tl.rl);
+    line_for(tl, total, [&](int bf) {
         int b, t;
         line_split(tl, !tl.row, dq, bf, b, t);
         const V2<T> *p = buf + (t + (tl.pad ? dl.div(t) : 0)) * tl.bp + b;
-        V2<T> x[R0], w[R0];
-        line_twiddles(w, tw, t);
+        V2<T> x[R0];
+        const LineTw<R0, Tile::fixed && sizeof(T) == 4, V2<T>> w(tw, t);
         x[0] = p[0];
 #pragma unroll
-        for (int u = 1; u < R0; ++u) x[u] = cmul_conj(p[u * leg], w[u]);
+        for (int u = 1; u < R0; ++u) x[u] = cmul_conj(p[u * leg], w.get(u));
         DftN<T, R0, true>::run(x);
         sink(b, t, q, x);
-    }
+    });
 }
 // Forward transform, operator, inverse transform of the tile's sequences.
-template <typename T, int R0, class Src, class Op, class Sink>
-__device__ __forceinline__ void line_pair(V2<T> *buf, LineTile tl, LinePlan pl, const V2<T> *tw, const Src &src, const Op &op,
+template <typename T, int R0, class Src, class Op, class Sink, class Tile, class Plan>
+__device__ __forceinline__ void line_pair(V2<T> *buf, Tile tl, Plan pl, const V2<T> *tw, const Src &src, const Op &op,
                                           const Sink &sink)
 {
     line_open<T, R0>(buf, tl, tw, src);

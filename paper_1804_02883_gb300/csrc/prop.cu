@@ -36,12 +36,19 @@ template <typename T> __device__ __forceinline__ T exp_t(T v);
 template <> __device__ __forceinline__ float exp_t<float>(float v) { return expf(v); }
 template <> __device__ __forceinline__ double exp_t<double>(double v) { return exp(v); }
 
+// Place of site i in the packed-row layout of the cluster solve, in floats
+// (site (y, x) -> packed row y / 2, component y & 1; power-of-two grids).
+__device__ __forceinline__ size_t packed_site(const GroupGeom &g, long long i)
+{
+    const long long y = i >> g.logx, x = i & (g.nx - 1);
+    return (size_t)((y >> 1) * g.nx + x) * 2 + (y & 1);
+}
+
 // Boltzmann factors E_{A,B} = exp(-N w_{A,B} ds / 2) and exp(-w_S) in the bulk
 // precision; exp(-w_S) into the S slot of phi_out and its block sums for Q_S
-// (per-thread sums of at most a few terms in the bulk type, FP64 across
-// threads and blocks).
+// in FP64.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) prop_prep(GroupGeom g, const double *omega, V2<T> *efac, double *phi_out, double *part)
+__global__ void __launch_bounds__(kThreads) prop_prep(GroupGeom g, const double *omega, V2<T> *efac, T *fac, double *phi_out, double *part)
 {
     __shared__ double red[32];
     const int run = blockIdx.y;
@@ -49,15 +56,23 @@ __global__ void __launch_bounds__(kThreads) prop_prep(GroupGeom g, const double 
     const double *wa = omega + (size_t)run * 3 * n, *wb = wa + n, *ws = wb + n;
     double *es = phi_out + (size_t)run * 3 * n + 2 * n;
     const T c = (T)(-0.5 * g.nseg * g.ds);
-    T acc = 0;
+    double acc = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        efac[(size_t)run * n + i] = mk<T>(exp_t<T>(c * (T)wa[i]), exp_t<T>(c * (T)wb[i]));
+        const T ea = exp_t<T>(c * (T)wa[i]), eb = exp_t<T>(c * (T)wb[i]);
+        efac[(size_t)run * n + i] = mk<T>(ea, eb);
+        if (fac) {  // node factors of the cluster solve
+            const size_t o = packed_site(g, i), hn = (size_t)n;
+            T *f = fac + (size_t)run * 3 * hn;
+            f[o] = ea * ea;
+            f[hn + o] = eb * eb;
+            f[2 * hn + o] = ea * eb;
+        }
         // exp(-w_S) in the bulk precision (FP32 in MIXED_FP32), kept in FP64
-        const T e = exp_t<T>(-(T)ws[i]);
-        es[i] = (double)e;
+        const double e = (double)exp_t<T>(-(T)ws[i]);
+        es[i] = e;
         acc += e;
     }
-    const double s = block_sum((double)acc, red);
+    const double s = block_sum(acc, red);
     if (threadIdx.x == 0) part[(size_t)run * kMaxPart + kMaxPart / 2 + blockIdx.x] = s;
 }
 
@@ -126,7 +141,8 @@ __global__ void __launch_bounds__(kThreads) prop_finalize(GroupGeom g, int nrow_
 // rounding of FP32 relative to the change itself.  The solvent change de goes
 // to the S slot of phi, its block sums to the S partials.
 __global__ void __launch_bounds__(kThreads) prop_prep_delta(GroupGeom g, const double *omega, const double *omega_t,
-                                                            float2 *rho, float *cdiff, double *phi_out, double *part)
+                                                            float2 *rho, float *cdiff, const float2 *efac, float *fac,
+                                                            double *phi_out, double *part)
 {
     __shared__ double red[32];
     const int run = blockIdx.y;
@@ -135,191 +151,34 @@ __global__ void __launch_bounds__(kThreads) prop_prep_delta(GroupGeom g, const d
     const double *ta = omega_t + (size_t)run * 3 * n, *tb = ta + n, *ts = tb + n;
     double *ds_out = phi_out + (size_t)run * 3 * n + 2 * n;
     const float c = (float)(-0.5 * g.nseg * g.ds);
-    float acc = 0.f;
+    double acc = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float da = (float)(wa[i] - ta[i]), db = (float)(wb[i] - tb[i]);
         const float qa = expm1f(c * da), qb = expm1f(c * db);
         rho[(size_t)run * n + i] = make_float2(qa, qb);
         if (cdiff) {
-            // (1 + rho_d)(1 + rho_a) - 1 for the block pairs (A, A), (B, B),
-            // (A, B) of a node's departing and arriving half-steps, in the
-            // packed-row layout of the cluster solve (site (y, x) -> packed
-            // row y / 2, component y & 1; power-of-two grids: shift and mask)
-            const long long y = i >> g.logx, x = i & (g.nx - 1), hn = n / 2;
-            const size_t o = (size_t)((y >> 1) * g.nx + x) * 2 + (y & 1);
-            cdiff[((size_t)run * 3 + 0) * hn * 2 + o] = qa * (2.f + qa);
-            cdiff[((size_t)run * 3 + 1) * hn * 2 + o] = qb * (2.f + qb);
-            cdiff[((size_t)run * 3 + 2) * hn * 2 + o] = qa + qb + qa * qb;
+            // (1 + rho_d)(1 + rho_a) - 1 and the node factors E'_d E'_a for the
+            // block pairs (A, A), (B, B), (A, B) of a node's departing and
+            // arriving half-steps, in the packed-row layout
+            const size_t o = packed_site(g, i), hn = (size_t)n;
+            float *cd = cdiff + (size_t)run * 3 * hn, *f = fac + (size_t)run * 3 * hn;
+            cd[o] = qa * (2.f + qa);
+            cd[hn + o] = qb * (2.f + qb);
+            cd[2 * hn + o] = qa + qb + qa * qb;
+            const float2 e = efac[(size_t)run * n + i];
+            const float pa = 1.f + qa, pb = 1.f + qb;
+            f[o] = e.x * e.x * (pa * pa);
+            f[hn + o] = e.y * e.y * (pb * pb);
+            f[2 * hn + o] = e.x * e.y * (pa * pb);
         }
         // e~_S exactly as the first solve formed it
         const float es = expf(-(float)ts[i]);
-        const float de = es * expm1f(-(float)(ws[i] - ts[i]));
-        ds_out[i] = (double)de;
+        const double de = (double)(es * expm1f(-(float)(ws[i] - ts[i])));
+        ds_out[i] = de;
         acc += de;
     }
-    const double s = block_sum((double)acc, red);
+    const double s = block_sum(acc, red);
     if (threadIdx.x == 0) part[(size_t)run * kMaxPart + kMaxPart / 2 + blockIdx.x] = s;
-}
-
-// ---------------------------------------------------------------------------
-// Streaming passes on radix-8 tiles (MIXED_FP32, grids too large for the
-// cluster-resident solve, 64..2048 points per axis).  The chain z = g + i g'
-// is transformed by column tiles then row tiles per contour step, as above;
-// the row pass stores z at every node (full history, FP32), and the contour
-// sums are one pass over the history afterwards (prop_contour_stream):
-// I(r) = sum_j w_j g(s_j) g'(1 - s_j) with g'(1 - s_j) the g' chain at its
-// node N_s - j.
-// ---------------------------------------------------------------------------
-
-struct Stream8K {
-    GroupGeom g;
-    float2 *chain;        // [run][n]
-    float2 *hist;         // [run][N_s + 1][n] (the reference of a differential solve)
-    float2 *hd;           // differential solve: (dg, dg') at every node, [run][N_s + 1][n]
-    const float2 *rho;    // differential solve: (rho_A, rho_B), [run][n]
-    const float2 *efac;   // [run][n]
-    double *part;
-    const float2 *twx, *twy;  // pass tables of each axis' best radix plan (fft8.cuh layout)
-    const float2 *twy8, *twy16;  // column tables of the radix-8 and radix-16 plans (tile-dependent)
-    const float *kx, *ky;
-};
-
-// node 0: g = g' = 1; chain <- E(s_0) z_0 (differential solve: change 0,
-// chain d a_0 = E rho of the departing half-step)
-template <bool DIFF>
-__global__ void __launch_bounds__(kThreads) prop_start8(Stream8K k)
-{
-    const int run = blockIdx.y;
-    const long long n = k.g.n;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float2 e = k.efac[(size_t)run * n + i];
-        if (!DIFF) {
-            k.hist[(size_t)run * (k.g.ns + 1) * n + i] = make_float2(1.f, 1.f);
-            k.chain[(size_t)run * n + i] = make_float2(fac_g<float>(e, k.g, 0, false), fac_gp<float>(e, k.g, 0, false));
-        } else {
-            const float2 q = k.rho[(size_t)run * n + i];
-            k.hd[(size_t)run * (k.g.ns + 1) * n + i] = make_float2(0.f, 0.f);
-            k.chain[(size_t)run * n + i] = make_float2(fac_g<float>(e, k.g, 0, false) * fac_g<float>(q, k.g, 0, false),
-                                                       fac_gp<float>(e, k.g, 0, false) * fac_gp<float>(q, k.g, 0, false));
-        }
-    }
-}
-
-template <int LOGY, int CW>
-__global__ void __launch_bounds__(ColTile<LOGY, CW>::T) prop_col8(Stream8K k)
-{
-    using CT = ColTile<LOGY, CW>;
-    using CL = ColLayout<LOGY, CT::C>;
-    constexpr int NY = CT::NY, C = CT::C, P = CT::P, T = CT::T;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *buf = reinterpret_cast<float2 *>(smem_raw);
-    const int nx = k.g.nx, run = blockIdx.y, x0 = blockIdx.x * C, tid = threadIdx.x;
-    float2 *data = k.chain + (size_t)run * k.g.n;
-#pragma unroll
-    for (int u = 0; u < P / T; ++u) {
-        const int i = tid + u * T;
-        buf[i] = data[(size_t)(i / C) * nx + x0 + (i % C)];
-    }
-    __syncthreads();
-    // twiddle tables and Fourier factors straight from global memory (L1):
-    // shared memory holds only the tile, so more tiles are in flight per SM
-    transform_pair<LOGY, T, CL, P, ScaleBins, CT::MR>(buf, CT::MR == 4 ? k.twy16 : k.twy8, ScaleBins{k.ky}, tid);
-    constexpr int RLOG_L = inv_rlog(LOGY, npasses(LOGY, CT::MR) - 1, CT::MR), RR = 1 << RLOG_L, PER_L = NY / RR, NB_L = P / RR / T;
-    float2 h[NB_L][RR];
-    int bb[NB_L], tt[NB_L];
-    last_inverse<LOGY, NB_L, T, CL, CT::MR>(buf, h, bb, tt, tid);
-#pragma unroll
-    for (int j = 0; j < NB_L; ++j)
-#pragma unroll
-        for (int r = 0; r < RR; ++r) data[(size_t)(tt[j] + r * PER_L) * nx + x0 + bb[j]] = h[j][r];
-}
-
-// Row pass of contour node m: Tx, node factors, history store, next half
-// step; at m = N_s block sums of g for Q_P.  Differential solve (DIFF): the
-// chain carries d a; dg_m = E'_a U + rho_a g~_m is stored, the chain goes on
-// with d a_m = E'_d dg_m + E_d rho_d g~_m (as in prop_row), dQ_P partials.
-template <int LOGX, bool DIFF>
-__global__ void __launch_bounds__(RowTile<LOGX>::T) prop_row8(Stream8K k, int m)
-{
-    using RT = RowTile<LOGX>;
-    using RL = RowLayout<LOGX>;
-    constexpr int NX = RT::NX, P = RT::P, T = RT::T;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[32];
-    float2 *buf = reinterpret_cast<float2 *>(smem_raw);
-    const int run = blockIdx.y, tid = threadIdx.x;
-    const long long n = k.g.n, base = (long long)blockIdx.x * P;
-    const int ns = k.g.ns;
-    float2 *data = k.chain + (size_t)run * n + base;
-#pragma unroll
-    for (int u = 0; u < P / T; ++u) {
-        const int i = tid + u * T;
-        buf[RL::at(i / NX, i % NX)] = data[i];
-    }
-    __syncthreads();
-    transform_pair<LOGX, T, RL, P, ScaleBins, RT::MR>(buf, k.twx, ScaleBins{k.kx}, tid);
-    constexpr int RLOG_L = inv_rlog(LOGX, npasses(LOGX, RT::MR) - 1, RT::MR), RR = 1 << RLOG_L, PER_L = NX / RR, NB_L = P / RR / T;
-    float2 h[NB_L][RR];
-    int bb[NB_L], tt[NB_L];
-    last_inverse<LOGX, NB_L, T, RL, RT::MR>(buf, h, bb, tt, tid);
-    const float2 *efac = k.efac + (size_t)run * n + base;
-    float2 *hist = k.hist + ((size_t)run * (ns + 1) + m) * n + base;
-    float qsum = 0.f;
-    // per batch of RR points: every load first, then the stores (the
-    // history and chain stores could alias the inputs as far as the compiler
-    // knows, which would serialise each load behind the previous stores)
-    if (DIFF) {
-        const float2 *rho = k.rho + (size_t)run * n + base;
-        float2 *hd = k.hd + ((size_t)run * (ns + 1) + m) * n + base;
-#pragma unroll
-        for (int j = 0; j < NB_L; ++j) {
-            float2 e[RR], q[RR], gr[RR];
-#pragma unroll
-            for (int r = 0; r < RR; ++r) {
-                const int i = bb[j] * NX + tt[j] + r * PER_L;
-                e[r] = efac[i];
-                q[r] = rho[i];
-                gr[r] = hist[i];
-            }
-#pragma unroll
-            for (int r = 0; r < RR; ++r) {
-                const int i = bb[j] * NX + tt[j] + r * PER_L;
-                const float2 u = h[j][r];
-                const float ea = fac_g<float>(e[r], k.g, m, true), eap = fac_gp<float>(e[r], k.g, m, true);
-                const float qa = fac_g<float>(q[r], k.g, m, true), qap = fac_gp<float>(q[r], k.g, m, true);
-                const float2 dg = make_float2(ea * (1.f + qa) * u.x + qa * gr[r].x, eap * (1.f + qap) * u.y + qap * gr[r].y);
-                hd[i] = dg;
-                if (m == ns) {
-                    qsum += dg.x;
-                } else {
-                    const float ed = fac_g<float>(e[r], k.g, m, false), edp = fac_gp<float>(e[r], k.g, m, false);
-                    const float qd = fac_g<float>(q[r], k.g, m, false), qdp = fac_gp<float>(q[r], k.g, m, false);
-                    data[i] = make_float2(ed * (1.f + qd) * dg.x + ed * qd * gr[r].x,
-                                          edp * (1.f + qdp) * dg.y + edp * qdp * gr[r].y);
-                }
-            }
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < NB_L; ++j) {
-            float2 e[RR];
-#pragma unroll
-            for (int r = 0; r < RR; ++r) e[r] = efac[bb[j] * NX + tt[j] + r * PER_L];
-#pragma unroll
-            for (int r = 0; r < RR; ++r) {
-                const int i = bb[j] * NX + tt[j] + r * PER_L;
-                const float eg = fac_g<float>(e[r], k.g, m, true), egp = fac_gp<float>(e[r], k.g, m, true);
-                const float2 z = make_float2(eg * h[j][r].x, egp * h[j][r].y);
-                hist[i] = z;
-                if (m == ns) qsum += z.x;
-                else data[i] = make_float2(fac_g<float>(e[r], k.g, m, false) * z.x, fac_gp<float>(e[r], k.g, m, false) * z.y);
-            }
-        }
-    }
-    if (m == ns) {
-        const double s = block_sum((double)qsum, red);
-        if (tid == 0) k.part[(size_t)run * kMaxPart + blockIdx.x] = s;
-    }
 }
 
 // Contour sums and normalisation over the full history (Eqs. (9)-(11)):
@@ -439,172 +298,7 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
     }
 }
 
-// The contour loop of the radix-8 streaming solve for (LX, LY), column tiles
-// of CW columns (diff: the differential solve's row passes).
-template <int LX, int LY, int CW>
-static void stream8_run(Stream8K &k, const Group &G, cudaStream_t s, const SolveProbe *probe, bool diff)
-{
-    using RT = RowTile<LX>;
-    using CT = ColTile<LY, CW>;
-    const size_t sr = (size_t)RT::ROWS * RowLayout<LX>::PITCH * sizeof(float2), sc = (size_t)CT::P * sizeof(float2);
-    static std::atomic<bool> conf{false};  // attribute set (idempotent if two threads race)
-    if (!conf) {
-        cudaFuncSetAttribute(prop_row8<LX, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
-        cudaFuncSetAttribute(prop_row8<LX, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sr);
-        cudaFuncSetAttribute(prop_col8<LY, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
-        conf = true;
-    }
-    const dim3 gr((unsigned)(G.g.n / RT::P), G.g.nruns), gc(G.g.nx / CT::C, G.g.nruns);
-    for (int m = 1; m <= G.g.ns; ++m) {
-        const bool pa = probe && m == probe->m_acc, ps = probe && m == probe->m_store;
-        if (pa) cudaEventRecordWithFlags(probe->ev[2], s, cudaEventRecordExternal);
-        prop_col8<LY, CW><<<gc, CT::T, sc, s>>>(k);
-        if (pa) cudaEventRecordWithFlags(probe->ev[3], s, cudaEventRecordExternal);
-        if (ps) cudaEventRecordWithFlags(probe->ev[0], s, cudaEventRecordExternal);
-        if (diff) prop_row8<LX, true><<<gr, RT::T, sr, s>>>(k, m);
-        else prop_row8<LX, false><<<gr, RT::T, sr, s>>>(k, m);
-        if (ps) cudaEventRecordWithFlags(probe->ev[1], s, cudaEventRecordExternal);
-        if (pa) cudaEventRecordWithFlags(probe->ev[4], s, cudaEventRecordExternal);
-    }
-}
-template <int LX, int LY>
-static bool stream8_dispatch_y(int logy, Stream8K &k, const Group &G, cudaStream_t s, const SolveProbe *probe, bool diff)
-{
-    if constexpr (LY > 11) {
-        return false;
-    } else {
-        if (logy != LY) return stream8_dispatch_y<LX, LY + 1>(logy, k, G, s, probe, diff);
-        switch (G.colw_prop) {
-        case 4: stream8_run<LX, LY, 4>(k, G, s, probe, diff); break;
-        case 8: stream8_run<LX, LY, 8>(k, G, s, probe, diff); break;
-        case 16: stream8_run<LX, LY, 16>(k, G, s, probe, diff); break;
-        default: stream8_run<LX, LY, ColTile<LY>::C>(k, G, s, probe, diff); break;
-        }
-        return true;
-    }
-}
-template <int LX>
-static bool stream8_dispatch(int logx, int logy, Stream8K &k, const Group &G, cudaStream_t s, const SolveProbe *probe,
-                             bool diff = false)
-{
-    if constexpr (LX > 11) {
-        return false;
-    } else {
-        if (logx != LX) return stream8_dispatch<LX + 1>(logx, logy, k, G, s, probe, diff);
-        return stream8_dispatch_y<LX, 6>(logy, k, G, s, probe, diff);
-    }
-}
-
-static Stream8K stream8_args(const Group &G)
-{
-    Stream8K k8;
-    k8.g = G.g;
-    k8.chain = reinterpret_cast<float2 *>(G.chain);
-    k8.hist = reinterpret_cast<float2 *>(G.hist);
-    k8.hd = reinterpret_cast<float2 *>(G.hd);
-    k8.rho = reinterpret_cast<const float2 *>(G.rho);
-    k8.efac = reinterpret_cast<const float2 *>(G.efac);
-    k8.part = G.part;
-    k8.twx = best_mr(G.g.logx) == 4 ? G.tab16x : G.tab8x;
-    k8.twy = best_mr(G.g.logy) == 4 ? G.tab16y : G.tab8y;
-    k8.twy8 = G.tab8y;
-    k8.twy16 = G.tab16y;
-    k8.kx = reinterpret_cast<const float *>(G.kx);
-    k8.ky = reinterpret_cast<const float *>(G.ky);
-    return k8;
-}
-
-// Column tile autotuner of the streaming propagator column pass (see
-// tune_column_tiles): times prop_col8 at each width on the group's chain
-// buffer (scratch until the next solve starts it) and keeps the fastest.
-template <int LY>
-static float time_col8(int w, Stream8K &k, const Group &G, cudaStream_t s, cudaEvent_t a, cudaEvent_t b)
-{
-    auto one = [&](auto tag) {
-        constexpr int CW = decltype(tag)::value;
-        using CT = ColTile<LY, CW>;
-        const size_t sc = (size_t)CT::P * sizeof(float2);
-        if (sc > 227 * 1024 ||
-            cudaFuncSetAttribute(prop_col8<LY, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc) != cudaSuccess) {
-            cudaGetLastError();  // this width does not fit: not a candidate
-            return 1e30f;
-        }
-        const dim3 gc(G.g.nx / CT::C, G.g.nruns);
-        float best = 1e30f;
-        for (int rep = 0; rep < 4; ++rep) {
-            cudaEventRecord(a, s);
-            prop_col8<LY, CW><<<gc, CT::T, sc, s>>>(k);
-            cudaEventRecord(b, s);
-            cudaEventSynchronize(b);
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, a, b);
-            if (rep > 0 && ms < best) best = ms;
-        }
-        return cudaGetLastError() == cudaSuccess ? best : 1e30f;
-    };
-    switch (w) {
-    case 4: return one(std::integral_constant<int, 4>{});
-    case 8: return one(std::integral_constant<int, 8>{});
-    default: return one(std::integral_constant<int, 16>{});
-    }
-}
-template <int LY>
-static int tune_col8_at(int logy, Stream8K &k, const Group &G, cudaStream_t s)
-{
-    if constexpr (LY > 11) {
-        return 0;
-    } else {
-        if (logy != LY) return tune_col8_at<LY + 1>(logy, k, G, s);
-        cudaEvent_t a, b;
-        if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) return 0;
-        float best = 1e30f;
-        int best_w = 0;
-        for (int w : kColWidths) {
-            if (G.g.nx % w) continue;
-            const float t = time_col8<LY>(w, k, G, s, a, b);
-            if (t < best) {
-                best = t;
-                best_w = w;
-            }
-        }
-        cudaEventDestroy(a);
-        cudaEventDestroy(b);
-        return best_w;
-    }
-}
-
-cudaError_t tune_stream_tiles(Group &G, cudaStream_t s)
-{
-    if (!(G.prec == EPD_LB_MIXED_FP32 && G.hist_full && G.tab8x)) return cudaSuccess;
-    if (const char *env = std::getenv("EPD_LB_COLUMN_TILE")) {
-        const int w = std::atoi(env);
-        if (w == 4 || w == 8 || w == 16) {
-            G.colw_prop = w;
-            return cudaSuccess;
-        }
-    }
-    Stream8K k8 = stream8_args(G);
-    cudaError_t e = cudaMemsetAsync(G.chain, 0, (size_t)G.g.nruns * G.g.n * sizeof(float2), s);
-    if (e != cudaSuccess) return e;
-    G.colw_prop = tune_col8_at<6>(G.g.logy, k8, G, s);
-    return cudaGetLastError();
-}
-
-bool stream8_eligible(int prec, int logx, int logy)
-{
-    return prec == EPD_LB_MIXED_FP32 && !cluster_shape_exists(logx, logy) && logx >= 6 && logy >= 6 && logx <= 11 &&
-           logy <= 11 && logx + logy >= 11;
-}
-
-static int grid_for(long long n)
-{
-    long long b = (n + kThreads - 1) / kThreads;
-    if (b > 1024) b = 1024;
-    return (int)b;
-}
-
-template <typename T>
-static PropK<T> prop_args(const Group &G)
+template <typename T> static PropK<T> prop_args(const Group &G)
 {
     PropK<T> k;
     k.g = G.g;
@@ -625,22 +319,93 @@ static PropK<T> prop_args(const Group &G)
     return k;
 }
 
-// Q partial blocks of the radix-8 row pass (one per row tile)
-static int stream8_row_blocks(const GroupGeom &g) { return (int)(g.n / (g.nx >= 2048 ? g.nx : 2048)); }
+// Column tile autotuner of the power-of-two streaming column pass (see
+// tune_column_tiles): times it at each width on the group's chain buffer
+// (scratch until the next solve starts it) and keeps the fastest.
+cudaError_t tune_stream_tiles(Group &G, cudaStream_t s)
+{
+    if (!(G.prec == EPD_LB_MIXED_FP32 && G.hist_full)) return cudaSuccess;
+    if (const char *env = std::getenv("EPD_LB_COLUMN_TILE")) {
+        const int w = std::atoi(env);
+        if ((w == 4 || w == 8 || w == 16) && stream_col_fits(G.g.ny, w)) {
+            G.colw_prop = w;
+            return cudaSuccess;
+        }
+    }
+    const PropK<float> k = prop_args<float>(G);
+    cudaError_t e = cudaMemsetAsync(G.chain, 0, (size_t)G.g.nruns * G.g.n * sizeof(float2), s);
+    if (e != cudaSuccess) return e;
+    cudaEvent_t a, b;
+    if ((e = cudaEventCreate(&a)) != cudaSuccess) return e;
+    if ((e = cudaEventCreate(&b)) != cudaSuccess) {
+        cudaEventDestroy(a);
+        return e;
+    }
+    float best = 1e30f;
+    for (int w : kColWidths) {
+        if (!stream_col_fits(G.g.ny, w)) continue;
+        for (int rep = 0; rep < 4 && !e; ++rep) {
+            cudaEventRecord(a, s);
+            e = stream_col(k, w, s);
+            cudaEventRecord(b, s);
+            cudaEventSynchronize(b);
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, a, b);
+            if (!e && rep > 0 && ms < best) {
+                best = ms;
+                G.colw_prop = w;
+            }
+        }
+    }
+    cudaEventDestroy(a);
+    cudaEventDestroy(b);
+    return e ? e : cudaGetLastError();
+}
 
-// The contour loop of the generic streaming solve (column pass, row pass per
-// node); blocks: the Q partials of the last row pass per run.
+bool stream8_eligible(int prec, int logx, int logy)
+{
+    return prec == EPD_LB_MIXED_FP32 && !cluster_shape_exists(logx, logy) && logx >= 6 && logy >= 6 && logx <= 11 &&
+           logy <= 11 && logx + logy >= 11;
+}
+
+// Blocks of the pointwise passes: four sites per thread (the FP64 block sums
+// of the solvent factor cost ten FP64 additions per thread), at most 1024.
+// Depends on one run's grid only: so does the order of the sums.
+static int grid_for(long long n)
+{
+    const long long b = (n + 4 * kThreads - 1) / (4 * kThreads);
+    return (int)(b > 1024 ? 1024 : b);
+}
+
+// One pass of either axis: compile-time tiles on the power-of-two FP32 grids
+// that have them (hist_full), the general passes otherwise.
+static cudaError_t col_pass(const PropK<float> &k, const Group &G, cudaStream_t s)
+{
+    return G.hist_full ? stream_col(k, G.colw_prop, s) : line_col(k, s);
+}
+static cudaError_t col_pass(const PropK<double> &k, const Group &, cudaStream_t s) { return line_col(k, s); }
+static cudaError_t row_pass(const PropK<float> &k, const Group &G, int m, bool diff, int *blocks, cudaStream_t s)
+{
+    return G.hist_full ? stream_row(k, m, diff, blocks, s) : line_row(k, m, diff, blocks, s);
+}
+static cudaError_t row_pass(const PropK<double> &k, const Group &, int m, bool diff, int *blocks, cudaStream_t s)
+{
+    return line_row(k, m, diff, blocks, s);
+}
+
+// The contour loop of the streaming solves (column pass, row pass per node);
+// blocks: the Q partials of the last row pass per run.
 template <typename T>
-static cudaError_t generic_loop(const PropK<T> &k, bool diff, int *blocks, cudaStream_t s, const SolveProbe *probe)
+static cudaError_t generic_loop(const Group &G, const PropK<T> &k, bool diff, int *blocks, cudaStream_t s, const SolveProbe *probe)
 {
     cudaError_t e = cudaSuccess;
     for (int m = 1; m <= k.g.ns && !e; ++m) {
         const bool pa = probe && m == probe->m_acc, ps = probe && m == probe->m_store;
         if (pa) cudaEventRecordWithFlags(probe->ev[2], s, cudaEventRecordExternal);
-        e = line_col(k, s);
+        e = col_pass(k, G, s);
         if (pa) cudaEventRecordWithFlags(probe->ev[3], s, cudaEventRecordExternal);
         if (ps) cudaEventRecordWithFlags(probe->ev[0], s, cudaEventRecordExternal);
-        if (!e) e = line_row(k, m, diff, blocks, s);
+        if (!e) e = row_pass(k, G, m, diff, blocks, s);
         if (ps) cudaEventRecordWithFlags(probe->ev[1], s, cudaEventRecordExternal);
         if (pa) cudaEventRecordWithFlags(probe->ev[4], s, cudaEventRecordExternal);
     }
@@ -654,23 +419,14 @@ static cudaError_t solve_t(Group &G, const double *omega, double *phi, double *q
     PropK<T> k = prop_args<T>(G);
 
     const int pg = grid_for(g.n);
-    prop_prep<T><<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, omega, reinterpret_cast<V2<T> *>(G.efac), phi, G.part);
+    prop_prep<T><<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, omega, reinterpret_cast<V2<T> *>(G.efac), reinterpret_cast<T *>(G.facp), phi, G.part);
     if (sizeof(T) == sizeof(float) && G.hc && G.twx_full && cluster_solve_supported(G)) {
         // whole contour in one cluster-resident launch, then the contour sums
         return launch_cluster_solve(G, s, false, pg, phi, q, probe);
     }
-    if (sizeof(T) == sizeof(float) && G.hist_full && G.tab8x) {
-        // radix-8 streaming passes with the full history, then the contour pass
-        Stream8K k8 = stream8_args(G);
-        prop_start8<false><<<dim3(pg, g.nruns), kThreads, 0, s>>>(k8);
-        if (!stream8_dispatch<6>(g.logx, g.logy, k8, G, s, probe)) return cudaErrorInvalidConfiguration;
-        prop_contour_stream<false><<<dim3((unsigned)((g.n + kThreads - 1) / kThreads), g.nruns), kThreads, 0, s>>>(
-            g, k8.hist, nullptr, stream8_row_blocks(g), pg, G.part, phi, q, nullptr, nullptr, G.err);
-        return cudaGetLastError();
-    }
     prop_start<T, false><<<dim3(pg, g.nruns), kThreads, 0, s>>>(k);
     int blocks = 0;
-    if (cudaError_t e = generic_loop<T>(k, false, &blocks, s, probe)) return e;
+    if (cudaError_t e = generic_loop<T>(G, k, false, &blocks, s, probe)) return e;
     if (sizeof(T) == sizeof(float) && k.hnodes == g.ns + 1)  // full history: the sums are one pass over it
         prop_contour_stream<false><<<dim3((unsigned)((g.n + kThreads - 1) / kThreads), g.nruns), kThreads, 0, s>>>(
             g, reinterpret_cast<const float2 *>(G.hist), nullptr, blocks, pg, G.part, phi, q, nullptr, nullptr, G.err);
@@ -687,18 +443,10 @@ static cudaError_t stream_delta(Group &G, int pg, double *phi, double *q, const 
 {
     const GroupGeom &g = G.g;
     const dim3 gcon((unsigned)((g.n + kThreads - 1) / kThreads), g.nruns);
-    if (G.hist_full && G.tab8x) {
-        Stream8K k8 = stream8_args(G);
-        prop_start8<true><<<dim3(pg, g.nruns), kThreads, 0, s>>>(k8);
-        if (!stream8_dispatch<6>(g.logx, g.logy, k8, G, s, probe, true)) return cudaErrorInvalidConfiguration;
-        prop_contour_stream<true><<<gcon, kThreads, 0, s>>>(g, k8.hist, k8.hd, stream8_row_blocks(g), pg, G.part, phi, q,
-                                                           phi_ref, q_ref, G.err);
-        return cudaGetLastError();
-    }
     PropK<float> k = prop_args<float>(G);
     prop_start<float, true><<<dim3(pg, g.nruns), kThreads, 0, s>>>(k);
     int blocks = 0;
-    if (cudaError_t e = generic_loop<float>(k, true, &blocks, s, probe)) return e;
+    if (cudaError_t e = generic_loop<float>(G, k, true, &blocks, s, probe)) return e;
     prop_contour_stream<true><<<gcon, kThreads, 0, s>>>(g, reinterpret_cast<const float2 *>(G.hist),
                                                        reinterpret_cast<const float2 *>(G.hd), blocks, pg, G.part, phi,
                                                        q, phi_ref, q_ref, G.err);
@@ -718,7 +466,8 @@ cudaError_t launch_solve_delta_at(Group &G, const double *omega, const double *o
     const GroupGeom &g = G.g;
     const int pg = grid_for(g.n);
     prop_prep_delta<<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, omega, omega_ref, reinterpret_cast<float2 *>(G.rho),
-                                                          reinterpret_cast<float *>(G.cdiff), phi, G.part);
+                                                          reinterpret_cast<float *>(G.cdiff), reinterpret_cast<const float2 *>(G.efac),
+                                                          reinterpret_cast<float *>(G.facd), phi, G.part);
     if (!G.hc) return stream_delta(G, pg, phi, q, phi_ref, q_ref, s, probe);
     return launch_cluster_solve(G, s, true, pg, phi, q, probe, phi_ref, q_ref);
 }
@@ -759,7 +508,7 @@ static cudaError_t solve3d_t(const Solve3 &S, const double *omega, double *phi, 
     const PropK<T> kz = view(S.vz, S.twx, S.twz, S.kx, S.kz);
     const GroupGeom &g = S.vx;
     const int pg = grid_for(g.n);
-    prop_prep<T><<<dim3(pg, 1), kThreads, 0, s>>>(g, omega, reinterpret_cast<V2<T> *>(S.efac), phi, S.part);
+    prop_prep<T><<<dim3(pg, 1), kThreads, 0, s>>>(g, omega, reinterpret_cast<V2<T> *>(S.efac), (T *)nullptr, phi, S.part);
     prop_start<T, false><<<dim3(pg, 1), kThreads, 0, s>>>(kx);
     int blocks = 0;
     cudaError_t e = cudaSuccess;

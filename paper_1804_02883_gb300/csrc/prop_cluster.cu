@@ -71,6 +71,7 @@ struct PropCK {
     const float2 *href;   // reference states a~_m (DIFF)
     const float2 *efac;   // (E_A, E_B) [run][n]
     const float2 *rho;    // (rho_A, rho_B) [run][n] (DIFF)
+    const float2 *fac;    // E_d E_a (plain) or E'_d E'_a (DIFF) for the block pairs (A,A), (B,B), (A,B), packed rows [run][3][NY/2][NX]
     const float2 *cdiff;  // (1 + rho_d)(1 + rho_a) - 1 for (A,A), (B,B), (A,B), packed rows [run][3][NY/2][NX] (DIFF)
     int *err;             // bit 2: an exchange wait gave up
     const float2 *twx, *twy;  // radix-8 pass tables (fft8.cuh layout)
@@ -94,12 +95,8 @@ struct ClusterGeom {
     static constexpr int MRX = (best_mr(LOGX) == 4 && P % (16 * T) == 0) ? 4 : 3;
     static constexpr int MRY = (best_mr(LOGY) == 4 && P % (16 * T) == 0) ? 4 : 3;
     static constexpr int TABX = tabs_total(LOGX, MRX), TABY = tabs_total(LOGY, MRY);
-    // row buffer, column buffer, pass tables, Fourier factors, the node
-    // factors of the epilogue sites in either packing (P points each; the
-    // differential solve reads the coefficients of a~ from L2, which
-    // measured faster than a shared-memory copy beside the factors)
-    static constexpr size_t SMEM =
-        (size_t)(R2 * PITCH + P + TABX + TABY + 2 * P) * sizeof(float2) + (NX + NY) * sizeof(float);
+    // row buffer, column buffer, pass tables, Fourier factors
+    static constexpr size_t SMEM = (size_t)(R2 * PITCH + P + TABX + TABY) * sizeof(float2) + (NX + NY) * sizeof(float);
     static constexpr size_t SMEM_DIFF = SMEM;
 };
 
@@ -206,10 +203,6 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
     float2 *taby = tabx + G::TABX;
     float *kx = reinterpret_cast<float *>(taby + G::TABY);
     float *ky = kx + NX;
-    // node factors of the two real sites of each epilogue point, thread-major
-    // ([point of the thread][thread]: conflict-free), rows then columns:
-    // E_d E_a (plain) or E'_d E'_a (DIFF)
-    float2 *fac_r = reinterpret_cast<float2 *>(ky + NY), *fac_c = fac_r + P;
     cg::cluster_group cl = cg::this_cluster();
     const int crank = (int)cl.block_rank();
     const int slot = blockIdx.x / C;
@@ -233,6 +226,7 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
     // [NY/2][NX]; rho (2 + rho) of blocks A, B in the same layout
     float2 *hout = k.hout + (size_t)(run * 2 + chain) * (ns + 1) * HN;
     const float2 *href = DIFF ? k.href + (size_t)(run * 2 + chain) * (ns + 1) * HN : nullptr;
+    const float2 *fac = k.fac + (size_t)run * 3 * HN;
     const float2 *cdiff = DIFF ? k.cdiff + (size_t)run * 3 * HN : nullptr;
 
     // blocks of the two half-step factors at contour node j of this chain
@@ -279,75 +273,22 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
     constexpr int RLOG_C = inv_rlog(LOGY, npasses(LOGY, G::MRY) - 1, G::MRY), RC = 1 << RLOG_C, PER_C = NY / RC;
     constexpr int NB_C = P / RC / T;
     static_assert(PER_C % 2 == 0 && (P / RC) % 32 == 0, "column pairs of the last column pass");
-    // per-site factors E^2 (plain) or E'^2 (DIFF) of this thread's epilogue
-    // sites in either packing (fac_r, fac_c), reloaded when the block (A or
-    // B) changes; each thread reads only what it wrote
-    int cur_r = -1, cur_c = -1;
     int failed = 0;
-    // the factors of packed-row point (kk, x) for blocks d (departing) and a
-    // (arriving): real sites 2kk (re) and 2kk + 1 (im) of column x
-    auto factors = [&](int kk, int x, bool bd, bool ba) {
-        const int s0 = 2 * kk * NX + x;
-        const float2 e0 = efac[s0], e1 = efac[s0 + NX];
-        const float f0 = (bd ? e0.y : e0.x) * (ba ? e0.y : e0.x), f1 = (bd ? e1.y : e1.x) * (ba ? e1.y : e1.x);
-        if constexpr (!DIFF) {
-            return f2(f0, f1);
-        } else {
-            const float2 r0 = rho[s0], r1 = rho[s0 + NX];
-            return f2(f0 * ((1.f + (bd ? r0.y : r0.x)) * (1.f + (ba ? r0.y : r0.x))),
-                      f1 * ((1.f + (bd ? r1.y : r1.x)) * (1.f + (ba ? r1.y : r1.x))));
-        }
-    };
     // a_m = E_d E_a U (plain) or d a_m = E'_d E'_a U + c a~_m (DIFF) at
     // packed-row point (kk, x), U = T(a_{m-1}) there, c = (1 + rho_d)(1 +
     // rho_a) - 1 from plane cp of cdiff (0: A A, 1: B B, 2: A B)
-    auto finish = [&](float2 u, float2 f, int m, int cp, int kk, int x) {
+    auto finish = [&](float2 u, int m, int cp, int kk, int x) {
+        const size_t e = (size_t)kk * NX + x;
+        const float2 f = fac[(size_t)cp * HN + e];
         if constexpr (!DIFF) {
             return f2(f.x * u.x, f.y * u.y);
         } else {
-            const size_t e = (size_t)kk * NX + x;
             const float2 ar = href[(size_t)m * HN + e];  // a~_m
             const float2 c = cdiff[(size_t)cp * HN + e];
             return f2(f.x * u.x + c.x * ar.x, f.y * u.y + c.y * ar.y);
         }
     };
 
-    // per-site factors of this thread's epilogue points in the row packing
-    // (fac_r) and the column packing (fac_c) for blocks (bd, ba)
-    auto fill_r = [&](bool bd, bool ba) {
-#pragma unroll
-        for (int j = 0; j < NB_L; ++j) {
-            int b, t;
-            RL::template split<PER_L>(bfly<true, NB_L, T>(tid, j), b, t);
-#pragma unroll
-            for (int r = 0; r < RR; ++r) fac_r[(j * RR + r) * T + tid] = factors(krow0 + b, t + r * PER_L, bd, ba);
-        }
-    };
-    auto fill_c = [&](bool bd, bool ba) {
-#pragma unroll
-        for (int j = 0; j < NB_C; ++j) {
-            int c, t;
-            col_pair_split<W2>(tid + j * T, c, t);
-#pragma unroll
-            for (int r = 0; r < RC; ++r) {
-                const int kk = (t + r * PER_C) >> 1, xx = 2 * (jcol0 + c) + (t & 1);
-                fac_c[(j * RC + r) * T + tid] = factors(kk, xx, bd, ba);
-            }
-        }
-    };
-    // The factors of the first step (both packings; they depend only on the
-    // fields of this solve, final before the first launch), then the state
-    // the previous launch of a phased schedule stored: a launch made as a
-    // programmatic dependent of the previous one runs this prologue while
-    // that one finishes, and waits for it only here (griddepcontrol.wait
-    // returns at once in a launch without that dependency).
-    if (nsteps > 0) {
-        const int m1 = m_begin + 1;
-        const int bd1 = dep_b(m1), ba1 = arr_b(m1);
-        fill_r(bd1, ba1);
-        fill_c(bd1, ba1);
-        cur_r = cur_c = 2 * bd1 + ba1;
-    }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -393,13 +334,16 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
         const bool second = hs & 1, cols = starts_in_columns(m) != second;
         const unsigned par = (unsigned)(i >> 1) & 1u;  // uses of this step's barrier so far in this launch
         const bool rearm = i + 2 < nsteps;
-        const int bd = dep_b(m), ba = arr_b(m), key = 2 * bd + ba, cp = bd == ba ? bd : 2;
-        if (DIFF && !second) {
+        const int bd = dep_b(m), ba = arr_b(m), cp = bd == ba ? bd : 2;
+        if (!second) {
             // a~_m and c of this step's epilogue sites into L1 ahead of use
             // (the packing the step ends in)
             auto pf = [&](size_t e) {
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(href + (size_t)m * HN + e));
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(cdiff + (size_t)cp * HN + e));
+                if (DIFF) {
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(href + (size_t)m * HN + e));
+                    asm volatile("prefetch.global.L1 [%0];" ::"l"(cdiff + (size_t)cp * HN + e));
+                }
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(fac + (size_t)cp * HN + e));
             };
             if (cols) {
 #pragma unroll
@@ -456,16 +400,12 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
             } else {
                 // node factors in the packed-row form (x = 2J + (y & 1) of
                 // packed row y / 2), the result back in the column buffer
-                if (key != cur_c) {
-                    cur_c = key;
-                    fill_c(bd, ba);
-                }
 #pragma unroll
                 for (int j = 0; j < NB_C; ++j)
 #pragma unroll
                     for (int r = 0; r < RC; ++r) {
                         const int kk = (ct[j] + r * PER_C) >> 1, xx = 2 * (jcol0 + cc[j]) + (ct[j] & 1);
-                        x[j][r] = finish(pair_transpose<16>(x[j][r], ct[j] & 1), fac_c[(j * RC + r) * T + tid], m, cp, kk, xx);
+                        x[j][r] = finish(pair_transpose<16>(x[j][r], ct[j] & 1), m, cp, kk, xx);
                     }
                 __syncthreads();  // every thread has read its columns: they are rewritten below
 #pragma unroll
@@ -504,16 +444,12 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
                 if (tid == 0 && rearm) mbar_expect(bar_col, XBYTES);
             } else {
                 // node factors; the result stays in the row buffer
-                if (key != cur_r) {
-                    cur_r = key;
-                    fill_r(bd, ba);
-                }
                 // every value first: the stores come after
 #pragma unroll
                 for (int j = 0; j < NB_L; ++j)
 #pragma unroll
                     for (int r = 0; r < RR; ++r)
-                        h[j][r] = finish(h[j][r], fac_r[(j * RR + r) * T + tid], m, cp, krow0 + bb[j], tt[j] + r * PER_L);
+                        h[j][r] = finish(h[j][r], m, cp, krow0 + bb[j], tt[j] + r * PER_L);
 #pragma unroll
                 for (int j = 0; j < NB_L; ++j)
 #pragma unroll
@@ -639,7 +575,7 @@ template <bool DIFF>
 __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
 {
     extern __shared__ __align__(16) float2 stg[];
-    __shared__ double bc;
+    __shared__ double bc, fac[4];
     const int run = blockIdx.y;
     const int nx = k.g.nx, ny = k.g.ny, ns = k.g.ns, na = k.g.na;
     const long long n = k.g.n;
@@ -681,22 +617,25 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
     constexpr int NST = CS::NSTAGE;
 #pragma unroll
     for (int c = 0; c < NST; ++c) issue(c, c * U);
+    // The FP64 divisions by one thread per block: at 2 FP64 lanes per SM the
+    // four or five of every thread were 40% of this kernel (plain pass 65 ->
+    // 47 us, differential 96 -> 84 us on 4 x 256 x 512, N_s = 64, cold).
     const double *pr = k.part + (size_t)run * kMaxPart;
-    const double sq = sum_partials(pr, k.nq, 1, &bc) / (double)n;
-    const double ss = sum_partials(pr + kMaxPart / 2, k.ns_part, 1, &bc) / (double)n;
-    double qp, qs;
-    if (DIFF) {
-        qp = k.q_t[2 * run] + sq;
-        qs = k.q_t[2 * run + 1] + ss;
-    } else {
-        qp = sq;
-        qs = ss;
+    const double tp = sum_partials(pr, k.nq, 1, &bc), ts = sum_partials(pr + kMaxPart / 2, k.ns_part, 1, &bc);
+    if (tid == 0) {
+        const double sq = tp / (double)n, ss = ts / (double)n;
+        const double qp = DIFF ? k.q_t[2 * run] + sq : sq, qs = DIFF ? k.q_t[2 * run + 1] + ss : ss;
+        fac[0] = k.g.phi_p * k.g.ds / qp;
+        fac[1] = (1.0 - k.g.phi_p) / qs;
+        fac[2] = sq / qp;
+        fac[3] = ss / qs;
+        if (blockIdx.x == 0) {
+            k.q[2 * run] = qp;
+            k.q[2 * run + 1] = qs;
+            if (!(qp > 0.0) || !(qs > 0.0) || !isfinite(qp) || !isfinite(qs)) atomicOr(k.err, 1);
+        }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        k.q[2 * run] = qp;
-        k.q[2 * run + 1] = qs;
-        if (!(qp > 0.0) || !(qs > 0.0) || !isfinite(qp) || !isfinite(qs)) atomicOr(k.err, 1);
-    }
+    __syncthreads();
     if (!valid) {
         cp_async_wait<0>();
         return;
@@ -774,27 +713,26 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
         issue(st, (ch + NST) * U);  // this stage's values are consumed
     }
     const double ia0 = sa0.value(), ib0 = sb0.value(), ia1 = sa1.value(), ib1 = sb1.value();
-    const double ds = k.g.ds, php = k.g.phi_p;
+    const double cp = fac[0], cs_ = fac[1];
     double *pa = k.phi + (size_t)run * 3 * n, *pb = pa + n, *ps = pb + n;
     if (!DIFF) {
-        const double c = php * ds / qp;
-        pa[s0] = c * ia0;
-        pb[s0] = c * ib0;
-        pa[s1] = c * ia1;
-        pb[s1] = c * ib1;
-        const double cs_ = (1.0 - php) / qs;
+        pa[s0] = cp * ia0;
+        pb[s0] = cp * ib0;
+        pa[s1] = cp * ia1;
+        pb[s1] = cp * ib1;
         ps[s0] *= cs_;
         ps[s1] *= cs_;
     } else {
         // Phi = Phi~ + (phi_p dI - Phi~ dQ) / (Q~ + dQ), the solvent with de
         const double *ta = k.phi_t + (size_t)run * 3 * n, *tb = ta + n, *tsol = tb + n;
-        const double rq = 1.0 / qp, rqs = 1.0 / qs, c = php * ds;
-        pa[s0] = ta[s0] + (c * ia0 - ta[s0] * sq) * rq;
-        pb[s0] = tb[s0] + (c * ib0 - tb[s0] * sq) * rq;
-        pa[s1] = ta[s1] + (c * ia1 - ta[s1] * sq) * rq;
-        pb[s1] = tb[s1] + (c * ib1 - tb[s1] * sq) * rq;
-        ps[s0] = tsol[s0] + ((1.0 - php) * ps[s0] - tsol[s0] * ss) * rqs;
-        ps[s1] = tsol[s1] + ((1.0 - php) * ps[s1] - tsol[s1] * ss) * rqs;
+        const double rp = fac[2], rs_ = fac[3];
+        const double a0 = ta[s0], a1 = ta[s1], b0 = tb[s0], b1 = tb[s1], t0 = tsol[s0], t1 = tsol[s1], e0_ = ps[s0], e1_ = ps[s1];
+        pa[s0] = a0 + (cp * ia0 - a0 * rp);
+        pb[s0] = b0 + (cp * ib0 - b0 * rp);
+        pa[s1] = a1 + (cp * ia1 - a1 * rp);
+        pb[s1] = b1 + (cp * ib1 - b1 * rp);
+        ps[s0] = t0 + (cs_ * e0_ - t0 * rs_);
+        ps[s1] = t1 + (cs_ * e1_ - t1 * rs_);
     }
 }
 
@@ -955,6 +893,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     k.efac = reinterpret_cast<const float2 *>(G.efac);
     k.rho = reinterpret_cast<const float2 *>(G.rho);
     k.cdiff = reinterpret_cast<const float2 *>(G.cdiff);
+    k.fac = reinterpret_cast<const float2 *>(diff ? G.facd : G.facp);
     k.err = G.err;
     k.twx = sh->mrx == 4 ? G.tab16x : G.tab8x;
     k.twy = sh->mry == 4 ? G.tab16y : G.tab8y;

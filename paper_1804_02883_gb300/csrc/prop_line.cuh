@@ -74,26 +74,26 @@ template <typename T> struct LineScale {  // the Fourier factor of Eq. (8)
     __device__ __forceinline__ V2<T> operator()(T f, V2<T> v) const { return cscale(v, f); }
 };
 
-// Column pass: Ty = IFFT_y Ky FFT_y on 2^logb adjacent columns.
-template <typename T, int R0>
-__global__ void __launch_bounds__(256) prop_col(PropK<T> k, int logb)
+// Column pass: Ty = IFFT_y Ky FFT_y on the tile's adjacent columns.
+template <typename T, int R0, class Tile, class Plan>
+__device__ __forceinline__ void col_tile(const PropK<T> &k, const Tile &tl, const Plan &pl)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V2<T> *buf = reinterpret_cast<V2<T> *>(smem_raw);
-    const int ny = k.g.ny, nx = k.g.nx, x0 = blockIdx.x << logb;
+    const int nx = k.g.nx, x0 = blockIdx.x << tl.logb;
     V2<T> *data = k.chain + (size_t)blockIdx.y * k.g.n + x0;
     line_dependents();
     line_pair<T, R0>(
-        buf, LineTile(false, ny, logb, k.g.py), k.g.py, k.twy,
+        buf, tl, pl, k.twy,
         [&](int b, int t, int q, V2<T>(&x)[R0]) {
-            const bool in = x0 + b < nx;
+            const bool in = Tile::fixed || x0 + b < nx;  // whole tiles on power-of-two grids
             const int i0 = t * nx + b, di = q * nx;
 #pragma unroll
             for (int u = 0; u < R0; ++u) x[u] = in ? data[i0 + u * di] : mk<T>((T)0, (T)0);
         },
         LineScale<T>{k.ky},
         [&](int b, int t, int q, V2<T>(&x)[R0]) {
-            if (x0 + b >= nx) return;
+            if (!Tile::fixed && x0 + b >= nx) return;
             const int i0 = t * nx + b, di = q * nx;
 #pragma unroll
             for (int u = 0; u < R0; ++u) data[i0 + u * di] = x[u];
@@ -105,6 +105,12 @@ __global__ void __launch_bounds__(256) prop_col(PropK<T> k, int logb)
 struct RowWeights {
     double a1, b1, a2, b2;
 };
+inline RowWeights row_weights(const GroupGeom &g, int m)
+{
+    const int ns = g.ns, na = g.na, s2 = ns - m;
+    return {weight_a(m, na, g.ds), weight_b(m, na, ns, g.ds), s2 == m ? 0.0 : weight_a(s2, na, g.ds),
+            s2 == m ? 0.0 : weight_b(s2, na, ns, g.ds)};
+}
 
 // Row pass producing contour node m (1 <= m <= ns): Tx, node factors, history
 // store / contour accumulation, Q_P partial sums at m = ns, next half step.
@@ -117,13 +123,13 @@ struct RowWeights {
 // With the full history (hnodes = N_s + 1) the contour sums are a pass of
 // their own (prop_contour_stream); otherwise node m >= N_s / 2 meets its
 // mirror from the half history here.
-template <typename T, int R0, bool DIFF>
-__global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, RowWeights w)
+template <typename T, int R0, bool DIFF, class Tile, class Plan>
+__device__ __forceinline__ void row_tile(const PropK<T> &k, const Tile &tl, const Plan &pl, int m, const RowWeights &w)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     V2<T> *buf = reinterpret_cast<V2<T> *>(smem_raw);
-    const int nx = k.g.nx, ny = k.g.ny, run = blockIdx.y, y0 = blockIdx.x << logb;
+    const int nx = Tile::fixed ? tl.n : k.g.nx, ny = k.g.ny, run = blockIdx.y, y0 = blockIdx.x << tl.logb;
     const int ns = k.g.ns, na = k.g.na, jr = k.g.jr, hlo = k.g.half_lo, hhi = k.g.half_hi, s2 = ns - m;
     const long long n = k.g.n, base = (long long)y0 * nx;
     V2<T> *data = k.chain + (size_t)run * n + base;
@@ -137,16 +143,16 @@ __global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, Row
     constexpr int CH = R0 % 4 == 0 ? 4 : (R0 % 5 == 0 ? 5 : (R0 % 3 == 0 ? 3 : 2));
     line_dependents();
     line_pair<T, R0>(
-        buf, LineTile(true, nx, logb, k.g.px), k.g.px, k.twx,
+        buf, tl, pl, k.twx,
         [&](int b, int t, int q, V2<T>(&x)[R0]) {
-            const bool in = y0 + b < ny;
+            const bool in = Tile::fixed || y0 + b < ny;
             const int i0 = b * nx + t;
 #pragma unroll
             for (int u = 0; u < R0; ++u) x[u] = in ? data[i0 + u * q] : mk<T>((T)0, (T)0);
         },
         LineScale<T>{k.kx},
         [&](int b, int t, int q, V2<T>(&x)[R0]) {
-            if (y0 + b >= ny) return;
+            if (!Tile::fixed && y0 + b >= ny) return;
             const int i0 = b * nx + t;
             if constexpr (DIFF) {
                 const float2 *rho = k.rho + (size_t)run * n + base;
@@ -226,6 +232,17 @@ __global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, Row
     }
 }
 
+template <typename T, int R0>
+__global__ void __launch_bounds__(256) prop_col(PropK<T> k, int logb)
+{
+    col_tile<T, R0>(k, LineTile(false, k.g.ny, logb, k.g.py), k.g.py);
+}
+template <typename T, int R0, bool DIFF>
+__global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, RowWeights w)
+{
+    row_tile<T, R0, DIFF>(k, LineTile(true, k.g.nx, logb, k.g.px), k.g.px, m, w);
+}
+
 template <typename K, typename... A>
 cudaError_t launch_line(bool dependent, K kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
 {
@@ -263,15 +280,13 @@ template <typename T> cudaError_t line_col_t(const PropK<T> &k, cudaStream_t s)
 
 template <typename T, bool DIFF> cudaError_t line_row_t(const PropK<T> &k, int m, int *blocks, cudaStream_t s)
 {
-    const int n = k.g.nx, ny = k.g.ny, r0 = k.g.px.r(0), ns = k.g.ns, na = k.g.na;
+    const int n = k.g.nx, ny = k.g.ny, r0 = k.g.px.r(0);
     const int l = line_logb(true, n, k.g.px, ny, k.g.nruns, sizeof(V2<T>), 3, 0, kMaxPart / 2);
     const dim3 grid((ny + (1 << l) - 1) >> l, k.g.nruns);
     *blocks = (int)grid.x;
     const size_t sm = LineTile(true, n, l, k.g.px).points() * sizeof(V2<T>);
-    const int th = line_threads(n, r0, l), s2 = ns - m;
-    const double ds = k.g.ds;
-    const RowWeights w = {weight_a(m, na, ds), weight_b(m, na, ns, ds), s2 == m ? 0.0 : weight_a(s2, na, ds),
-                          s2 == m ? 0.0 : weight_b(s2, na, ns, ds)};
+    const int th = line_threads(n, r0, l);
+    const RowWeights w = row_weights(k.g, m);
     switch (r0) {
     case 2: return launch_line(k.dependent, prop_row<T, 2, DIFF>, grid, th, sm, s, k, m, l, w);
     case 4: return launch_line(k.dependent, prop_row<T, 4, DIFF>, grid, th, sm, s, k, m, l, w);
@@ -289,5 +304,11 @@ cudaError_t line_col(const PropK<float> &k, cudaStream_t s);
 cudaError_t line_col(const PropK<double> &k, cudaStream_t s);
 cudaError_t line_row(const PropK<float> &k, int m, bool diff, int *blocks, cudaStream_t s);
 cudaError_t line_row(const PropK<double> &k, int m, bool diff, int *blocks, cudaStream_t s);
+// The same on power-of-two grids of 64..2048 points per axis in FP32, on
+// compile-time tiles (prop_stream.cu); colw: columns per tile (4, 8, 16; 0: by
+// the rule of line_logb).
+cudaError_t stream_col(const PropK<float> &k, int colw, cudaStream_t s);
+cudaError_t stream_row(const PropK<float> &k, int m, bool diff, int *blocks, cudaStream_t s);
+bool stream_col_fits(int ny, int colw);  // whether a tile of colw columns fits an SM
 
 } // namespace epdlb

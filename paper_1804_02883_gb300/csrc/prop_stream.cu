@@ -1,0 +1,123 @@
+// prop_stream.cu -- the streaming propagator passes on power-of-two grids of
+// 64..2048 points per axis in FP32 (MIXED_FP32 grids without a cluster shape,
+// such as 1024 x 2048): the passes of prop_line.cuh on tiles known at compile
+// time.
+//
+// Bound: instruction issue, then the L2 traffic of the chain.  With the axis,
+// the tile and the radices fixed, offsets are immediates, and a transform pair
+// of 1024 points is eight accesses of shared memory per point and five
+// barriers (ten and nine as load, Stockham passes and store).  Radix 32 would
+// save two more of each but holds 168-250 registers: 512 x 512 (9 runs, N_s =
+// 24) 2.27 ms a step with 32.16, 2.14 with 8.8.8.  1024 x 2048, N_s = 128:
+// 8.9 -> 8.1 ms a step.
+#include "prop_line.cuh"
+
+namespace epdlb {
+namespace {
+
+template <int LOGN, int LOGB> constexpr int tile_threads()
+{
+    return ((1 << LOGN) / LinePlanCT<LOGN>::r(0)) << LOGB;
+}
+template <int LOGN, int LOGB, bool ROW> using TileOf = LineTileCT<LOGN, LOGB, ROW, tile_threads<LOGN, LOGB>()>;
+
+template <int LOGY, int LOGB>
+__global__ void __launch_bounds__(tile_threads<LOGY, LOGB>()) stream_col_k(PropK<float> k)
+{
+    col_tile<float, LinePlanCT<LOGY>::r(0)>(k, TileOf<LOGY, LOGB, false>(), LinePlanCT<LOGY>());
+}
+template <int LOGX, int LOGB, bool DIFF>
+__global__ void __launch_bounds__(tile_threads<LOGX, LOGB>()) stream_row_k(PropK<float> k, int m, RowWeights w)
+{
+    row_tile<float, LinePlanCT<LOGX>::r(0), DIFF>(k, TileOf<LOGX, LOGB, true>(), LinePlanCT<LOGX>(), m, w);
+}
+
+constexpr size_t kMaxTile = 200 * 1024;
+
+template <int LOGY, int LOGB> cudaError_t col_at(const PropK<float> &k, cudaStream_t s)
+{
+    constexpr size_t sm = (size_t)TileOf<LOGY, LOGB, false>::POINTS * sizeof(float2);
+    if constexpr (sm > kMaxTile || tile_threads<LOGY, LOGB>() > 512) {
+        return cudaErrorInvalidConfiguration;
+    } else {
+        static const cudaError_t set =
+            cudaFuncSetAttribute(stream_col_k<LOGY, LOGB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (set) return set;
+        return launch_line(k.dependent, stream_col_k<LOGY, LOGB>, dim3(k.g.nx >> LOGB, k.g.nruns), tile_threads<LOGY, LOGB>(), sm, s, k);
+    }
+}
+template <int LOGX, int LOGB> cudaError_t row_at(const PropK<float> &k, int m, bool diff, const RowWeights &w, cudaStream_t s)
+{
+    constexpr size_t sm = (size_t)TileOf<LOGX, LOGB, true>::POINTS * sizeof(float2);
+    static const cudaError_t set = [] {
+        cudaError_t e = cudaFuncSetAttribute(stream_row_k<LOGX, LOGB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        return e ? e : cudaFuncSetAttribute(stream_row_k<LOGX, LOGB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    }();
+    if (set) return set;
+    const dim3 grid(k.g.ny >> LOGB, k.g.nruns);
+    constexpr int th = tile_threads<LOGX, LOGB>();
+    return diff ? launch_line(k.dependent, stream_row_k<LOGX, LOGB, true>, grid, th, sm, s, k, m, w)
+                : launch_line(k.dependent, stream_row_k<LOGX, LOGB, false>, grid, th, sm, s, k, m, w);
+}
+
+template <int LOGY> cudaError_t col_by(const PropK<float> &k, int colw, cudaStream_t s)
+{
+    if (!colw) {
+        colw = LOGY >= 10 ? 8 : 16;
+        while (colw > 4 && (long long)(k.g.nx / colw) * k.g.nruns < 4 * 152) colw /= 2;
+    }
+    switch (colw) {
+    case 4: return col_at<LOGY, 2>(k, s);
+    case 16: return col_at<LOGY, 4>(k, s);
+    default: return col_at<LOGY, 3>(k, s);
+    }
+}
+// rows per tile: 128 threads (64 on the shortest axes); 32 or 64 threads while
+// the launch has fewer than two tiles per SM
+template <int LOGX> cudaError_t row_by(const PropK<float> &k, int m, bool diff, int *blocks, const RowWeights &w, cudaStream_t s)
+{
+    constexpr int big = LOGX == 11 ? 0 : (LOGX == 10 ? 1 : (LOGX == 9 ? 2 : 3)), small = LOGX <= 7 ? 2 : (LOGX == 8 ? 1 : 0);
+    if (big == small || (long long)(k.g.ny >> big) * k.g.nruns >= 2 * 152) {
+        *blocks = k.g.ny >> big;
+        return row_at<LOGX, big>(k, m, diff, w, s);
+    }
+    *blocks = k.g.ny >> small;
+    return row_at<LOGX, small>(k, m, diff, w, s);
+}
+
+} // namespace
+
+bool stream_col_fits(int ny, int colw)
+{
+    const int log = ilog2(ny), r0 = ct_radix(log, 0);
+    return (size_t)(ny + ny / ct_radix(log, ct_radix(log, -1) - 1)) * colw * sizeof(float2) <= kMaxTile && ny / r0 * colw <= 512;
+}
+
+cudaError_t stream_col(const PropK<float> &k, int colw, cudaStream_t s)
+{
+    switch (k.g.logy) {
+    case 6: return col_by<6>(k, colw, s);
+    case 7: return col_by<7>(k, colw, s);
+    case 8: return col_by<8>(k, colw, s);
+    case 9: return col_by<9>(k, colw, s);
+    case 10: return col_by<10>(k, colw, s);
+    case 11: return col_by<11>(k, colw, s);
+    default: return cudaErrorInvalidConfiguration;
+    }
+}
+
+cudaError_t stream_row(const PropK<float> &k, int m, bool diff, int *blocks, cudaStream_t s)
+{
+    const RowWeights w = row_weights(k.g, m);
+    switch (k.g.logx) {
+    case 6: return row_by<6>(k, m, diff, blocks, w, s);
+    case 7: return row_by<7>(k, m, diff, blocks, w, s);
+    case 8: return row_by<8>(k, m, diff, blocks, w, s);
+    case 9: return row_by<9>(k, m, diff, blocks, w, s);
+    case 10: return row_by<10>(k, m, diff, blocks, w, s);
+    case 11: return row_by<11>(k, m, diff, blocks, w, s);
+    default: return cudaErrorInvalidConfiguration;
+    }
+}
+
+} // namespace epdlb
