@@ -446,6 +446,7 @@ static void form_groups(const epd_lb_params *p, int nruns, std::vector<Group> &g
         groups[gi].run_params.push_back(p[r]);
     }
     for (auto &G : groups) {
+        G.crowded = groups.size() > 1;
         fill_geom(G);
     }
 }

@@ -81,6 +81,7 @@ struct Group {
     void *rho = nullptr;      // (rho_A, rho_B) = expm1(-N d omega ds / 2), [run][n] float2
     void *cdiff = nullptr;    // (1 + rho_d)(1 + rho_a) - 1 for (A,A), (B,B), (A,B), packed rows [run][3][ny/2][nx] float2
     void *facp = nullptr, *facd = nullptr;  // E_d E_a of a plain solve, E'_d E'_a of a differential one, for (A,A), (B,B), (A,B), packed rows as cdiff
+    bool crowded = false;     // the handle steps other groups beside this one
     bool stateless = false;   // one solve on a caller's stream, not a handle's captured step
     bool diff = false;        // the step uses the reference + differential solve pair
     bool phi_stale = false;   // omega was replaced since phi was last computed

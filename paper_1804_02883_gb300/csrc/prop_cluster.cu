@@ -95,9 +95,10 @@ struct ClusterGeom {
     static constexpr int MRX = (best_mr(LOGX) == 4 && P % (16 * T) == 0) ? 4 : 3;
     static constexpr int MRY = (best_mr(LOGY) == 4 && P % (16 * T) == 0) ? 4 : 3;
     static constexpr int TABX = tabs_total(LOGX, MRX), TABY = tabs_total(LOGY, MRY);
-    // row buffer, column buffer, pass tables, Fourier factors
+    // row buffer, column buffer, pass tables, Fourier factors; with CACHE the
+    // node factors of the epilogue sites in either packing (P points each)
     static constexpr size_t SMEM = (size_t)(R2 * PITCH + P + TABX + TABY) * sizeof(float2) + (NX + NY) * sizeof(float);
-    static constexpr size_t SMEM_DIFF = SMEM;
+    static constexpr size_t SMEM_CACHE = SMEM + (size_t)2 * P * sizeof(float2);
 };
 
 // Distributed-shared-memory pushes: st.async of 8 bytes into a CTA of the
@@ -181,8 +182,14 @@ __device__ __forceinline__ float2 pair_transpose(float2 v, bool odd)
 // exchange of the field between the packings per contour step.
 __device__ __forceinline__ bool starts_in_columns(int m) { return m & 1; }
 
-// MINB: CTAs per SM the register budget is sized for (65536 / (T MINB) each)
-template <int LOGX, int LOGY, int C, int T, int MINB, bool DIFF>
+// MINB: CTAs per SM the register budget is sized for (65536 / (T MINB) each).
+// CACHE: the node factors E_d E_a of the thread's epilogue sites are kept in
+// shared memory, refilled when the block changes (a launch that runs the whole
+// contour at one CTA per SM); otherwise they are read from their planes each
+// step (64 KB per CTA less; 128 x 128, one run: 3.31 ms per 4 steps alone,
+// cached 3.15; 4 x 256 x 512 in 8 phased launches, each of which would refill
+// them: 5.03 ms per 4 steps, cached 5.16).
+template <int LOGX, int LOGY, int C, int T, int MINB, bool DIFF, bool CACHE>
 __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
 {
     using G = ClusterGeom<LOGX, LOGY, C, T>;
@@ -203,6 +210,8 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
     float2 *taby = tabx + G::TABX;
     float *kx = reinterpret_cast<float *>(taby + G::TABY);
     float *ky = kx + NX;
+    // CACHE: thread-major ([point of the thread][thread]: conflict-free), rows then columns
+    float2 *fac_r = reinterpret_cast<float2 *>(ky + NY), *fac_c = fac_r + P;
     cg::cluster_group cl = cg::this_cluster();
     const int crank = (int)cl.block_rank();
     const int slot = blockIdx.x / C;
@@ -274,12 +283,13 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
     constexpr int NB_C = P / RC / T;
     static_assert(PER_C % 2 == 0 && (P / RC) % 32 == 0, "column pairs of the last column pass");
     int failed = 0;
+    int cur_r = -1, cur_c = -1;  // block pairs cached
     // a_m = E_d E_a U (plain) or d a_m = E'_d E'_a U + c a~_m (DIFF) at
     // packed-row point (kk, x), U = T(a_{m-1}) there, c = (1 + rho_d)(1 +
     // rho_a) - 1 from plane cp of cdiff (0: A A, 1: B B, 2: A B)
-    auto finish = [&](float2 u, int m, int cp, int kk, int x) {
+    auto finish = [&](float2 u, const float2 *cached, int m, int cp, int kk, int x) {
         const size_t e = (size_t)kk * NX + x;
-        const float2 f = fac[(size_t)cp * HN + e];
+        const float2 f = CACHE ? *cached : fac[(size_t)cp * HN + e];
         if constexpr (!DIFF) {
             return f2(f.x * u.x, f.y * u.y);
         } else {
@@ -289,6 +299,32 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
         }
     };
 
+    // fills of the cached factors: every epilogue point of the thread in the
+    // row packing (fac_r) and the column packing (fac_c)
+    auto fill_r = [&](int cp) {
+#pragma unroll
+        for (int j = 0; j < NB_L; ++j) {
+            int b, t;
+            RL::template split<PER_L>(bfly<true, NB_L, T>(tid, j), b, t);
+#pragma unroll
+            for (int r = 0; r < RR; ++r) fac_r[(j * RR + r) * T + tid] = fac[(size_t)cp * HN + (size_t)(krow0 + b) * NX + t + r * PER_L];
+        }
+    };
+    auto fill_c = [&](int cp) {
+#pragma unroll
+        for (int j = 0; j < NB_C; ++j) {
+            int c, t;
+            col_pair_split<W2>(tid + j * T, c, t);
+#pragma unroll
+            for (int r = 0; r < RC; ++r)
+                fac_c[(j * RC + r) * T + tid] =
+                    fac[(size_t)cp * HN + (size_t)((t + r * PER_C) >> 1) * NX + 2 * (jcol0 + c) + (t & 1)];
+        }
+    };
+    // A launch made as a programmatic dependent of the previous one of a phased
+    // schedule runs this prologue while that one finishes, and waits for it
+    // only here, before it reads the stored states (griddepcontrol.wait returns
+    // at once in a launch without that dependency).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -335,7 +371,7 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
         const unsigned par = (unsigned)(i >> 1) & 1u;  // uses of this step's barrier so far in this launch
         const bool rearm = i + 2 < nsteps;
         const int bd = dep_b(m), ba = arr_b(m), cp = bd == ba ? bd : 2;
-        if (!second) {
+        if (!second && (DIFF || !CACHE)) {
             // a~_m and c of this step's epilogue sites into L1 ahead of use
             // (the packing the step ends in)
             auto pf = [&](size_t e) {
@@ -343,7 +379,7 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(href + (size_t)m * HN + e));
                     asm volatile("prefetch.global.L1 [%0];" ::"l"(cdiff + (size_t)cp * HN + e));
                 }
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(fac + (size_t)cp * HN + e));
+                if (!CACHE) asm volatile("prefetch.global.L1 [%0];" ::"l"(fac + (size_t)cp * HN + e));
             };
             if (cols) {
 #pragma unroll
@@ -398,6 +434,7 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
                 // next use depends on
                 if (tid == 0 && rearm) mbar_expect(bar_row, XBYTES);
             } else {
+                if (CACHE && cp != cur_c) fill_c(cur_c = cp);
                 // node factors in the packed-row form (x = 2J + (y & 1) of
                 // packed row y / 2), the result back in the column buffer
 #pragma unroll
@@ -405,7 +442,7 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
 #pragma unroll
                     for (int r = 0; r < RC; ++r) {
                         const int kk = (ct[j] + r * PER_C) >> 1, xx = 2 * (jcol0 + cc[j]) + (ct[j] & 1);
-                        x[j][r] = finish(pair_transpose<16>(x[j][r], ct[j] & 1), m, cp, kk, xx);
+                        x[j][r] = finish(pair_transpose<16>(x[j][r], ct[j] & 1), &fac_c[(j * RC + r) * T + tid], m, cp, kk, xx);
                     }
                 __syncthreads();  // every thread has read its columns: they are rewritten below
 #pragma unroll
@@ -444,12 +481,13 @@ __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
                 if (tid == 0 && rearm) mbar_expect(bar_col, XBYTES);
             } else {
                 // node factors; the result stays in the row buffer
+                if (CACHE && cp != cur_r) fill_r(cur_r = cp);
                 // every value first: the stores come after
 #pragma unroll
                 for (int j = 0; j < NB_L; ++j)
 #pragma unroll
                     for (int r = 0; r < RR; ++r)
-                        h[j][r] = finish(h[j][r], m, cp, krow0 + bb[j], tt[j] + r * PER_L);
+                        h[j][r] = finish(h[j][r], &fac_r[(j * RR + r) * T + tid], m, cp, krow0 + bb[j], tt[j] + r * PER_L);
 #pragma unroll
                 for (int j = 0; j < NB_L; ++j)
 #pragma unroll
@@ -742,26 +780,40 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
 
 struct ClusterShape {
     int logx, logy, c, t;
-    const void *fn;       // plain and reference solves
-    const void *fn_diff;  // differential solve
-    size_t smem, smem_diff;
+    // forms of the kernel (ChainForm): plain and reference solves, differential solve
+    const void *fn[3], *fn_diff[3];
+    size_t smem[3];
     int mrx, mry;         // radix plans of the row and column transforms (log2 of the largest radix)
 };
+// CHAIN_SOLO: the whole register file for one CTA per SM, factors cached;
+// CHAIN_SHARE: half of it, factors from planes; CHAIN_PHASED: the whole, from
+// planes.  The tiles below 4096 points fit several CTAs per SM in any form.
+enum ChainForm { CHAIN_SOLO = 0, CHAIN_SHARE = 1, CHAIN_PHASED = 2 };
 
 template <int LOGX, int LOGY, int C, int T, int MINB = 1024 / T>
 static ClusterShape shape_of()
 {
-    return ClusterShape{LOGX, LOGY, C, T, (const void *)prop_chain<LOGX, LOGY, C, T, MINB, false>,
-                        (const void *)prop_chain<LOGX, LOGY, C, T, MINB, true>, ClusterGeom<LOGX, LOGY, C, T>::SMEM,
-                        ClusterGeom<LOGX, LOGY, C, T>::SMEM_DIFF, ClusterGeom<LOGX, LOGY, C, T>::MRX,
-                        ClusterGeom<LOGX, LOGY, C, T>::MRY};
+    constexpr int SHARE = MINB == 1 ? 2 : MINB;
+    constexpr bool PH = C >= 8;  // smaller clusters are never one too many by far: phased launches take the solo form
+    using G = ClusterGeom<LOGX, LOGY, C, T>;
+    return ClusterShape{LOGX, LOGY, C, T,
+                        {(const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, true>,
+                         (const void *)prop_chain<LOGX, LOGY, C, T, SHARE, false, false>,
+                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, !PH>},
+                        {(const void *)prop_chain<LOGX, LOGY, C, T, MINB, true, true>,
+                         (const void *)prop_chain<LOGX, LOGY, C, T, SHARE, true, false>,
+                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, true, !PH>},
+                        {G::SMEM_CACHE, G::SMEM, PH ? G::SMEM : G::SMEM_CACHE}, G::MRX, G::MRY};
 }
 
-// Instantiated grids (log2 nx, log2 ny).  Tiles of 4096 points take 256
-// threads (one or two butterflies per thread and pass) with the SM's whole
-// register file (both packings' per-site factors stay in registers; at 128
-// registers a thread spilled 220-480 bytes); the smaller tiles fit several
-// CTAs per SM.
+// Instantiated grids (log2 nx, log2 ny).  A tile of 4096 points has 256
+// threads (one or two butterflies per thread and pass).  With the SM's whole
+// register file (255 registers) a chain runs fastest; at 128 registers a
+// second CTA shares the SM and fills the exchange waits of the first: slower
+// for one chain, more chains per second.  One handle with one group whose
+// chains have an SM per CTA takes the first form (4 x 256 x 512, alone: 1.40
+// ms a step, 1.47 with the second), a handle with several groups, or more
+// chains than fit so, the second (32-run ensemble, 2 steps: 13.6 -> 12.2 ms).
 static const ClusterShape *find_shape(int logx, int logy)
 {
     static const ClusterShape shapes[] = {
@@ -775,10 +827,9 @@ static const ClusterShape *find_shape(int logx, int logy)
     return nullptr;
 }
 
-static const void *chain_fn(const ClusterShape *s, bool diff) { return diff ? s->fn_diff : s->fn; }
+static const void *chain_fn(const ClusterShape *s, bool diff, ChainForm f) { return diff ? s->fn_diff[f] : s->fn[f]; }
 
-static void set_cluster_cfg(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, const ClusterShape *s, int nclusters,
-                            bool diff)
+static void set_cluster_cfg(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, const ClusterShape *s, int nclusters, ChainForm f)
 {
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = s->c;
@@ -786,7 +837,7 @@ static void set_cluster_cfg(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, 
     attr.val.clusterDim.z = 1;
     cfg.gridDim = dim3(s->c * nclusters, 1, 1);
     cfg.blockDim = dim3(s->t, 1, 1);
-    cfg.dynamicSmemBytes = diff ? s->smem_diff : s->smem;
+    cfg.dynamicSmemBytes = s->smem[f];
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
 }
@@ -805,12 +856,12 @@ static int g_solo_clusters[16][16][2];
 
 static int count_solo_clusters(const ClusterShape *s, bool diff)
 {
-    const void *fn = chain_fn(s, diff);
-    const size_t sm = std::max(kSoloSmem, diff ? s->smem_diff : s->smem);
+    const void *fn = chain_fn(s, diff, CHAIN_PHASED);
+    const size_t sm = std::max(kSoloSmem, s->smem[CHAIN_PHASED]);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
-    set_cluster_cfg(cfg, attr, s, 1, diff);
+    set_cluster_cfg(cfg, attr, s, 1, CHAIN_PHASED);
     cfg.dynamicSmemBytes = sm;
     int nclusters = 0;
     if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess) return 0;
@@ -828,19 +879,21 @@ bool cluster_solve_supported(const Group &G)
     int &st = checked[s->logx][s->logy];
     if (st == 0) {
         st = 2;
-        auto ok = [&](bool diff) {
-            const void *fn = chain_fn(s, diff);
-            const size_t sm = diff ? s->smem_diff : s->smem;
+        auto ok = [&](bool diff, ChainForm f) {
+            const void *fn = chain_fn(s, diff, f);
+            const size_t sm = s->smem[f];
             if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) return false;
             if (s->c > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
                 return false;
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute attr;
-            set_cluster_cfg(cfg, attr, s, 1, diff);
+            set_cluster_cfg(cfg, attr, s, 1, f);
             int nclusters = 0;
             return cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters > 0;
         };
-        if (ok(false) && ok(true)) {
+        bool all = true;
+        for (ChainForm f : {CHAIN_SOLO, CHAIN_SHARE, CHAIN_PHASED}) all = all && ok(false, f) && ok(true, f);
+        if (all) {
             st = 1;
             g_solo_clusters[s->logx][s->logy][0] = count_solo_clusters(s, false);
             g_solo_clusters[s->logx][s->logy][1] = count_solo_clusters(s, true);
@@ -864,6 +917,7 @@ int cluster_chain_launches(const Group &G, bool diff)
     const char *env = std::getenv("EPD_LB_CHAIN_SCHEDULE");
     if (env && !std::strcmp(env, "single")) return 1;
     if (env && !std::strcmp(env, "phased")) return can ? nch : 1;
+    if (G.crowded) return 1;
     return (can && nch == solo + 1) ? nch : 1;
 }
 
@@ -907,11 +961,13 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     // launch j and runs N_s / (nch - 1) steps in each of the others).
     const int nch = 2 * G.g.nruns, launches = cluster_chain_launches(G, diff);
     const bool phased = launches > 1;
+    const int solo = g_solo_clusters[sh->logx][sh->logy][diff ? 1 : 0];
+    const ChainForm form = phased ? CHAIN_PHASED : (G.crowded || nch > solo ? CHAIN_SHARE : CHAIN_SOLO);
     k.nseg = phased ? nch - 1 : 0;
     k.skip = 0;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
-    set_cluster_cfg(cfg, attr, sh, phased ? nch - 1 : nch, diff);
+    set_cluster_cfg(cfg, attr, sh, phased ? nch - 1 : nch, form);
     if (phased) cfg.dynamicSmemBytes = std::max(kSoloSmem, cfg.dynamicSmemBytes);
     cfg.stream = s;
     if (probe) {
@@ -932,7 +988,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
             c2.attrs = attrs;
             c2.numAttrs = 2;
         }
-        cudaError_t e = cudaLaunchKernelExC(&c2, chain_fn(sh, diff), args);
+        cudaError_t e = cudaLaunchKernelExC(&c2, chain_fn(sh, diff, form), args);
         if (e != cudaSuccess) return e;
     }
     if (probe) cudaEventRecordWithFlags(probe->ev[1], s, cudaEventRecordExternal);
