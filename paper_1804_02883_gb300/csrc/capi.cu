@@ -1284,6 +1284,84 @@ extern "C" void epd_lb_destroy(epd_lb *h)
 // Stateless single-chain solve on device pointers.
 // ---------------------------------------------------------------------------
 
+// Tables of a stateless call, written on the device: twiddles exp(-2 pi i t /
+// n), t < n, the Fourier factors exp(-R_G^2 k^2 ds) / n of Eq. (8), and the
+// pass tables of the cluster solve (fft8.cuh layout).  Formed in FP64.  (The
+// host built them per call, six to ten pageable copies and a synchronisation:
+// 0.1 ms of a 128 x 128 solve.)
+struct AxisTables {
+    int n;
+    void *tw, *kf;                // may be null
+    float2 *tab[2];               // pass tables of the radix-8 and radix-16 plans, or null
+};
+struct CallTables {
+    AxisTables ax[3];
+    double dx, rg, ds;
+};
+namespace {
+template <typename T> __global__ void call_tables(CallTables c)
+{
+    const AxisTables a = c.ax[blockIdx.y];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, n = a.n;
+    auto twiddle = [n](int t) {
+        double s, k;
+        sincospi(2.0 * (double)t / (double)n, &s, &k);
+        return make_double2(k, -s);
+    };
+    // one entry per thread and kind: an FP64 sine or exponential is ~10 us of
+    // dependent instructions, so nothing is computed after it
+    if (blockIdx.z == 0) {
+        if (i < n && a.tw) {
+            const double2 w = twiddle(i);
+            reinterpret_cast<V2<T> *>(a.tw)[i] = mk<T>((T)w.x, (T)w.y);
+        }
+        return;
+    }
+    if (blockIdx.z == 1) {
+        if (i < n && a.kf) {
+            const double k = 2.0 * 3.14159265358979323846 * (double)signed_bin(i, n) / ((double)n * c.dx);
+            reinterpret_cast<T *>(a.kf)[i] = (T)(exp(-c.rg * c.rg * k * k * c.ds) / (double)n);
+        }
+        return;
+    }
+    const int v = blockIdx.z - 2;
+    if (a.tab[v]) {
+        const int logn = ilog2(n), mr = 3 + v, np = npasses(logn, mr);
+        for (int e = i; e < tabs_total(logn, mr); e += gridDim.x * blockDim.x) {
+            for (int I = 0; I < 2 * (np - 1); ++I) {  // the pass the entry belongs to
+                const bool inv = I >= np - 1;
+                const int p = inv ? I - (np - 1) : I;
+                const int slog = inv ? inv_slog(logn, p, mr) : fwd_slog(logn, p, mr), rlog = inv ? inv_rlog(logn, p, mr) : fwd_rlog(logn, p, mr);
+                const int off = inv ? inv_off(logn, p, mr) : fwd_off(logn, p, mr), M = n >> (slog + rlog);
+                const int r = e - off;
+                if (r < 0 || r >= tab_rows(rlog) * M) continue;
+                const int row = r / M, k = rlog >= 3 ? (1 << row) : row + 1;
+                const double2 w = twiddle(((r % M) << slog) * k);
+                a.tab[v][e] = make_float2((float)w.x, (float)w.y);
+            }
+        }
+    }
+}
+} // namespace
+static cudaError_t launch_call_tables(const CallTables &c, int axes, bool fp64, cudaStream_t s)
+{
+    int m = 1;
+    for (int i = 0; i < axes; ++i) m = std::max(m, c.ax[i].n);
+    bool tabs = false;
+    for (int i = 0; i < axes; ++i) tabs = tabs || c.ax[i].tab[0] || c.ax[i].tab[1];
+    if (tabs) m *= 4;  // a pass table has at most 4 n entries
+    const dim3 grid((m + 63) / 64, axes, tabs ? 4 : 2);
+    if (fp64) call_tables<double><<<grid, 64, 0, s>>>(c);
+    else call_tables<float><<<grid, 64, 0, s>>>(c);
+    return cudaGetLastError();
+}
+static cudaError_t launch_group_tables(const Group &G, cudaStream_t s)
+{
+    const CallTables c = {{{G.g.nx, G.twx, G.kx, {G.tab8x, G.tab16x}}, {G.g.ny, G.twy, G.ky, {G.tab8y, G.tab16y}}, {}},
+                          G.g.dx, G.g.rg, G.g.ds};
+    return launch_call_tables(c, 2, G.prec == EPD_LB_PLAIN_FP64, s);
+}
+
 // Only the buffers a solve touches: chain, history, factors, contour sums,
 // partials and tables.
 static size_t carve_solve(Group &G, char *base)
@@ -1313,6 +1391,36 @@ static size_t carve_solve(Group &G, char *base)
     G.ky = take((size_t)G.g.ny * tb);
     G.twx_d = (double2 *)take((size_t)G.g.nx * sizeof(double2));
     G.twy_d = (double2 *)take((size_t)G.g.ny * sizeof(double2));
+    return align_up(off);
+}
+
+// The same for the cluster-resident solve of one run (MIXED_FP32 grids with a
+// cluster shape): its stored states, factors, planes and pass tables; 0 for
+// other problems.
+static size_t carve_solve_cluster(Group &G, char *base)
+{
+    if (G.prec != EPD_LB_MIXED_FP32 || !G.g.pow2 || !cluster_shape_exists(G.g.logx, G.g.logy)) return 0;
+    const size_t n = (size_t)G.g.n;
+    size_t off = 0;
+    auto take = [&](size_t bytes) -> void * {
+        off = align_up(off);
+        void *p = base ? base + off : nullptr;
+        off += bytes;
+        return p;
+    };
+    G.stateless = true;
+    G.err = (int *)take(256);
+    G.part = (double *)take(kMaxPart * sizeof(double));
+    G.efac = take(n * sizeof(float2));
+    G.facp = take(3 * n * sizeof(float));
+    G.hc = take(cluster_state_floats2(G.g.nx, G.g.ny, G.g.ns) * sizeof(float2));
+    G.twx = G.twy = nullptr;
+    G.kx = take((size_t)G.g.nx * sizeof(float));
+    G.ky = take((size_t)G.g.ny * sizeof(float));
+    G.tab8x = (float2 *)take((size_t)tabs_total(G.g.logx) * sizeof(float2));
+    G.tab8y = (float2 *)take((size_t)tabs_total(G.g.logy) * sizeof(float2));
+    G.tab16x = best_mr(G.g.logx) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logx, 4) * sizeof(float2)) : nullptr;
+    G.tab16y = best_mr(G.g.logy) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logy, 4) * sizeof(float2)) : nullptr;
     return align_up(off);
 }
 
@@ -1384,24 +1492,10 @@ static size_t solve3_layout(const epd_lb_params *p, int nz, Solve3 &S, char *bas
     return align_up(off);
 }
 
-// Twiddles exp(-2 pi i t / n), t < n, and (kf not null) factors exp(-R_G^2 k^2 ds) / n of one axis.
-template <typename T>
-static cudaError_t upload_axis(int n, double dx, double rg, double ds, void *tw, void *kf, cudaStream_t s)
+static cudaError_t launch_box_tables(const epd_lb_params &p, int nz, const Solve3 &S, cudaStream_t s)
 {
-    const double pi = 3.14159265358979323846;
-    std::vector<T> t(2 * (size_t)n), k((size_t)n);
-    for (int j = 0; j < n; ++j) {
-        const double a = 2.0 * pi * (double)j / (double)n;
-        t[2 * j] = (T)std::cos(a);
-        t[2 * j + 1] = (T)-std::sin(a);
-        const int mm = j <= n / 2 ? j : j - n;
-        const double kk = 2.0 * pi * (double)mm / ((double)n * dx);
-        k[j] = (T)(std::exp(-rg * rg * kk * kk * ds) / (double)n);
-    }
-    cudaError_t e = cudaMemcpyAsync(tw, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice, s);
-    if (!e && kf) e = cudaMemcpyAsync(kf, k.data(), k.size() * sizeof(T), cudaMemcpyHostToDevice, s);
-    if (!e) e = cudaStreamSynchronize(s);  // the host vectors go out of scope
-    return e;
+    const CallTables c = {{{p.nx, S.twx, S.kx, {}}, {p.ny, S.twy, S.ky, {}}, {nz, S.twz, S.kz, {}}}, p.dx, p.rg, 1.0 / (double)p.ns};
+    return launch_call_tables(c, 3, S.prec == EPD_LB_PLAIN_FP64, s);
 }
 
 extern "C" int epd_prop_solve3d_workspace_bytes(const epd_lb_params *p, int32_t nz, size_t *bytes)
@@ -1424,15 +1518,8 @@ extern "C" int epd_prop_solve3d(const epd_lb_params *p, int32_t nz, const double
     if (workspace_bytes < need || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
     solve3_layout(p, nz, S, (char *)workspace_dev);
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const double ds = 1.0 / (double)p->ns;
     cudaError_t e = cudaMemsetAsync(S.err, 0, sizeof(int), s);
-    auto up = [&](int n, void *tw, void *kf) {
-        return p->precision == EPD_LB_MIXED_FP32 ? upload_axis<float>(n, p->dx, p->rg, ds, tw, kf, s)
-                                                 : upload_axis<double>(n, p->dx, p->rg, ds, tw, kf, s);
-    };
-    if (!e) e = up(p->nx, S.twx, S.kx);
-    if (!e) e = up(p->ny, S.twy, S.ky);
-    if (!e) e = up(nz, S.twz, S.kz);
+    if (!e) e = launch_box_tables(*p, nz, S, s);
     if (!e) e = launch_solve3d(S, omega_dev, phi_dev, q_dev, s);
     return e ? EPD_LB_ECUDA : EPD_LB_OK;
 }
@@ -1502,19 +1589,12 @@ extern "C" int epd_step3d(const epd_lb_params *p, int32_t nz, double *omega_dev,
     if (workspace_bytes < need || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
     step3_layout(p, nz, T, (char *)workspace_dev);
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const double ds = 1.0 / (double)p->ns;
     cudaError_t e = cudaMemsetAsync(T.S.err, 0, sizeof(int), s);
-    auto up = [&](int n, void *tw, void *kf) {
-        return p->precision == EPD_LB_MIXED_FP32 ? upload_axis<float>(n, p->dx, p->rg, ds, tw, kf, s)
-                                                 : upload_axis<double>(n, p->dx, p->rg, ds, tw, kf, s);
-    };
-    if (!e) e = up(p->nx, T.S.twx, T.S.kx);
-    if (!e) e = up(p->ny, T.S.twy, T.S.ky);
-    if (!e) e = up(nz, T.S.twz, T.S.kz);
+    if (!e) e = launch_box_tables(*p, nz, T.S, s);
     // FP64 twiddles of the EPD transforms
-    if (!e) e = upload_axis<double>(p->nx, p->dx, p->rg, ds, (void *)T.twx, nullptr, s);
-    if (!e) e = upload_axis<double>(p->ny, p->dx, p->rg, ds, (void *)T.twy, nullptr, s);
-    if (!e) e = upload_axis<double>(nz, p->dx, p->rg, ds, (void *)T.twz, nullptr, s);
+    const CallTables c = {{{p->nx, (void *)T.twx, nullptr, {}}, {p->ny, (void *)T.twy, nullptr, {}}, {nz, (void *)T.twz, nullptr, {}}},
+                          p->dx, p->rg, 1.0 / (double)p->ns};
+    if (!e) e = launch_call_tables(c, 3, true, s);
     if (!e) e = launch_step3d(T, omega_dev, pop_dev, vel_dev, phi_dev, q_dev, force_dev, s);
     return e ? EPD_LB_ECUDA : EPD_LB_OK;
 }
@@ -1552,6 +1632,7 @@ extern "C" int epd_prop_solve_workspace_bytes(const epd_lb_params *p, size_t *by
     Group G;
     if (!bytes || !solve_group(p, G)) return EPD_LB_EINVAL;
     *bytes = carve_solve(G, nullptr);
+    *bytes = std::max(*bytes, carve_solve_cluster(G, nullptr));
     return EPD_LB_OK;
 }
 
@@ -1561,10 +1642,20 @@ extern "C" int epd_prop_solve(const epd_lb_params *p, const double *omega_dev, d
     Group G;
     if (!solve_group(p, G) || !omega_dev || !phi_dev || !q_dev || !workspace_dev) return EPD_LB_EINVAL;
     if (workspace_bytes < carve_solve(G, nullptr) || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
-    carve_solve(G, (char *)workspace_dev);
+    // the cluster-resident solve where the grid has one and the workspace
+    // holds its states (128 x 128, N_s = 64: 0.76 ms as streaming passes, 0.30
+    // resident); a workspace of the streaming passes' size still does
+    Group C = G;
+    const size_t cluster_bytes = carve_solve_cluster(C, nullptr);
+    if (cluster_bytes && workspace_bytes >= cluster_bytes && cluster_solve_supported(G)) {
+        carve_solve_cluster(C, (char *)workspace_dev);
+        G = C;
+    } else {
+        carve_solve(G, (char *)workspace_dev);
+    }
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (cudaMemsetAsync(G.err, 0, sizeof(int), s) != cudaSuccess) return EPD_LB_ECUDA;
-    if (upload_tables_e(G, s) != cudaSuccess) return EPD_LB_ECUDA;
+    if (launch_group_tables(G, s) != cudaSuccess) return EPD_LB_ECUDA;
     if (launch_solve(G, omega_dev, phi_dev, q_dev, s) != cudaSuccess) return EPD_LB_ECUDA;
     return EPD_LB_OK;
 }
@@ -1585,37 +1676,6 @@ __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 // Device address of g_noalloc_scratch on each device (host code must not use
 // the symbol itself as an address).
 std::atomic<void *> g_noalloc_addr[kNoallocDevices];
-
-// Twiddles exp(-2 pi i t / n), t < n, and Fourier factors
-// exp(-R_G^2 k^2 ds) / n (Eq. (8)), computed on the device in FP64.
-template <typename T>
-__global__ void noalloc_tables(int nx, int ny, double dx, double rg, double ds, V2<T> *twx, V2<T> *twy, T *kx, T *ky)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    auto twiddle = [](int t, int n, V2<T> *out) {
-        double s, c;
-        sincospi(2.0 * (double)t / (double)n, &s, &c);
-        out[t] = mk<T>((T)c, (T)(-s));
-    };
-    auto factor = [&](int m, int n, T *out) {
-        const double k = 2.0 * 3.14159265358979323846 * (double)signed_bin(m, n) / ((double)n * dx);
-        out[m] = (T)(exp(-rg * rg * k * k * ds) / (double)n);
-    };
-    if (i < nx) twiddle(i, nx, twx);
-    if (i < ny) twiddle(i, ny, twy);
-    if (i < nx) factor(i, nx, kx);
-    if (i < ny) factor(i, ny, ky);
-}
-
-template <typename T>
-cudaError_t noalloc_launch_tables(Group &G, cudaStream_t s)
-{
-    const int m = std::max(G.g.nx, G.g.ny);
-    noalloc_tables<T><<<(m + kThreads - 1) / kThreads, kThreads, 0, s>>>(
-        G.g.nx, G.g.ny, G.g.dx, G.g.rg, G.g.ds, reinterpret_cast<V2<T> *>(G.twx), reinterpret_cast<V2<T> *>(G.twy),
-        reinterpret_cast<T *>(G.kx), reinterpret_cast<T *>(G.ky));
-    return cudaGetLastError();
-}
 
 } // namespace
 
@@ -1642,8 +1702,7 @@ extern "C" int epd_prop_solve_noalloc(const epd_lb_params *p, const double *omeg
     // the error word must start at zero; every other scratch buffer is written
     // before it is read within the call
     if (cudaMemsetAsync(G.err, 0, sizeof(int), s) != cudaSuccess) return EPD_LB_ECUDA;
-    const cudaError_t e = G.prec == EPD_LB_MIXED_FP32 ? noalloc_launch_tables<float>(G, s) : noalloc_launch_tables<double>(G, s);
-    if (e != cudaSuccess) return EPD_LB_ECUDA;
+    if (launch_group_tables(G, s) != cudaSuccess) return EPD_LB_ECUDA;
     if (launch_solve(G, omega_dev, phi_dev, q_dev, s) != cudaSuccess) return EPD_LB_ECUDA;
     return EPD_LB_OK;
 }

@@ -377,16 +377,17 @@ static int grid_for(long long n)
     return (int)(b > 1024 ? 1024 : b);
 }
 
-// One pass of either axis: compile-time tiles on the power-of-two FP32 grids
-// that have them (hist_full), the general passes otherwise.
+// One pass of either axis: compile-time tiles on the FP32 grids that have them
+// (powers of two, 64..2048 points per axis), the general passes otherwise.
+static bool has_stream_tiles(const GroupGeom &g) { return g.pow2 && g.logx >= 6 && g.logx <= 11 && g.logy >= 6 && g.logy <= 11; }
 static cudaError_t col_pass(const PropK<float> &k, const Group &G, cudaStream_t s)
 {
-    return G.hist_full ? stream_col(k, G.colw_prop, s) : line_col(k, s);
+    return has_stream_tiles(k.g) ? stream_col(k, G.colw_prop, s) : line_col(k, s);
 }
 static cudaError_t col_pass(const PropK<double> &k, const Group &, cudaStream_t s) { return line_col(k, s); }
-static cudaError_t row_pass(const PropK<float> &k, const Group &G, int m, bool diff, int *blocks, cudaStream_t s)
+static cudaError_t row_pass(const PropK<float> &k, const Group &, int m, bool diff, int *blocks, cudaStream_t s)
 {
-    return G.hist_full ? stream_row(k, m, diff, blocks, s) : line_row(k, m, diff, blocks, s);
+    return has_stream_tiles(k.g) ? stream_row(k, m, diff, blocks, s) : line_row(k, m, diff, blocks, s);
 }
 static cudaError_t row_pass(const PropK<double> &k, const Group &, int m, bool diff, int *blocks, cudaStream_t s)
 {
@@ -420,7 +421,7 @@ static cudaError_t solve_t(Group &G, const double *omega, double *phi, double *q
 
     const int pg = grid_for(g.n);
     prop_prep<T><<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, omega, reinterpret_cast<V2<T> *>(G.efac), reinterpret_cast<T *>(G.facp), phi, G.part);
-    if (sizeof(T) == sizeof(float) && G.hc && G.twx_full && cluster_solve_supported(G)) {
+    if (sizeof(T) == sizeof(float) && G.hc && G.tab8x && cluster_solve_supported(G)) {
         // whole contour in one cluster-resident launch, then the contour sums
         return launch_cluster_solve(G, s, false, pg, phi, q, probe);
     }

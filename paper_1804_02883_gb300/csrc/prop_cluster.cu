@@ -794,7 +794,7 @@ template <int LOGX, int LOGY, int C, int T, int MINB = 1024 / T>
 static ClusterShape shape_of()
 {
     constexpr int SHARE = MINB == 1 ? 2 : MINB;
-    constexpr bool PH = C >= 8;  // smaller clusters are never one too many by far: phased launches take the solo form
+    constexpr bool PH = C >= 8;  // below that a launch holds many clusters and one more costs little: no form of their own
     using G = ClusterGeom<LOGX, LOGY, C, T>;
     return ClusterShape{LOGX, LOGY, C, T,
                         {(const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, true>,

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(256) prop_col(PropK<T> k, int logb)
     col_tile<T, R0>(k, LineTile(false, k.g.ny, logb, k.g.py), k.g.py);
 }
 template <typename T, int R0, bool DIFF>
-__global__ void __launch_bounds__(256) prop_row(PropK<T> k, int m, int logb, RowWeights w)
+__global__ void __launch_bounds__(256, 2) prop_row(PropK<T> k, int m, int logb, RowWeights w)
 {
     row_tile<T, R0, DIFF>(k, LineTile(true, k.g.nx, logb, k.g.px), k.g.px, m, w);
 }

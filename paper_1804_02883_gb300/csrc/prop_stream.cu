@@ -1,6 +1,6 @@
 // prop_stream.cu -- the streaming propagator passes on power-of-two grids of
-// 64..2048 points per axis in FP32 (MIXED_FP32 grids without a cluster shape,
-// such as 1024 x 2048): the passes of prop_line.cuh on tiles known at compile
+// 64..2048 points per axis in FP32 (grids without a cluster shape, such as 1024
+// x 2048, and stateless solves): the passes of prop_line.cuh on tiles known at compile
 // time.
 //
 // Bound: instruction issue, then the L2 traffic of the chain.  With the axis,

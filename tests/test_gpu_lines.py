@@ -38,3 +38,27 @@ def test_solve_on_every_plan(ny, nx, precision):
     ph, qh = h.solve(0, om)
     h.close()
     assert rel_err(ph, phi) < tol and rel_err(qh, q) < tol
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ny,nx,ns", [(64, 64, 8), (128, 128, 6), (64, 512, 4), (512, 256, 6), (512, 512, 4), (64, 2048, 4)])
+def test_stateless_solve_takes_either_workspace(ny, nx, ns):
+    """MIXED_FP32 on powers of two: the cluster-resident solve with the queried
+    workspace, the streaming passes with one that only holds half the history
+    (the size documented for the allocation-free call); grids without a
+    cluster shape stream with both."""
+    import torch
+
+    run = P.RunParams(nx=nx, ny=ny, ns=ns, precision=P.MIXED_FP32, f_a=0.5)
+    om = W.random_omega(ny, nx, 12)
+    phi, q = O.solve(oracle_params(run), om)
+    od = torch.from_numpy(om).cuda()
+    nb = P.epd_prop_solve_workspace_bytes(run)
+    for size in (nb, min(nb, ny * nx * (16 + (ns // 2 + 3) * 8) + 192 * 1024)):
+        pd = torch.empty_like(od)
+        qd = torch.empty(2, dtype=torch.float64, device="cuda")
+        ws = torch.empty(size + 256, dtype=torch.uint8, device="cuda")
+        P.epd_prop_solve(run, od.data_ptr(), pd.data_ptr(), qd.data_ptr(), (ws.data_ptr() + 255) & ~255, size,
+                         torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert rel_err(pd.cpu().numpy(), phi) < 2e-6 and rel_err(qd.cpu().numpy(), q) < 2e-6
