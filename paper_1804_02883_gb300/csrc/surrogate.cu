@@ -468,18 +468,40 @@ __global__ void __launch_bounds__(128) conv3x3_tc(ConvArgs a, const __grid_const
 }
 
 
+// Four 8 x 8 BF16 matrices from shared memory, transposed: lane l gives the
+// address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t saddr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(saddr)
+                 : "memory");
+}
+
 // Weight gradient of one layer: dW[tap][co][ci] = sum_p dZ[p][co] x[p + off(tap)][ci]
 // over an 8 x 16 tile per step, `tiles` consecutive tiles per CTA; 9 warps, warp
 // = tap.  Partial sums per CTA to part[blk][tap][co][ci] (deterministic
-// reduction later).  CO, CI multiples of 16 and 8.
+// reduction later).  CO, CI multiples of 16.  Both operands lie in shared
+// memory as the tensors do, channels contiguous per pixel, while the sum runs
+// over pixels: transposing matrix loads make the fragments (rows of channels
+// padded by 16 bytes: the eight rows of a matrix on different banks), and the
+// next tile streams in by asynchronous copies meanwhile.  What bounded it
+// before were the 2-byte shared loads and packs that gathered the fragments:
+// 103 us per 32 x 32 layer on 4 x 256 x 512.
+template <int CI, int CO, int D> struct DwGeom {
+    static constexpr int CS = CI + 8, DS = CO + 8;
+    static constexpr int HH = Halo<D>::HH, HW = Halo<D>::HW;
+    static constexpr int XB = HH * HW * CS, ZB = TP * DS;  // BF16 values of a stage
+    static constexpr size_t SMEM = (size_t)2 * (XB + ZB) * sizeof(__nv_bfloat16);
+};
 template <int CI, int CO, int D>
 __global__ void __launch_bounds__(288) conv3x3_dw(const __nv_bfloat16 *x, const __nv_bfloat16 *dz, float *part, int nx, int ny,
                                                  int tiles_x, int tiles_per_cta, int ntiles_total)
 {
-    constexpr int CS = CI + 8, DS = TP + 8;
-    constexpr int HH = Halo<D>::HH, HW = Halo<D>::HW;
-    __shared__ __align__(16) __nv_bfloat16 tile[HH * HW * CS];
-    __shared__ __align__(16) __nv_bfloat16 dzt[CO * DS];  // [co][p], transposed
+    using G = DwGeom<CI, CO, D>;
+    constexpr int CS = G::CS, DS = G::DS, HH = G::HH, HW = G::HW;
+    static_assert(CI % 16 == 0 && CO % 16 == 0, "pairs of 8-channel matrices");
+    extern __shared__ __align__(16) __nv_bfloat16 dw_smem[];
     const int tid = threadIdx.x, lane = tid & 31, tap = tid >> 5;
     const int g = lane >> 2, t = lane & 3, dy = (tap / 3) * D, dx = (tap % 3) * D;
     const long long n = (long long)nx * ny;
@@ -491,51 +513,57 @@ __global__ void __launch_bounds__(288) conv3x3_dw(const __nv_bfloat16 *x, const 
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
     const int tiles_per_img = tiles_x * (ny / TH);
-    for (int it = 0; it < tiles_per_cta; ++it) {
-        const int tidx = blockIdx.x * tiles_per_cta + it;
-        if (tidx >= ntiles_total) break;
-        const int b = tidx / tiles_per_img, r = tidx % tiles_per_img;
-        const int ty0 = (r / tiles_x) * TH, tx0 = (r % tiles_x) * TW;
-        const __nv_bfloat16 *xin = x + (size_t)b * n * CI;
-        const __nv_bfloat16 *dzin = dz + (size_t)b * n * CO;
-        __syncthreads();
-        for (int e = tid; e < HH * HW * (CI / 8); e += 288) {
-            const int pix = e / (CI / 8), ch = (e % (CI / 8)) * 8;
-            const int hy = pix / HW, hx = pix % HW;
-            const int gy = halo_wrap(ty0 + hy - D, ny), gx = halo_wrap(tx0 + hx - D, nx);
-            *reinterpret_cast<uint4 *>(&tile[pix * CS + ch]) = *reinterpret_cast<const uint4 *>(&xin[((size_t)gy * nx + gx) * CI + ch]);
+    const int first = blockIdx.x * tiles_per_cta, count = min(tiles_per_cta, ntiles_total - first);
+    auto load = [&](int it) {
+        if (it < count) {
+            const int tidx = first + it, b = tidx / tiles_per_img, r = tidx % tiles_per_img;
+            const int ty0 = (r / tiles_x) * TH, tx0 = (r % tiles_x) * TW;
+            const __nv_bfloat16 *xin = x + (size_t)b * n * CI;
+            const __nv_bfloat16 *dzin = dz + (size_t)b * n * CO;
+            __nv_bfloat16 *xs = dw_smem + (it & 1) * (G::XB + G::ZB), *zs = xs + G::XB;
+            for (int e = tid; e < HH * HW * (CI / 8); e += 288) {
+                const int pix = e / (CI / 8), ch = (e % (CI / 8)) * 8;
+                const int hy = pix / HW, hx = pix % HW;
+                const int gy = halo_wrap(ty0 + hy - D, ny), gx = halo_wrap(tx0 + hx - D, nx);
+                cp_async16(&xs[pix * CS + ch], &xin[((size_t)gy * nx + gx) * CI + ch]);
+            }
+            for (int e = tid; e < TP * (CO / 8); e += 288) {
+                const int p = e / (CO / 8), ch = (e % (CO / 8)) * 8;
+                cp_async16(&zs[p * DS + ch], &dzin[((size_t)(ty0 + p / TW) * nx + tx0 + p % TW) * CO + ch]);
+            }
         }
-        for (int e = tid; e < TP * CO; e += 288) {
-            const int p = e / CO, co = e % CO;
-            const int gy = ty0 + p / TW, gx = tx0 + p % TW;
-            dzt[co * DS + p] = dzin[((size_t)gy * nx + gx) * CO + co];
-        }
+        cp_async_commit();
+    };
+    load(0);
+    for (int it = 0; it < count; ++it) {
+        load(it + 1);
+        cp_async_wait<1>();
         __syncthreads();
+        const __nv_bfloat16 *xs = dw_smem + (it & 1) * (G::XB + G::ZB), *zs = xs + G::XB;
+        // A (co x pixels): matrices (co 0-7, k 0-7), (co 8-15, k 0-7), (co 0-7, k 8-15), (co 8-15, k 8-15)
+        const uint32_t za = (uint32_t)__cvta_generic_to_shared(zs + ((lane & 7) + ((lane >> 4) & 1) * 8) * DS + ((lane >> 3) & 1) * 8);
+        // B (pixels x ci): matrices (k 0-7, ci 0-7), (k 8-15, ci 0-7), (k 0-7, ci 8-15), (k 8-15, ci 8-15)
+        const uint32_t xa = (uint32_t)__cvta_generic_to_shared(xs + (dy * HW + dx + (lane & 7) + ((lane >> 3) & 1) * 8) * CS + ((lane >> 4) & 1) * 8);
 #pragma unroll
         for (int kc = 0; kc < TP / 16; ++kc) {  // 16 pixels = one tile row
-            const int py = kc;
             uint32_t af[CO / 16][4];
 #pragma unroll
-            for (int mt = 0; mt < CO / 16; ++mt) {
-                const int r0 = (mt * 16 + g) * DS + kc * 16 + 2 * t, r1 = r0 + 8 * DS;
-                af[mt][0] = *reinterpret_cast<const uint32_t *>(&dzt[r0]);
-                af[mt][1] = *reinterpret_cast<const uint32_t *>(&dzt[r1]);
-                af[mt][2] = *reinterpret_cast<const uint32_t *>(&dzt[r0 + 8]);
-                af[mt][3] = *reinterpret_cast<const uint32_t *>(&dzt[r1 + 8]);
-            }
+            for (int mt = 0; mt < CO / 16; ++mt) ldmatrix_x4_trans(af[mt], za + (uint32_t)(kc * 16 * DS + mt * 16) * 2);
 #pragma unroll
-            for (int nt = 0; nt < CI / 8; ++nt) {
-                const int ci = nt * 8 + g;
-                const int k0 = 2 * t, k1 = 2 * t + 8;  // pixel columns in the row
-                const __nv_bfloat16 *row = &tile[((py + dy) * HW + dx) * CS + ci];
-                uint32_t bf[2];
-                bf[0] = pack2(row[(k0)*CS], row[(k0 + 1) * CS]);
-                bf[1] = pack2(row[(k1)*CS], row[(k1 + 1) * CS]);
+            for (int np = 0; np < CI / 16; ++np) {
+                uint32_t bf[4];
+                ldmatrix_x4_trans(bf, xa + (uint32_t)(kc * HW * CS + np * 16) * 2);
+                const uint32_t b0[2] = {bf[0], bf[1]}, b1[2] = {bf[2], bf[3]};
 #pragma unroll
-                for (int mt = 0; mt < CO / 16; ++mt) mma16816(acc[mt][nt], af[mt], bf);
+                for (int mt = 0; mt < CO / 16; ++mt) {
+                    mma16816(acc[mt][2 * np], af[mt], b0);
+                    mma16816(acc[mt][2 * np + 1], af[mt], b1);
+                }
             }
         }
+        __syncthreads();  // this stage is filled again by the next load
     }
+    cp_async_wait<0>();
     float *out = part + (size_t)blockIdx.x * 9 * CO * CI + (size_t)tap * CO * CI;
 #pragma unroll
     for (int mt = 0; mt < CO / 16; ++mt)
@@ -558,9 +586,8 @@ constexpr int kRedBlocks = 64;  // blocks per plane of the two-pass reductions
 // Fixed-order sums over planes of n values in one launch, grid (kRedBlocks,
 // planes): every block writes part[plane][block]; the last block to finish
 // (a self-resetting counter) adds each plane's partials in block order and
-// writes out[plane] = sum * scale.  KIND 0: the FP64 values, 1: exp(-v) in
-// FP32 (solvent weight of Eq. (11)), 2: channel c = plane % 2 of the FP32
-// [sample][pixel][8] network output.
+// writes out[plane] = sum * scale.  KIND 0: the FP64 values, 2: channel c =
+// plane % 2 of the FP32 [sample][pixel][8] network output.
 __device__ __forceinline__ void finish_planes(const double *part, int planes, double scale, double *out, unsigned *cnt)
 {
     __shared__ bool last;
@@ -572,10 +599,14 @@ __device__ __forceinline__ void finish_planes(const double *part, int planes, do
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int p = threadIdx.x; p < planes; p += blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < kRedBlocks; ++b) s += part[(size_t)p * kRedBlocks + b];
-        out[p] = s * scale;
+    // a warp per plane: two partials per lane, then a fixed shuffle tree (one
+    // thread's chain of 64 dependent FP64 additions was 3 us)
+    static_assert(kRedBlocks == 64, "two partials per lane");
+    const int lane = threadIdx.x & 31;
+    for (int p = threadIdx.x >> 5; p < planes; p += blockDim.x >> 5) {
+        double s = part[(size_t)p * kRedBlocks + lane] + part[(size_t)p * kRedBlocks + 32 + lane];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) out[p] = s * scale;
     }
 }
 
@@ -591,11 +622,6 @@ __global__ void __launch_bounds__(256) plane_partials(const void *f, long long n
     if (KIND == 0) {
         const double *p = reinterpret_cast<const double *>(f) + (size_t)plane * n;
         for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) s += p[i];
-    } else if (KIND == 1) {
-        const double *p = reinterpret_cast<const double *>(f) + ((size_t)plane * 3 + 2) * n;
-        float acc = 0.f;
-        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) acc += expf(-(float)p[i]);
-        s = (double)acc;
     } else {
         const float *p = reinterpret_cast<const float *>(f) + (size_t)(plane / 2) * n * 8 + (plane % 2);
         float acc = 0.f;
@@ -607,124 +633,165 @@ __global__ void __launch_bounds__(256) plane_partials(const void *f, long long n
     finish_planes(part, gridDim.y, scale, out, cnt);
 }
 
-// x0[b][p][16] = s_in (omega_c - <omega_c>) for c < 3, 0 for the padding.
-__global__ void prep_input(const double *omega, const double *mean, double s_in, long long n, int nb, __nv_bfloat16 *x0)
+// Means of the fields a pass needs, in one launch, grid (kRedBlocks, 4 nb):
+// planes 0..2 of a sample the FP64 means of omega; plane 3 the solvent weight,
+// <exp(-omega_S)> (TAN = false) or <e q>, e = exp(-omega0_S), q = expm1(-(omega_S
+// - omega0_S)) (TAN), in FP32 per thread, FP64 beyond.  out: [nb][3] means,
+// solvent: [nb].
+template <bool TAN>
+__global__ void __launch_bounds__(256) field_partials(const double *omega, const double *omega0, long long n, double *part, double scale,
+                                                      double *out, double *solvent, unsigned *cnt)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * nb) return;
-    const long long b = i / n, p = i % n;
-    __align__(16) __nv_bfloat16 v[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) v[c] = __float2bfloat16_rn((float)(s_in * (omega[(b * 3 + c) * n + p] - mean[b * 3 + c])));
-    uint4 *dst = reinterpret_cast<uint4 *>(x0 + (size_t)i * 16);
-    dst[0] = *reinterpret_cast<uint4 *>(&v[0]);
-    dst[1] = *reinterpret_cast<uint4 *>(&v[8]);
+    __shared__ double red[32];
+    __shared__ bool last;
+    const int plane = blockIdx.y, b = plane >> 2, c = plane & 3;
+    const long long chunk = (n + kRedBlocks - 1) / kRedBlocks, lo = blockIdx.x * chunk;
+    const long long hi = lo + chunk < n ? lo + chunk : n;
+    const double *w = omega + ((size_t)b * 3 + (c < 3 ? c : 2)) * n;
+    double s = 0.0;
+    if (c < 3) {
+        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) s += w[i];
+    } else {
+        float acc = 0.f;
+        if (TAN) {
+            const double *w0 = omega0 + ((size_t)b * 3 + 2) * n;
+            for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x)
+                acc += expf(-(float)w0[i]) * expm1f(-(float)(w[i] - w0[i]));
+        } else {
+            for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) acc += expf(-(float)w[i]);
+        }
+        s = (double)acc;
+    }
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) part[(size_t)plane * kRedBlocks + blockIdx.x] = s;
+    __threadfence();  // this block's partial before its arrival
+    if (threadIdx.x == 0) {
+        const unsigned total = gridDim.x * gridDim.y;
+        last = atomicInc(cnt, total - 1) == total - 1;  // wraps to 0 for the next use
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31;
+    for (int p = threadIdx.x >> 5; p < (int)gridDim.y; p += blockDim.x >> 5) {
+        double t = part[(size_t)p * kRedBlocks + lane] + part[(size_t)p * kRedBlocks + 32 + lane];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) ((p & 3) < 3 ? out[(p >> 2) * 3 + (p & 3)] : solvent[p >> 2]) = t * scale;
+    }
+}
+
+// Network input of a pixel: 16 BF16 channels, three in use.
+__device__ __forceinline__ void store_input(__nv_bfloat16 *dst, float a, float b, float c)
+{
+    const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
+    uint4 *d = reinterpret_cast<uint4 *>(dst);
+    d[0] = make_uint4(pack2(__float2bfloat16_rn(a), __float2bfloat16_rn(b)), pack2(__float2bfloat16_rn(c), z), 0u, 0u);
+    d[1] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// The pointwise kernels below take grid (pixels, samples): a 64-bit division
+// per pixel for the sample, and FP64 divisions per pixel, cost them more than
+// their traffic (densities_tangent 32 us, densities_out 20, loss_grad 56 on
+// 4 x 256 x 512).
+
+// x0[b][p][16] = s_in (omega_c - <omega_c>) for c < 3, 0 for the padding.
+__global__ void __launch_bounds__(256) prep_input(const double *omega, const double *mean, double s_in, long long n, __nv_bfloat16 *x0)
+{
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.y;
+    if (p >= n) return;
+    const double *w = omega + (size_t)b * 3 * n + p, *m = mean + b * 3;
+    store_input(x0 + ((size_t)b * n + p) * 16, (float)(s_in * (w[0] - m[0])), (float)(s_in * (w[n] - m[1])),
+                (float)(s_in * (w[2 * n] - m[2])));
 }
 
 // Tangent input: dx0[b][p][16] = s_in ((omega_c - omega0_c) - <omega_c - omega0_c>)
 // for c < 3 (the FP64 difference of the two fields, then BF16), 0 for the padding.
-__global__ void prep_tangent(const double *omega, const double *omega0, const double *mean, const double *mean0, double s_in,
-                             long long n, int nb, __nv_bfloat16 *t0)
+__global__ void __launch_bounds__(256) prep_tangent(const double *omega, const double *omega0, const double *mean, const double *mean0,
+                                                    double s_in, long long n, __nv_bfloat16 *t0)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * nb) return;
-    const long long b = i / n, p = i % n;
-    __align__(16) __nv_bfloat16 v[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const size_t q = (b * 3 + c) * n + p;
-        v[c] = __float2bfloat16_rn((float)(s_in * ((omega[q] - omega0[q]) - (mean[b * 3 + c] - mean0[b * 3 + c]))));
-    }
-    uint4 *dst = reinterpret_cast<uint4 *>(t0 + (size_t)i * 16);
-    dst[0] = *reinterpret_cast<uint4 *>(&v[0]);
-    dst[1] = *reinterpret_cast<uint4 *>(&v[8]);
-}
-
-// Block partials of sum e q over one plane per sample, e = exp(-omega0_S),
-// q = expm1(-(omega_S - omega0_S)) (FP32, accurate relative to the change).
-__global__ void __launch_bounds__(256) solvent_change_partials(const double *omega, const double *omega0, long long n, double *part,
-                                                               double scale, double *out, unsigned *cnt)
-{
-    __shared__ double red[32];
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int b = blockIdx.y;
-    const long long chunk = (n + kRedBlocks - 1) / kRedBlocks, lo = blockIdx.x * chunk;
-    const long long hi = lo + chunk < n ? lo + chunk : n;
-    const double *w = omega + ((size_t)b * 3 + 2) * n, *w0 = omega0 + ((size_t)b * 3 + 2) * n;
-    float acc = 0.f;
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x)
-        acc += expf(-(float)w0[i]) * expm1f(-(float)(w[i] - w0[i]));
-    const double s = block_sum((double)acc, red);
-    if (threadIdx.x == 0) part[(size_t)b * kRedBlocks + blockIdx.x] = s;
-    finish_planes(part, gridDim.y, scale, out, cnt);
+    if (p >= n) return;
+    const double *w = omega + (size_t)b * 3 * n + p, *w0 = omega0 + (size_t)b * 3 * n + p, *m = mean + b * 3, *m0 = mean0 + b * 3;
+    float v[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] = (float)(s_in * ((w[c * n] - w0[c * n]) - (m[c] - m0[c])));
+    store_input(t0 + ((size_t)b * n + p) * 16, v[0], v[1], v[2]);
 }
 
 // Densities after a field change: Phi_A, Phi_B = the densities at omega0
 // plus s_out (dy4 - <dy4>) (the tangent output); Phi_S of Eq. (11) at omega
 // as the densities at omega0 plus the exact change,
 //   Phi_S = Phi0_S + Phi0_S (q - m) / (1 + m),  m = <e q> / <e>,
-// every term of the size of the change (e, q as in solvent_change_partials).
-__global__ void densities_tangent(const float *t4, const double *tmean, const double *phi0, const double *omega,
-                                  const double *omega0, const double *e_mean, const double *eq_mean, double s_out, long long n,
-                                  int nb, double *phi)
+// every term of the size of the change (e, q as in field_partials).
+__global__ void __launch_bounds__(256) densities_tangent(const float *t4, const double *tmean, const double *phi0, const double *omega,
+                                                         const double *omega0, const double *e_mean, const double *eq_mean, double s_out,
+                                                         long long n, double *phi)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * nb) return;
-    const long long b = i / n, p = i % n;
-    const float2 y = *reinterpret_cast<const float2 *>(&t4[(size_t)i * 8]);
-    phi[(b * 3 + 0) * n + p] = phi0[(b * 3 + 0) * n + p] + s_out * ((double)y.x - tmean[2 * b]);
-    phi[(b * 3 + 1) * n + p] = phi0[(b * 3 + 1) * n + p] + s_out * ((double)y.y - tmean[2 * b + 1]);
-    const size_t q = (b * 3 + 2) * n + p;
-    const double dq = (double)expm1f(-(float)(omega[q] - omega0[q])), m = eq_mean[b] / e_mean[b];
-    phi[q] = phi0[q] + phi0[q] * (dq - m) / (1.0 + m);
+    __shared__ double k[4];
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.y;
+    if (threadIdx.x == 0) {
+        const double m = eq_mean[b] / e_mean[b];
+        k[0] = tmean[2 * b];
+        k[1] = tmean[2 * b + 1];
+        k[2] = m;
+        k[3] = 1.0 / (1.0 + m);
+    }
+    __syncthreads();
+    if (p >= n) return;
+    const float2 y = *reinterpret_cast<const float2 *>(&t4[((size_t)b * n + p) * 8]);
+    const size_t q = (size_t)b * 3 * n + p;
+    const double a0 = phi0[q], b0 = phi0[q + n], s0 = phi0[q + 2 * n];
+    const double dq = (double)expm1f(-(float)(omega[q + 2 * n] - omega0[q + 2 * n]));
+    phi[q] = a0 + s_out * ((double)y.x - k[0]);
+    phi[q + n] = b0 + s_out * ((double)y.y - k[1]);
+    phi[q + 2 * n] = s0 + s0 * (dq - k[2]) * k[3];
 }
 
 // Densities from the network output: Phi_A, Phi_B with exact means, Phi_S from
 // Eq. (11) (exp(-w_S) in FP32, Q_S the per-sample mean of the same values).
-__global__ void densities_out(const float *y4, const double *ymean, const double *omega, const double *qs_mean, double s_out,
-                              double pa_bar, double pb_bar, double ps_bar, long long n, int nb, double *phi)
+__global__ void __launch_bounds__(256) densities_out(const float *y4, const double *ymean, const double *omega, const double *qs_mean,
+                                                     double s_out, double pa_bar, double pb_bar, double ps_bar, long long n, double *phi)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * nb) return;
-    const long long b = i / n, p = i % n;
-    const float2 y = *reinterpret_cast<const float2 *>(&y4[(size_t)i * 8]);
-    phi[(b * 3 + 0) * n + p] = pa_bar + s_out * ((double)y.x - ymean[2 * b]);
-    phi[(b * 3 + 1) * n + p] = pb_bar + s_out * ((double)y.y - ymean[2 * b + 1]);
-    phi[(b * 3 + 2) * n + p] = ps_bar * (double)expf(-(float)omega[(b * 3 + 2) * n + p]) / qs_mean[b];
+    __shared__ double k[3];
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.y;
+    if (threadIdx.x == 0) {
+        k[0] = ymean[2 * b];
+        k[1] = ymean[2 * b + 1];
+        k[2] = ps_bar / qs_mean[b];
+    }
+    __syncthreads();
+    if (p >= n) return;
+    const float2 y = *reinterpret_cast<const float2 *>(&y4[((size_t)b * n + p) * 8]);
+    const size_t q = (size_t)b * 3 * n + p;
+    phi[q] = pa_bar + s_out * ((double)y.x - k[0]);
+    phi[q + n] = pb_bar + s_out * ((double)y.y - k[1]);
+    phi[q + 2 * n] = k[2] * (double)expf(-(float)omega[q + 2 * n]);
 }
 
 // Loss and output gradient: targets t_c = (Phi_c - <Phi_c>) / s_out for
 // c = A, B; loss = mean over samples, channels, pixels of (y - t)^2; dZ4 =
 // 2 (y - t) / count in BF16 ([b][p][16], channels >= 2 zero).  Per-block
-// partial loss sums to lpart.
-__global__ void __launch_bounds__(256) loss_grad(const float *y4, const double *phi_t, const double *tmean, double s_out, long long n,
-                                                 int nb, __nv_bfloat16 *dz4, double *lpart)
+// partial loss sums to lpart.  inv_s = 1 / s_out, two_c = 2 / count.
+__global__ void __launch_bounds__(256) loss_grad(const float *y4, const double *phi_t, const double *tmean, double inv_s, double two_c,
+                                                 long long n, __nv_bfloat16 *dz4, double *lpart)
 {
     __shared__ double red[32];
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.y;
     double l = 0.0;
-    if (i < n * nb) {
-        const long long b = i / n, p = i % n;
-        const double cnt = 2.0 * (double)n * (double)nb;
-        __align__(16) __nv_bfloat16 v[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const double tc = (phi_t[(b * 3 + c) * n + p] - tmean[b * 3 + c]) / s_out;
-            const double d = (double)y4[(size_t)i * 8 + c] - tc;
-            l += d * d;
-            v[c] = __float2bfloat16_rn((float)(2.0 * d / cnt));
-        }
-        uint4 *dst = reinterpret_cast<uint4 *>(dz4 + (size_t)i * 16);
-        dst[0] = *reinterpret_cast<uint4 *>(&v[0]);
-        dst[1] = *reinterpret_cast<uint4 *>(&v[8]);
+    if (p < n) {
+        const float2 y = *reinterpret_cast<const float2 *>(&y4[((size_t)b * n + p) * 8]);
+        const double *ph = phi_t + (size_t)b * 3 * n + p;
+        const double d0 = (double)y.x - (ph[0] - tmean[b * 3]) * inv_s, d1 = (double)y.y - (ph[n] - tmean[b * 3 + 1]) * inv_s;
+        l = d0 * d0 + d1 * d1;
+        store_input(dz4 + ((size_t)b * n + p) * 16, (float)(two_c * d0), (float)(two_c * d1), 0.f);
     }
     l = block_sum(l, red);
-    if (threadIdx.x == 0) lpart[blockIdx.x] = l;
+    if (threadIdx.x == 0) lpart[(size_t)b * gridDim.x + blockIdx.x] = l;
 }
 
 // Sum of `cnt` per-block partials (fixed order) -> out[0] / denom.
@@ -935,7 +1002,6 @@ static void plane_means(const Work &w, const void *f, int kind, int planes, doub
     const dim3 g(kRedBlocks, planes);
     const double sc = 1.0 / (double)w.n;
     if (kind == 0) plane_partials<0><<<g, 256, 0, s>>>(f, w.n, w.red, sc, out, w.cnt);
-    else if (kind == 1) plane_partials<1><<<g, 256, 0, s>>>(f, w.n, w.red, sc, out, w.cnt);
     else plane_partials<2><<<g, 256, 0, s>>>(f, w.n, w.red, sc, out, w.cnt);
 }
 
@@ -1057,13 +1123,13 @@ cudaError_t forward(Work &w, const float *params, const double *omega, double *p
     cudaError_t e;
     if ((e = ready_counter(w, s))) return e;
     if (!w.prepacked && (e = pack_all(w, params, false, s))) return e;
-    plane_means(w, omega, 0, w.nb * 3, w.means, s);
-    prep_input<<<blocks(w.n * w.nb), 256, 0, s>>>(omega, w.means, s_in, w.n, w.nb, reinterpret_cast<__nv_bfloat16 *>(w.x0));
+    // (the partials in the output's buffer, written later)
+    field_partials<false><<<dim3(kRedBlocks, 4 * w.nb), 256, 0, s>>>(omega, nullptr, w.n, (double *)w.y4, 1.0 / (double)w.n, w.means, w.qs, w.cnt);
+    const dim3 px(blocks(w.n), w.nb);
+    prep_input<<<px, 256, 0, s>>>(omega, w.means, s_in, w.n, reinterpret_cast<__nv_bfloat16 *>(w.x0));
     if ((e = forward_layers(w, params, s))) return e;
     plane_means(w, w.y4, 2, w.nb * 2, w.ymean, s);
-    plane_means(w, omega, 1, w.nb, w.qs, s);
-    densities_out<<<blocks(w.n * w.nb), 256, 0, s>>>((const float *)w.y4, w.ymean, omega, w.qs, s_out, pa_bar, pb_bar, ps_bar, w.n, w.nb,
-                                                     phi);
+    densities_out<<<px, 256, 0, s>>>((const float *)w.y4, w.ymean, omega, w.qs, s_out, pa_bar, pb_bar, ps_bar, w.n, phi);
     return cudaGetLastError();
 }
 
@@ -1074,18 +1140,18 @@ cudaError_t tangent(Work &w, const float *params, const double *omega, const dou
     // means of omega0 (w.means) and <exp(-omega0_S)> (w.qs)
     cudaError_t e;
     if ((e = ready_counter(w, s))) return e;
-    plane_means(w, omega, 0, w.nb * 3, w.means2, s);
-    prep_tangent<<<blocks(w.n * w.nb), 256, 0, s>>>(omega, omega0, w.means2, w.means, s_in, w.n, w.nb,
-                                                    reinterpret_cast<__nv_bfloat16 *>(w.t0));
+    // <e q> and the partials in the forward pass's output buffer, which is free
+    // again; <e> at omega0 is in qs
+    double *eq = (double *)w.y4;
+    field_partials<true><<<dim3(kRedBlocks, 4 * w.nb), 256, 0, s>>>(omega, omega0, w.n, eq + w.nb, 1.0 / (double)w.n, w.means2, eq, w.cnt);
+    const dim3 px(blocks(w.n), w.nb);
+    prep_tangent<<<px, 256, 0, s>>>(omega, omega0, w.means2, w.means, s_in, w.n, reinterpret_cast<__nv_bfloat16 *>(w.t0));
     conv<16, 32, EP_JVP, kD0>(w, w.t0, w.wf[0], nullptr, w.t[0], nullptr, nullptr, 32, s, w.y[0]);
     conv<32, 32, EP_JVP, kD1>(w, w.t[0], w.wf[1], nullptr, w.t[1], nullptr, nullptr, 32, s, w.y[1]);
     conv<32, 32, EP_JVP, kD2>(w, w.t[1], w.wf[2], nullptr, w.t[0], nullptr, nullptr, 32, s, w.y[2]);
     conv<32, 8, EP_LINEAR, kD3>(w, w.t[0], w.wf[3], nullptr, nullptr, (float *)w.t4, nullptr, 2, s);
     plane_means(w, w.t4, 2, w.nb * 2, w.ymean, s);
-    // <e q> into means2 (free again); <e> at omega0 is in qs
-    solvent_change_partials<<<dim3(kRedBlocks, w.nb), 256, 0, s>>>(omega, omega0, w.n, w.red, 1.0 / (double)w.n, w.means2, w.cnt);
-    densities_tangent<<<blocks(w.n * w.nb), 256, 0, s>>>((const float *)w.t4, w.ymean, phi0, omega, omega0, w.qs, w.means2, s_out,
-                                                         w.n, w.nb, phi);
+    densities_tangent<<<px, 256, 0, s>>>((const float *)w.t4, w.ymean, phi0, omega, omega0, w.qs, eq, s_out, w.n, phi);
     (void)ps_bar;
     return cudaGetLastError();
 }
@@ -1095,9 +1161,15 @@ static void dw(Work &w, const void *x, const void *dzp, cudaStream_t s)
 {
     const int tiles_x = w.nx / TW;
     const int ntiles = w.nb * tiles_x * (w.ny / TH);
-    const int per = (ntiles + w.nblk_dw - 1) / w.nblk_dw;
+    // two CTAs per SM: fewer partials for reduce_dw, whose FP64 sums are
+    // bound by the FP64 unit (512 CTAs: 22 us per 32 x 32 layer)
+    const int cap = std::min(w.nblk_dw, 2 * 152), per = (ntiles + cap - 1) / cap;
     const int nblk = (ntiles + per - 1) / per;
-    conv3x3_dw<CI, CO, D><<<nblk, 288, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(x), reinterpret_cast<const __nv_bfloat16 *>(dzp),
+    constexpr size_t smem = DwGeom<CI, CO, D>::SMEM;
+    static const cudaError_t set =
+        cudaFuncSetAttribute(conv3x3_dw<CI, CO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    (void)set;  // a failure shows at the launch
+    conv3x3_dw<CI, CO, D><<<nblk, 288, smem, s>>>(reinterpret_cast<const __nv_bfloat16 *>(x), reinterpret_cast<const __nv_bfloat16 *>(dzp),
                                             w.dwpart, w.nx, w.ny, tiles_x, per, ntiles);
     w.nblk_dw = nblk;
 }
@@ -1122,13 +1194,15 @@ cudaError_t gradients(Work &w, const float *params, const double *omega, const d
     if ((e = ready_counter(w, s))) return e;
     if ((e = pack_all(w, params, true, s))) return e;
     plane_means(w, omega, 0, w.nb * 3, w.means, s);
-    prep_input<<<blocks(w.n * w.nb), 256, 0, s>>>(omega, w.means, s_in, w.n, w.nb, reinterpret_cast<__nv_bfloat16 *>(w.x0));
+    const dim3 px(blocks(w.n), w.nb);
+    prep_input<<<px, 256, 0, s>>>(omega, w.means, s_in, w.n, reinterpret_cast<__nv_bfloat16 *>(w.x0));
     if ((e = forward_layers(w, params, s))) return e;
     plane_means(w, phi_t, 0, w.nb * 3, w.tmean, s);
-    const unsigned lb = blocks(w.n * w.nb);
-    loss_grad<<<lb, 256, 0, s>>>((const float *)w.y4, phi_t, w.tmean, s_out, w.n, w.nb, reinterpret_cast<__nv_bfloat16 *>(w.dz4),
+    const double count = 2.0 * (double)w.n * w.nb;
+    // n is a multiple of 256 (sides multiples of 16): nb n / 256 partials
+    loss_grad<<<px, 256, 0, s>>>((const float *)w.y4, phi_t, w.tmean, 1.0 / s_out, 2.0 / count, w.n, reinterpret_cast<__nv_bfloat16 *>(w.dz4),
                                  w.lpart);
-    sum_parts<<<1, 256, 0, s>>>(w.lpart, (int)lb, 2.0 * (double)w.n * w.nb, loss_dev);
+    sum_parts<<<1, 256, 0, s>>>(w.lpart, (int)(px.x * px.y), count, loss_dev);
     // layer 4: dW from y3 and dZ4; dZ3 = (W4^T dZ4) (1 - y3^2)
     layer_grads(w, 3, w.y[2], w.dz4, 16, 32, s);
     conv<16, 32, EP_DX, kD3>(w, w.dz4, w.wb[3], nullptr, w.dz[0], nullptr, (const float *)w.yf[2], 32, s);
