@@ -847,29 +847,35 @@ __global__ void __launch_bounds__(256) bias_grad_part(const __nv_bfloat16 *dz, l
 #pragma unroll
     for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = (double)acc[j];
     __syncthreads();
-    if (threadIdx.x < CO) {
-        const int c = threadIdx.x, gc = c / 8, j = c % 8;
-        double t = 0.0;
-        for (int k = gc; k < (int)blockDim.x; k += c8n) t += red[k][j];
-        part[(size_t)blockIdx.x * CO + c] = t;
+    // channel c of slice sl: 256 / CO slices, then a fixed tree over them (one
+    // thread's chain of 64-128 dependent FP64 additions was 4-8 us)
+    const int c = threadIdx.x % CO, sl = threadIdx.x / CO, nsl = 256 / CO, gc = c / 8, j = c % 8;
+    const int rows = 256 / c8n, per = rows / nsl;  // rows of red per channel group, and per slice
+    double t = 0.0;
+    for (int k = sl * per; k < (sl + 1) * per; ++k) t += red[k * c8n + gc][j];
+    __shared__ double sums[256];
+    sums[threadIdx.x] = t;
+    __syncthreads();
+    if (sl == 0) {
+        double u = 0.0;
+        for (int k = 0; k < nsl; ++k) u += sums[k * CO + c];
+        part[(size_t)blockIdx.x * CO + c] = u;
     }
 }
-// (one block of 256 threads: 8 slices of the blocks per channel, the
-// slices' sums added in a fixed order)
-__global__ void __launch_bounds__(256) bias_grad_finish(const double *part, int nblk, int CO, int co_real, float *gb)
+// (one block of 1024 threads: 32 slices of the blocks per channel, the
+// slices' sums by a fixed shuffle tree)
+__global__ void __launch_bounds__(1024) bias_grad_finish(const double *part, int nblk, int CO, int co_real, float *gb)
 {
-    __shared__ double red[8][32];
+    __shared__ double red[32][33];
     const int c = threadIdx.x & 31, sl = threadIdx.x >> 5;
     double t = 0.0;
     if (c < CO)
-        for (int b = sl; b < nblk; b += 8) t += part[(size_t)b * CO + c];
-    red[sl][c] = t;
+        for (int b = sl; b < nblk; b += 32) t += part[(size_t)b * CO + c];
+    red[c][sl] = t;
     __syncthreads();
-    if (sl == 0 && c < co_real) {
-        double u = 0.0;
-        for (int k = 0; k < 8; ++k) u += red[k][c];
-        gb[c] = (float)u;
-    }
+    double u = red[sl][c];  // warp sl: channel sl, lane c: slice c
+    for (int o = 16; o > 0; o >>= 1) u += __shfl_down_sync(0xffffffffu, u, o);
+    if (c == 0 && sl < co_real) gb[sl] = (float)u;
 }
 
 // Adam on the FP32 master parameters (Kingma and Ba, 2015).
@@ -1183,7 +1189,7 @@ static void layer_grads(Work &w, int l, const void *x, const void *dzp, int CO, 
     else dw<32, 16, kD3>(w, x, dzp, s);
     reduce_dw<<<(9 * CO * CI + 31) / 32, 256, 0, s>>>(w.dwpart, w.nblk_dw, kCout[l], kCin[l], CO, CI, w.grad + param_offset_w(l));
     bias_grad_part<<<kBiasBlocks, 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(dzp), (long long)w.nb * w.n, CO, w.bpart);
-    bias_grad_finish<<<1, 256, 0, s>>>(w.bpart, kBiasBlocks, CO, kCout[l], w.grad + param_offset_b(l));
+    bias_grad_finish<<<1, 1024, 0, s>>>(w.bpart, kBiasBlocks, CO, kCout[l], w.grad + param_offset_b(l));
     w.nblk_dw = ntiles_cap;
 }
 
