@@ -104,12 +104,16 @@ __device__ __forceinline__ void col_tile(const PropK<T> &k, const Tile &tl, cons
 // (block A, B) and of its mirror N_s - m.
 struct RowWeights {
     double a1, b1, a2, b2;
+    bool a, b;  // whether a block has a weight there at all (compared on the host: FP64 comparisons were 9% of an FP32 row pass)
 };
 inline RowWeights row_weights(const GroupGeom &g, int m)
 {
     const int ns = g.ns, na = g.na, s2 = ns - m;
-    return {weight_a(m, na, g.ds), weight_b(m, na, ns, g.ds), s2 == m ? 0.0 : weight_a(s2, na, g.ds),
-            s2 == m ? 0.0 : weight_b(s2, na, ns, g.ds)};
+    RowWeights w = {weight_a(m, na, g.ds), weight_b(m, na, ns, g.ds), s2 == m ? 0.0 : weight_a(s2, na, g.ds),
+                    s2 == m ? 0.0 : weight_b(s2, na, ns, g.ds), false, false};
+    w.a = w.a1 != 0.0 || w.a2 != 0.0;
+    w.b = w.b1 != 0.0 || w.b2 != 0.0;
+    return w;
 }
 
 // Row pass producing contour node m (1 <= m <= ns): Tx, node factors, history
@@ -189,8 +193,8 @@ __device__ __forceinline__ void row_tile(const PropK<T> &k, const Tile &tl, cons
             } else {
                 const bool store_all = k.hnodes == ns + 1, acc = !store_all && m >= hhi;
                 // only the block(s) with a weight at this node or its mirror
-                const bool use_a = acc && (m == hhi || w.a1 != 0.0 || w.a2 != 0.0);
-                const bool use_b = acc && (m == hhi || w.b1 != 0.0 || w.b2 != 0.0);
+                const bool use_a = acc && (m == hhi || w.a);
+                const bool use_b = acc && (m == hhi || w.b);
                 double *ia = k.ia + (size_t)run * n + base, *ib = k.ib + (size_t)run * n + base;
 #pragma unroll
                 for (int u0 = 0; u0 < R0; u0 += CH) {
