@@ -34,9 +34,9 @@ UNIT = "site·contour-steps/s"
 HBM_FALLBACK = 6800.0
 # FP32 (non-tensor) units of a GB300 at its maximum SM clock
 FP32_SMS, FP32_LANES, FP32_MHZ = 152, 128, 2070.0
-# dram__bytes_read.sum + dram__bytes_write.sum of the 8 prop_chain<9,8,16,256,1,1>
+# dram__bytes_read.sum + dram__bytes_write.sum of the 8 prop_chain<9,8,16,256,1,1,0>
 # launches of one differential solve of the channel workload (ncu, one capture)
-CHAIN_DIFF_TRAFFIC_BYTES = 391.25e6 + 7.20e6
+CHAIN_DIFF_TRAFFIC_BYTES = 363.49e6 + 8.22e6
 
 
 def max_over_ranks(x: float, dist=None, device="cpu") -> float:
@@ -803,8 +803,8 @@ def main():
                     "peak_source": "derived FP32 peak: 152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"}
     else:
         # streaming passes, per site and contour step (FP32 complex z = g + i g'):
-        # radix-8 row pass = chain read 8 + write 8, factors 8, history store 8;
-        # radix-2 row pass accumulating the contour sums also reads the history
+        # row pass = chain read 8 + write 8, factors 8, history store 8;
+        # the general row pass accumulating the contour sums also reads the history
         # and read-modify-writes the FP64 sums; column pass = chain read + write
         # MIXED (differential second solve, whose passes are the timed ones):
         # chain read + write 16, factors 8, rho 8, reference node 8, change
@@ -818,7 +818,7 @@ def main():
             gbs = bps * nsite / (kt[k] * 1e-3) / 1e9
             kernels[k] = {"ms": kt[k], "bytes_per_site": bps, "achieved_gbs": gbs, "frac": gbs / hbm}
         dom = "prop_row_accumulate"
-        name = ("prop_row8 (row pass of one contour step, radix-8 streaming" if radix8 else "prop_row (row pass, streaming") + \
+        name = ("stream_row_k (row pass of one contour step, streaming on power-of-two tiles" if radix8 else "prop_row (row pass, streaming") + \
             (", differential second solve)" if h.tiles(0)["differential"] else ")")
         roofline = {"bound": "hbm", "kernel": name, "achieved": kernels[dom]["achieved_gbs"], "peak": hbm,
                     "unit": "GB/s", "frac": kernels[dom]["achieved_gbs"] / hbm, "traffic": None,

@@ -72,7 +72,7 @@ enum {
  * Parameters of one run (Sec. 2 model, Sec. 3 and Sec. 4 set-up).
  *  nx, ny      grid sites per axis in [8, 2048], even and of the form 2^a 3^b 5^c
  *              (the paper's 150 x 150 included); nx is the flow axis.  Axes that
- *              are not powers of two take mixed-radix (2, 3, 4, 5) transforms in
+ *              are not powers of two take transforms of radices 2 to 16 in
  *              the streaming passes.
  *  ns          contour steps N_s in [2, 512]; even for MIXED_FP32 on
  *              power-of-two grids (the paper's N_s = N = 17 runs elsewhere)
@@ -237,8 +237,8 @@ int epd_lb_enable_timing(epd_lb *h, int32_t on);
 int epd_lb_kernel_times(epd_lb *h, double *ms);
 
 /* Launch configuration chosen for a run's group (batching and tiling of the
- * hot path; not in the paper).  out[0]: solve path, 0 = streaming radix-2 /
- * mixed-radix passes, 1 = streaming radix-8 passes with the full contour history, 2 =
+ * hot path; not in the paper).  out[0]: solve path, 0 = general streaming
+ * passes, 1 = streaming passes on power-of-two tiles with the full contour history, 2 =
  * cluster-resident solve; out[1]: CTAs per cluster (path 2) or 0; out[2]: the
  * column tile width of the radix-8 column passes (EPD and streaming
  * propagator; 4, 8 or 16 columns), chosen at epd_lb_init by timing each
@@ -457,7 +457,10 @@ int epd_lb3d_step(const epd_lb_params *p, int32_t nz, const double *pop_in_dev, 
  * omega_dev (3*ny*nx doubles) -> phi_dev (3*ny*nx doubles), q_dev[2] =
  * (Q_P, Q_S).  workspace_dev of epd_prop_solve_workspace_bytes bytes holds the
  * propagator history and the transform buffers; cuda_stream may be NULL (the
- * legacy default stream).  Asynchronous.
+ * legacy default stream).  Asynchronous.  In EPD_LB_MIXED_FP32 on the grids of
+ * the cluster-resident solve the queried size holds that solve's states; a
+ * workspace of the streaming passes' size (half the history, about
+ * nx*ny*(16 + (ns/2 + 3)*8) + 40 KiB bytes) is taken as well, with those passes.
  */
 int epd_prop_solve_workspace_bytes(const epd_lb_params *p, size_t *bytes);
 int epd_prop_solve(const epd_lb_params *p, const double *omega_dev, double *phi_dev, double *q_dev,

@@ -479,7 +479,7 @@ class EpdLb:
 
     def tiles(self, run: int) -> dict:
         """Launch configuration of a run's group: solve path (0 streaming
-        radix-2, 1 streaming radix-8, 2 cluster), CTAs per cluster, the
+        passes, 1 streaming on power-of-two tiles, 2 cluster), CTAs per cluster, the
         autotuned column tile widths (EPD passes; streaming propagator
         passes), whether the differential second solve is used, and the
         chain-kernel launches per cluster solve."""

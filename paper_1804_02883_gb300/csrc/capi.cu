@@ -87,8 +87,11 @@ size_t carve_group(Group &G, char *base, size_t off)
         G.hd = take(hs);
         G.rho = take(R * n * sizeof(float2));
         G.cdiff = take(R * 3 * n * sizeof(float));
-        G.facp = take(R * 3 * n * sizeof(float));
-        G.facd = take(R * 3 * n * sizeof(float));
+        // the factor planes (12 bytes per site) in the streaming passes' contour
+        // sums (two adjoining arrays of 8; sizes on these grids are multiples
+        // of the alignment), which this solve does not use
+        G.facp = G.ia;
+        G.facd = G.ia2;
     } else if (stream_diff) {
         G.hd = take(R * (size_t)(G.g.ns + 1) * n * sizeof(float2));
         G.rho = take(R * n * sizeof(float2));
@@ -386,9 +389,9 @@ static std::string validate(const epd_lb_params &p)
                       p.ny, kMinN, kMaxN);
         return buf;
     }
-    // the MIXED power-of-two paths (cluster-resident and radix-8 streaming
-    // solves) pair contour nodes symmetrically and need N_s even; the radix-2
-    // streaming solve (PLAIN_FP64, mixed-radix grids) takes any N_s, such as
+    // the MIXED power-of-two paths (cluster-resident and streaming solves) pair
+    // contour nodes symmetrically and need N_s even; the general streaming
+    // solve (PLAIN_FP64, other grids) takes any N_s, such as
     // the paper's N_s = N = 17
     const bool any_ns = p.precision == EPD_LB_PLAIN_FP64 || !(pow2(p.nx) && pow2(p.ny));
     if (p.ns < 2 || p.ns > 512 || ((p.ns & 1) && !any_ns)) {
@@ -1287,8 +1290,8 @@ extern "C" void epd_lb_destroy(epd_lb *h)
 // Tables of a stateless call, written on the device: twiddles exp(-2 pi i t /
 // n), t < n, the Fourier factors exp(-R_G^2 k^2 ds) / n of Eq. (8), and the
 // pass tables of the cluster solve (fft8.cuh layout).  Formed in FP64.  (The
-// host built them per call, six to ten pageable copies and a synchronisation:
-// 0.1 ms of a 128 x 128 solve.)
+// host built them per call: six to ten pageable copies and a synchronisation,
+// where this launch is 11 us beside the 0.34 ms of a 128 x 128 solve.)
 struct AxisTables {
     int n;
     void *tw, *kf;                // may be null
@@ -1643,8 +1646,8 @@ extern "C" int epd_prop_solve(const epd_lb_params *p, const double *omega_dev, d
     if (!solve_group(p, G) || !omega_dev || !phi_dev || !q_dev || !workspace_dev) return EPD_LB_EINVAL;
     if (workspace_bytes < carve_solve(G, nullptr) || ((uintptr_t)workspace_dev & 255)) return EPD_LB_ENOMEM;
     // the cluster-resident solve where the grid has one and the workspace
-    // holds its states (128 x 128, N_s = 64: 0.76 ms as streaming passes, 0.30
-    // resident); a workspace of the streaming passes' size still does
+    // holds its states (128 x 128, N_s = 64: 0.76 ms a call as streaming passes,
+    // 0.35 resident); a workspace of the streaming passes' size still does
     Group C = G;
     const size_t cluster_bytes = carve_solve_cluster(C, nullptr);
     if (cluster_bytes && workspace_bytes >= cluster_bytes && cluster_solve_supported(G)) {

@@ -68,8 +68,8 @@ struct Group {
     // FP64 fields, [run][species][n]
     double *omega, *omega_t, *phi, *phi_t;
     double *q, *q_t;   // [run][2]
-    double *ia, *ib;   // contour sums, [run][n]
-    double *ia2, *ib2; // contour sums of the g' chain's terms (cluster solve), [run][n]
+    double *ia, *ib;   // contour sums of the streaming solves, [run][n]; cluster solve: facp
+    double *ia2, *ib2; // cluster solve: facd, [run][n]
     // differential second solve (MIXED_FP32).  Cluster solve: states of both
     // chains at every node, in the padded row layout
     // [run][chain][ns+1][ny/2][nx + nx/8] float2 (hc: plain / reference
@@ -85,10 +85,10 @@ struct Group {
     bool stateless = false;   // one solve on a caller's stream, not a handle's captured step
     bool diff = false;        // the step uses the reference + differential solve pair
     bool phi_stale = false;   // omega was replaced since phi was last computed
-    bool hist_full = false;   // streaming radix-8 solve (hist holds all N_s + 1 nodes)
+    bool hist_full = false;   // MIXED streaming solve on power-of-two tiles (hist holds all N_s + 1 nodes)
     int hnodes = 0;           // nodes of hist per run: N_s + 1 (MIXED streaming solves) or half_lo + 1
     int colw = 0;             // radix-8 EPD column tile width chosen by the autotuner (0: default)
-    int colw_prop = 0;        // radix-8 streaming propagator column tile width (0: default)
+    int colw_prop = 0;        // column tile width of the streaming propagator on power-of-two tiles (0: default)
     // exact step (CG inversion of App. C), FP64 [run][3][n] unless noted
     double *cg_target = nullptr;  // Phi~ = Phi(t) - dt div(v Phi(t))
     double *cg_dir = nullptr;     // search direction d
@@ -209,7 +209,7 @@ bool cluster_shape_exists(int logx, int logy);
 // differential one): 1, or 2 nruns when the chains are one more than the
 // clusters that fit at one CTA per SM (the phased schedule); 0 without a shape.
 int cluster_chain_launches(const Group &G, bool diff);
-// MIXED grids solved by the radix-8 streaming passes with the full history
+// MIXED grids solved by the streaming passes on power-of-two tiles with the full history
 bool stream8_eligible(int prec, int logx, int logy);
 size_t cluster_state_floats2(int nx, int ny, int ns);  // per run, both chains
 // Chain launch plus contour sums and normalisation into phi, q (diff: the

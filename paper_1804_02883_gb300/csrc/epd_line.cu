@@ -8,7 +8,9 @@
 // are small (line_logb) so that a 64 x 64 grid has 64-128 CTAs instead of 2,
 // and what a row pass forms from FP64 fields (mu, omega) it leaves in the
 // transform's type for the column pass.  The x spectrum of the force travels
-// in the plan's digit-reversed order.
+// in the plan's digit-reversed order.  The FP64 unit bounds the FP64 passes (4 x
+// 256 x 512: 180 us a column pass), latency the FP32 ones: the seven passes of
+// a 64 x 150 x 150 step 0.48 -> 0.42 ms as kernel time (cold, serialised).
 #include "common.cuh"
 #include "engine.h"
 #include "epd.cuh"

@@ -317,7 +317,7 @@ __device__ __forceinline__ int line_bin(LinePlan pl, int n, int p)
 
 // Twiddles of a butterfly, tw[u j] (tw[i] = exp(-2 pi i i / n)), read before
 // its points: with few warps per SM the reads' latency is exposed, and taken
-// one by one next to their uses it cost the FP64 passes 40%.  PROD: the powers
+// one by one next to their uses it is exposed at every butterfly.  PROD: the powers
 // of two are read, the others are products, w_u = w_(u mod 8) w_(u - u mod 8)
 // (power-of-two axes in FP32: a gather at stride u j touches a line per lane,
 // and fewer factors stay in registers).

@@ -480,7 +480,7 @@ cudaError_t launch_observables(Group &G, int run, int parity, double *part, doub
 // its 370 MB 54 us), so the moments come from the sums and differences of
 // opposite populations, the post-collision populations from their even and
 // odd parts, 1 / rho once, and the ghost part joins the moments (linear):
-// 2.09 -> 0.40 ms on 64 x 128 x 128 (the directions were a table in constant
+// 2.09 -> 0.38 ms on 64 x 128 x 128 (the directions were a table in constant
 // memory, every product formed: ~900 per site).
 __global__ void __launch_bounds__(kThreads) lb3d_step_k(int nx, int ny, int nz, double gs, double gb, double gg,
                                                         const double *__restrict__ in, const double *__restrict__ force,

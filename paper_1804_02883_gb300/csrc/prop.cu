@@ -16,14 +16,15 @@
 // the chains run through the second half, node m of g meets node N_s - m of g'
 // from the history (and vice versa), and the trapezoid sums of Eqs. (9)-(10)
 // are accumulated in FP64 on the fly.  In MIXED_FP32 every node is stored:
-// the full history is the reference of the differential second solve
-// (prop_row<T, true> and the radix-8 passes below), whose contour sums are a
-// separate pass over the stored nodes (prop_contour_stream).
+// the full history is the reference of the differential second solve, and the
+// contour sums are a separate pass over the stored nodes (prop_contour_stream).
+// The column and row passes are in prop_line.cuh (every grid, both precisions)
+// and prop_stream.cu (FP32 on power-of-two grids); this file holds the pointwise
+// and contour passes and the solves' host side.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdlib>
-#include <type_traits>
 
 #include "common.cuh"
 #include "engine.h"
@@ -99,10 +100,9 @@ __global__ void __launch_bounds__(kThreads) prop_start(PropK<T> k)
 }
 
 // Normalisation, Eqs. (9)-(11) with Q as spatial means.
-// ia2/ib2 (may be null): sums of the second chain's terms (cluster solve).
 __global__ void __launch_bounds__(kThreads) prop_finalize(GroupGeom g, int nrow_blocks, int nprep_blocks, const double *ia,
-                                                      const double *ib, const double *ia2, const double *ib2,
-                                                      const double *part, double *phi, double *q, int *err)
+                                                      const double *ib, const double *part, double *phi, double *q,
+                                                      int *err)
 {
     __shared__ double bc, fac[2];
     const int run = blockIdx.y;
@@ -125,10 +125,9 @@ __global__ void __launch_bounds__(kThreads) prop_finalize(GroupGeom g, int nrow_
     const double cp = fac[0], cs = fac[1];
     double *pa = phi + (size_t)run * 3 * n, *pb = pa + n, *ps = pb + n;
     const double *ja = ia + (size_t)run * n, *jb = ib + (size_t)run * n;
-    const double *ja2 = ia2 ? ia2 + (size_t)run * n : nullptr, *jb2 = ib2 ? ib2 + (size_t)run * n : nullptr;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        pa[i] = cp * (ja2 ? ja[i] + ja2[i] : ja[i]);
-        pb[i] = cp * (jb2 ? jb[i] + jb2[i] : jb[i]);
+        pa[i] = cp * ja[i];
+        pb[i] = cp * jb[i];
         ps[i] = cs * ps[i];
     }
 }
@@ -432,7 +431,7 @@ static cudaError_t solve_t(Group &G, const double *omega, double *phi, double *q
         prop_contour_stream<false><<<dim3((unsigned)((g.n + kThreads - 1) / kThreads), g.nruns), kThreads, 0, s>>>(
             g, reinterpret_cast<const float2 *>(G.hist), nullptr, blocks, pg, G.part, phi, q, nullptr, nullptr, G.err);
     else
-        prop_finalize<<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, blocks, pg, G.ia, G.ib, nullptr, nullptr, G.part, phi, q, G.err);
+        prop_finalize<<<dim3(pg, g.nruns), kThreads, 0, s>>>(g, blocks, pg, G.ia, G.ib, G.part, phi, q, G.err);
     return cudaGetLastError();
 }
 
@@ -519,7 +518,7 @@ static cudaError_t solve3d_t(const Solve3 &S, const double *omega, double *phi, 
         if (!e) e = line_row(kx, m, false, &blocks, s);
     }
     if (e) return e;
-    prop_finalize<<<dim3(pg, 1), kThreads, 0, s>>>(g, blocks, pg, S.ia, S.ib, nullptr, nullptr, S.part, phi, q, S.err);
+    prop_finalize<<<dim3(pg, 1), kThreads, 0, s>>>(g, blocks, pg, S.ia, S.ib, S.part, phi, q, S.err);
     return cudaGetLastError();
 }
 

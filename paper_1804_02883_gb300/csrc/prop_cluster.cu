@@ -656,8 +656,9 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
 #pragma unroll
     for (int c = 0; c < NST; ++c) issue(c, c * U);
     // The FP64 divisions by one thread per block: at 2 FP64 lanes per SM the
-    // four or five of every thread were 40% of this kernel (plain pass 65 ->
-    // 47 us, differential 96 -> 84 us on 4 x 256 x 512, N_s = 64, cold).
+    // four or five of every thread were a sixth of the plain pass (4 x 256 x 512,
+    // N_s = 64, cold: 65 -> 56 us; the differential one, bound by its two
+    // histories, 97 -> 95 us).
     const double *pr = k.part + (size_t)run * kMaxPart;
     const double tp = sum_partials(pr, k.nq, 1, &bc), ts = sum_partials(pr + kMaxPart / 2, k.ns_part, 1, &bc);
     if (tid == 0) {

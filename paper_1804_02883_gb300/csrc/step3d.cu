@@ -14,7 +14,8 @@
 // and an elementwise pass per derivative.  The force is one 3D transform
 // forward, in the plans' digit-reversed order, and two back: f_x + i f_y as one
 // complex field, f_z as another.  FP64 instructions bound all of it (2 lanes
-// per SM and cycle).  64 x 128 x 128 (ns = 16): these operators 5.1 -> 1.9 ms.
+// per SM and cycle).  64 x 128 x 128 (ns = 16): these operators 5.2 -> 2.4 ms
+// of kernel time (cold, serialised).
 #include <algorithm>
 #include <cmath>
 
