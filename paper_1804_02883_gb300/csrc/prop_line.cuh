@@ -8,6 +8,10 @@
 // pass; FP64: the FP64 unit (2 lanes per SM and cycle), so what counts there
 // is FP64 instructions per point and an even load of the SMs.  A CTA holds few
 // lines (line_logb) so that every grid gives each SM several tiles.
+// Per launch (cold, serialised), 64 x 150 x 150 in FP32, 32 runs as Stockham
+// passes -> 64 runs now: column 24.3 -> 14.6 us, row 37.7 -> 24.4 us (1.9 TB/s
+// of the chain, factors and history; no instruction to issue for a third of the
+// stalls).  FP64, 4 x 256 x 512, N_s = 64: 53 and 73 us, a step 20.4 -> 15.0 ms.
 #pragma once
 
 #include "common.cuh"
@@ -260,6 +264,11 @@ cudaError_t launch_line(bool dependent, K kernel, dim3 grid, int threads, size_t
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = dependent ? 1 : 0;
+    // tiles past the default limit: wide column tiles on long axes, and the
+    // row tiles of 3D boxes that fill the Q partials (per launch, so on
+    // whichever device is current)
+    if (smem > 48 * 1024)
+        if (cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

@@ -9,7 +9,10 @@
 // barriers (ten and nine as load, Stockham passes and store).  Radix 32 would
 // save two more of each but holds 168-250 registers: 512 x 512 (9 runs, N_s =
 // 24) 2.27 ms a step with 32.16, 2.14 with 8.8.8.  1024 x 2048, N_s = 128:
-// 8.9 -> 8.1 ms a step.
+// 8.9 -> 8.1 ms a step; per launch (cold, serialised) column 19.9 -> 15.5 us
+// (2.2 TB/s), differential row 23.5 -> 21.4 us (4.7 TB/s), plain row 17.9 -> 20.0 us
+// (in digit-reversed order both transforms of a pair read twiddles; the pair of
+// passes is what gains).
 #include "prop_line.cuh"
 
 namespace epdlb {
@@ -40,20 +43,12 @@ template <int LOGY, int LOGB> cudaError_t col_at(const PropK<float> &k, cudaStre
     if constexpr (sm > kMaxTile || tile_threads<LOGY, LOGB>() > 512) {
         return cudaErrorInvalidConfiguration;
     } else {
-        static const cudaError_t set =
-            cudaFuncSetAttribute(stream_col_k<LOGY, LOGB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (set) return set;
         return launch_line(k.dependent, stream_col_k<LOGY, LOGB>, dim3(k.g.nx >> LOGB, k.g.nruns), tile_threads<LOGY, LOGB>(), sm, s, k);
     }
 }
 template <int LOGX, int LOGB> cudaError_t row_at(const PropK<float> &k, int m, bool diff, const RowWeights &w, cudaStream_t s)
 {
     constexpr size_t sm = (size_t)TileOf<LOGX, LOGB, true>::POINTS * sizeof(float2);
-    static const cudaError_t set = [] {
-        cudaError_t e = cudaFuncSetAttribute(stream_row_k<LOGX, LOGB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        return e ? e : cudaFuncSetAttribute(stream_row_k<LOGX, LOGB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    }();
-    if (set) return set;
     const dim3 grid(k.g.ny >> LOGB, k.g.nruns);
     constexpr int th = tile_threads<LOGX, LOGB>();
     return diff ? launch_line(k.dependent, stream_row_k<LOGX, LOGB, true>, grid, th, sm, s, k, m, w)

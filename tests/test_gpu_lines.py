@@ -3,6 +3,7 @@ to four radices, every first, inner and last radix, lines fewer than a tile,
 columns that do not fill their last tile.  Single-chain solves against the
 FP64 oracle: 1e-12 in FP64; FP32 2e-6 (transforms of O(1) fields over two
 chains of N_s steps round to about 1e-7 of the largest value per step)."""
+import numpy as np
 import pytest
 
 import oracle as O
@@ -62,3 +63,21 @@ def test_stateless_solve_takes_either_workspace(ny, nx, ns):
                          torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert rel_err(pd.cpu().numpy(), phi) < 2e-6 and rel_err(qd.cpu().numpy(), q) < 2e-6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [P.PLAIN_FP64, P.MIXED_FP32])
+@pytest.mark.parametrize("nz,ny,nx", [(128, 144, 200), (160, 256, 100)])
+def test_box_with_more_rows_than_partials(nz, ny, nx, precision):
+    """Boxes of many x rows take more rows per tile to fit the Q partials, in
+    more shared memory than a kernel has by default.  Fields constant along z
+    give the 2D solve's densities in every plane (the same bounds as above)."""
+    run = P.RunParams(nx=nx, ny=ny, ns=2, precision=precision)
+    om = W.random_omega(ny, nx, 13)
+    phi, q = P.prop_solve3d(run, np.repeat(om[:, None], nz, axis=1))
+    h = P.EpdLb([run])
+    ph, qh = h.solve(0, om)
+    h.close()
+    tol = 1e-12 if precision == P.PLAIN_FP64 else 4e-6  # FP32: both sides round
+    assert rel_err(phi, np.repeat(ph[:, None], nz, axis=1)) < tol
+    assert rel_err(q, qh) < tol
