@@ -166,19 +166,22 @@ __device__ __forceinline__ void row_tile(const PropK<T> &k, const Tile &tl, cons
                 const float2 *rho = k.rho + (size_t)run * n + base;
                 V2<T> *hd = k.hd + ((size_t)run * (ns + 1) + m) * n + base;
                 const V2<T> *gref = hist + (size_t)m * n;
+                // eight points' operands in flight where the tile is known at compile time
+                // (1024 x 2048: 21.4 -> 19.3 us a launch)
+                constexpr int CD = Tile::fixed && R0 % 8 == 0 ? 8 : CH;
 #pragma unroll
-                for (int u0 = 0; u0 < R0; u0 += CH) {
-                    V2<T> eb[CH], grb[CH];
-                    float2 qb[CH];
+                for (int u0 = 0; u0 < R0; u0 += CD) {
+                    V2<T> eb[CD], grb[CD];
+                    float2 qb[CD];
 #pragma unroll
-                    for (int c = 0; c < CH; ++c) {
+                    for (int c = 0; c < CD; ++c) {
                         const int i = i0 + (u0 + c) * q;
                         eb[c] = efac[i];
                         grb[c] = gref[i];
                         qb[c] = rho[i];
                     }
 #pragma unroll
-                    for (int c = 0; c < CH; ++c) {
+                    for (int c = 0; c < CD; ++c) {
                         const int i = i0 + (u0 + c) * q;
                         const V2<T> e = eb[c], gr = grb[c], h = x[u0 + c];
                         const float2 r = qb[c];
