@@ -203,6 +203,23 @@ __device__ __forceinline__ void row_tile(const PropK<T> &k, const Tile &tl, cons
                 const bool use_a = acc && (m == hhi || w.a);
                 const bool use_b = acc && (m == hhi || w.b);
                 double *ia = k.ia + (size_t)run * n + base, *ib = k.ib + (size_t)run * n + base;
+                if constexpr (Tile::fixed) {
+                    if (store_all) {  // no sums: the factors of all the thread's points at once (1024 x 2048, 2 steps: 16.1 -> 15.3 ms)
+                        V2<T> eb[R0];
+#pragma unroll
+                        for (int u = 0; u < R0; ++u) eb[u] = efac[i0 + u * q];
+#pragma unroll
+                        for (int u = 0; u < R0; ++u) {
+                            const int i = i0 + u * q;
+                            const V2<T> e = eb[u], h = x[u];
+                            const V2<T> z = mk<T>((bag ? e.y : e.x) * h.x, (bap ? e.y : e.x) * h.y);
+                            hist[(size_t)m * n + i] = z;
+                            if (m == ns) qsum += (double)z.x;
+                            else data[i] = mk<T>((bdg ? e.y : e.x) * z.x, (bdp ? e.y : e.x) * z.y);
+                        }
+                        return;
+                    }
+                }
 #pragma unroll
                 for (int u0 = 0; u0 < R0; u0 += CH) {
                     V2<T> eb[CH], hvb[CH];
