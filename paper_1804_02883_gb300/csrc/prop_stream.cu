@@ -57,9 +57,9 @@ template <int LOGX, int LOGB> cudaError_t row_at(const PropK<float> &k, int m, b
 
 template <int LOGY> cudaError_t col_by(const PropK<float> &k, int colw, cudaStream_t s)
 {
-    if (!colw) {
+    if (!colw) {  // the widest that fits, narrower while the launch has fewer than four tiles per SM
         colw = LOGY >= 10 ? 8 : 16;
-        while (colw > 4 && (long long)(k.g.nx / colw) * k.g.nruns < 4 * 152) colw /= 2;
+        while (colw > 4 && (!stream_col_fits(1 << LOGY, colw) || (long long)(k.g.nx / colw) * k.g.nruns < 4 * 152)) colw /= 2;
     }
     switch (colw) {
     case 4: return col_at<LOGY, 2>(k, s);

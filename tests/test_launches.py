@@ -1,0 +1,22 @@
+"""Launches of the library's host side, checked without a GPU (fake_runtime)."""
+import pytest
+
+import paper_1804_02883_gb300 as P
+from paper_1804_02883_gb300 import workloads as W
+from fake_runtime import FakeRuntime
+
+
+@pytest.fixture(scope="module")
+def rt(tmp_path_factory):
+    return FakeRuntime(str(tmp_path_factory.mktemp("fake")))
+
+
+@pytest.mark.parametrize("ny", [64, 128, 256, 512, 1024, 2048])
+def test_default_column_tiles_launch_for_every_batch(rt, ny):
+    """epd_lb_init solves Phi(0) before it times the column widths: the default
+    width has to launch whatever the batch."""
+    for nx in (64, 128, 256, 512, 1024, 2048):
+        for runs in (1, 2, 3, 5, 10, 19, 38, 64):
+            r = W.with_(W.plain_small(), nx=nx, ny=ny, ns=2, precision=P.MIXED_FP32, f0=0.0)
+            rc, _ = rt.init([W.with_(r, seed=s) for s in range(runs)])
+            assert rc == 0, (nx, runs)
