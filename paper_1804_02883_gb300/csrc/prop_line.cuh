@@ -271,6 +271,8 @@ __global__ void __launch_bounds__(256, 2) prop_row(PropK<T> k, int m, int logb, 
     row_tile<T, R0, DIFF>(k, LineTile(true, k.g.nx, logb, k.g.px), k.g.px, m, w);
 }
 
+constexpr size_t kMaxTile = 200 * 1024;  // shared memory of a tile at most
+
 template <typename K, typename... A>
 cudaError_t launch_line(bool dependent, K kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
 {
@@ -284,11 +286,13 @@ cudaError_t launch_line(bool dependent, K kernel, dim3 grid, int threads, size_t
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = dependent ? 1 : 0;
-    // tiles past the default limit: wide column tiles on long axes, and the
-    // row tiles of 3D boxes that fill the Q partials (per launch, so on
-    // whichever device is current)
+    // Tiles past the default limit: wide column tiles on long axes, and the
+    // row tiles of 3D boxes that fill the Q partials.  The limit belongs to the
+    // function on the current device and every host thread sees it, so each
+    // such launch sets the same value, on whichever device is current.
+    if (smem > kMaxTile) return cudaErrorInvalidConfiguration;
     if (smem > 48 * 1024)
-        if (cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) return e;
+        if (cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxTile)) return e;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

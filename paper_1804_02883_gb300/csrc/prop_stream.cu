@@ -35,8 +35,6 @@ __global__ void __launch_bounds__(tile_threads<LOGX, LOGB>()) stream_row_k(PropK
     row_tile<float, LinePlanCT<LOGX>::r(0), DIFF>(k, TileOf<LOGX, LOGB, true>(), LinePlanCT<LOGX>(), m, w);
 }
 
-constexpr size_t kMaxTile = 200 * 1024;
-
 template <int LOGY, int LOGB> cudaError_t col_at(const PropK<float> &k, cudaStream_t s)
 {
     constexpr size_t sm = (size_t)TileOf<LOGY, LOGB, false>::POINTS * sizeof(float2);

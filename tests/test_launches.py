@@ -20,3 +20,14 @@ def test_default_column_tiles_launch_for_every_batch(rt, ny):
             r = W.with_(W.plain_small(), nx=nx, ny=ny, ns=2, precision=P.MIXED_FP32, f0=0.0)
             rc, _ = rt.init([W.with_(r, seed=s) for s in range(runs)])
             assert rc == 0, (nx, runs)
+
+
+def test_shared_memory_limits_never_fall(rt):
+    """The limit is the function's, shared by every host thread: a launch that
+    lowered it would fail another thread's launch of a wider tile.  Boxes whose
+    row tiles (58 and 52 KB) are one kernel's, the wider one first and last."""
+    boxes = [(160, 256, 100), (256, 320, 50), (160, 256, 100)]
+    for precision in (P.PLAIN_FP64, P.MIXED_FP32):
+        for nz, ny, nx in boxes:
+            assert rt.solve3d(W.with_(W.plain_small(), nx=nx, ny=ny, ns=2, precision=precision), nz) == 0
+            assert rt.L.fake_lowered() == 0
