@@ -1671,14 +1671,13 @@ extern "C" int epd_prop_solve(const epd_lb_params *p, const double *omega_dev, d
 namespace {
 
 constexpr size_t kNoallocBytes = EPD_PROP_SOLVE_NOALLOC_MAX_BYTES;
-constexpr int kNoallocDevices = 64;
 
 // One copy per device that loads this library, held until the process exits.
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
 // Device address of g_noalloc_scratch on each device (host code must not use
 // the symbol itself as an address).
-std::atomic<void *> g_noalloc_addr[kNoallocDevices];
+std::atomic<void *> g_noalloc_addr[kMaxDevices];
 
 } // namespace
 
@@ -1694,7 +1693,7 @@ extern "C" int epd_prop_solve_noalloc(const epd_lb_params *p, const double *omeg
     if (carve_solve(G, nullptr) > kNoallocBytes) return EPD_LB_ETOOLARGE;
 
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNoallocDevices) return EPD_LB_ECUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return EPD_LB_ECUDA;
     void *base = g_noalloc_addr[dev].load();
     if (!base) {
         if (cudaGetSymbolAddress(&base, g_noalloc_scratch) != cudaSuccess || !base) return EPD_LB_ECUDA;

@@ -2,6 +2,7 @@
 // launchers of the kernels that make up one hybrid LB/EPD time step.
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <string>
@@ -116,6 +117,25 @@ struct Group {
     float2 *tab8x = nullptr, *tab8y = nullptr;  // radix-8 pass tables (fft8.cuh layout); null with twx_full
     float2 *tab16x = nullptr, *tab16y = nullptr;  // radix-16 plan tables of 256-point axes (else null)
     int *err;                      // device error word (shared by the handle)
+};
+
+constexpr int kMaxDevices = 64;    // devices of a process
+
+// Kernel attributes (shared-memory limits, cluster sizes) belong to a function
+// on one device: set(), cudaSuccess if it worked, once on each device that
+// launches (setting them twice does no harm, so two threads may race).
+struct PerDevice {
+    std::atomic<bool> done[kMaxDevices] = {};
+    template <class F> cudaError_t once(F set)
+    {
+        int d = 0;
+        if (cudaError_t e = cudaGetDevice(&d)) return e;
+        if (d < 0 || d >= kMaxDevices) return set();
+        if (done[d]) return cudaSuccess;
+        const cudaError_t e = set();
+        if (e == cudaSuccess) done[d] = true;
+        return e;
+    }
 };
 
 constexpr int kMaxPart = 4096;     // partial sums per run and reduction

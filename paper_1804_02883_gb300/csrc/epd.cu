@@ -16,7 +16,6 @@
 // out of every derivative, and FP32 rounding then scales with the
 // fluctuations rather than with mu itself), omega (zero-mean noise), and
 // dPhi^D.  Pointwise combinations with the fields are done in FP64.
-#include <atomic>
 #include <cmath>
 #include <cstdlib>
 
@@ -275,11 +274,9 @@ static bool row8_at(int logx, const EpdK &k, dim3 grid_yz, cudaStream_t s)
     } else {
         if (logx != L) return row8_at<MODE, L + 1>(logx, k, grid_yz, s);
         using RT = RowTile<L>;
-        static std::atomic<bool> conf{false};  // attribute set (idempotent if two threads race)
-        if (!conf) {
-            conf = cudaFuncSetAttribute(epd_row8<L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RT::SMEM) == cudaSuccess;
-            if (!conf) return false;
-        }
+        static PerDevice conf;
+        if (conf.once([] { return cudaFuncSetAttribute(epd_row8<L, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RT::SMEM); }))
+            return false;
         const int blocks = (int)(k.g.n / RT::P);
         epd_row8<L, MODE><<<dim3(blocks, grid_yz.y, grid_yz.z), RT::T, RT::SMEM, s>>>(k);
         return true;
@@ -290,11 +287,9 @@ static bool col8_launch(const EpdK &k, dim3 grid_yz, cudaStream_t s)
 {
     using CT = ColTile<L, CW>;
     if (k.g.nx % CT::C) return false;
-    static std::atomic<bool> conf{false};  // attribute set (idempotent if two threads race)
-    if (!conf) {
-        conf = cudaFuncSetAttribute(epd_col8<L, MODE, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CT::SMEM) == cudaSuccess;
-        if (!conf) return false;
-    }
+    static PerDevice conf;
+    if (conf.once([] { return cudaFuncSetAttribute(epd_col8<L, MODE, CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CT::SMEM); }))
+        return false;
     epd_col8<L, MODE, CW><<<dim3(k.g.nx / CT::C, grid_yz.y, grid_yz.z), CT::T, CT::SMEM, s>>>(k);
     return true;
 }

@@ -22,7 +22,6 @@
 // and prop_stream.cu (FP32 on power-of-two grids); this file holds the pointwise
 // and contour passes and the solves' host side.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdlib>
 

@@ -51,7 +51,6 @@
 // of the second solve; only the rounding changes: FP32 relative to the
 // change, not to Phi.
 #include <algorithm>
-#include <atomic>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -844,8 +843,8 @@ static void set_cluster_cfg(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, 
 }
 
 // Clusters of a shape that fit at once at one CTA per SM (more than half of
-// an SM's shared memory per CTA), per shape and solve kind; 0: unknown or
-// none.  Filled by cluster_solve_supported, outside any stream capture.
+// an SM's shared memory per CTA), per device, shape and solve kind; 0: unknown
+// or none.  Filled by cluster_solve_supported, outside any stream capture.
 constexpr size_t kSoloSmem = 116 * 1024;
 // phased launches as programmatic dependents (EPD_LB_CHAIN_PDL=0 in the
 // environment turns it off, for timing one against the other)
@@ -853,7 +852,18 @@ static const bool g_chain_pdl = [] {
     const char *e = std::getenv("EPD_LB_CHAIN_PDL");
     return !(e && e[0] == '0');
 }();
-static int g_solo_clusters[16][16][2];
+static int g_solo_clusters[kMaxDevices][16][16][2];
+
+static int current_device()
+{
+    int d = 0;
+    return cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < kMaxDevices ? d : -1;
+}
+static int solo_clusters(const ClusterShape *s, bool diff)
+{
+    const int d = current_device();
+    return d < 0 ? 0 : g_solo_clusters[d][s->logx][s->logy][diff ? 1 : 0];
+}
 
 static int count_solo_clusters(const ClusterShape *s, bool diff)
 {
@@ -874,10 +884,13 @@ bool cluster_solve_supported(const Group &G)
     if (G.prec != EPD_LB_MIXED_FP32) return false;
     const ClusterShape *s = find_shape(G.g.logx, G.g.logy);
     if (!s) return false;
+    // the kernels' attributes are set here, on each device once
+    const int dev = current_device();
+    if (dev < 0) return false;
     static std::mutex mu;  // handles may be created on several threads
     std::lock_guard<std::mutex> lock(mu);
-    static int checked[16][16] = {};  // 0 unknown, 1 ok, 2 not launchable
-    int &st = checked[s->logx][s->logy];
+    static int checked[kMaxDevices][16][16] = {};  // 0 unknown, 1 ok, 2 not launchable
+    int &st = checked[dev][s->logx][s->logy];
     if (st == 0) {
         st = 2;
         auto ok = [&](bool diff, ChainForm f) {
@@ -896,8 +909,8 @@ bool cluster_solve_supported(const Group &G)
         for (ChainForm f : {CHAIN_SOLO, CHAIN_SHARE, CHAIN_PHASED}) all = all && ok(false, f) && ok(true, f);
         if (all) {
             st = 1;
-            g_solo_clusters[s->logx][s->logy][0] = count_solo_clusters(s, false);
-            g_solo_clusters[s->logx][s->logy][1] = count_solo_clusters(s, true);
+            g_solo_clusters[dev][s->logx][s->logy][0] = count_solo_clusters(s, false);
+            g_solo_clusters[dev][s->logx][s->logy][1] = count_solo_clusters(s, true);
         }
         cudaGetLastError();
     }
@@ -910,7 +923,7 @@ int cluster_chain_launches(const Group &G, bool diff)
 {
     const ClusterShape *sh = find_shape(G.g.logx, G.g.logy);
     if (!sh) return 0;
-    const int nch = 2 * G.g.nruns, solo = g_solo_clusters[sh->logx][sh->logy][diff ? 1 : 0];
+    const int nch = 2 * G.g.nruns, solo = solo_clusters(sh, diff);
     // solo > 0: the one-CTA-per-SM shared-memory size is set for this shape
     const bool can = solo > 0 && nch >= 2 && G.g.ns >= nch - 1;
     // EPD_LB_CHAIN_SCHEDULE=single|phased forces a schedule (the results are
@@ -962,7 +975,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     // launch j and runs N_s / (nch - 1) steps in each of the others).
     const int nch = 2 * G.g.nruns, launches = cluster_chain_launches(G, diff);
     const bool phased = launches > 1;
-    const int solo = g_solo_clusters[sh->logx][sh->logy][diff ? 1 : 0];
+    const int solo = solo_clusters(sh, diff);
     const ChainForm form = phased ? CHAIN_PHASED : (G.crowded || nch > solo ? CHAIN_SHARE : CHAIN_SOLO);
     k.nseg = phased ? nch - 1 : 0;
     k.skip = 0;
@@ -1011,15 +1024,12 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     c.err = G.err;
     const int npk = G.g.nx * G.g.ny / 2;
     const dim3 grid((npk + kThreads - 1) / kThreads, G.g.nruns), gq(kQBlocks, G.g.nruns);
-    static std::atomic<bool> conf{false};  // attribute set (idempotent if two threads race)
-    if (!conf) {
-        cudaError_t e1 = cudaFuncSetAttribute(prop_contour<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)ContourStage<true>::SMEM);
-        cudaError_t e2 = cudaFuncSetAttribute(prop_contour<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)ContourStage<false>::SMEM);
-        if (e1 || e2) return e1 ? e1 : e2;
-        conf = true;
-    }
+    static PerDevice conf;
+    if (cudaError_t e = conf.once([] {
+            const cudaError_t e1 = cudaFuncSetAttribute(prop_contour<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<true>::SMEM);
+            return e1 ? e1 : cudaFuncSetAttribute(prop_contour<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<false>::SMEM);
+        }))
+        return e;
     if (diff) {
         prop_qsum<true><<<gq, kThreads, 0, s>>>(c);
         prop_contour<true><<<grid, kThreads, ContourStage<true>::SMEM, s>>>(c);

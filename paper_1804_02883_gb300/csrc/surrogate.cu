@@ -34,7 +34,6 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <mutex>
 #include <cuda.h>
@@ -1066,11 +1065,8 @@ static void conv(Work &w, const void *in, const void *wt, const float *bias, voi
                  cudaStream_t s, const void *ycur = nullptr)
 {
     constexpr size_t smem = ConvTC<KP, NP, D>::SMEM;
-    static std::atomic<bool> conf{false};  // attribute set (idempotent if two threads race)
-    if (!conf) {
-        cudaFuncSetAttribute(conv3x3_tc<KP, NP, MODE, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        conf = true;
-    }
+    static PerDevice conf;  // (a failure shows at the launch)
+    conf.once([] { return cudaFuncSetAttribute(conv3x3_tc<KP, NP, MODE, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
     ConvArgs a;
     CUtensorMap map;
     a.use_tma = halo_map(&map, in, KP, w.nx, w.ny, w.nb, HaloTC<D>::HW, HaloTC<D>::HH) ? 1 : 0;
@@ -1172,8 +1168,8 @@ static void dw(Work &w, const void *x, const void *dzp, cudaStream_t s)
     const int cap = std::min(w.nblk_dw, 2 * 152), per = (ntiles + cap - 1) / cap;
     const int nblk = (ntiles + per - 1) / per;
     constexpr size_t smem = DwGeom<CI, CO, D>::SMEM;
-    // (on whichever device is current; a failure shows at the launch)
-    cudaFuncSetAttribute(conv3x3_dw<CI, CO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static PerDevice conf;  // (a failure shows at the launch)
+    conf.once([] { return cudaFuncSetAttribute(conv3x3_dw<CI, CO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
     conv3x3_dw<CI, CO, D><<<nblk, 288, smem, s>>>(reinterpret_cast<const __nv_bfloat16 *>(x), reinterpret_cast<const __nv_bfloat16 *>(dzp),
                                             w.dwpart, w.nx, w.ny, tiles_x, per, ntiles);
     w.nblk_dw = nblk;

@@ -31,3 +31,24 @@ def test_shared_memory_limits_never_fall(rt):
         for nz, ny, nx in boxes:
             assert rt.solve3d(W.with_(W.plain_small(), nx=nx, ny=ny, ns=2, precision=precision), nz) == 0
             assert rt.L.fake_lowered() == 0
+
+
+CLUSTER_GRIDS = [(64, 64), (64, 128), (128, 64), (128, 128), (128, 256), (256, 128), (256, 256), (128, 512), (512, 128), (256, 512), (512, 256)]
+
+
+def test_kernel_attributes_are_set_on_every_device(rt):
+    """Shared-memory limits and cluster sizes belong to a device: a process that
+    used one device solves, steps and runs the network on the next."""
+    for dev in (0, 1):
+        rt.L.fake_device(dev)
+        try:
+            for ny, nx in CLUSTER_GRIDS:
+                r = W.with_(W.plain_small(), nx=nx, ny=ny, ns=2, precision=P.MIXED_FP32, f0=0.0)
+                assert rt.solve(r) == 0
+                assert any("prop_chain" in l[0] for l in rt.launches())
+                rc, out = rt.init([r])
+                assert rc == 0 and any("epd_row8" in l[0] for l in out)
+            assert rt.sur_forward(W.with_(W.plain_small(), nx=64, ny=64), 2) == 0
+            assert sum("conv3x3_tc" in l[0] for l in rt.launches()) == 4
+        finally:
+            rt.L.fake_device(0)
