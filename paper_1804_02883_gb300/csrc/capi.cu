@@ -448,10 +448,7 @@ static void form_groups(const epd_lb_params *p, int nruns, std::vector<Group> &g
         groups[gi].run_ids.push_back(r);
         groups[gi].run_params.push_back(p[r]);
     }
-    for (auto &G : groups) {
-        G.crowded = groups.size() > 1;
-        fill_geom(G);
-    }
+    for (auto &G : groups) fill_geom(G);
 }
 
 } // namespace epdlb
@@ -475,6 +472,7 @@ struct epd_lb {
     double *obs = nullptr;
     double *part = nullptr;  // partials of the two-stage reductions
     int parity = 0;
+    bool crowded = false;  // the groups' chains want more SMs than there are
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     bool timing = false;
     bool timed_cluster = false;  // the timed solve ran as one cluster-resident launch
@@ -600,6 +598,15 @@ static cudaError_t enqueue_step(epd_lb *h, int parity, cudaStream_t s, int mode 
 {
     cudaError_t e;
     const size_t ng = h->groups.size();
+    struct Crowd {  // for the launches recorded here: elsewhere a group runs alone
+        epd_lb *h;
+        explicit Crowd(epd_lb *h_) : h(h_) { set(h->crowded); }
+        ~Crowd() { set(false); }
+        void set(bool v)
+        {
+            for (auto &G : h->groups) G.crowded = v;
+        }
+    } crowd(h);
     for (size_t gi = 1; gi < ng; ++gi) {
         if ((e = cudaEventRecord(h->fork_ev[gi - 1], s))) return e;
         if ((e = cudaStreamWaitEvent(h->side[gi - 1], h->fork_ev[gi - 1], 0))) return e;
@@ -726,6 +733,9 @@ extern "C" int epd_lb_init(const epd_lb_params *p, int32_t nruns, void *workspac
         h->join_ev.push_back(b);
     }
     h->parity = 0;
+    int sms = 0;
+    for (auto &G : h->groups) sms += group_sms(G);
+    h->crowded = h->groups.size() > 1 && sms > kSMs;
     if (int rc = build_graphs(h)) return bail(rc);
     *out = h;
     return EPD_LB_OK;
@@ -1253,7 +1263,9 @@ extern "C" int epd_lb_tiles(epd_lb *h, int32_t run, int32_t *out)
     out[2] = G->colw;
     out[3] = G->diff ? 1 : 0;
     out[4] = G->colw_prop;
-    out[5] = cluster ? cluster_chain_launches(*G, G->diff) : 0;
+    Group V = *G;
+    V.crowded = h->crowded && !h->cg_max;
+    out[5] = cluster ? cluster_chain_launches(V, V.diff) : 0;
     return EPD_LB_OK;
 }
 

@@ -82,7 +82,7 @@ struct Group {
     void *rho = nullptr;      // (rho_A, rho_B) = expm1(-N d omega ds / 2), [run][n] float2
     void *cdiff = nullptr;    // (1 + rho_d)(1 + rho_a) - 1 for (A,A), (B,B), (A,B), packed rows [run][3][ny/2][nx] float2
     void *facp = nullptr, *facd = nullptr;  // E_d E_a of a plain solve, E'_d E'_a of a differential one, for (A,A), (B,B), (A,B), packed rows as cdiff
-    bool crowded = false;     // the handle steps other groups beside this one
+    bool crowded = false;     // while a step of several groups is recorded: they want more SMs than there are
     bool stateless = false;   // one solve on a caller's stream, not a handle's captured step
     bool diff = false;        // the step uses the reference + differential solve pair
     bool phi_stale = false;   // omega was replaced since phi was last computed
@@ -119,6 +119,7 @@ struct Group {
     int *err;                      // device error word (shared by the handle)
 };
 
+constexpr int kSMs = 152;          // of a GB300
 constexpr int kMaxDevices = 64;    // devices of a process
 
 // Kernel attributes (shared-memory limits, cluster sizes) belong to a function
@@ -229,6 +230,9 @@ bool cluster_shape_exists(int logx, int logy);
 // differential one): 1, or 2 nruns when the chains are one more than the
 // clusters that fit at one CTA per SM (the phased schedule); 0 without a shape.
 int cluster_chain_launches(const Group &G, bool diff);
+// SMs that a group's step takes beside others: the chain CTAs of a launch at
+// one per SM, or the tiles of a streaming pass up to half the chip.
+int group_sms(const Group &G);
 // MIXED grids solved by the streaming passes on power-of-two tiles with the full history
 bool stream8_eligible(int prec, int logx, int logy);
 size_t cluster_state_floats2(int nx, int ny, int ns);  // per run, both chains

@@ -810,10 +810,12 @@ static ClusterShape shape_of()
 // threads (one or two butterflies per thread and pass).  With the SM's whole
 // register file (255 registers) a chain runs fastest; at 128 registers a
 // second CTA shares the SM and fills the exchange waits of the first: slower
-// for one chain, more chains per second.  One handle with one group whose
-// chains have an SM per CTA takes the first form (4 x 256 x 512, alone: 1.40
-// ms a step, 1.47 with the second), a handle with several groups, or more
-// chains than fit so, the second (32-run ensemble, 2 steps: 13.6 -> 12.2 ms).
+// for one chain, more chains per second.  Chains that have an SM per CTA take
+// the first form (4 x 256 x 512, alone: 1.40 ms a step, 1.47 with the second),
+// more chains than fit so, or groups side by side that want more SMs than there
+// are (group_sms), the second (32-run ensemble, 2 steps: 13.6 -> 12.2 ms; 1 of
+// 128 x 128 beside 1 of 128 x 256, 12 SMs, takes 0.85 ms a step so, 0.77 in the
+// first form; 4 of 256 x 512 in turns beside 1 of 128 x 128 1.72 and 1.39).
 static const ClusterShape *find_shape(int logx, int logy)
 {
     static const ClusterShape shapes[] = {
@@ -933,6 +935,18 @@ int cluster_chain_launches(const Group &G, bool diff)
     if (env && !std::strcmp(env, "phased")) return can ? nch : 1;
     if (G.crowded) return 1;
     return (can && nch == solo + 1) ? nch : 1;
+}
+
+int group_sms(const Group &G)
+{
+    const ClusterShape *sh = G.hc ? find_shape(G.g.logx, G.g.logy) : nullptr;
+    // A streaming group's short launches share the SMs they get: half the chip.
+    // Beside a 1024 x 1024 one, ms a step with the chains' SMs to themselves and
+    // shared: 8 of 128 x 128 (32 SMs) 1.20 and 1.43, 4 of 256 x 256 (64) 1.34 and
+    // 1.53, 2 of 256 x 512 (64) 3.03 and 3.17, 4 of 256 x 512 (112) 2.08 and 1.84.
+    if (!sh) return std::min(kSMs / 2, G.g.nruns * G.g.ny);
+    const int nch = 2 * G.g.nruns;
+    return std::min(kSMs, sh->c * (cluster_chain_launches(G, G.diff) > 1 ? nch - 1 : nch));
 }
 
 size_t cluster_state_floats2(int nx, int ny, int ns) { return (size_t)2 * (ns + 1) * (ny / 2) * nx; }

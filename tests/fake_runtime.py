@@ -43,6 +43,17 @@ class FakeRuntime:
             self.L.epd_lb_destroy(h)
         return rc, out
 
+    def step_exact(self, runs, iterations):
+        """(return code of one exact step of that many iterations, its launches)."""
+        h = ctypes.c_void_p()
+        rc = self.L.epd_lb_init(binding._params_array(runs), len(runs), None, 0, None, ctypes.byref(h))
+        rc = rc or self.L.epd_lb_set_inversion(h, iterations, ctypes.c_double(0.0))
+        self.L.fake_reset()
+        rc = rc or self.L.epd_lb_step(h, ctypes.c_int64(1))
+        out = self.launches()
+        self.L.epd_lb_destroy(h)
+        return rc, out
+
     def solve(self, run):
         self.L.fake_reset()
         n = ctypes.c_size_t()

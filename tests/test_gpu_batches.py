@@ -24,3 +24,21 @@ def test_wide_batches_of_long_columns_step(ny, nx, runs):
     assert rel_err(hb.densities(runs - 1)[0], hs.densities(0)[0]) < 1e-5
     hb.close()
     hs.close()
+
+
+def test_forms_of_the_chain_kernel_give_the_same_bits():
+    # a run stepped alone (whole register file, cached factors), in a batch
+    # that takes turns or shares SMs, and beside groups that fill the chip
+    r = W.with_(W.plain_small(), nx=512, ny=256, ns=16, precision=P.MIXED_FP32, f0=1e-6, seed=9)
+    others = [W.with_(r, seed=20 + s) for s in range(7)]
+    crowd = [W.with_(r, ns=n, seed=n) for n in (8, 10, 12, 14)]
+    ref = None
+    for runs in ([r], [r] + others[:3], [r] + others, [r] + crowd):
+        h = P.EpdLb(runs)
+        h.step(2)
+        h.sync()
+        got = (*h.densities(0), h.velocity(0), h.get_state(0)[0])
+        h.close()
+        ref = ref or got
+        for a, b in zip(got, ref):
+            assert np.array_equal(a, b)

@@ -52,3 +52,33 @@ def test_kernel_attributes_are_set_on_every_device(rt):
             assert sum("conv3x3_tc" in l[0] for l in rt.launches()) == 4
         finally:
             rt.L.fake_device(0)
+
+
+def _chains(out):
+    """Template arguments (.., CTAs the registers are sized for, differential, cached) of the chain launches."""
+    return [l[1] for l in out if "prop_chain" in l[0]]
+
+
+def test_chains_share_an_sm_only_where_the_groups_fill_the_chip(rt):
+    """Groups stepped side by side take the half-register form once their
+    clusters are more than the SMs; two small ones, and the benchmark batch
+    beside a small run, keep the whole register file, the batch its turns."""
+    def run(ny, nx, n, ns=16):
+        r = W.with_(W.plain_small(), nx=nx, ny=ny, ns=ns, precision=P.MIXED_FP32, f0=0.0)
+        return [W.with_(r, seed=s) for s in range(n)]
+
+    rc, out = rt.init(run(128, 128, 1) + run(128, 256, 1))
+    assert rc == 0 and _chains(out) and all(a[-1] == 1 for a in _chains(out))
+    rc, out = rt.init(run(256, 512, 4) + run(128, 128, 1))
+    wide = [a for a in _chains(out) if a[:2] == (9, 8)]
+    # Phi(0), then two solves a step in two graphs, 8 launches each
+    assert rc == 0 and len(wide) == 5 * 8 and all(a[4] == 1 for a in wide)
+    rc, out = rt.init(W.ensemble_32())
+    step = _chains(out)[len({(r.ny, r.nx, r.ns) for r in W.ensemble_32()}):]  # after the solves of Phi(0)
+    assert rc == 0 and step and all(a[-3] == 2 and a[-1] == 0 for a in step if a[2] >= 4)
+
+
+def test_groups_of_an_exact_step_run_alone(rt):
+    """The exact step takes its groups one after the other."""
+    rc, out = rt.step_exact(W.ensemble_32(), 2)
+    assert rc == 0 and _chains(out) and all(a[-1] == 1 for a in _chains(out) if a[2] < 16)
