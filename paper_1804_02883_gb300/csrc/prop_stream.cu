@@ -70,7 +70,7 @@ template <int LOGY> cudaError_t col_by(const PropK<float> &k, int colw, cudaStre
 template <int LOGX> cudaError_t row_by(const PropK<float> &k, int m, bool diff, int *blocks, const RowWeights &w, cudaStream_t s)
 {
     constexpr int big = LOGX == 11 ? 0 : (LOGX == 10 ? 1 : (LOGX == 9 ? 2 : 3)), small = LOGX <= 7 ? 2 : (LOGX == 8 ? 1 : 0);
-    if (big == small || (long long)(k.g.ny >> big) * k.g.nruns >= 2 * 152) {
+    if (big == small || (long long)(k.g.ny >> big) * row_tile_runs(k.g, m) >= 2 * 152) {
         *blocks = k.g.ny >> big;
         return row_at<LOGX, big>(k, m, diff, w, s);
     }

@@ -42,3 +42,21 @@ def test_forms_of_the_chain_kernel_give_the_same_bits():
         ref = ref or got
         for a, b in zip(got, ref):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,ny,nx,runs", [(P.PLAIN_FP64, 64, 64, 33), (P.MIXED_FP32, 150, 150, 17), (P.PLAIN_FP64, 90, 96, 24),
+                                                  (P.MIXED_FP32, 64, 1024, 11), (P.MIXED_FP32, 512, 512, 9), (P.MIXED_FP32, 256, 2048, 3)])
+def test_a_batch_equals_its_runs_stepped_alone(precision, ny, nx, runs):
+    # batches past the sizes where the row passes take more rows per tile
+    rs = [W.with_(W.plain_small(), nx=nx, ny=ny, ns=6, precision=precision, f0=0.0, seed=s + 1) for s in range(runs)]
+    hb = P.EpdLb(rs)
+    hb.step(2)
+    hb.sync()
+    for k in (0, runs - 1):
+        hs = P.EpdLb([rs[k]])
+        hs.step(2)
+        hs.sync()
+        for a, b in zip((*hb.densities(k), hb.velocity(k), hb.get_state(k)[0]), (*hs.densities(0), hs.velocity(0), hs.get_state(0)[0])):
+            assert np.array_equal(a, b)
+        hs.close()
+    hb.close()

@@ -82,3 +82,18 @@ def test_groups_of_an_exact_step_run_alone(rt):
     """The exact step takes its groups one after the other."""
     rc, out = rt.step_exact(W.ensemble_32(), 2)
     assert rc == 0 and _chains(out) and all(a[-1] == 1 for a in _chains(out) if a[2] < 16)
+
+
+@pytest.mark.parametrize("precision,ny,nx", [(P.PLAIN_FP64, 64, 64), (P.MIXED_FP32, 150, 150), (P.MIXED_FP32, 64, 1024), (P.MIXED_FP32, 1024, 512)])
+def test_q_is_summed_over_the_same_tiles_in_every_batch(rt, precision, ny, nx):
+    """The last row pass of a solve leaves the Q partials: its tile, and so the
+    order of the sum, is that of one run whatever the batch."""
+    tiles = set()
+    for n in (1, 2, 10, 16, 32, 64):
+        r = W.with_(W.plain_small(), nx=nx, ny=ny, ns=4, precision=precision, f0=0.0)
+        rc, out = rt.init([W.with_(r, seed=s) for s in range(n)])
+        assert rc == 0
+        for a, b in zip(out, out[1:]):
+            if "prop_finalize" in b[0] or "prop_contour_stream" in b[0]:
+                tiles.add((a[1], a[2][0], a[3]))
+    assert len({t[1:] for t in tiles}) == 1, tiles
