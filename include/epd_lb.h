@@ -457,8 +457,11 @@ int epd_lb3d_step(const epd_lb_params *p, int32_t nz, const double *pop_in_dev, 
  * omega_dev (3*ny*nx doubles) -> phi_dev (3*ny*nx doubles), q_dev[2] =
  * (Q_P, Q_S).  workspace_dev of epd_prop_solve_workspace_bytes bytes holds the
  * propagator history and the transform buffers; cuda_stream may be NULL (the
- * legacy default stream).  Asynchronous.  In EPD_LB_MIXED_FP32 on the grids of
- * the cluster-resident solve the queried size holds that solve's states; a
+ * legacy default stream).  Asynchronous, so the return value says only that the
+ * work was enqueued: q_dev holds positive, finite Q_P and Q_S after a good
+ * solve; a bounded device wait that gave up (the exchange of the cluster-resident
+ * solve, see EPD_LB_ETIMEOUT) makes q_dev and phi_dev NaN.  In EPD_LB_MIXED_FP32
+ * on the grids of the cluster-resident solve the queried size holds that solve's states; a
  * workspace of the streaming passes' size (half the history, about
  * nx*ny*(16 + (ns/2 + 3)*8) + 40 KiB bytes) is taken as well, with those passes.
  */

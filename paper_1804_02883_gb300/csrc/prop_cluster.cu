@@ -520,6 +520,7 @@ struct ContourK {
     const double *phi_t, *q_t;  // first solve's densities (differential solve)
     double *phi, *q;
     int *err;
+    bool stateless;  // nobody reads err: a give-up makes Q and the densities NaN
 };
 
 // Compensated (Kahan) FP32 sum: value() = sum minus the carried rounding
@@ -662,7 +663,9 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
     const double tp = sum_partials(pr, k.nq, 1, &bc), ts = sum_partials(pr + kMaxPart / 2, k.ns_part, 1, &bc);
     if (tid == 0) {
         const double sq = tp / (double)n, ss = ts / (double)n;
-        const double qp = DIFF ? k.q_t[2 * run] + sq : sq, qs = DIFF ? k.q_t[2 * run + 1] + ss : ss;
+        const bool lost = !DIFF && k.stateless && (*k.err & 4);
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        const double qp = DIFF ? k.q_t[2 * run] + sq : (lost ? nan : sq), qs = DIFF ? k.q_t[2 * run + 1] + ss : (lost ? nan : ss);
         fac[0] = k.g.phi_p * k.g.ds / qp;
         fac[1] = (1.0 - k.g.phi_p) / qs;
         fac[2] = sq / qp;
@@ -1036,6 +1039,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     c.phi = phi;
     c.q = q;
     c.err = G.err;
+    c.stateless = G.stateless;
     const int npk = G.g.nx * G.g.ny / 2;
     const dim3 grid((npk + kThreads - 1) / kThreads, G.g.nruns), gq(kQBlocks, G.g.nruns);
     static PerDevice conf;
