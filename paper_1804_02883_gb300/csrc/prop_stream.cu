@@ -65,12 +65,13 @@ template <int LOGY> cudaError_t col_by(const PropK<float> &k, int colw, cudaStre
     default: return col_at<LOGY, 3>(k, s);
     }
 }
-// rows per tile: 128 threads (64 on the shortest axes); 32 or 64 threads while
-// the launch has fewer than two tiles per SM
+// rows per tile: 64 to 256 threads; 16 to 64 while the launch has fewer than two
+// tiles per SM, but for the last pass, whose tiles set the order of the Q_P sum
+// and follow the grid alone
 template <int LOGX> cudaError_t row_by(const PropK<float> &k, int m, bool diff, int *blocks, const RowWeights &w, cudaStream_t s)
 {
     constexpr int big = LOGX == 11 ? 0 : (LOGX == 10 ? 1 : (LOGX == 9 ? 2 : 3)), small = LOGX <= 7 ? 2 : (LOGX == 8 ? 1 : 0);
-    if (big == small || (long long)(k.g.ny >> big) * row_tile_runs(k.g, m) >= 2 * 152) {
+    if (big == small || m == k.g.ns || (long long)(k.g.ny >> big) * k.g.nruns >= 2 * 152) {
         *blocks = k.g.ny >> big;
         return row_at<LOGX, big>(k, m, diff, w, s);
     }
