@@ -1307,7 +1307,7 @@ extern "C" void epd_lb_destroy(epd_lb *h)
 struct AxisTables {
     int n;
     void *tw, *kf;                // may be null
-    float2 *tab[2];               // pass tables of the radix-8 and radix-16 plans, or null
+    float2 *tab[2];               // pass tables of the radix-8 and radix-16 plans (kReadAll), or null
 };
 struct CallTables {
     AxisTables ax[3];
@@ -1341,7 +1341,7 @@ template <typename T> __global__ void call_tables(CallTables c)
     }
     const int v = blockIdx.z - 2;
     if (a.tab[v]) {
-        const int logn = ilog2(n), mr = 3 + v, np = npasses(logn, mr);
+        const int logn = ilog2(n), mr = (3 + v) | kReadAll, np = npasses(logn, mr);
         for (int e = i; e < tabs_total(logn, mr); e += gridDim.x * blockDim.x) {
             for (int I = 0; I < 2 * (np - 1); ++I) {  // the pass the entry belongs to
                 const bool inv = I >= np - 1;
@@ -1349,8 +1349,8 @@ template <typename T> __global__ void call_tables(CallTables c)
                 const int slog = inv ? inv_slog(logn, p, mr) : fwd_slog(logn, p, mr), rlog = inv ? inv_rlog(logn, p, mr) : fwd_rlog(logn, p, mr);
                 const int off = inv ? inv_off(logn, p, mr) : fwd_off(logn, p, mr), M = n >> (slog + rlog);
                 const int r = e - off;
-                if (r < 0 || r >= tab_rows(rlog) * M) continue;
-                const int row = r / M, k = rlog >= 3 ? (1 << row) : row + 1;
+                if (r < 0 || r >= tab_rows(rlog, mr) * M) continue;
+                const int row = r / M, k = row + 1;
                 const double2 w = twiddle(((r % M) << slog) * k);
                 a.tab[v][e] = make_float2((float)w.x, (float)w.y);
             }
@@ -1432,10 +1432,10 @@ static size_t carve_solve_cluster(Group &G, char *base)
     G.twx = G.twy = nullptr;
     G.kx = take((size_t)G.g.nx * sizeof(float));
     G.ky = take((size_t)G.g.ny * sizeof(float));
-    G.tab8x = (float2 *)take((size_t)tabs_total(G.g.logx) * sizeof(float2));
-    G.tab8y = (float2 *)take((size_t)tabs_total(G.g.logy) * sizeof(float2));
-    G.tab16x = best_mr(G.g.logx) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logx, 4) * sizeof(float2)) : nullptr;
-    G.tab16y = best_mr(G.g.logy) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logy, 4) * sizeof(float2)) : nullptr;
+    G.tab8x = (float2 *)take((size_t)tabs_total(G.g.logx, 3 | kReadAll) * sizeof(float2));
+    G.tab8y = (float2 *)take((size_t)tabs_total(G.g.logy, 3 | kReadAll) * sizeof(float2));
+    G.tab16x = best_mr(G.g.logx) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logx, 4 | kReadAll) * sizeof(float2)) : nullptr;
+    G.tab16y = best_mr(G.g.logy) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logy, 4 | kReadAll) * sizeof(float2)) : nullptr;
     return align_up(off);
 }
 

@@ -16,11 +16,13 @@
 namespace epdlb {
 
 // Radix plan: passes of radix 2^mr (8 by default, 16 where a kernel picks
-// mr = 4), the last forward pass takes the remainder.
-__host__ __device__ constexpr int npasses(int logn, int mr = 3) { return (logn + mr - 1) / mr; }
+// mr = 4), the last forward pass takes the remainder.  mr | kReadAll: every
+// twiddle is read from the tables, none formed as a product.
+constexpr int kReadAll = 8;
+__host__ __device__ constexpr int npasses(int logn, int mr = 3) { return (logn + (mr & 7) - 1) / (mr & 7); }
 __host__ __device__ constexpr int fwd_rlog(int logn, int i, int mr = 3)
 {
-    return i < npasses(logn, mr) - 1 ? mr : logn - mr * (npasses(logn, mr) - 1);
+    return i < npasses(logn, mr) - 1 ? (mr & 7) : logn - (mr & 7) * (npasses(logn, mr) - 1);
 }
 __host__ __device__ constexpr int fwd_slog(int logn, int i, int mr = 3) { return i == 0 ? 0 : fwd_slog(logn, i - 1, mr) + fwd_rlog(logn, i - 1, mr); }
 __host__ __device__ constexpr int inv_rlog(int logn, int i, int mr = 3) { return fwd_rlog(logn, npasses(logn, mr) - 1 - i, mr); }
@@ -28,17 +30,18 @@ __host__ __device__ constexpr int inv_slog(int logn, int i, int mr = 3) { return
 // Twiddle tables: one per pass that needs twiddles (forward passes
 // 0..np-2, inverse passes 0..np-2), rows x M entries, M = N / (S R): rows
 // k = 1, 2, 4 for radix 8 and k = 1, 2, 4, 8 for radix 16 (the others are
-// products), k = 1..R-1 otherwise.
-__host__ __device__ constexpr int tab_rows(int rlog) { return rlog >= 3 ? rlog : (1 << rlog) - 1; }
-__host__ __device__ constexpr int tab_len(int logn, int slog, int rlog) { return tab_rows(rlog) * ((1 << logn) >> (slog + rlog)); }
+// products), k = 1..R-1 otherwise and with kReadAll.
+__host__ __device__ constexpr bool tab_powers(int rlog, int mr) { return rlog >= 3 && !(mr & kReadAll); }
+__host__ __device__ constexpr int tab_rows(int rlog, int mr) { return tab_powers(rlog, mr) ? rlog : (1 << rlog) - 1; }
+__host__ __device__ constexpr int tab_len(int logn, int slog, int rlog, int mr) { return tab_rows(rlog, mr) * ((1 << logn) >> (slog + rlog)); }
 __host__ __device__ constexpr int fwd_off(int logn, int i, int mr = 3)
 {
-    return i == 0 ? 0 : fwd_off(logn, i - 1, mr) + tab_len(logn, fwd_slog(logn, i - 1, mr), fwd_rlog(logn, i - 1, mr));
+    return i == 0 ? 0 : fwd_off(logn, i - 1, mr) + tab_len(logn, fwd_slog(logn, i - 1, mr), fwd_rlog(logn, i - 1, mr), mr);
 }
 __host__ __device__ constexpr int inv_off(int logn, int i, int mr = 3)
 {
     return i == 0 ? fwd_off(logn, npasses(logn, mr) - 1, mr)
-                  : inv_off(logn, i - 1, mr) + tab_len(logn, inv_slog(logn, i - 1, mr), inv_rlog(logn, i - 1, mr));
+                  : inv_off(logn, i - 1, mr) + tab_len(logn, inv_slog(logn, i - 1, mr), inv_rlog(logn, i - 1, mr), mr);
 }
 __host__ __device__ constexpr int tabs_total(int logn, int mr = 3) { return inv_off(logn, npasses(logn, mr) - 1, mr); }
 // radix 16 where it takes fewer passes than radix 8 (128, 256, 1024, 2048
@@ -158,11 +161,11 @@ template <int LOGN, int W> struct ColLayout {
 // Twiddles w[k] = w1^k, k = 1..R-1, of one butterfly from a pass table laid
 // out [row][p] (row length M): radix 8 reads w1, w2, w4 and radix 16 also w8,
 // and forms the rest by products (at most three roundings more than a table
-// entry).
-template <int R>
+// entry); READ: every one is read.
+template <int R, bool READ>
 __device__ __forceinline__ void twiddles(float2 (&w)[R], const float2 *tab, int M, int p)
 {
-    if constexpr (R == 8) {
+    if constexpr (R == 8 && !READ) {
         w[1] = tab[p];
         w[2] = tab[M + p];
         w[4] = tab[2 * M + p];
@@ -170,7 +173,7 @@ __device__ __forceinline__ void twiddles(float2 (&w)[R], const float2 *tab, int 
         w[5] = fmul(w[1], w[4]);
         w[6] = fmul(w[2], w[4]);
         w[7] = fmul(w[3], w[4]);
-    } else if constexpr (R == 16) {
+    } else if constexpr (R == 16 && !READ) {
         w[1] = tab[p];
         w[2] = tab[M + p];
         w[4] = tab[2 * M + p];
@@ -210,7 +213,7 @@ template <bool WS> __device__ __forceinline__ void pass_sync()
 
 // One in-place Stockham pass (radix 2^RLOG, stride 2^SLOG): load, wait, write.
 // tab: this pass's twiddles [k-1][p] (unused in a forward last pass).
-template <int LOGN, int SLOG, int RLOG, bool INV, int NB, int T, class L, bool WS = false>
+template <int LOGN, int SLOG, int RLOG, bool INV, int NB, int T, class L, bool WS = false, bool READ = false>
 __device__ __forceinline__ void pass(float2 *buf, const float2 *tab, int tid)
 {
     constexpr int N = 1 << LOGN, R = 1 << RLOG, S = 1 << SLOG, PER = N / R, M = N / (S * R);
@@ -229,7 +232,7 @@ __device__ __forceinline__ void pass(float2 *buf, const float2 *tab, int tid)
         const int q = tt[j] & (S - 1), p = tt[j] >> SLOG;
         if (M > 1) {
             float2 w[R];
-            twiddles<R>(w, tab, M, p);
+            twiddles<R, READ>(w, tab, M, p);
 #pragma unroll
             for (int k = 1; k < R; ++k) x[j][k] = INV ? fmulc(x[j][k], w[k]) : fmul(x[j][k], w[k]);
         }
@@ -242,7 +245,7 @@ __device__ __forceinline__ void pass(float2 *buf, const float2 *tab, int tid)
 // Forward last pass, spectral operator, inverse first pass (same points per
 // thread).  op(b, bin, v) returns the operator applied to bin `bin` (natural
 // order) of sequence b.
-template <int LOGN, int RLOG, int NB, int T, class L, class Op, bool WS = false>
+template <int LOGN, int RLOG, int NB, int T, class L, class Op, bool WS = false, bool READ = false>
 __device__ __forceinline__ void middle(float2 *buf, const float2 *tab_inv0, const Op &op, int tid)
 {
     constexpr int N = 1 << LOGN, R = 1 << RLOG, PER = N / R;
@@ -262,7 +265,7 @@ __device__ __forceinline__ void middle(float2 *buf, const float2 *tab_inv0, cons
         for (int k = 0; k < R; ++k) x[j][k] = op(bb[j], tt[j] + k * PER, x[j][k]);
         Dft<RLOG, true>::run(x[j]);
         float2 w[R];
-        twiddles<R>(w, tab_inv0, PER, tt[j]);
+        twiddles<R, READ>(w, tab_inv0, PER, tt[j]);
 #pragma unroll
         for (int k = 1; k < R; ++k) x[j][k] = fmulc(x[j][k], w[k]);
 #pragma unroll
@@ -289,7 +292,7 @@ __device__ __forceinline__ void inverse_first(float2 *buf, const float2 *tab_inv
     for (int j = 0; j < NB; ++j) {
         Dft<RLOG, true>::run(x[j]);
         float2 w[R];
-        twiddles<R>(w, tab_inv0, PER, tt[j]);
+        twiddles<R, false>(w, tab_inv0, PER, tt[j]);
 #pragma unroll
         for (int k = 1; k < R; ++k) x[j][k] = fmulc(x[j][k], w[k]);
 #pragma unroll
@@ -304,7 +307,7 @@ struct FwdPasses {
     {
         if constexpr (I < npasses(LOGN, MR) - 1) {
             constexpr int RLOG = fwd_rlog(LOGN, I, MR);
-            pass<LOGN, fwd_slog(LOGN, I, MR), RLOG, false, P / (1 << RLOG) / T, T, L, WS>(buf, tabs + fwd_off(LOGN, I, MR), tid);
+            pass<LOGN, fwd_slog(LOGN, I, MR), RLOG, false, P / (1 << RLOG) / T, T, L, WS, (MR & kReadAll) != 0>(buf, tabs + fwd_off(LOGN, I, MR), tid);
             FwdPasses<LOGN, I + 1, T, L, P, MR, WS>::run(buf, tabs, tid);
         }
     }
@@ -315,7 +318,7 @@ struct InvPasses {
     {
         if constexpr (I < npasses(LOGN, MR) - 1) {
             constexpr int RLOG = inv_rlog(LOGN, I, MR);
-            pass<LOGN, inv_slog(LOGN, I, MR), RLOG, true, P / (1 << RLOG) / T, T, L, WS>(buf, tabs + inv_off(LOGN, I, MR), tid);
+            pass<LOGN, inv_slog(LOGN, I, MR), RLOG, true, P / (1 << RLOG) / T, T, L, WS, (MR & kReadAll) != 0>(buf, tabs + inv_off(LOGN, I, MR), tid);
             InvPasses<LOGN, I + 1, T, L, P, MR, WS>::run(buf, tabs, tid);
         }
     }
@@ -328,7 +331,7 @@ __device__ __forceinline__ void transform_pair(float2 *buf, const float2 *tabs, 
 {
     FwdPasses<LOGN, 0, T, L, P, MR, WS>::run(buf, tabs, tid);
     constexpr int RM = fwd_rlog(LOGN, npasses(LOGN, MR) - 1, MR);
-    middle<LOGN, RM, P / (1 << RM) / T, T, L, Op, WS>(buf, tabs + inv_off(LOGN, 0, MR), op, tid);
+    middle<LOGN, RM, P / (1 << RM) / T, T, L, Op, WS, (MR & kReadAll) != 0>(buf, tabs + inv_off(LOGN, 0, MR), op, tid);
     InvPasses<LOGN, 1, T, L, P, MR, WS>::run(buf, tabs, tid);
 }
 
@@ -394,10 +397,10 @@ inline void build_tables_host(int logn, const float *tw, float *out, int mr = 3)
         const int slog = invp ? inv_slog(logn, pi, mr) : fwd_slog(logn, pi, mr);
         const int rlog = invp ? inv_rlog(logn, pi, mr) : fwd_rlog(logn, pi, mr);
         const int off = invp ? inv_off(logn, pi, mr) : fwd_off(logn, pi, mr);
-        const int M = (1 << logn) >> (slog + rlog), len = tab_rows(rlog) * M;
+        const int M = (1 << logn) >> (slog + rlog), len = tab_rows(rlog, mr) * M;
         for (int e = 0; e < len; ++e) {
             const int row = e / M, p = e % M;
-            const int k = rlog >= 3 ? (1 << row) : row + 1;
+            const int k = tab_powers(rlog, mr) ? (1 << row) : row + 1;
             const int j = (p << slog) * k;
             out[2 * (off + e)] = tw[2 * j];
             out[2 * (off + e) + 1] = tw[2 * j + 1];

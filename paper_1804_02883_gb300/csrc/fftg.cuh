@@ -228,7 +228,7 @@ template <typename T, bool INV> struct DftN<T, 15, INV> : DftPf<T, 3, 5, INV> {}
 // consecutive points (the global order) where the legs are far enough apart.
 // No access then meets the same bank more than twice.
 struct LineTile {
-    static constexpr bool fixed = false;
+    static constexpr bool fixed = false, products = false;
     int n, logb, bp, rl, pad;
     bool row;
     __host__ __device__ LineTile(bool row_, int n_, int logb_, LinePlan pl)
@@ -242,7 +242,7 @@ struct LineTile {
 // The same with everything known at compile time, for the power-of-two axes
 // of the streaming solves: offsets become immediates, indices shifts, loops
 // straight code (a third fewer instructions per point than above).
-// NT: threads of the block.
+// NT: threads of the block; READ: every twiddle is read (LineTw).
 constexpr int ct_radix(int logn, int i)
 {
     // 64 = 8.8, 128 = 16.8, 256 = 16.16, 512 = 8.8.8, 1024 = 16.8.8, 2048 = 16.8.16
@@ -253,8 +253,8 @@ template <int LOGN> struct LinePlanCT {
     static constexpr int nf = ct_radix(LOGN, -1);
     static __host__ __device__ constexpr int r(int i) { return ct_radix(LOGN, i); }
 };
-template <int LOGN, int LOGB, bool ROW, int NT> struct LineTileCT {
-    static constexpr bool fixed = true;
+template <int LOGN, int LOGB, bool ROW, int NT, bool READ> struct LineTileCT {
+    static constexpr bool fixed = true, products = !READ;
     static constexpr int n = 1 << LOGN, logb = LOGB, bp = ROW ? (1 << LOGB) | 1 : 1 << LOGB;
     static constexpr int rl = LinePlanCT<LOGN>::r(LinePlanCT<LOGN>::nf - 1), pad = 1, nt = NT;
     static constexpr bool row = ROW;
@@ -268,7 +268,7 @@ template <class Tile> struct TileDiv {
     __device__ __forceinline__ int div(int a) const { return f.div(a); }
     __device__ __forceinline__ int d() const { return f.d; }
 };
-template <int LOGN, int LOGB, bool ROW, int NT> struct TileDiv<LineTileCT<LOGN, LOGB, ROW, NT>> {
+template <int LOGN, int LOGB, bool ROW, int NT, bool READ> struct TileDiv<LineTileCT<LOGN, LOGB, ROW, NT, READ>> {
     int v;
     __device__ __forceinline__ explicit TileDiv(int d) : v(d) {}
     __device__ __forceinline__ int div(int a) const { return (int)((unsigned)a / (unsigned)v); }  // a shift once inlined
@@ -364,7 +364,7 @@ __device__ __forceinline__ void line_pass(V2<T> *buf, Tile tl, int M, int S, con
         const int blk = dm.div(t), j = t - blk * M;
         V2<T> *p = buf + (j + (tl.pad ? dl.div(j) : 0)) * tl.bp + blk * R * leg + b;
         V2<T> x[R];
-        const LineTw<R, Tile::fixed && sizeof(T) == 4, V2<T>> w(tw, j * S);
+        const LineTw<R, Tile::products && sizeof(T) == 4, V2<T>> w(tw, j * S);
 #pragma unroll
         for (int u = 0; u < R; ++u) x[u] = p[u * leg];
         if (INV) {
@@ -491,7 +491,7 @@ __device__ __forceinline__ void line_open(V2<T> *buf, Tile tl, const V2<T> *__re
         line_split(tl, !tl.row, dq, bf, b, t);
         V2<T> x[R0];
         src(b, t, q, x);
-        const LineTw<R0, Tile::fixed && sizeof(T) == 4, V2<T>> w(tw, t);
+        const LineTw<R0, Tile::products && sizeof(T) == 4, V2<T>> w(tw, t);
         DftN<T, R0, false>::run(x);
         V2<T> *p = buf + (t + (tl.pad ? dl.div(t) : 0)) * tl.bp + b;
         p[0] = x[0];
@@ -511,7 +511,7 @@ __device__ __forceinline__ void line_close(const V2<T> *buf, Tile tl, const V2<T
         line_split(tl, !tl.row, dq, bf, b, t);
         const V2<T> *p = buf + (t + (tl.pad ? dl.div(t) : 0)) * tl.bp + b;
         V2<T> x[R0];
-        const LineTw<R0, Tile::fixed && sizeof(T) == 4, V2<T>> w(tw, t);
+        const LineTw<R0, Tile::products && sizeof(T) == 4, V2<T>> w(tw, t);
         x[0] = p[0];
 #pragma unroll
         for (int u = 1; u < R0; ++u) x[u] = cmul_conj(p[u * leg], w.get(u));

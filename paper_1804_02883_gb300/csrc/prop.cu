@@ -316,7 +316,7 @@ template <typename T> static PropK<T> prop_args(const Group &G)
     k.twy = reinterpret_cast<const V2<T> *>(G.twy);
     k.kx = reinterpret_cast<const T *>(G.kx);
     k.ky = reinterpret_cast<const T *>(G.ky);
-    k.dependent = G.stateless;
+    k.stateless = G.stateless;
     return k;
 }
 
@@ -502,7 +502,7 @@ static cudaError_t solve3d_t(const Solve3 &S, const double *omega, double *phi, 
         k.twy = reinterpret_cast<const V2<T> *>(tw_col);
         k.kx = reinterpret_cast<const T *>(k_row);
         k.ky = reinterpret_cast<const T *>(k_col);
-        k.dependent = true;
+        k.stateless = true;
         return k;
     };
     const PropK<T> kx = view(S.vx, S.twx, S.twy, S.kx, S.ky);

@@ -83,7 +83,8 @@ struct PropCK {
     int nseg, skip;
 };
 
-template <int LOGX, int LOGY, int C, int T>
+// READ: every twiddle from the tables (stateless solves, see ChainForm).
+template <int LOGX, int LOGY, int C, int T, bool READ = false>
 struct ClusterGeom {
     static constexpr int NX = 1 << LOGX, NY = 1 << LOGY, R2 = NY / 2 / C, W2 = NX / 2 / C;
     static constexpr int P = R2 * NX;  // complex points per CTA in either packing
@@ -91,8 +92,8 @@ struct ClusterGeom {
     static constexpr int HN = NY / 2 * NX;  // stored complex points per chain and node
     // radix 16 where it saves passes (fft8.cuh best_mr) and every thread gets
     // whole 16-point butterflies
-    static constexpr int MRX = (best_mr(LOGX) == 4 && P % (16 * T) == 0) ? 4 : 3;
-    static constexpr int MRY = (best_mr(LOGY) == 4 && P % (16 * T) == 0) ? 4 : 3;
+    static constexpr int MRX = ((best_mr(LOGX) == 4 && P % (16 * T) == 0) ? 4 : 3) | (READ ? kReadAll : 0);
+    static constexpr int MRY = ((best_mr(LOGY) == 4 && P % (16 * T) == 0) ? 4 : 3) | (READ ? kReadAll : 0);
     static constexpr int TABX = tabs_total(LOGX, MRX), TABY = tabs_total(LOGY, MRY);
     // row buffer, column buffer, pass tables, Fourier factors; with CACHE the
     // node factors of the epilogue sites in either packing (P points each)
@@ -188,10 +189,10 @@ __device__ __forceinline__ bool starts_in_columns(int m) { return m & 1; }
 // step (64 KB per CTA less; 128 x 128, one run: 3.31 ms per 4 steps alone,
 // cached 3.15; 4 x 256 x 512 in 8 phased launches, each of which would refill
 // them: 5.03 ms per 4 steps, cached 5.16).
-template <int LOGX, int LOGY, int C, int T, int MINB, bool DIFF, bool CACHE>
+template <int LOGX, int LOGY, int C, int T, int MINB, bool DIFF, bool CACHE, bool READ = false>
 __global__ void __launch_bounds__(T, MINB) prop_chain(PropCK k)
 {
-    using G = ClusterGeom<LOGX, LOGY, C, T>;
+    using G = ClusterGeom<LOGX, LOGY, C, T, READ>;
     constexpr int NX = G::NX, NY = G::NY, R2 = G::R2, W2 = G::W2, P = G::P, HN = G::HN;
     constexpr int NWARP = T / 32;
     static_assert(P == W2 * NY, "layout sizes");
@@ -784,14 +785,19 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
 struct ClusterShape {
     int logx, logy, c, t;
     // forms of the kernel (ChainForm): plain and reference solves, differential solve
-    const void *fn[3], *fn_diff[3];
-    size_t smem[3];
+    const void *fn[4], *fn_diff[4];
+    size_t smem[4];
     int mrx, mry;         // radix plans of the row and column transforms (log2 of the largest radix)
 };
 // CHAIN_SOLO: the whole register file for one CTA per SM, factors cached;
 // CHAIN_SHARE: half of it, factors from planes; CHAIN_PHASED: the whole, from
 // planes.  The tiles below 4096 points fit several CTAs per SM in any form.
-enum ChainForm { CHAIN_SOLO = 0, CHAIN_SHARE = 1, CHAIN_PHASED = 2 };
+// CHAIN_READ: the first with every twiddle read, for stateless solves (plain
+// only), which keep the accuracy of single reads: an RMS error of 3.4e-7 on 128 x
+// 128, N_s = 64, 4.4e-7 with products (256 x 512: 2.6e-7, 3.5e-7), for 0.346 ms
+// instead of 0.344.  A handle's solves form products (4 x 256 x 512 a step: 1.37
+// ms, 1.39 with every twiddle read).
+enum ChainForm { CHAIN_SOLO = 0, CHAIN_SHARE = 1, CHAIN_PHASED = 2, CHAIN_READ = 3 };
 
 template <int LOGX, int LOGY, int C, int T, int MINB = 1024 / T>
 static ClusterShape shape_of()
@@ -799,14 +805,16 @@ static ClusterShape shape_of()
     constexpr int SHARE = MINB == 1 ? 2 : MINB;
     constexpr bool PH = C >= 8;  // below that a launch holds many clusters and one more costs little: no form of their own
     using G = ClusterGeom<LOGX, LOGY, C, T>;
+    using GR = ClusterGeom<LOGX, LOGY, C, T, true>;
     return ClusterShape{LOGX, LOGY, C, T,
                         {(const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, true>,
                          (const void *)prop_chain<LOGX, LOGY, C, T, SHARE, false, false>,
-                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, !PH>},
+                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, !PH>,
+                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, false, true, true>},
                         {(const void *)prop_chain<LOGX, LOGY, C, T, MINB, true, true>,
                          (const void *)prop_chain<LOGX, LOGY, C, T, SHARE, true, false>,
-                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, true, !PH>},
-                        {G::SMEM_CACHE, G::SMEM, PH ? G::SMEM : G::SMEM_CACHE}, G::MRX, G::MRY};
+                         (const void *)prop_chain<LOGX, LOGY, C, T, MINB, true, !PH>, nullptr},
+                        {G::SMEM_CACHE, G::SMEM, PH ? G::SMEM : G::SMEM_CACHE, GR::SMEM_CACHE}, G::MRX, G::MRY};
 }
 
 // Instantiated grids (log2 nx, log2 ny).  A tile of 4096 points has 256
@@ -912,6 +920,7 @@ bool cluster_solve_supported(const Group &G)
         };
         bool all = true;
         for (ChainForm f : {CHAIN_SOLO, CHAIN_SHARE, CHAIN_PHASED}) all = all && ok(false, f) && ok(true, f);
+        all = all && ok(false, CHAIN_READ);
         if (all) {
             st = 1;
             g_solo_clusters[dev][s->logx][s->logy][0] = count_solo_clusters(s, false);
@@ -928,6 +937,7 @@ int cluster_chain_launches(const Group &G, bool diff)
 {
     const ClusterShape *sh = find_shape(G.g.logx, G.g.logy);
     if (!sh) return 0;
+    if (G.stateless) return 1;
     const int nch = 2 * G.g.nruns, solo = solo_clusters(sh, diff);
     // solo > 0: the one-CTA-per-SM shared-memory size is set for this shape
     const bool can = solo > 0 && nch >= 2 && G.g.ns >= nch - 1;
@@ -970,7 +980,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
                                  const SolveProbe *probe, const double *phi_ref, const double *q_ref)
 {
     const ClusterShape *sh = find_shape(G.g.logx, G.g.logy);
-    if (!sh || !G.hc || (diff && !G.hd)) return cudaErrorInvalidValue;
+    if (!sh || !G.hc || (diff && (!G.hd || G.stateless))) return cudaErrorInvalidValue;
     PropCK k;
     k.g = G.g;
     k.hout = reinterpret_cast<float2 *>(diff ? G.hd : G.hc);
@@ -993,7 +1003,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     const int nch = 2 * G.g.nruns, launches = cluster_chain_launches(G, diff);
     const bool phased = launches > 1;
     const int solo = solo_clusters(sh, diff);
-    const ChainForm form = phased ? CHAIN_PHASED : (G.crowded || nch > solo ? CHAIN_SHARE : CHAIN_SOLO);
+    const ChainForm form = G.stateless ? CHAIN_READ : (phased ? CHAIN_PHASED : (G.crowded || nch > solo ? CHAIN_SHARE : CHAIN_SOLO));
     k.nseg = phased ? nch - 1 : 0;
     k.skip = 0;
     cudaLaunchConfig_t cfg = {};

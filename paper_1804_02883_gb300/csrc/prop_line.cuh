@@ -31,7 +31,7 @@ template <typename T> struct PropK {
     double *ia, *ib, *part;
     const V2<T> *twx, *twy;
     const T *kx, *ky;
-    bool dependent;  // launches as programmatic dependents (see line_dependents)
+    bool stateless;  // launches as programmatic dependents (see line_dependents), every twiddle read
 };
 
 // Boltzmann factor (E_A, E_B) of the half-step at node j of chain g (fac_g)
@@ -305,13 +305,13 @@ template <typename T> cudaError_t line_col_t(const PropK<T> &k, cudaStream_t s)
     const size_t sm = LineTile(false, n, l, k.g.py).points() * sizeof(V2<T>);
     const int th = line_threads(n, r0, l);
     switch (r0) {
-    case 2: return launch_line(k.dependent, prop_col<T, 2>, grid, th, sm, s, k, l);
-    case 4: return launch_line(k.dependent, prop_col<T, 4>, grid, th, sm, s, k, l);
-    case 6: return launch_line(k.dependent, prop_col<T, 6>, grid, th, sm, s, k, l);
-    case 8: return launch_line(k.dependent, prop_col<T, 8>, grid, th, sm, s, k, l);
-    case 10: return launch_line(k.dependent, prop_col<T, 10>, grid, th, sm, s, k, l);
-    case 12: return launch_line(k.dependent, prop_col<T, 12>, grid, th, sm, s, k, l);
-    default: return launch_line(k.dependent, prop_col<T, 16>, grid, th, sm, s, k, l);
+    case 2: return launch_line(k.stateless, prop_col<T, 2>, grid, th, sm, s, k, l);
+    case 4: return launch_line(k.stateless, prop_col<T, 4>, grid, th, sm, s, k, l);
+    case 6: return launch_line(k.stateless, prop_col<T, 6>, grid, th, sm, s, k, l);
+    case 8: return launch_line(k.stateless, prop_col<T, 8>, grid, th, sm, s, k, l);
+    case 10: return launch_line(k.stateless, prop_col<T, 10>, grid, th, sm, s, k, l);
+    case 12: return launch_line(k.stateless, prop_col<T, 12>, grid, th, sm, s, k, l);
+    default: return launch_line(k.stateless, prop_col<T, 16>, grid, th, sm, s, k, l);
     }
 }
 
@@ -330,13 +330,13 @@ template <typename T, bool DIFF> cudaError_t line_row_t(const PropK<T> &k, int m
     const int th = line_threads(n, r0, l);
     const RowWeights w = row_weights(k.g, m);
     switch (r0) {
-    case 2: return launch_line(k.dependent, prop_row<T, 2, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 4: return launch_line(k.dependent, prop_row<T, 4, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 6: return launch_line(k.dependent, prop_row<T, 6, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 8: return launch_line(k.dependent, prop_row<T, 8, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 10: return launch_line(k.dependent, prop_row<T, 10, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 12: return launch_line(k.dependent, prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
-    default: return launch_line(k.dependent, prop_row<T, 16, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 2: return launch_line(k.stateless, prop_row<T, 2, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 4: return launch_line(k.stateless, prop_row<T, 4, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 6: return launch_line(k.stateless, prop_row<T, 6, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 8: return launch_line(k.stateless, prop_row<T, 8, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 10: return launch_line(k.stateless, prop_row<T, 10, DIFF>, grid, th, sm, s, k, m, l, w);
+    case 12: return launch_line(k.stateless, prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
+    default: return launch_line(k.stateless, prop_row<T, 16, DIFF>, grid, th, sm, s, k, m, l, w);
     }
 }
 

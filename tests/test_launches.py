@@ -55,7 +55,8 @@ def test_kernel_attributes_are_set_on_every_device(rt):
 
 
 def _chains(out):
-    """Template arguments (.., CTAs the registers are sized for, differential, cached) of the chain launches."""
+    """Template arguments of the chain launches: log2 nx and ny, CTAs, threads, CTAs per SM
+    the registers are sized for, differential, cached, every twiddle read."""
     return [l[1] for l in out if "prop_chain" in l[0]]
 
 
@@ -68,20 +69,20 @@ def test_chains_share_an_sm_only_where_the_groups_fill_the_chip(rt):
         return [W.with_(r, seed=s) for s in range(n)]
 
     rc, out = rt.init(run(128, 128, 1) + run(128, 256, 1))
-    assert rc == 0 and _chains(out) and all(a[-1] == 1 for a in _chains(out))
+    assert rc == 0 and _chains(out) and all(a[6] == 1 for a in _chains(out))
     rc, out = rt.init(run(256, 512, 4) + run(128, 128, 1))
     wide = [a for a in _chains(out) if a[:2] == (9, 8)]
     # Phi(0), then two solves a step in two graphs, 8 launches each
     assert rc == 0 and len(wide) == 5 * 8 and all(a[4] == 1 for a in wide)
     rc, out = rt.init(W.ensemble_32())
     step = _chains(out)[len({(r.ny, r.nx, r.ns) for r in W.ensemble_32()}):]  # after the solves of Phi(0)
-    assert rc == 0 and step and all(a[-3] == 2 and a[-1] == 0 for a in step if a[2] >= 4)
+    assert rc == 0 and step and all(a[4] == 2 and a[6] == 0 for a in step if a[2] >= 4)
 
 
 def test_groups_of_an_exact_step_run_alone(rt):
     """The exact step takes its groups one after the other."""
     rc, out = rt.step_exact(W.ensemble_32(), 2)
-    assert rc == 0 and _chains(out) and all(a[-1] == 1 for a in _chains(out) if a[2] < 16)
+    assert rc == 0 and _chains(out) and all(a[6] == 1 for a in _chains(out) if a[2] < 16)
 
 
 @pytest.mark.parametrize("precision,ny,nx", [(P.PLAIN_FP64, 64, 64), (P.MIXED_FP32, 150, 150), (P.MIXED_FP32, 64, 1024), (P.MIXED_FP32, 1024, 512)])
