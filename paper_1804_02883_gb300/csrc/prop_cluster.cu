@@ -54,6 +54,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -521,7 +522,6 @@ struct ContourK {
     const double *phi_t, *q_t;  // first solve's densities (differential solve)
     double *phi, *q;
     int *err;
-    bool stateless;  // nobody reads err: a give-up makes Q and the densities NaN
 };
 
 // Compensated (Kahan) FP32 sum: value() = sum minus the carried rounding
@@ -537,6 +537,28 @@ struct KSum {
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
+
+// Sum of products with every rounding error carried (two-sum of exact
+// products): good to ~2^-47 per term.
+struct PairSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float w, float x, float y)  // w: a power of two
+    {
+        const float p = x * y, t = w * p, u = s + t, v = u - s;
+        c += ((s - (u - v)) + (t - v)) + w * fmaf(x, y, -p);
+        s = u;
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+// 1 / (a b) in FP64 for FP32 a, b: Newton steps from the FP32 reciprocal (an
+// FP64 division is several times as many instructions)
+__device__ __forceinline__ double inverse64(float a, float b)
+{
+    const double p = (double)a * (double)b;
+    double r = (double)(1.f / (a * b));
+    r = r * fma(-p, r, 2.0);
+    return r * fma(-p, r, 2.0);
+}
 
 // Trapezoid weights over [0, s_{N_A}] and [s_{N_A}, 1] in units of ds.
 __device__ __forceinline__ void node_weights(int j, int na, int ns, float &wa, float &wb)
@@ -566,8 +588,9 @@ __global__ void selftest_wait(int *err, long long limit)
 
 // Q partials from node N_s of the g chain: Q_P = mean g_{N_s} with
 // g = a / E (plain); dQ_P = mean dg_{N_s}, dg = (d a - rho a~) / E' (DIFF).
-// Block sums into part[run][block].
-template <bool DIFF>
+// Block sums into part[run][block].  F64 (stateless solves): quotients and sums
+// in FP64.
+template <bool DIFF, bool F64>
 __global__ void __launch_bounds__(kThreads) prop_qsum(ContourK k)
 {
     __shared__ double red[32];
@@ -581,12 +604,15 @@ __global__ void __launch_bounds__(kThreads) prop_qsum(ContourK k)
     const float2 *d_ns = DIFF ? k.hd + (size_t)run * 2 * cs + (size_t)ns * k.hn : nullptr;
     const float2 *efac = k.efac + (size_t)run * n;
     const float2 *rho = DIFF ? k.rho + (size_t)run * n : nullptr;
-    float acc = 0.f;
+    static_assert(!(DIFF && F64), "stateless solves are plain");
+    typename std::conditional<F64, double, float>::type acc = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npk; i += gridDim.x * blockDim.x) {
         const int kk = i >> k.g.logx, x = i & (nx - 1), s0 = 2 * kk * nx + x, s1 = s0 + nx;
         const float2 e0 = efac[s0], e1 = efac[s1], a = a_ns[i];
         const float E0 = bm ? e0.y : e0.x, E1 = bm ? e1.y : e1.x;
-        if (!DIFF) {
+        if constexpr (F64) {
+            acc += (double)a.x * inverse64(E0, 1.f) + (double)a.y * inverse64(E1, 1.f);
+        } else if (!DIFF) {
             acc += a.x / E0 + a.y / E1;
         } else {
             const float2 r0 = rho[s0], r1 = rho[s1], d = d_ns[i];
@@ -606,11 +632,15 @@ template <bool DIFF> struct ContourStage {
 };
 
 // One thread per packed site (real rows 2kk and 2kk+1 at column x).
-// Products in FP32, partial sums over at most 8 nodes of equal weights in
-// FP32, then FP64.  The node states stream through shared memory by
+// Products in FP32, compensated FP32 sums.  PAIRS (stateless solves): exact
+// products of the stored states summed exactly per block of the contour, the
+// node factors of the block (A below N_A, B above, the junction's own) divided
+// out of the sums in FP64: 4e-13 of FP64 sums, where three roundings per product
+// and the compensated sum leave 1e-8 (128 x 128, N_s = 64: 0.346 -> 0.348 ms a
+// solve).  The node states stream through shared memory by
 // asynchronous copies, each thread staging only its own elements (no
 // barriers), so that the loads in flight do not hold registers.
-template <bool DIFF>
+template <bool DIFF, bool PAIRS>
 __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
 {
     extern __shared__ __align__(16) float2 stg[];
@@ -664,7 +694,7 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
     const double tp = sum_partials(pr, k.nq, 1, &bc), ts = sum_partials(pr + kMaxPart / 2, k.ns_part, 1, &bc);
     if (tid == 0) {
         const double sq = tp / (double)n, ss = ts / (double)n;
-        const bool lost = !DIFF && k.stateless && (*k.err & 4);
+        const bool lost = PAIRS && (*k.err & 4);  // nobody reads a stateless call's error word
         const double nan = __longlong_as_double(0x7ff8000000000000ll);
         const double qp = DIFF ? k.q_t[2 * run] + sq : (lost ? nan : sq), qs = DIFF ? k.q_t[2 * run + 1] + ss : (lost ? nan : ss);
         fac[0] = k.g.phi_p * k.g.ds / qp;
@@ -705,6 +735,8 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
                 rs[bk][c] = 1.f / (e[bk][c] * (1.f + q[bk][c]));
             }
     }
+    PairSum qa0, qb0, qa1, qb1;        // PAIRS: the nodes below and above the junction
+    float2 ja = f2(0.f, 0.f), jb = ja;  // and the junction's states
     // compensated (Kahan) FP32 sums per block and real site; the trapezoid
     // weights 1 and 1/2 scale the terms exactly
     KSum sa0, sb0, sa1, sb1;
@@ -727,6 +759,19 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
             // (selects: a run-time index would move these small arrays to local memory)
             auto pick = [](const float (&v)[2][2], bool b, int c) { return b ? v[1][c] : v[0][c]; };
             const float2 a = b[0], bb = b[kThreads];
+            if constexpr (PAIRS) {
+                if (m < na) {
+                    qa0.add(wa, a.x, bb.x);
+                    qa1.add(wa, a.y, bb.y);
+                } else if (m > na) {
+                    qb0.add(wb, a.x, bb.x);
+                    qb1.add(wb, a.y, bb.y);
+                } else {
+                    ja = a;
+                    jb = bb;
+                }
+                continue;
+            }
             float t0, t1;
             if (!DIFF) {
                 t0 = a.x * bb.x * (bk == bp ? pick(r2, bk, 0) : ri[0][0] * ri[1][0]);
@@ -754,7 +799,23 @@ __global__ void __launch_bounds__(kThreads) prop_contour(ContourK k)
         }
         issue(st, (ch + NST) * U);  // this stage's values are consumed
     }
-    const double ia0 = sa0.value(), ib0 = sb0.value(), ia1 = sa1.value(), ib1 = sb1.value();
+    double ia0, ib0, ia1, ib1;
+    if constexpr (PAIRS) {
+        float wa, wb;
+        node_weights(na, na, ns, wa, wb);
+        const bool bk = half_step_block(k.g.jr, 0, na, ns, na, false), bp = half_step_block(k.g.jr, 1, ns - na, ns, na, false);
+        const double j0 = (double)ja.x * (double)jb.x * inverse64(bk ? e0.y : e0.x, bp ? e0.y : e0.x);
+        const double j1 = (double)ja.y * (double)jb.y * inverse64(bk ? e1.y : e1.x, bp ? e1.y : e1.x);
+        ia0 = fma(qa0.value(), inverse64(e0.x, e0.x), wa * j0);
+        ib0 = fma(qb0.value(), inverse64(e0.y, e0.y), wb * j0);
+        ia1 = fma(qa1.value(), inverse64(e1.x, e1.x), wa * j1);
+        ib1 = fma(qb1.value(), inverse64(e1.y, e1.y), wb * j1);
+    } else {
+        ia0 = sa0.value();
+        ib0 = sb0.value();
+        ia1 = sa1.value();
+        ib1 = sb1.value();
+    }
     const double cp = fac[0], cs_ = fac[1];
     double *pa = k.phi + (size_t)run * 3 * n, *pb = pa + n, *ps = pb + n;
     if (!DIFF) {
@@ -1049,21 +1110,26 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     c.phi = phi;
     c.q = q;
     c.err = G.err;
-    c.stateless = G.stateless;
     const int npk = G.g.nx * G.g.ny / 2;
     const dim3 grid((npk + kThreads - 1) / kThreads, G.g.nruns), gq(kQBlocks, G.g.nruns);
     static PerDevice conf;
     if (cudaError_t e = conf.once([] {
-            const cudaError_t e1 = cudaFuncSetAttribute(prop_contour<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<true>::SMEM);
-            return e1 ? e1 : cudaFuncSetAttribute(prop_contour<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<false>::SMEM);
+            cudaError_t e = cudaFuncSetAttribute(prop_contour<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<true>::SMEM);
+            if (!e) e = cudaFuncSetAttribute(prop_contour<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<false>::SMEM);
+            return e ? e : cudaFuncSetAttribute(prop_contour<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ContourStage<false>::SMEM);
         }))
         return e;
     if (diff) {
-        prop_qsum<true><<<gq, kThreads, 0, s>>>(c);
-        prop_contour<true><<<grid, kThreads, ContourStage<true>::SMEM, s>>>(c);
+        prop_qsum<true, false><<<gq, kThreads, 0, s>>>(c);
+        prop_contour<true, false><<<grid, kThreads, ContourStage<true>::SMEM, s>>>(c);
+    } else if (G.stateless) {
+        // 64 threads a block while 256 would leave SMs empty
+        const int th = npk < kSMs * kThreads ? 64 : kThreads;
+        prop_qsum<false, true><<<gq, kThreads, 0, s>>>(c);
+        prop_contour<false, true><<<dim3((npk + th - 1) / th, G.g.nruns), th, ContourStage<false>::SMEM, s>>>(c);
     } else {
-        prop_qsum<false><<<gq, kThreads, 0, s>>>(c);
-        prop_contour<false><<<grid, kThreads, ContourStage<false>::SMEM, s>>>(c);
+        prop_qsum<false, false><<<gq, kThreads, 0, s>>>(c);
+        prop_contour<false, false><<<grid, kThreads, ContourStage<false>::SMEM, s>>>(c);
     }
     return cudaGetLastError();
 }

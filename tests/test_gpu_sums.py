@@ -76,3 +76,48 @@ def test_stateless_solves_are_as_accurate_as_radix_2(ny, nx, ns):
     # with the queried workspace, and the streaming passes with a small one
     for nbytes in (None, ny * nx * (16 + (ns // 2 + 3) * 8) + 192 * 1024):
         assert rms_error(ny, nx, ns, nbytes) <= RADIX2_RMS[ny, nx, ns]
+
+
+@pytest.mark.parametrize("jr", [0, 1])
+@pytest.mark.parametrize("ny,nx,ns,f_a", [(64, 64, 32, 0.5), (128, 128, 64, 0.3), (128, 512, 10, 0.882), (512, 256, 12, 0.0), (256, 512, 8, 1.0)])
+def test_resident_stateless_sums_equal_fp64_sums(ny, nx, ns, f_a, jr):
+    # the states a_m = E_dep(m) g_m that the cluster kernel leaves in the
+    # workspace (error word and partials, factors (E_A, E_B), three factor planes, the
+    # states of both chains in pairs of rows), summed here in FP64
+    import torch
+
+    run = W.with_(W.plain_small(), nx=nx, ny=ny, ns=ns, f_a=f_a, precision=P.MIXED_FP32, junction_rule=jr)
+    om = torch.from_numpy(W.random_omega(ny, nx, 7)).cuda()
+    pd, qd = torch.empty_like(om), torch.empty(2, dtype=torch.float64, device="cuda")
+    nb = P.epd_prop_solve_workspace_bytes(run)
+    ws = torch.zeros(nb + 256, dtype=torch.uint8, device="cuda")
+    off = -ws.data_ptr() % 256
+    P.epd_prop_solve(run, om.data_ptr(), pd.data_ptr(), qd.data_ptr(), ws.data_ptr() + off, nb, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    phi, q = pd.cpu().numpy(), qd.cpu().numpy()
+    raw, n = ws[off:].cpu().numpy(), ny * nx
+    o = 256 + 4096 * 8
+    e = raw[o:o + 8 * n].view(np.float32).reshape(ny, nx, 2).astype(np.float64)
+    o += 8 * n + 12 * n
+    a = raw[o:o + 8 * (ns + 1) * n].view(np.float32).reshape(2, ns + 1, ny // 2, nx, 2)
+    a = a.transpose(0, 1, 2, 4, 3).reshape(2, ns + 1, ny, nx).astype(np.float64)
+    na = int(np.round(f_a * ns))
+
+    def block(chain, m):  # of the departing half-step
+        if jr == 0:
+            return int((m if chain == 0 else ns - m) >= na)
+        j = m - 1 if m == ns else m
+        return int((j if chain == 0 else ns - 1 - j) >= na)
+
+    want = np.zeros((2, ny, nx))
+    for m in range(ns + 1):
+        t = (a[0, m] / e[..., block(0, m)]) * (a[1, ns - m] / e[..., block(1, ns - m)])
+        if na and m <= na:
+            want[0] += t * (0.5 if m in (0, na) else 1.0)
+        if na < ns and m >= na:
+            want[1] += t * (0.5 if m in (na, ns) else 1.0)
+    qp = (a[0, ns] / e[..., block(0, ns)]).mean()
+    assert abs(q[0] / qp - 1) < 1e-12
+    want *= run.phi_p / ns / qp
+    for s in range(2):
+        assert rel_err(phi[s], want[s]) < 4e-12
