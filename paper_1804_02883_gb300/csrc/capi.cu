@@ -13,6 +13,7 @@
 #include "common.cuh"
 #include "engine.h"
 #include "fft8.cuh"
+#include "fftg.cuh"
 #include "surrogate.h"
 
 namespace epdlb {
@@ -294,10 +295,12 @@ static void host_tables(const Group &G, std::vector<T> &twx, std::vector<T> &twy
         outd.resize(2 * (size_t)n);
         for (int t = 0; t < n; ++t) {
             const double a = 2.0 * pi * (double)t / (double)n;
-            outd[2 * t] = std::cos(a);
-            outd[2 * t + 1] = -std::sin(a);
-            out[2 * t] = (T)outd[2 * t];
-            out[2 * t + 1] = (T)outd[2 * t + 1];
+            const V2<double> w = unit_pair<double>(std::cos(a), -std::sin(a));
+            const V2<T> v = unit_pair<T>(std::cos(a), -std::sin(a));
+            outd[2 * t] = w.x;
+            outd[2 * t + 1] = w.y;
+            out[2 * t] = v.x;
+            out[2 * t + 1] = v.y;
         }
     };
     tw(G.g.nx, twx, twxd);
@@ -333,8 +336,9 @@ static cudaError_t upload_tables_t(Group &G, cudaStream_t s)
             std::vector<float> t(2 * (size_t)n);
             for (int j = 0; j < n; ++j) {
                 const double a = 2.0 * pi * (double)j / (double)n;
-                t[2 * j] = (float)std::cos(a);
-                t[2 * j + 1] = (float)-std::sin(a);
+                const float2 w = unit_pair<float>(std::cos(a), -std::sin(a));
+                t[2 * j] = w.x;
+                t[2 * j + 1] = w.y;
             }
             return t;
         };
@@ -1328,7 +1332,7 @@ template <typename T> __global__ void call_tables(CallTables c)
     if (blockIdx.z == 0) {
         if (i < n && a.tw) {
             const double2 w = twiddle(i);
-            reinterpret_cast<V2<T> *>(a.tw)[i] = mk<T>((T)w.x, (T)w.y);
+            reinterpret_cast<V2<T> *>(a.tw)[i] = unit_pair<T>(w.x, w.y);
         }
         return;
     }
@@ -1352,7 +1356,7 @@ template <typename T> __global__ void call_tables(CallTables c)
                 if (r < 0 || r >= tab_rows(rlog, mr) * M) continue;
                 const int row = r / M, k = row + 1;
                 const double2 w = twiddle(((r % M) << slog) * k);
-                a.tab[v][e] = make_float2((float)w.x, (float)w.y);
+                a.tab[v][e] = unit_pair<float>(w.x, w.y);
             }
         }
     }

@@ -121,3 +121,19 @@ def test_resident_stateless_sums_equal_fp64_sums(ny, nx, ns, f_a, jr):
     want *= run.phi_p / ns / qp
     for s in range(2):
         assert rel_err(phi[s], want[s]) < 4e-12
+
+
+# the same of the passes of radices 2 to 5 on grids that are not powers of two
+RADIX5_RMS = {
+    (150, 150, 17): 6.0607e-8, (270, 384, 24): 1.0300e-7, (96, 90, 32): 1.6063e-7, (32, 64, 32): 2.5659e-7,
+    (128, 432, 24): 1.0157e-7, (320, 480, 24): 9.2380e-8, (200, 240, 33): 1.2030e-7, (54, 162, 48): 3.3837e-7,
+    (486, 30, 40): 2.3627e-7, (36, 250, 48): 2.9919e-7, (1458, 40, 16): 5.9600e-8, (48, 96, 48): 3.5349e-7,
+    (90, 1024, 24): 9.0197e-8, (180, 300, 32): 1.1285e-7,
+}
+
+
+def test_general_grids_are_as_accurate_as_small_radices():
+    # on one grid a few per cent either way are chance; over these the errors
+    # are no larger
+    ratio = [rms_error(*g) / e for g, e in RADIX5_RMS.items()]
+    assert np.exp(np.mean(np.log(ratio))) <= 1.0, ratio
