@@ -478,8 +478,8 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t sad
 }
 
 // Weight gradient of one layer: dW[tap][co][ci] = sum_p dZ[p][co] x[p + off(tap)][ci]
-// over an 8 x 16 tile per step, `tiles` consecutive tiles per CTA; 9 warps, warp
-// = tap.  Partial sums per CTA to part[blk][tap][co][ci] (deterministic
+// over an 8 x 16 tile per step, consecutive tiles per CTA, `seg` of them per FP32
+// accumulator and the accumulators added; 9 warps, warp = tap.  Partial sums per CTA to part[blk][tap][co][ci] (deterministic
 // reduction later).  CO, CI multiples of 16.  Both operands lie in shared
 // memory as the tensors do, channels contiguous per pixel, while the sum runs
 // over pixels: transposing matrix loads make the fragments (rows of channels
@@ -495,7 +495,7 @@ template <int CI, int CO, int D> struct DwGeom {
 };
 template <int CI, int CO, int D>
 __global__ void __launch_bounds__(288) conv3x3_dw(const __nv_bfloat16 *x, const __nv_bfloat16 *dz, float *part, int nx, int ny,
-                                                 int tiles_x, int tiles_per_cta, int ntiles_total)
+                                                 int tiles_x, int tiles_per_cta, int seg, int ntiles_total)
 {
     using G = DwGeom<CI, CO, D>;
     constexpr int CS = G::CS, DS = G::DS, HH = G::HH, HW = G::HW;
@@ -504,14 +504,15 @@ __global__ void __launch_bounds__(288) conv3x3_dw(const __nv_bfloat16 *x, const 
     const int tid = threadIdx.x, lane = tid & 31, tap = tid >> 5;
     const int g = lane >> 2, t = lane & 3, dy = (tap / 3) * D, dx = (tap % 3) * D;
     const long long n = (long long)nx * ny;
-    float acc[CO / 16][CI / 8][4];
+    float acc[CO / 16][CI / 8][4], sum[CO / 16][CI / 8][4];
 #pragma unroll
     for (int mt = 0; mt < CO / 16; ++mt)
 #pragma unroll
         for (int nt = 0; nt < CI / 8; ++nt)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
+            for (int i = 0; i < 4; ++i) acc[mt][nt][i] = sum[mt][nt][i] = 0.f;
     const int tiles_per_img = tiles_x * (ny / TH);
+    int left = seg;
     const int first = blockIdx.x * tiles_per_cta, count = min(tiles_per_cta, ntiles_total - first);
     auto load = [&](int it) {
         if (it < count) {
@@ -561,6 +562,18 @@ __global__ void __launch_bounds__(288) conv3x3_dw(const __nv_bfloat16 *x, const 
             }
         }
         __syncthreads();  // this stage is filled again by the next load
+        if (--left == 0 || it + 1 == count) {
+            left = seg;
+#pragma unroll
+            for (int mt = 0; mt < CO / 16; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < CI / 8; ++nt)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        sum[mt][nt][i] += acc[mt][nt][i];
+                        acc[mt][nt][i] = 0.f;
+                    }
+        }
     }
     cp_async_wait<0>();
     float *out = part + (size_t)blockIdx.x * 9 * CO * CI + (size_t)tap * CO * CI;
@@ -569,10 +582,10 @@ __global__ void __launch_bounds__(288) conv3x3_dw(const __nv_bfloat16 *x, const 
 #pragma unroll
         for (int nt = 0; nt < CI / 8; ++nt) {
             const int co = mt * 16 + g, ci = nt * 8 + 2 * t;
-            out[co * CI + ci] = acc[mt][nt][0];
-            out[co * CI + ci + 1] = acc[mt][nt][1];
-            out[(co + 8) * CI + ci] = acc[mt][nt][2];
-            out[(co + 8) * CI + ci + 1] = acc[mt][nt][3];
+            out[co * CI + ci] = sum[mt][nt][0];
+            out[co * CI + ci + 1] = sum[mt][nt][1];
+            out[(co + 8) * CI + ci] = sum[mt][nt][2];
+            out[(co + 8) * CI + ci + 1] = sum[mt][nt][3];
         }
 }
 
@@ -1163,15 +1176,18 @@ static void dw(Work &w, const void *x, const void *dzp, cudaStream_t s)
 {
     const int tiles_x = w.nx / TW;
     const int ntiles = w.nb * tiles_x * (w.ny / TH);
-    // two CTAs per SM: fewer partials for reduce_dw, whose FP64 sums are
-    // bound by the FP64 unit (512 CTAs: 22 us per 32 x 32 layer)
-    const int cap = std::min(w.nblk_dw, 2 * 152), per = (ntiles + cap - 1) / cap;
+    // Two CTAs per SM: fewer partials for reduce_dw, whose FP64 sums are bound by
+    // the FP64 unit (512 CTAs: 22 us per 32 x 32 layer).  A value still goes
+    // through no more roundings than with 512 CTAs of per512 tiles, each tile's 8
+    // chunks of 16 pixels in turn: sums of one tile less, and these added.
+    const int per512 = (ntiles + 511) / 512, cap = per512 == 1 ? w.nblk_dw : std::min(w.nblk_dw, 2 * kSMs);
+    const int per = (ntiles + cap - 1) / cap, seg = std::max(1, per512 - 1);
     const int nblk = (ntiles + per - 1) / per;
     constexpr size_t smem = DwGeom<CI, CO, D>::SMEM;
     static PerDevice conf;  // (a failure shows at the launch)
     conf.once([] { return cudaFuncSetAttribute(conv3x3_dw<CI, CO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); });
     conv3x3_dw<CI, CO, D><<<nblk, 288, smem, s>>>(reinterpret_cast<const __nv_bfloat16 *>(x), reinterpret_cast<const __nv_bfloat16 *>(dzp),
-                                            w.dwpart, w.nx, w.ny, tiles_x, per, ntiles);
+                                            w.dwpart, w.nx, w.ny, tiles_x, per, seg, ntiles);
     w.nblk_dw = nblk;
 }
 

@@ -31,6 +31,8 @@ class FakeRuntime:
         L.epd_prop_solve.argtypes = [ctypes.c_void_p] * 5 + [ctypes.c_size_t, ctypes.c_void_p]
         L.epd_sur_forward.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_double, ctypes.c_double] + \
             [ctypes.c_void_p] * 3 + [ctypes.c_size_t, ctypes.c_void_p]
+        L.epd_sur_gradients.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_double, ctypes.c_double] + \
+            [ctypes.c_void_p] * 5 + [ctypes.c_size_t, ctypes.c_void_p]
         L.epd_prop_solve3d.argtypes = [ctypes.c_void_p, ctypes.c_int32] + [ctypes.c_void_p] * 4 + [ctypes.c_size_t, ctypes.c_void_p]
 
     def init(self, runs):
@@ -71,6 +73,12 @@ class FakeRuntime:
         n = ctypes.c_size_t()
         assert self.L.epd_sur_workspace_bytes(run.ny, run.nx, batch, 0, ctypes.byref(n)) == 0
         return self.L.epd_sur_forward(ctypes.byref(run.c()), batch, PTR, 1.0, 1.0, PTR, PTR, PTR, n, None)
+
+    def sur_gradients(self, run, batch):
+        self.L.fake_reset()
+        n = ctypes.c_size_t()
+        assert self.L.epd_sur_workspace_bytes(run.ny, run.nx, batch, 1, ctypes.byref(n)) == 0
+        return self.L.epd_sur_gradients(ctypes.byref(run.c()), batch, PTR, 1.0, 1.0, PTR, PTR, PTR, PTR, PTR, n, None)
 
     def launches(self):
         """(mangled kernel name, integral template arguments, grid, block, shared memory, cluster) of every launch."""

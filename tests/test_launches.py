@@ -98,3 +98,27 @@ def test_q_is_summed_over_the_same_tiles_in_every_batch(rt, precision, ny, nx):
             if "prop_finalize" in b[0] or "prop_contour_stream" in b[0]:
                 tiles.add((a[1], a[2][0], a[3]))
     assert len({t[1:] for t in tiles}) == 1, tiles
+
+
+def _dw_split(tiles):
+    """CTAs of the weight-gradient kernel, and tiles per CTA and per accumulator (restated)."""
+    per512 = -(-tiles // 512)
+    cap = min(512, tiles) if per512 == 1 else 304
+    per = -(-tiles // cap)
+    return -(-tiles // per), per, max(1, per512 - 1)
+
+
+def test_weight_gradient_values_pass_few_roundings():
+    """8 chunks of 16 pixels a tile in turn, then the accumulators added: no more
+    roundings than the chunks of one in 512 of the tiles, whose partials (the CTAs')
+    are added in FP64."""
+    for tiles in range(1, 70000):
+        _, per, seg = _dw_split(tiles)
+        assert 8 * min(seg, per) + -(-per // seg) - 1 <= 8 * -(-tiles // 512), tiles
+
+
+@pytest.mark.parametrize("batch,ny,nx", [(4, 256, 512), (1, 256, 256), (8, 512, 512), (1, 16, 16), (3, 48, 80), (2, 240, 160)])
+def test_weight_gradient_ctas(rt, batch, ny, nx):
+    assert rt.sur_gradients(W.with_(W.plain_small(), nx=nx, ny=ny), batch) == 0
+    dw = [l for l in rt.launches() if "conv3x3_dw" in l[0]]
+    assert len(dw) == 4 and all(l[2][0] == _dw_split(batch * ny * nx // 128)[0] for l in dw)
