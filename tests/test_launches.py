@@ -122,3 +122,9 @@ def test_weight_gradient_ctas(rt, batch, ny, nx):
     assert rt.sur_gradients(W.with_(W.plain_small(), nx=nx, ny=ny), batch) == 0
     dw = [l for l in rt.launches() if "conv3x3_dw" in l[0]]
     assert len(dw) == 4 and all(l[2][0] == _dw_split(batch * ny * nx // 128)[0] for l in dw)
+
+
+@pytest.mark.parametrize("batch", [1, 16000, 16384, 21845, 30000])
+def test_network_takes_large_batches_of_small_grids(rt, batch):
+    """The planes of a batch are a grid dimension: 65535 in y, 2^31 - 1 in x."""
+    assert rt.sur_forward(W.with_(W.plain_small(), nx=16, ny=16), batch) == 0
