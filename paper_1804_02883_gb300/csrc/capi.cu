@@ -38,10 +38,8 @@ size_t carve_group(Group &G, char *base, size_t off)
     G.phi_t = (double *)take(R * 3 * n * sizeof(double));
     G.q = (double *)take(R * 2 * sizeof(double));
     G.q_t = (double *)take(R * 2 * sizeof(double));
-    G.ia = (double *)take(R * n * sizeof(double));
-    G.ib = (double *)take(R * n * sizeof(double));
-    G.ia2 = (double *)take(R * n * sizeof(double));
-    G.ib2 = (double *)take(R * n * sizeof(double));
+    G.ia = (double *)take(2 * R * n * sizeof(double));
+    G.ib = G.ia ? G.ia + R * n : nullptr;
     G.cz = (double2 *)take(R * 4 * n * sizeof(double2));
     G.part = (double *)take(R * kMaxPart * sizeof(double));
     G.f0_lat = (double *)take(R * sizeof(double));
@@ -69,10 +67,8 @@ size_t carve_group(Group &G, char *base, size_t off)
     G.twx_d = (double2 *)take((size_t)G.g.nx * sizeof(double2));
     G.twy_d = (double2 *)take((size_t)G.g.ny * sizeof(double2));
     // radix-8/16 and cluster tables: power-of-two axes only
-    G.twx_full = G.twy_full = G.tab8x = G.tab8y = G.tab16x = G.tab16y = nullptr;
+    G.tab8x = G.tab8y = G.tab16x = G.tab16y = nullptr;
     if (G.g.pow2) {
-        G.twx_full = (float2 *)take((size_t)G.g.nx * sizeof(float2));
-        G.twy_full = (float2 *)take((size_t)G.g.ny * sizeof(float2));
         G.tab8x = (float2 *)take((size_t)tabs_total(G.g.logx) * sizeof(float2));
         G.tab8y = (float2 *)take((size_t)tabs_total(G.g.logy) * sizeof(float2));
         G.tab16x = best_mr(G.g.logx) == 4 ? (float2 *)take((size_t)tabs_total(G.g.logx, 4) * sizeof(float2)) : nullptr;
@@ -88,11 +84,10 @@ size_t carve_group(Group &G, char *base, size_t off)
         G.hd = take(hs);
         G.rho = take(R * n * sizeof(float2));
         G.cdiff = take(R * 3 * n * sizeof(float));
-        // the factor planes (12 bytes per site) in the streaming passes' contour
-        // sums (two adjoining arrays of 8; sizes on these grids are multiples
-        // of the alignment), which this solve does not use
+        // the plain solve's factor planes (12 bytes per site) in the streaming
+        // passes' contour sums (16), which this solve does not use
         G.facp = G.ia;
-        G.facd = G.ia2;
+        G.facd = take(R * 3 * n * sizeof(float));
     } else if (stream_diff) {
         G.hd = take(R * (size_t)(G.g.ns + 1) * n * sizeof(float2));
         G.rho = take(R * n * sizeof(float2));
@@ -128,8 +123,6 @@ static Group run_view(const Group &G, int r)
     V.q_t += 2 * r;
     V.ia += (size_t)r * n;
     V.ib += (size_t)r * n;
-    V.ia2 += (size_t)r * n;
-    V.ib2 += (size_t)r * n;
     V.cz += (size_t)r * 4 * n;
     V.part += (size_t)r * kMaxPart;
     V.f0_lat += r;
@@ -169,9 +162,9 @@ static Group run_view(const Group &G, int r)
 static bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
 // Radices of the in-place transforms (fftg.cuh) of an even length 2^a 3^b 5^c:
-// the first from {2, 4, 6, 8, 10, 12, 16}, the last from {1, 2, 3, 4, 5, 8, 9,
-// 10, 15, 16}, {3, 4, 5, 8, 9} between (every such length to 2048 has a plan
-// of at most four).  Cost per plan: instructions per point of each radix, the
+// the first from {2, 4, 6, 8, 10, 12}, the last from {1, 2, 3, 4, 5, 8, 9, 10, 15,
+// 16} (1: z axes of 2 to 6 planes), {3, 4, 5, 8, 9} between; every such length to
+// 2048 has a plan of two to four.  Cost per plan: instructions per point of each radix, the
 // twiddles and shared-memory trip of each pass, a shorter contiguous run of
 // the first pass's legs (0.5 r_0), and w times the largest radix, the serial
 // instructions of one thread.  Large radices save passes where every SM has
@@ -186,7 +179,7 @@ static bool pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 // results do not depend on the batch it is in.
 LinePlan line_plan(int n, long long sites, bool fp64)
 {
-    static const int first[] = {2, 4, 6, 8, 10, 12, 16}, inner[] = {3, 4, 5, 8, 9}, last[] = {1, 2, 3, 4, 5, 8, 9, 10, 15, 16};
+    static const int first[] = {2, 4, 6, 8, 10, 12}, inner[] = {3, 4, 5, 8, 9}, last[] = {1, 2, 3, 4, 5, 8, 9, 10, 15, 16};
     const double w = fp64 ? (sites <= (1 << 15) ? 2.0 : (sites < (1 << 20) ? 1.0 : 0.3)) : (sites <= (1 << 14) ? 1.0 : 0.3);
     auto cost = [](int r) {
         static const double c[17] = {0, 0, 2, 4, 4, 7.2, 6, 0, 6.5, 9.8, 9.2, 0, 8, 0, 0, 11.2, 10};
@@ -330,7 +323,7 @@ static cudaError_t upload_tables_t(Group &G, cudaStream_t s)
     if ((e = cudaMemcpyAsync(G.ky, ky.data(), ky.size() * sizeof(T), cudaMemcpyHostToDevice, s))) return e;
     if ((e = cudaMemcpyAsync(G.twx_d, twxd.data(), twxd.size() * sizeof(double), cudaMemcpyHostToDevice, s))) return e;
     if ((e = cudaMemcpyAsync(G.twy_d, twyd.data(), twyd.size() * sizeof(double), cudaMemcpyHostToDevice, s))) return e;
-    if (G.twx_full) {
+    if (G.tab8x) {
         const double pi = 3.14159265358979323846;
         auto full = [&](int n) {
             std::vector<float> t(2 * (size_t)n);
@@ -343,8 +336,6 @@ static cudaError_t upload_tables_t(Group &G, cudaStream_t s)
             return t;
         };
         const std::vector<float> fx = full(G.g.nx), fy = full(G.g.ny);
-        if ((e = cudaMemcpyAsync(G.twx_full, fx.data(), fx.size() * sizeof(float), cudaMemcpyHostToDevice, s))) return e;
-        if ((e = cudaMemcpyAsync(G.twy_full, fy.data(), fy.size() * sizeof(float), cudaMemcpyHostToDevice, s))) return e;
         std::vector<float> tx(2 * (size_t)tabs_total(G.g.logx)), ty(2 * (size_t)tabs_total(G.g.logy));
         build_tables_host(G.g.logx, fx.data(), tx.data());
         build_tables_host(G.g.logy, fy.data(), ty.data());
@@ -723,7 +714,7 @@ extern "C" int epd_lb_init(const epd_lb_params *p, int32_t nruns, void *workspac
         if (tune_stream_tiles(G, h->stream) != cudaSuccess) return bail(EPD_LB_ECUDA);
         // cluster grids: when the cluster solve launches; MIXED streaming
         // grids always
-        G.diff = G.hd != nullptr && (G.hc ? G.twx_full != nullptr && cluster_solve_supported(G) : true);
+        G.diff = G.hd != nullptr && (G.hc ? cluster_solve_supported(G) : true);
     }
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return bail(EPD_LB_ECUDA);
     for (size_t gi = 1; gi < h->groups.size(); ++gi) {
@@ -1261,7 +1252,7 @@ extern "C" int epd_lb_tiles(epd_lb *h, int32_t run, int32_t *out)
     if (!out) return EPD_LB_EINVAL;
     if (int rc = locate(h, run, &G, &m)) return rc;
     (void)m;
-    const bool cluster = G->hc && G->twx_full && cluster_solve_supported(*G);
+    const bool cluster = G->hc && cluster_solve_supported(*G);
     out[0] = cluster ? 2 : (G->hist_full ? 1 : 0);
     out[1] = cluster ? cluster_ctas(*G) : 0;
     out[2] = G->colw;

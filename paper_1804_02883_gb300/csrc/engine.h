@@ -69,8 +69,7 @@ struct Group {
     // FP64 fields, [run][species][n]
     double *omega, *omega_t, *phi, *phi_t;
     double *q, *q_t;   // [run][2]
-    double *ia, *ib;   // contour sums of the streaming solves, [run][n]; cluster solve: facp
-    double *ia2, *ib2; // cluster solve: facd, [run][n]
+    double *ia, *ib;   // contour sums of the streaming solves, [run][n]; cluster solve: facp in both
     // differential second solve (MIXED_FP32).  Cluster solve: states of both
     // chains at every node, in the padded row layout
     // [run][chain][ns+1][ny/2][nx + nx/8] float2 (hc: plain / reference
@@ -113,8 +112,7 @@ struct Group {
     // transform tables
     void *twx, *twy, *kx, *ky;     // bulk precision: twiddles, exp(-rg^2 k^2 ds)/N
     double2 *twx_d, *twy_d;        // FP64 twiddles for the EPD/force passes
-    float2 *twx_full, *twy_full;   // FP32 twiddles exp(-2 pi i j/N), j < N (cluster solve); may be null
-    float2 *tab8x = nullptr, *tab8y = nullptr;  // radix-8 pass tables (fft8.cuh layout); null with twx_full
+    float2 *tab8x = nullptr, *tab8y = nullptr;  // radix-8 pass tables (fft8.cuh layout), power-of-two grids
     float2 *tab16x = nullptr, *tab16y = nullptr;  // radix-16 plan tables of 256-point axes (else null)
     int *err;                      // device error word (shared by the handle)
 };

@@ -361,7 +361,7 @@ static EpdK make_k(Group &G)
     return k;
 }
 
-static cudaError_t aux(Group &G, cudaStream_t s)
+cudaError_t launch_aux_convection(Group &G, cudaStream_t s)
 {
     EpdK k = make_k(G);
     k.omega_dst = G.omega_t;
@@ -375,7 +375,7 @@ static cudaError_t aux(Group &G, cudaStream_t s)
     return e ? e : epd_line_col(k, COL_CONVECT, d, s);
 }
 
-static cudaError_t diffusion(Group &G, cudaStream_t s)
+cudaError_t launch_diffusion(Group &G, cudaStream_t s)
 {
     EpdK k = make_k(G);
     k.omega_dst = G.omega;
@@ -389,7 +389,7 @@ static cudaError_t diffusion(Group &G, cudaStream_t s)
     return e ? e : epd_line_col(k, COL_DIFFUSE, d, s);
 }
 
-static cudaError_t force(Group &G, cudaStream_t s)
+cudaError_t launch_force(Group &G, cudaStream_t s)
 {
     EpdK k = make_k(G);
     if (use_r8(G)) {
@@ -469,21 +469,6 @@ cudaError_t launch_convect_phi(Group &G, const double *phi, double *phi_dst, cud
     k.twy = G.twy_d;
     const cudaError_t e = epd_line_row(k, ROW_DIVX, true, s);
     return e ? e : epd_line_col(k, COL_DIVY, true, s);
-}
-
-cudaError_t launch_aux_convection(Group &G, cudaStream_t s)
-{
-    return aux(G, s);
-}
-
-cudaError_t launch_diffusion(Group &G, cudaStream_t s)
-{
-    return diffusion(G, s);
-}
-
-cudaError_t launch_force(Group &G, cudaStream_t s)
-{
-    return force(G, s);
 }
 
 } // namespace epdlb

@@ -335,12 +335,8 @@ template <int LOGN, int LOGB, bool ROW, int NT, bool READ> struct TileDiv<LineTi
 template <class Tile, class F> __device__ __forceinline__ void line_for(const Tile &, int total, F f)
 {
     if constexpr (Tile::fixed) {
-        if (total % Tile::nt == 0) {
 #pragma unroll
-            for (int i = 0; i < total / Tile::nt; ++i) f((int)threadIdx.x + i * Tile::nt);
-        } else if ((int)threadIdx.x < total) {  // fewer butterflies than threads
-            f((int)threadIdx.x);
-        }
+        for (int i = 0; i < total / Tile::nt; ++i) f((int)threadIdx.x + i * Tile::nt);  // one butterfly of the largest radix per thread: whole rounds
     } else {
         for (int bf = threadIdx.x; bf < total; bf += blockDim.x) f(bf);
     }
@@ -615,8 +611,7 @@ template <typename T, bool INV> __device__ __forceinline__ void line_pass_by(int
     case 8: line_pass_call<T, 8, INV>(buf, tl, M, S, tw); break;
     case 9: line_pass_call<T, 9, INV>(buf, tl, M, S, tw); break;
     case 10: line_pass_call<T, 10, INV>(buf, tl, M, S, tw); break;
-    case 12: line_pass_call<T, 12, INV>(buf, tl, M, S, tw); break;
-    default: line_pass_call<T, 16, INV>(buf, tl, M, S, tw); break;
+    default: line_pass_call<T, 12, INV>(buf, tl, M, S, tw); break;
     }
 }
 // FWD: forward transform; then op in digit-reversed order; BWD: inverse.

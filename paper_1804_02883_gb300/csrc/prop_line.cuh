@@ -310,8 +310,7 @@ template <typename T> cudaError_t line_col_t(const PropK<T> &k, cudaStream_t s)
     case 6: return launch_line(k.stateless, prop_col<T, 6>, grid, th, sm, s, k, l);
     case 8: return launch_line(k.stateless, prop_col<T, 8>, grid, th, sm, s, k, l);
     case 10: return launch_line(k.stateless, prop_col<T, 10>, grid, th, sm, s, k, l);
-    case 12: return launch_line(k.stateless, prop_col<T, 12>, grid, th, sm, s, k, l);
-    default: return launch_line(k.stateless, prop_col<T, 16>, grid, th, sm, s, k, l);
+    default: return launch_line(k.stateless, prop_col<T, 12>, grid, th, sm, s, k, l);
     }
 }
 
@@ -335,8 +334,7 @@ template <typename T, bool DIFF> cudaError_t line_row_t(const PropK<T> &k, int m
     case 6: return launch_line(k.stateless, prop_row<T, 6, DIFF>, grid, th, sm, s, k, m, l, w);
     case 8: return launch_line(k.stateless, prop_row<T, 8, DIFF>, grid, th, sm, s, k, m, l, w);
     case 10: return launch_line(k.stateless, prop_row<T, 10, DIFF>, grid, th, sm, s, k, m, l, w);
-    case 12: return launch_line(k.stateless, prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
-    default: return launch_line(k.stateless, prop_row<T, 16, DIFF>, grid, th, sm, s, k, m, l, w);
+    default: return launch_line(k.stateless, prop_row<T, 12, DIFF>, grid, th, sm, s, k, m, l, w);
     }
 }
 

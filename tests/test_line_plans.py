@@ -9,7 +9,9 @@ import paper_1804_02883_gb300 as P
 from test_gpu_line_plans import BOX, MORE
 from test_gpu_lines import GRIDS
 
-FIRST, INNER, LAST = {2, 4, 6, 8, 10, 12}, {3, 4, 5, 8, 9}, {2, 3, 4, 5, 8, 9, 10, 15, 16}
+BOXES = [(2, 8, 8)]  # of test_gpu_solve3d.py
+
+FIRST, INNER, LAST = {2, 4, 6, 8, 10, 12}, {3, 4, 5, 8, 9}, {1, 2, 3, 4, 5, 8, 9, 10, 15, 16}
 
 
 class Plan(ctypes.Structure):
@@ -24,7 +26,7 @@ def plan(n, sites, fp64):
 
 
 def lengths():
-    for n in range(8, 2049, 2):
+    for n in range(2, 2049, 2):  # z axes start at 2, x and y at 8
         m = n
         for p in (2, 3, 5):
             while m % p == 0:
@@ -52,6 +54,7 @@ def test_every_length_has_a_plan_that_a_test_runs(fp64):
             assert p[0] in FIRST and p[-1] in LAST and set(p[1:-1]) <= INNER, (n, sites, p)
             plans.append(p)
     ran = [plan(n, ny * nx, fp64) for ny, nx in GRIDS + MORE for n in (ny, nx)]
+    ran += [plan(n, ny * nx * nz, fp64) for nz, ny, nx in BOXES for n in (nz, ny, nx)]
     if fp64:
         ran += [plan(n, BOX[0] * BOX[1] * BOX[2], fp64) for n in BOX]
     want, got = used(plans), used(ran)
