@@ -645,8 +645,8 @@ __global__ void __launch_bounds__(256) plane_partials(const void *f, long long n
     finish_planes(part, gridDim.y, scale, out, cnt);
 }
 
-// Means of the fields a pass needs, in one launch, grid (4 nb, kRedBlocks)
-// (the planes in x: y ends at 65535):
+// Means of the fields a pass needs, in one launch of 4 nb planes of
+// kRedBlocks blocks (all in x: y ends at 65535):
 // planes 0..2 of a sample the FP64 means of omega; plane 3 the solvent weight,
 // <exp(-omega_S)> (TAN = false) or <e q>, e = exp(-omega0_S), q = expm1(-(omega_S
 // - omega0_S)) (TAN), in FP32 per thread, FP64 beyond.  out: [nb][3] means,
@@ -657,8 +657,8 @@ __global__ void __launch_bounds__(256) field_partials(const double *omega, const
 {
     __shared__ double red[32];
     __shared__ bool last;
-    const int plane = blockIdx.x, b = plane >> 2, c = plane & 3;
-    const long long chunk = (n + kRedBlocks - 1) / kRedBlocks, lo = blockIdx.y * chunk;
+    const int plane = blockIdx.x / kRedBlocks, blk = blockIdx.x % kRedBlocks, b = plane >> 2, c = plane & 3;
+    const long long chunk = (n + kRedBlocks - 1) / kRedBlocks, lo = blk * chunk;
     const long long hi = lo + chunk < n ? lo + chunk : n;
     const double *w = omega + ((size_t)b * 3 + (c < 3 ? c : 2)) * n;
     double s = 0.0;
@@ -676,17 +676,17 @@ __global__ void __launch_bounds__(256) field_partials(const double *omega, const
         s = (double)acc;
     }
     s = block_sum(s, red);
-    if (threadIdx.x == 0) part[(size_t)plane * kRedBlocks + blockIdx.y] = s;
+    if (threadIdx.x == 0) part[(size_t)plane * kRedBlocks + blk] = s;
     __threadfence();  // this block's partial before its arrival
     if (threadIdx.x == 0) {
-        const unsigned total = gridDim.x * gridDim.y;
+        const unsigned total = gridDim.x;
         last = atomicInc(cnt, total - 1) == total - 1;  // wraps to 0 for the next use
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
     const int lane = threadIdx.x & 31;
-    for (int p = threadIdx.x >> 5; p < (int)gridDim.x; p += blockDim.x >> 5) {
+    for (int p = threadIdx.x >> 5; p < (int)gridDim.x / kRedBlocks; p += blockDim.x >> 5) {
         double t = part[(size_t)p * kRedBlocks + lane] + part[(size_t)p * kRedBlocks + 32 + lane];
         for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
         if (lane == 0) ((p & 3) < 3 ? out[(p >> 2) * 3 + (p & 3)] : solvent[p >> 2]) = t * scale;
@@ -1140,7 +1140,7 @@ cudaError_t forward(Work &w, const float *params, const double *omega, double *p
     if ((e = ready_counter(w, s))) return e;
     if (!w.prepacked && (e = pack_all(w, params, false, s))) return e;
     // (the partials in the output's buffer, written later)
-    field_partials<false><<<dim3(4 * w.nb, kRedBlocks), 256, 0, s>>>(omega, nullptr, w.n, (double *)w.y4, 1.0 / (double)w.n, w.means, w.qs, w.cnt);
+    field_partials<false><<<4 * w.nb * kRedBlocks, 256, 0, s>>>(omega, nullptr, w.n, (double *)w.y4, 1.0 / (double)w.n, w.means, w.qs, w.cnt);
     const dim3 px(blocks(w.n), w.nb);
     prep_input<<<px, 256, 0, s>>>(omega, w.means, s_in, w.n, reinterpret_cast<__nv_bfloat16 *>(w.x0));
     if ((e = forward_layers(w, params, s))) return e;
@@ -1159,7 +1159,7 @@ cudaError_t tangent(Work &w, const float *params, const double *omega, const dou
     // <e q> and the partials in the forward pass's output buffer, which is free
     // again; <e> at omega0 is in qs
     double *eq = (double *)w.y4;
-    field_partials<true><<<dim3(4 * w.nb, kRedBlocks), 256, 0, s>>>(omega, omega0, w.n, eq + w.nb, 1.0 / (double)w.n, w.means2, eq, w.cnt);
+    field_partials<true><<<4 * w.nb * kRedBlocks, 256, 0, s>>>(omega, omega0, w.n, eq + w.nb, 1.0 / (double)w.n, w.means2, eq, w.cnt);
     const dim3 px(blocks(w.n), w.nb);
     prep_tangent<<<px, 256, 0, s>>>(omega, omega0, w.means2, w.means, s_in, w.n, reinterpret_cast<__nv_bfloat16 *>(w.t0));
     conv<16, 32, EP_JVP, kD0>(w, w.t0, w.wf[0], nullptr, w.t[0], nullptr, nullptr, 32, s, w.y[0]);
