@@ -4,8 +4,8 @@
 Workload (N = 1 per GPU): four independent 256 x 512 runs (flow along the
 512-site axis), N_s = 64, polymer fraction 0.2, one per reverse-Poiseuille
 amplitude 0, 1e-6, 4e-6, 1.6e-5 f*, seeded +-1e-3 noise (the paper's
-synthetic quench), mixed precision (FP32 propagators and LB, FP64 fields,
-contour sums, Q and EPD transforms).  One step = one coupled EPD/LB time step
+synthetic quench), mixed precision (FP32 propagators, LB and EPD
+transforms, FP64 fields and Q, compensated contour sums).  One step = one coupled EPD/LB time step
 of all four runs: 2 single-chain solves x 2 chains x N_s contour steps plus
 the EPD update, the force and one D2Q9 collide-stream per run.
 
@@ -34,7 +34,7 @@ UNIT = "site·contour-steps/s"
 HBM_FALLBACK = 6800.0
 # FP32 (non-tensor) units of a GB300 at its maximum SM clock
 FP32_SMS, FP32_LANES, FP32_MHZ = 152, 128, 2070.0
-# dram__bytes_read.sum + dram__bytes_write.sum of the 8 prop_chain<9,8,16,256,1,1,0>
+# dram__bytes_read.sum + dram__bytes_write.sum of the 8 prop_chain<9,8,16,256,1,1,0,0>
 # launches of one differential solve of the channel workload (ncu, one capture)
 CHAIN_DIFF_TRAFFIC_BYTES = 363.49e6 + 8.22e6
 
@@ -919,7 +919,7 @@ def main():
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": WORKLOADS[args.workload],
-                       "precision": "mixed (FP32 propagator, LB and EPD transforms; FP64 fields, contour sums, Q)",
+                       "precision": "mixed (FP32 propagator, LB and EPD transforms; FP64 fields and Q; compensated contour sums)",
                        "l2": "flushed (256 MB write) before every timed step", "parallelism": f"replicas x{world}"},
             "lb_mlups": lb_mlups,
             "fp64_plain": fp64,

@@ -60,8 +60,15 @@ enum {
 enum {
     EPD_LB_PLAIN_FP64 = 0,   /* every field and transform in FP64            */
     EPD_LB_MIXED_FP32 = 1    /* propagators, LB populations and the EPD/force
-                                transforms in FP32; fields omega and Phi,
-                                contour sums, Q and masses in FP64.  The
+                                transforms in FP32; fields omega and Phi, Q
+                                and masses in FP64.  Contour sums of the FP32
+                                propagators: FP64 in 3D and in streaming
+                                stateless solves; exact additions in pairs of
+                                FP32 values (good to about 2^-44) in a
+                                handle's streaming solves and in resident
+                                stateless ones; compensated FP32, with FP64
+                                totals, in a handle's resident solves and of
+                                the changes of the second solve.  The
                                 step's second solve is computed as its
                                 difference from the first (same result up to
                                 rounding, FP32 relative to the change that

@@ -15,7 +15,7 @@
 // with E = exp(-N w ds / 2).  The history holds nodes 0..floor(N_s/2): while
 // the chains run through the second half, node m of g meets node N_s - m of g'
 // from the history (and vice versa), and the trapezoid sums of Eqs. (9)-(10)
-// are accumulated in FP64 on the fly.  In MIXED_FP32 every node is stored:
+// are accumulated in FP64 on the fly.  A MIXED_FP32 handle stores every node:
 // the full history is the reference of the differential second solve, and the
 // contour sums are a separate pass over the stored nodes (prop_contour_stream).
 // The column and row passes are in prop_line.cuh (every grid, both precisions)

@@ -1078,7 +1078,7 @@ cudaError_t launch_cluster_solve(Group &G, cudaStream_t s, bool diff, int nprep_
     }
     void *args[] = {&k};
     // launches after the first of a phased schedule are programmatic
-    // dependents of the one before: their prologue (tables, node factors)
+    // dependents of the one before: their prologue (tables, barriers)
     // overlaps its end; they wait for it before reading the stored states
     cudaLaunchAttribute attrs[2] = {attr, {}};
     attrs[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;

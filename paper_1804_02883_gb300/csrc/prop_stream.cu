@@ -9,8 +9,8 @@
 // barriers (ten and nine as load, Stockham passes and store).  Radix 32 would
 // save two more of each but holds 168-250 registers: 512 x 512 (9 runs, N_s =
 // 24) 2.27 ms a step with 32.16, 2.14 with 8.8.8.  1024 x 2048, N_s = 128:
-// 8.8 -> 7.7 ms a step; per launch (cold, serialised) column 19.9 -> 15.5 us
-// (2.2 TB/s), differential row 23.5 -> 19.3 us (5.2 TB/s), plain row 17.9 -> 20.2 us
+// 8.8 -> 7.6 ms a step; per launch (cold, serialised) column 19.9 -> 15.6 us
+// (2.2 TB/s), differential row 23.5 -> 19.4 us (5.2 TB/s), plain row 17.9 -> 20.6 us
 // (in digit-reversed order both transforms of a pair read twiddles; the pair of
 // passes is what gains).
 //
