@@ -62,6 +62,18 @@ __host__ __device__ inline double ulp(double v)
     return v * 2.220446049250313e-16;
 }
 
+// a b rounded, never fused with what follows (by the compiler of either side)
+template <typename T> __host__ __device__ inline T mul_rounded(T a, T b)
+{
+#ifdef __CUDA_ARCH__
+    if constexpr (sizeof(T) == 4) return __fmul_rn(a, b);
+    else return __dmul_rn(a, b);
+#else
+    volatile T p = a * b;
+    return p;
+#endif
+}
+
 // The pair next to (c, s) = (cos, -sin) in T's numbers that is nearest to the
 // unit circle.  A forward and an inverse pass multiply by w and conj(w), so over a
 // contour every step adds the same |w|^2 - 1 at the same points; of the rounded
@@ -77,10 +89,9 @@ template <typename T> __host__ __device__ inline V2<T> unit_pair(double c, doubl
     best.x = c0;
     best.y = s0;
     if (c0 == (T)0 || s0 == (T)0) return best;
-    // c0^2 + s0^2 - 1, the products exact by FMA, the larger minus one first
-    const double p = (double)c0 * (double)c0, q = (double)s0 * (double)s0;
-    const double low = fma((double)c0, (double)c0, -p) + fma((double)s0, (double)s0, -q);
-    const T m0 = (T)((p > q ? (p - 1.0) + q : (q - 1.0) + p) + low);
+    // c0^2 + s0^2 - 1, the products exact by FMA, the larger minus one first (exact)
+    const T p = mul_rounded(c0, c0), q = mul_rounded(s0, s0), low = fma(c0, c0, -p) + fma(s0, s0, -q);
+    const T m0 = (p > q ? (p - (T)1) + q : (q - (T)1) + p) + low;
     const T uc = ulp(c0), us = ulp(s0);
     const T ec = (T)((double)c0 - c), es = (T)((double)s0 - s);
     T least = (T)1;
